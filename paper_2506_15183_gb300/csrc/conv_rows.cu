@@ -1,0 +1,476 @@
+// 3x3 convolution of the inpainter's wide, shallow layers (32 or 64 output channels on tiles
+// 32, 64 or 128 pixels wide) on the tensor cores: the row form.
+//
+// What bounds these layers: one tcgen05.mma of M = 128 pixels x N = Cout x K = 16 reads its
+// A tile (4 KB) and its weights (Cout x 32 bytes) from shared memory at 128 bytes per
+// cycle, and one thread issues at most one MMA per ~55 cycles (measured), so at N = 32 the
+// tensor core does 16 cycles of work per 55.  The three taps of a kernel column share
+// their input, so here they share the MMA: M is one image row (128 / W images side by
+// side, so the lanes of an accumulator are the same pixels of every row), the accumulators
+// of R rows lie next to each other in tensor memory, and input row r is multiplied once
+// with the weights of taps dy = 2, 1, 0 (N = 3 Cout) into the accumulators of rows r - 1, r,
+// r + 1: 56 cycles where three MMAs took 164 (N = 96), 96 where they took 164 (N = 192).
+//
+// The kernel columns share the copy of a row as well: tap dx reads the same shared-memory
+// row from a start one pixel (64 bytes) to the left or right (the swizzle is a function
+// of the shared-memory address, so any pixel start reads what the copy engine wrote), and
+// the lanes whose neighbour lies outside the image (x = 0 for dx = 0, x = W - 1 for dx = 2)
+// are left out by the MMA's lane mask, which is the convolution's zero padding.  A row is
+// copied once per 32 channels, (R + 2) / R times in all, instead of three times that.
+//
+// Per output element the products are accumulated in the order (channel block, dx, dy,
+// K half) of conv3x3_halo, so both forms give the same bits.
+//
+// One CTA per SM walks units of (image group, R rows).  Warp 0 streams rows (8 KB each) and
+// weights, warp 1 issues the MMAs, warps 2-5 read back one of two accumulator sets (256
+// columns each) while the other is being filled, zero it for its next use, and store: each
+// warp stages its 32 pixels of two rows and writes them with its own TMA store.  Where the
+// next level follows, the 2x2 maximum of the rows a warp holds goes to the pooled tensor
+// in the same pass.
+//
+// The issuing warp runs its loop as a whole (one lane elected per instruction): in uniform
+// control flow the descriptors are built in uniform registers, where a single-lane branch
+// cost about 100 more cycles per MMA (dec0a below 337 us).
+//
+// Measured, 870 tiles, halo form -> row form, us: enc0a 143 -> 83, enc0b 144 -> 106, enc1a 51
+// -> 34, enc1b 78 -> 50, dec1a 166 -> 129, dec1b 141 -> 118, dec0a 305 -> 174, dec0b 152 -> 83
+// (dec0b moves 456 MB: 67 us at the measured copy bandwidth).
+#include <algorithm>
+#include <cmath>
+
+#include "tc.cuh"
+#include "unet_internal.h"
+
+namespace yoro {
+
+namespace {
+
+__device__ unsigned g_rows_status;  // waits that ran out in this file's kernel
+
+constexpr int kRowBytes = kTileM * kKc * 2;     // one row of 128 pixels x 32 channels
+constexpr int kAccCols = 256;                   // tensor-memory columns of an accumulator set
+constexpr int kMaxRows = 24;                    // row slots (bounds the barrier array)
+constexpr int kStageBytes = 2 * 32 * kKc * 2;   // a warp's 32 pixels of two rows, 32 channels
+constexpr int kStores = 4 * 2 * kStageBytes;    // two staging buffers for each of four warps
+constexpr int kRowsThreads = 192;
+
+struct RowsArgs {
+    int T, H, W, Cin;
+    int nrows;         // row slots
+    int wslots;        // weight slots (9 taps of one channel block each); resident when wslots == Cin / 32
+    int y_coff, upsample, relu;
+    const float* bias;
+    const int* count;  // optional: tiles at or after *count are skipped
+    uint16_t* pool;    // optional: T x H/2 x W/2 x Cout, the 2x2 maximum of the output
+};
+
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b)
+{
+    const __nv_bfloat162 m =
+        __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+    return *reinterpret_cast<const uint32_t*>(&m);
+}
+
+// One 32-channel slice of one pixel: bias, ReLU, rounding to bfloat16.
+__device__ __forceinline__ void finish(const uint32_t (&r)[32], const float* bias, int relu, uint32_t (&q)[16])
+{
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        float v0 = __fadd_rn(__uint_as_float(r[2 * i]), bias[2 * i]);
+        float v1 = __fadd_rn(__uint_as_float(r[2 * i + 1]), bias[2 * i + 1]);
+        if (relu) {
+            v0 = fmaxf(v0, 0.0f);
+            v1 = fmaxf(v1, 0.0f);
+        }
+        q[i] = pack_bf16x2(v0, v1);
+    }
+}
+
+template <int COUT, int R>
+__global__ void __launch_bounds__(kRowsThreads, 1)
+    conv3x3_rows(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                 const __grid_constant__ CUtensorMap tmY, const RowsArgs a)
+{
+    extern __shared__ unsigned char smem_raw[];
+    const int W = a.W, H = a.H, NR = a.nrows, WS = a.wslots;
+    const int nimg = kTileM / W, bands = H / R;
+    const int cb_n = a.Cin / kKc;
+    const int tiles = a.count ? min(a.T, *a.count) : a.T;
+    const int units = (tiles + nimg - 1) / nimg * bands;
+    if ((int)blockIdx.x >= units) return;  // uniform
+
+    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                                           ~static_cast<uintptr_t>(1023));
+    // 1 KB of barriers first: the row before slot 0 that a dx = 0 operand starts 64 bytes into
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem);
+    uint64_t* empty = full + kMaxRows;
+    uint64_t* wfull = empty + kMaxRows;
+    uint64_t* wempty = wfull + 4;
+    uint64_t* afull = wempty + 4;
+    uint64_t* aempty = afull + 2;
+    uint64_t* drain = aempty + 2;
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
+    float* sbias = reinterpret_cast<float*>(smem + 512);  // COUT floats
+    unsigned char* rows = smem + 1024;
+    constexpr int kWBytes = 9 * COUT * kKc * 2;
+    unsigned char* wts = rows + NR * kRowBytes;
+    unsigned char* stage = wts + WS * kWBytes;
+    const bool resident = WS == cb_n;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < NR; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int s = 0; s < WS && s < 4; ++s) {
+            mbar_init(&wfull[s], 1);
+            mbar_init(&wempty[s], 1);
+        }
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(&afull[s], 1);
+            mbar_init(&aempty[s], 4);
+        }
+        mbar_init(drain, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                     "r"(2 * kAccCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    for (int c = threadIdx.x; c < COUT; c += kRowsThreads) sbias[c] = __ldg(a.bias + c);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tslot;
+
+    auto timed_out = [&]() {
+        atomicOr(&g_rows_status, kUnetTimeout);
+        *abort_flag = 1;
+    };
+    int issued = 0, wissued = 0;  // rows and weight slots that thread 0 has copied
+
+    if (warp == 0) {
+        if (lane == 0) {  // copies
+            int slot = 0, ph = 1, ws = 0, wph = 1;
+            bool ok = true;
+            for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+                const int g = u / bands, y0 = (u - g * bands) * R;
+                const uint64_t deadline = globaltimer() + kWaitNs;
+                for (int cb = 0; cb < cb_n && ok; ++cb) {
+                    if (!resident || u == (int)blockIdx.x) {
+                        if (!(ok = mbar_wait(&wempty[ws], wph, deadline))) break;
+                        unsigned char* dst = wts + ws * kWBytes;
+                        mbar_expect_tx(&wfull[ws], kWBytes);
+                        for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                            for (int j = 0; j < 3; ++j)  // blocks of a kernel column: taps dy = 2, 1, 0
+                                tma_load_2d(dst + (dx * 3 + j) * COUT * kKc * 2, &tmB, &wfull[ws],
+                                            (3 * (2 - j) + dx) * a.Cin + cb * kKc, 0);
+                        ++wissued;
+                        if (++ws == WS) {
+                            ws = 0;
+                            wph ^= 1;
+                        }
+                    }
+                    for (int r = -1; r <= R; ++r) {
+                        const int y = y0 + r;
+                        if (y < 0 || y >= H) continue;  // zero padding: the row is left out
+                        if (!(ok = mbar_wait(&empty[slot], ph, deadline))) break;
+                        mbar_expect_tx(&full[slot], kRowBytes);
+                        tma_load_4d(rows + slot * kRowBytes, &tmA, &full[slot], cb * kKc, 0, g * nimg, y);
+                        ++issued;
+                        if (++slot == NR) {
+                            slot = 0;
+                            ph ^= 1;
+                        }
+                    }
+                }
+            }
+            if (!ok) timed_out();
+        }
+    } else if (warp == 1) {  // MMAs: the whole warp runs the loop, one lane issues
+        constexpr uint32_t id1 = idesc_bf16(COUT), id2 = idesc_bf16(2 * COUT), id3 = idesc_bf16(3 * COUT);
+        const uint32_t el = elect_one();
+        const uint64_t drow = desc_sw64(smem_u32(rows));
+        const uint64_t dw = desc_sw64(smem_u32(wts));
+        // lanes x = 0 and x = W - 1 of each image
+        const uint32_t lo2 = W == 128 ? 0u : 1u, lo13 = W == 32 ? 1u : 0u;
+        const uint32_t hi3 = 0x80000000u, hi1 = W == 128 ? 0u : hi3, hi02 = W == 32 ? hi3 : 0u;
+        int slot0 = 0, ph0 = 0, ws = 0, wph = 0;
+        bool ok = true;
+        int it = 0;
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++it) {
+            const int g = u / bands, y0 = (u - g * bands) * R;
+            const bool top = y0 == 0, bottom = y0 + R == H;  // row -1 or R lies outside the image
+            const uint32_t acc = tmem + (uint32_t)((it & 1) * kAccCols);
+            const uint64_t deadline = globaltimer() + kWaitNs;
+            if (!(ok = mbar_wait_warp(&aempty[it & 1], (it >> 1) & 1, deadline))) break;
+            tc_fence_after();
+            for (int cb = 0; cb < cb_n && ok; ++cb) {
+                if (resident) ws = cb;
+                if (!resident || it == 0)
+                    if (!(ok = mbar_wait_warp(&wfull[ws], wph, deadline))) break;
+                int slot = slot0, ph = ph0;
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx) {
+                    const uint32_t m0 = dx == 0 ? 1u : dx == 2 ? hi02 : 0u;
+                    const uint32_t m1 = dx == 0 ? lo13 : dx == 2 ? hi1 : 0u;
+                    const uint32_t m2 = dx == 0 ? lo2 : dx == 2 ? hi02 : 0u;
+                    const uint32_t m3 = dx == 0 ? lo13 : dx == 2 ? hi3 : 0u;
+                    const uint64_t wb = dw + (uint64_t)((uint32_t)(ws * kWBytes + dx * 3 * COUT * kKc * 2) >> 4);
+                    slot = slot0;
+                    ph = ph0;
+#pragma unroll
+                    for (int r = -1; r <= R; ++r) {
+                        if ((r == -1 && top) || (r == R && bottom)) continue;
+                        if (dx == 0) {
+                            ok = ok && mbar_wait_warp(&full[slot], ph, deadline);
+                            tc_fence_after();
+                        }
+                        if (ok) {
+                            // output rows r - 1 .. r + 1 inside the unit
+                            const int lo = r < 1 ? 0 : r - 1, hi = r + 1 > R - 1 ? R - 1 : r + 1, n = hi - lo + 1;
+                            const uint32_t id = n == 3 ? id3 : n == 2 ? id2 : id1;
+                            const uint64_t da =
+                                drow + (uint64_t)((uint32_t)slot * (uint32_t)(kRowBytes >> 4) + (uint32_t)(4 * dx)) - 4;
+                            const uint64_t db = wb + (uint64_t)((lo - (r - 1)) * (COUT * kKc * 2 >> 4));
+                            const uint32_t d = acc + (uint32_t)(lo * COUT);
+                            mma_bf16_masked(el, d, da, db, id, m0, m1, m2, m3);
+                            mma_bf16_masked(el, d, da + 2, db + 2, id, m0, m1, m2, m3);
+                            if (dx == 2) mma_commit_elected(el, &empty[slot]);
+                        }
+                        if (++slot == NR) {
+                            slot = 0;
+                            ph ^= 1;
+                        }
+                    }
+                }
+                slot0 = slot;
+                ph0 = ph;
+                if (!resident) {
+                    if (ok) mma_commit_elected(el, &wempty[ws]);
+                    if (++ws == WS) {
+                        ws = 0;
+                        wph ^= 1;
+                    }
+                }
+            }
+            if (ok) mma_commit_elected(el, &afull[it & 1]);
+        }
+        if (!ok) {  // the MMAs issued so far: wait for them (bounded)
+            if (el) timed_out();
+            mma_commit_elected(el, drain);
+            mbar_wait_warp(drain, 0, globaltimer() + kWaitNs);
+        }
+    } else {  // read back, store
+        const int q = warp & 3;  // this warp's quarter of the tensor-memory lanes
+        const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
+        for (int c = 0; c < 2 * kAccCols; c += 32) tmem_zero32_async(tq + c);
+        tmem_wait_st();
+        tc_fence_before();
+        if (lane == 0) {
+            mbar_arrive(&aempty[0]);
+            mbar_arrive(&aempty[1]);
+        }
+        unsigned char* st = stage + (warp - 2) * 2 * kStageBytes;
+        const int img = W == 32 ? q : W == 64 ? q >> 1 : 0;           // image of the group
+        const int x0 = W == 32 ? 0 : W == 64 ? (q & 1) * 32 : q * 32;  // first pixel of the row
+        int it = 0, nst = 0;
+        for (int u = blockIdx.x; u < units; u += gridDim.x, ++it) {
+            const int g = u / bands, y0 = (u - g * bands) * R;
+            const int n = g * nimg + img;
+            const uint32_t acc = tq + (uint32_t)((it & 1) * kAccCols);
+            bool ok = mbar_wait(&afull[it & 1], (it >> 1) & 1, globaltimer() + 2 * kWaitNs);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok || *abort_flag) {
+                if (!ok && lane == 0) timed_out();
+                break;
+            }
+            __syncwarp();
+            tc_fence_after();
+            for (int rr = 0; rr < R; rr += 2) {
+#pragma unroll
+                for (int c0 = 0; c0 < COUT; c0 += 32) {
+                    uint32_t v0[32], v1[32];
+                    const uint32_t t0 = acc + (uint32_t)(rr * COUT + c0), t1 = t0 + COUT;
+                    tmem_ld32_async(t0, v0);
+                    tmem_ld32_async(t1, v1);
+                    tmem_wait_ld();
+                    tmem_zero32_async(t0);
+                    tmem_zero32_async(t1);
+                    uint32_t p0[16], p1[16];
+                    finish(v0, sbias + c0, a.relu, p0);
+                    finish(v1, sbias + c0, a.relu, p1);
+                    // a staging buffer is free once the store issued from it two slices ago has read it
+                    unsigned char* sb = st + (nst & 1) * kStageBytes;
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                    __syncwarp();
+                    const int sw = (lane >> 1) & 3;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        *reinterpret_cast<uint4*>(sb + lane * 64 + ((k ^ sw) << 4)) =
+                            make_uint4(p0[4 * k], p0[4 * k + 1], p0[4 * k + 2], p0[4 * k + 3]);
+                        *reinterpret_cast<uint4*>(sb + 2048 + lane * 64 + ((k ^ sw) << 4)) =
+                            make_uint4(p1[4 * k], p1[4 * k + 1], p1[4 * k + 2], p1[4 * k + 3]);
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (n < a.T) {
+                            if (!a.upsample) {
+                                tma_store_4d(&tmY, sb, a.y_coff + c0, x0, n, y0 + rr);
+                            } else {
+#pragma unroll
+                                for (int ab = 0; ab < 4; ++ab)
+                                    tma_store_5d(&tmY, sb, a.y_coff + c0, ab & 1, x0, ab >> 1, n * H + y0 + rr);
+                            }
+                        }
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    }
+                    ++nst;
+                    if (a.pool) {  // 2x2 maximum: the two rows, then the neighbouring pixel
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            const uint32_t m = max_bf16x2(p0[i], p1[i]);
+                            p0[i] = max_bf16x2(m, __shfl_xor_sync(0xffffffffu, m, 1));
+                        }
+                        if (n < a.T) {  // lanes 2i and 2i + 1 write 16 bytes of each 32 of pooled pixel i
+                            const size_t px = ((size_t)n * (H / 2) + ((y0 + rr) >> 1)) * (W / 2) + ((x0 + lane) >> 1);
+                            uint4* dst = reinterpret_cast<uint4*>(a.pool + px * COUT + c0) + (lane & 1);
+#pragma unroll
+                            for (int k = 0; k < 2; ++k)
+                                dst[2 * k] = (lane & 1) ? make_uint4(p0[8 * k + 4], p0[8 * k + 5], p0[8 * k + 6], p0[8 * k + 7])
+                                                        : make_uint4(p0[8 * k], p0[8 * k + 1], p0[8 * k + 2], p0[8 * k + 3]);
+                        }
+                    }
+                }
+            }
+            tmem_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&aempty[it & 1]);
+        }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x == 0 && *abort_flag) {  // copies still in flight after a timeout: wait for them (bounded)
+        const uint64_t d = globaltimer() + kWaitNs;
+        for (int i = max(0, issued - NR); i < issued; ++i) mbar_wait(&full[i % NR], (i / NR) & 1, d);
+        for (int i = max(0, wissued - WS); i < wissued; ++i) mbar_wait(&wfull[i % WS], (i / WS) & 1, d);
+    }
+    __syncthreads();
+    if (warp == 1) {  // the allocating warp frees
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kAccCols) : "memory");
+    }
+}
+
+size_t rows_smem(int nrows, int wslots, int cout)
+{
+    return 2048 + (size_t)nrows * kRowBytes + (size_t)wslots * 9 * cout * kKc * 2 + kStores;
+}
+
+}  // namespace
+
+// 16-pixel rows and 128 channels stay with the halo form: at N = 128 an MMA already does 64
+// cycles of work for 64 of operand reads, so sharing it between taps gains nothing.  The
+// form wins at every tile count measured (T = 64: dec0a 33.9 -> 25.0 us, enc0b 18.8 -> 14.9;
+// at T = 2 and 8 both are bound by the call, 11-12 us).
+bool conv_rows_takes(int H, int W, int Cout)
+{
+    return (W == 32 || W == 64 || W == 128) && (Cout == 32 || Cout == 64) && H % 2 == 0;
+}
+
+cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStream_t stream)
+{
+    EncodeTiled enc = tensor_map_encoder();
+    if (!enc) return cudaErrorNotSupported;
+    const int nimg = kTileM / c.W, groups = (c.T + nimg - 1) / nimg;
+    RowsArgs a;
+    a.T = c.T;
+    a.H = c.H;
+    a.W = c.W;
+    a.Cin = c.Cin;
+    // rows of a unit: an accumulator set's 256 columns, fewer while that leaves SMs without a unit
+    int R = kAccCols / c.Cout;
+    while (c.H % R) R /= 2;
+    while (R > 2 && groups * (c.H / R) < sms) R /= 2;
+    const int cb_n = c.Cin / kKc;
+    a.wslots = cb_n <= 3 && 9 * c.Cin * c.Cout * 2 <= 80 * 1024 ? cb_n : 2;
+    a.nrows = std::min(kMaxRows, (int)((smem_max - (int)rows_smem(0, a.wslots, c.Cout)) / kRowBytes));
+    if (a.nrows < R + 2) return cudaErrorInvalidValue;
+    a.y_coff = c.y_coff;
+    a.upsample = c.upsample;
+    a.relu = c.relu;
+    a.bias = c.bias;
+    a.count = c.count;
+    a.pool = static_cast<uint16_t*>(c.pool);
+
+    CUtensorMap ta, tb, ty;
+    const cuuint32_t one[5] = {1, 1, 1, 1, 1};
+    // {channel, x, image, y}: a box of one row of nimg images is 128 consecutive pixels
+    const cuuint64_t ci = (cuuint64_t)c.Cin, W = (cuuint64_t)c.W, H = (cuuint64_t)c.H, T = (cuuint64_t)c.T;
+    const cuuint64_t ad[4] = {ci, W, T, H};
+    const cuuint64_t as[3] = {ci * 2, H * W * ci * 2, W * ci * 2};
+    const cuuint32_t abox[4] = {(cuuint32_t)kKc, (cuuint32_t)c.W, (cuuint32_t)nimg, 1};
+    if (enc(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(c.x), ad, as, abox, one,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    const cuuint64_t bd[2] = {9 * ci, (cuuint64_t)c.Cout};
+    const cuuint64_t bs[1] = {9 * ci * 2};
+    const cuuint32_t bbox[2] = {(cuuint32_t)kKc, (cuuint32_t)c.Cout};
+    if (enc(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(c.wk), bd, bs, bbox, one,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    // a store's box: 32 channels x 32 pixels x two rows of one image
+    const cuuint64_t cs = (cuuint64_t)c.y_cstride;
+    CUresult r;
+    if (!c.upsample) {
+        const cuuint64_t d[4] = {cs, W, T, H};
+        const cuuint64_t s[3] = {cs * 2, H * W * cs * 2, W * cs * 2};
+        const cuuint32_t box[4] = {(cuuint32_t)kKc, 32, 1, 2};
+        r = enc(&ty, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, c.y, d, s, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    } else {  // {channel, b, x, a, n H + y}: pixel (2y + a, 2x + b)
+        const cuuint64_t d[5] = {cs, 2, W, 2, T * H};
+        const cuuint64_t s[4] = {cs * 2, 2 * cs * 2, 2 * W * cs * 2, 4 * W * cs * 2};
+        const cuuint32_t box[5] = {(cuuint32_t)kKc, 1, 32, 1, 2};
+        r = enc(&ty, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, c.y, d, s, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    }
+    if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+
+    const size_t smem = rows_smem(a.nrows, a.wslots, c.Cout);
+    const int grid = std::min(groups * (c.H / R), sms);
+    auto go = [&](auto kernel) -> cudaError_t {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+        if (e != cudaSuccess) return e;
+        kernel<<<grid, kRowsThreads, smem, stream>>>(ta, tb, ty, a);
+        return cudaGetLastError();
+    };
+    if (c.Cout == 64) return R == 4 ? go(conv3x3_rows<64, 4>) : go(conv3x3_rows<64, 2>);
+    return R == 8 ? go(conv3x3_rows<32, 8>) : R == 4 ? go(conv3x3_rows<32, 4>) : go(conv3x3_rows<32, 2>);
+}
+
+unsigned conv_rows_status_take()
+{
+    unsigned v = 0, z = 0;
+    if (cudaMemcpyFromSymbol(&v, g_rows_status, sizeof v) != cudaSuccess ||
+        cudaMemcpyToSymbol(g_rows_status, &z, sizeof z) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return v;
+}
+
+}  // namespace yoro

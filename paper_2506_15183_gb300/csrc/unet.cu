@@ -11,8 +11,10 @@
 // the accumulators with tcgen05.ld, adds the bias, applies ReLU, rounds to BF16 and
 // stores NHWC at a channel offset of a wider buffer (so a decoder's concatenation is
 // written in place), or, for the layer below a decoder level, to the 2 x 2 pixels of the
-// nearest upsampling.  Two forms:
-//   - conv3x3_halo, for tiles of whole rows of one image: a band of 256 / W rows goes
+// nearest upsampling.  Three forms:
+//   - conv3x3_rows (conv_rows.cu), for 32 or 64 output channels on tiles 32 to 128 pixels
+//     wide: one image row per accumulator, the three taps of a kernel column in one MMA.
+//   - conv3x3_halo, for the other tiles of whole rows of one image: a band of 256 / W rows goes
 //     into two accumulators (each CTA walks bands blockIdx.x, + gridDim.x, ..., as many
 //     CTAs as fit on the SMs at once); a K step is one (channel block, dx) pair, a single box of
 //     the rows plus one above and below, shared by the three dy taps through the start
@@ -22,7 +24,7 @@
 //     tiles, and 256 output channels): a K step is one (channel block, tap), the
 //     activation box {32 channels, W, rows, tiles} at the tap's offset and the weight box
 //     {32, Cout} of the K-major weights (k = tap * Cin + ci), in a 4-stage ring.
-// Both use CTAs of 128 threads, several per SM, so the copies of one overlap the set-up,
+// The last two use CTAs of 128 threads, several per SM, so the copies of one overlap the set-up,
 // MMAs and epilogue of the others.
 //
 // Every wait on an mbarrier has a deadline (1 s of %globaltimer): a wait that runs out
@@ -39,10 +41,11 @@
 #include <new>
 #include <vector>
 
+#include "tc.cuh"
+#include "unet_internal.h"
 #include "yoro.h"
 #include "yoro_internal.h"
 #include "yoro_unet.h"
-#include "unet_internal.h"
 
 namespace yoro {
 
@@ -50,151 +53,8 @@ namespace {
 
 __device__ unsigned g_unet_status;  // kernel-side failures of this file's kernels
 
-constexpr unsigned kUnetTimeout = 1u;
 constexpr int kStages = 4;
-constexpr int kTileM = 128;                  // pixels per CTA tile (MMA M)
-constexpr int kKc = 32;                      // channels per K step (64 bytes: the swizzle span)
-constexpr int kABytes = kTileM * kKc * 2;    // 8 KB
-constexpr uint64_t kWaitNs = 1000000000ull;  // 1 s
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ uint64_t globaltimer()
-{
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Wait for the phase of parity `parity` to complete; false if `deadline` passed first.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64_t deadline)
-{
-    while (!mbar_try_wait(bar, parity))
-        if (globaltimer() > deadline) return false;
-    return true;
-}
-
-__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1, int c2,
-                                            int c3)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], "
-        "[%2];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-        : "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
-            smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1)
-        : "memory");
-}
-
-// TMA tensor stores from shared memory (bulk-group completion): 4-D and 5-D boxes.
-__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, const void* src, int c0, int c1, int c2, int c3)
-{
-    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(
-                     reinterpret_cast<uint64_t>(map)),
-                 "r"(smem_u32(src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-                 : "memory");
-}
-
-__device__ __forceinline__ void tma_store_5d(const CUtensorMap* map, const void* src, int c0, int c1, int c2, int c3,
-                                             int c4)
-{
-    asm volatile("cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5, %6}], [%1];" ::"l"(
-                     reinterpret_cast<uint64_t>(map)),
-                 "r"(smem_u32(src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
-                 : "memory");
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Shared-memory matrix descriptor of a K-major operand whose rows (one M or N index
-// each) are 64 bytes of K, 64-byte swizzled by the copy engine: 8-row groups 512 bytes
-// apart (stride byte offset), leading byte offset unused for a swizzled K-major layout,
-// descriptor version 1, layout type 4 (64-byte swizzle).  The start address may move
-// by 32 bytes inside the swizzle span to select the second K = 16 half.
-__device__ __forceinline__ uint64_t desc_sw64(uint32_t saddr)
-{
-    uint64_t d = (uint64_t)((saddr >> 4) & 0x3fffu);
-    d |= (uint64_t)1u << 16;
-    d |= (uint64_t)(512u >> 4) << 32;
-    d |= (uint64_t)1u << 46;
-    d |= (uint64_t)4u << 61;
-    return d;
-}
-
-// Instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), BF16 A and B
-// (bits 7-9 and 10-12 = 1), both K-major, N / 8 at bit 17, M / 16 at bit 24.
-__device__ __forceinline__ uint32_t idesc_bf16(int n)
-{
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(accum)
-        : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t* bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-
-// 32 consecutive accumulator columns of this warp's 32 TMEM lanes (one lane per thread).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
-{
-    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t*>(&v);
-}
+constexpr int kABytes = kTileM * kKc * 2;  // 8 KB
 
 struct ConvArgs {
     int T, H, W;          // tiles and their size (the output has the input's size)
@@ -552,13 +412,9 @@ __global__ void __launch_bounds__(128, 1)
     }
 }
 
-// Driver entry point for tensor-map encoding, looked up once through the runtime (no
-// link against the driver library).
-using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+}  // namespace
 
-EncodeTiled encode_fn()
+EncodeTiled tensor_map_encoder()
 {
     static EncodeTiled fn = nullptr;
     if (!fn) {
@@ -572,6 +428,8 @@ EncodeTiled encode_fn()
     }
     return fn;
 }
+
+namespace {
 
 size_t conv_smem_bytes(int cout)
 {
@@ -626,7 +484,7 @@ unsigned unet_status_take()
         cudaGetLastError();
         return 0;
     }
-    return v;
+    return v | conv_rows_status_take();
 }
 
 // One 3x3 convolution (zero padding 1) of x (T tiles of H x W, NHWC bf16 with Cin
@@ -635,6 +493,7 @@ unsigned unet_status_take()
 // y_cstride channels (upsample: into the 2H x 2W grid of the nearest upsampling).
 // Shared memory of one SM (228 KB) and the SM count of the current device.
 constexpr size_t kSmemPerSm = 228 * 1024;
+constexpr int kSmemPerBlock = 227 * 1024;  // the most one CTA can take
 
 int sm_count()
 {
@@ -673,7 +532,7 @@ cudaError_t unet_conv3x3(const void* x, int T, int H, int W, int Cin, const void
     if (pixels % kTileM || (nb > 1 && T % nb)) return cudaErrorInvalidValue;
     if (y_cstride % 8 || y_coff % 8 || y_coff + Cout > y_cstride) return cudaErrorInvalidValue;
     if (reinterpret_cast<uintptr_t>(y) % 16) return cudaErrorInvalidValue;  // a TMA store's base
-    EncodeTiled enc = encode_fn();
+    EncodeTiled enc = tensor_map_encoder();
     if (!enc) return cudaErrorNotSupported;
 
     CUtensorMap ta, tb;
@@ -733,6 +592,10 @@ cudaError_t unet_conv3x3(const void* x, int T, int H, int W, int Cin, const void
     a.stages = kStages;
     int mt = 0, stages = 0;
     if (nb == 1) halo_shape(H, W, Cout, &mt, &stages);
+    if (mt && conv_rows_takes(H, W, Cout))
+        return conv_rows_launch(ConvCall{x, wk, y, bias, count, nullptr, T, H, W, Cin, Cout, y_cstride, y_coff, upsample,
+                                         relu},
+                                sm_count(), kSmemPerBlock, stream);
     if (mt) {
         const int rows = mt * kTileM / W;
         CUtensorMap th;

@@ -1,6 +1,7 @@
 // Internal interface of the learned inpainter (unet.cu, unet_train.cu).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cstddef>
@@ -25,6 +26,31 @@ struct UnetNet {
     int *flags, *list, *count;
     int max_grid_tiles;  // capacity of flags / list
 };
+
+// Driver entry point for tensor-map encoding, looked up once through the runtime (no link
+// against the driver library); nullptr if it is missing.
+using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiled tensor_map_encoder();
+
+// One 3x3 convolution (the arguments of unet_conv3x3) with an optional 2x2-pooled copy of
+// its output, T x H/2 x W/2 x Cout.
+struct ConvCall {
+    const void* x;
+    const void* wk;
+    void* y;
+    const float* bias;
+    const int* count;
+    void* pool;
+    int T, H, W, Cin, Cout, y_cstride, y_coff, upsample, relu;
+};
+
+// conv_rows.cu: the row form of the convolution.  conv_rows_takes(): whether a shape that
+// the halo form accepts can run as rows.
+bool conv_rows_takes(int H, int W, int Cout);
+cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStream_t stream);
+unsigned conv_rows_status_take();
 
 size_t unet_param_count();
 void unet_layer_dims(int i, int* cin, int* cout);
