@@ -39,6 +39,7 @@
 #include <cmath>
 
 #include "tc.cuh"
+#include "unet_device.cuh"
 #include "unet_internal.h"
 
 namespace yoro {
@@ -49,7 +50,7 @@ __device__ unsigned g_rows_status;  // waits that ran out in this file's kernel
 
 constexpr int kRowBytes = kTileM * kKc * 2;     // one row of 128 pixels x 32 channels
 constexpr int kAccCols = 256;                   // tensor-memory columns of an accumulator set
-constexpr int kMaxRows = 24;                    // row slots (bounds the barrier array)
+constexpr int kMaxRows = 22;                    // row slots (bounds the barrier array)
 constexpr int kStageBytes = 2 * 32 * kKc * 2;   // a warp's 32 pixels of two rows, 32 channels
 constexpr int kStores = 4 * 2 * kStageBytes;    // two staging buffers for each of four warps
 constexpr int kRowsThreads = 192;
@@ -61,15 +62,14 @@ struct RowsArgs {
     int y_coff, upsample, relu;
     const float* bias;
     const int* count;  // optional: tiles at or after *count are skipped
-    uint16_t* pool;    // optional: T x H/2 x W/2 x Cout, the 2x2 maximum of the output
+    uint16_t* pool;    // kPool: T x H/2 x W/2 x Cout, the 2x2 maximum of the output
+    const float* wout; // kColors, kCompose: the output layer
+    float* rgb;        // kColors: T x H x W x 3
+    const int* list;   // kCompose: the cells of the tiles
 };
 
-__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b)
-{
-    const __nv_bfloat162 m =
-        __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
-    return *reinterpret_cast<const uint32_t*>(&m);
-}
+// What the epilogue does with a pixel's channels.
+enum { kStore, kPool, kColors, kCompose };
 
 // One 32-channel slice of one pixel: bias, ReLU, rounding to bfloat16.
 __device__ __forceinline__ void finish(const uint32_t (&r)[32], const float* bias, int relu, uint32_t (&q)[16])
@@ -86,10 +86,12 @@ __device__ __forceinline__ void finish(const uint32_t (&r)[32], const float* bia
     }
 }
 
-template <int COUT, int R>
+struct NoFrames {};
+
+template <int COUT, int R, int MODE, class Frames>
 __global__ void __launch_bounds__(kRowsThreads, 1)
     conv3x3_rows(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                 const __grid_constant__ CUtensorMap tmY, const RowsArgs a)
+                 const __grid_constant__ CUtensorMap tmY, const RowsArgs a, const __grid_constant__ Frames ft)
 {
     extern __shared__ unsigned char smem_raw[];
     const int W = a.W, H = a.H, NR = a.nrows, WS = a.wslots;
@@ -111,7 +113,8 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     uint64_t* drain = aempty + 2;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
-    float* sbias = reinterpret_cast<float*>(smem + 512);  // COUT floats
+    float* sbias = reinterpret_cast<float*>(smem + 480);  // COUT floats
+    float* swout = reinterpret_cast<float*>(smem + 608);  // kColors, kCompose: 99 floats after 32 biases
     unsigned char* rows = smem + 1024;
     constexpr int kWBytes = 9 * COUT * kKc * 2;
     unsigned char* wts = rows + NR * kRowBytes;
@@ -144,6 +147,8 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     for (int c = threadIdx.x; c < COUT; c += kRowsThreads) sbias[c] = __ldg(a.bias + c);
+    if (MODE == kColors || MODE == kCompose)
+        for (int c = threadIdx.x; c < 99; c += kRowsThreads) swout[c] = __ldg(a.wout + c);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -294,7 +299,60 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
             }
             __syncwarp();
             tc_fence_after();
-            for (int rr = 0; rr < R; rr += 2) {
+            if constexpr (MODE == kColors || MODE == kCompose) {  // the output layer, a row of pixels at a time
+                bool live = n < tiles;
+                float* rgb = nullptr;
+                const uint8_t* mask = nullptr;
+                uint32_t* rgba = nullptr;
+                int pitch = 0, r0 = 0, r1 = R;  // rows of the unit that are written
+                if constexpr (MODE == kColors) {
+                    rgb = a.rgb + (((size_t)n * H + y0) * W + x0 + lane) * 3;
+                } else if (live) {
+                    const int cell = a.list[n];
+                    const int f = table_frame(ft, cell), tile = cell - ft.off[f];
+                    const int tx = tile % ft.ntx[f], ty = tile / ft.ntx[f];
+                    const int gx = window_origin(tx, ft.w[f]) + x0 + lane, gy = window_origin(ty, ft.h[f]) + y0;
+                    // the pixels of the window outside the cell belong to the neighbouring tile
+                    live = gx >= kTile * tx && gx < ft.w[f];
+                    r0 = max(0, kTile * ty - gy);
+                    r1 = min(R, ft.h[f] - gy);
+                    pitch = ft.w[f];
+                    mask = ft.mask[f] + (ptrdiff_t)gy * pitch + gx;
+                    rgba = ft.rgba[f] + (ptrdiff_t)gy * pitch + gx;
+                }
+#pragma unroll 1
+                for (int r = 0; r < R; ++r) {
+                    uint32_t v[32], p[16];
+                    const uint32_t t = acc + (uint32_t)(r * COUT);
+                    tmem_ld32_async(t, v);
+                    bool put = live && r >= r0 && r < r1;
+                    if constexpr (MODE == kCompose) {  // hole pixels only
+                        put = put && mask[(ptrdiff_t)r * pitch];
+                    }
+                    tmem_wait_ld();
+                    tmem_zero32_async(t);
+                    if (!__any_sync(0xffffffffu, put)) continue;
+                    finish(v, sbias, a.relu, p);
+                    float x[32], col[3];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        x[2 * i] = __uint_as_float(p[i] << 16);
+                        x[2 * i + 1] = __uint_as_float(p[i] & 0xffff0000u);
+                    }
+                    net_colors(x, swout, col);
+                    if (put) {
+                        if constexpr (MODE == kColors) {
+                            float* o = rgb + (size_t)r * W * 3;
+                            o[0] = col[0];
+                            o[1] = col[1];
+                            o[2] = col[2];
+                        } else {
+                            rgba[(ptrdiff_t)r * pitch] = net_rgba(col);
+                        }
+                    }
+                }
+            }
+            for (int rr = 0; rr < R && MODE < kColors; rr += 2) {
 #pragma unroll
                 for (int c0 = 0; c0 < COUT; c0 += 32) {
                     uint32_t v0[32], v1[32];
@@ -334,7 +392,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
                         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     }
                     ++nst;
-                    if (a.pool) {  // 2x2 maximum: the two rows, then the neighbouring pixel
+                    if constexpr (MODE == kPool) {  // 2x2 maximum: the two rows, then the neighbouring pixel
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
                             const uint32_t m = max_bf16x2(p0[i], p1[i]);
@@ -413,6 +471,10 @@ cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStrea
     a.bias = c.bias;
     a.count = c.count;
     a.pool = static_cast<uint16_t*>(c.pool);
+    a.wout = c.wout;
+    a.rgb = c.rgb;
+    a.list = c.list;
+    if ((c.rgb || c.frames) && (c.Cout != 32 || c.upsample || c.pool)) return cudaErrorInvalidValue;
 
     CUtensorMap ta, tb, ty;
     const cuuint32_t one[5] = {1, 1, 1, 1, 1};
@@ -452,14 +514,26 @@ cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStrea
 
     const size_t smem = rows_smem(a.nrows, a.wslots, c.Cout);
     const int grid = std::min(groups * (c.H / R), sms);
-    auto go = [&](auto kernel) -> cudaError_t {
+    auto go = [&](auto kernel, const auto& frames) -> cudaError_t {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
         if (e != cudaSuccess) return e;
-        kernel<<<grid, kRowsThreads, smem, stream>>>(ta, tb, ty, a);
+        kernel<<<grid, kRowsThreads, smem, stream>>>(ta, tb, ty, a, frames);
         return cudaGetLastError();
     };
-    if (c.Cout == 64) return R == 4 ? go(conv3x3_rows<64, 4>) : go(conv3x3_rows<64, 2>);
-    return R == 8 ? go(conv3x3_rows<32, 8>) : R == 4 ? go(conv3x3_rows<32, 4>) : go(conv3x3_rows<32, 2>);
+    const NoFrames none;
+#define YORO_ROWS32(MODE, FRAMES, TABLE)                                \
+    (R == 8   ? go(conv3x3_rows<32, 8, MODE, FRAMES>, TABLE)            \
+     : R == 4 ? go(conv3x3_rows<32, 4, MODE, FRAMES>, TABLE)            \
+              : go(conv3x3_rows<32, 2, MODE, FRAMES>, TABLE))
+    if (c.Cout == 64) {
+        if (c.pool) return R == 4 ? go(conv3x3_rows<64, 4, kPool, NoFrames>, none) : go(conv3x3_rows<64, 2, kPool, NoFrames>, none);
+        return R == 4 ? go(conv3x3_rows<64, 4, kStore, NoFrames>, none) : go(conv3x3_rows<64, 2, kStore, NoFrames>, none);
+    }
+    if (c.frames) return YORO_ROWS32(kCompose, FrameTable, *c.frames);
+    if (c.rgb) return YORO_ROWS32(kColors, NoFrames, none);
+    if (c.pool) return YORO_ROWS32(kPool, NoFrames, none);
+    return YORO_ROWS32(kStore, NoFrames, none);
+#undef YORO_ROWS32
 }
 
 unsigned conv_rows_status_take()

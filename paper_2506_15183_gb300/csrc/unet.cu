@@ -42,6 +42,7 @@
 #include <vector>
 
 #include "tc.cuh"
+#include "unet_device.cuh"
 #include "unet_internal.h"
 #include "yoro.h"
 #include "yoro_internal.h"
@@ -66,6 +67,7 @@ struct ConvArgs {
     int relu;
     int ncols;            // tensor-memory columns allocated (a power of two >= mt Cout, >= 32)
     const int* count;     // optional: tiles at or after *count are skipped (the tile list's length)
+    uint16_t* pool;       // optional (16-pixel rows only): T x H/2 x W/2 x Cout, the 2x2 maximum of the output
     int mt, stages;       // halo form: 128-pixel accumulators per CTA and copy stages
 };
 
@@ -108,6 +110,20 @@ __device__ __forceinline__ void epilogue_store(const ConvArgs& a, const CUtensor
             const int sw = (px >> 1) & 3;
 #pragma unroll
             for (int k = 0; k < 4; ++k) *reinterpret_cast<uint4*>(row + ((k ^ sw) << 4)) = q[k];
+            // 16-pixel rows: a warp holds two of them; the 2x2 maximum of its pixels
+            if (a.pool) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    qw[i] = max_bf16x2(qw[i], __shfl_xor_sync(0xffffffffu, qw[i], 16));
+                    qw[i] = max_bf16x2(qw[i], __shfl_xor_sync(0xffffffffu, qw[i], 1));
+                }
+                const int yy = y0 + ((j * kTileM + warp * 32) >> 4);  // the first of its rows
+                const size_t pp = ((size_t)n0 * (a.H >> 1) + (yy >> 1)) * 8 + ((lane & 15) >> 1);
+                // the four lanes of a pooled pixel write 16 bytes each
+                const int k = (lane & 1) + 2 * (lane >> 4);
+                reinterpret_cast<uint4*>(a.pool + pp * a.Cout + c0)[k] =
+                    k == 0 ? q[0] : k == 1 ? q[1] : k == 2 ? q[2] : q[3];
+            }
         }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the writes, seen by the copy engine
@@ -513,10 +529,13 @@ int sm_count()
 // Needs T H W a multiple of 128, W in {8, 16, 32, 64, 128} with 128 / W rows per tile or
 // whole tiles per 128 pixels, Cout in {32, 64, 128, 256}.  Returns cudaErrorInvalidValue
 // for shapes it does not take.
-cudaError_t unet_conv3x3(const void* x, int T, int H, int W, int Cin, const void* wk, const float* bias, void* y,
-                         int Cout, int y_cstride, int y_coff, int upsample, int relu, cudaStream_t stream,
-                         const int* count)
+cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
 {
+    const int T = call.T, H = call.H, W = call.W, Cin = call.Cin, Cout = call.Cout;
+    const int y_cstride = call.y_cstride, y_coff = call.y_coff, upsample = call.upsample;
+    const void *x = call.x, *wk = call.wk;
+    void* y = call.y;
+    if (call.pool && (W < 16 || W > 64 || H % 2 || upsample)) return cudaErrorInvalidValue;
     if (T < 1 || H < 1 || W < 1 || Cin < kKc || Cin % kKc || (Cout != 32 && Cout != 64 && Cout != 128 && Cout != 256))
         return cudaErrorInvalidValue;
     if (W > kTileM || kTileM % W) return cudaErrorInvalidValue;
@@ -580,22 +599,23 @@ cudaError_t unet_conv3x3(const void* x, int T, int H, int W, int Cin, const void
     a.W = W;
     a.Cin = Cin;
     a.Cout = Cout;
-    a.bias = bias;
+    a.bias = call.bias;
     a.y = static_cast<__nv_bfloat16*>(y);
     a.y_cstride = y_cstride;
     a.y_coff = y_coff;
     a.upsample = upsample;
-    a.relu = relu;
+    a.relu = call.relu;
     a.ncols = Cout < 32 ? 32 : Cout;
-    a.count = count;
+    a.count = call.count;
+    a.pool = static_cast<uint16_t*>(call.pool);
     a.mt = 0;
     a.stages = kStages;
     int mt = 0, stages = 0;
     if (nb == 1) halo_shape(H, W, Cout, &mt, &stages);
     if (mt && conv_rows_takes(H, W, Cout))
-        return conv_rows_launch(ConvCall{x, wk, y, bias, count, nullptr, T, H, W, Cin, Cout, y_cstride, y_coff, upsample,
-                                         relu},
-                                sm_count(), kSmemPerBlock, stream);
+        return conv_rows_launch(call, sm_count(), kSmemPerBlock, stream);
+    // the output layer rides on the row form only; the other forms pool 16-pixel rows
+    if (call.rgb || call.frames || (call.pool && W != 16)) return cudaErrorInvalidValue;
     if (mt) {
         const int rows = mt * kTileM / W;
         CUtensorMap th;
@@ -642,40 +662,11 @@ cudaError_t unet_conv3x3(const void* x, int T, int H, int W, int Cin, const void
 
 namespace {
 
-constexpr int kTile = 64;  // inference tile: 64 x 64 pixels
 constexpr int kInCh = 6;   // network input channels (padded to 32 in memory)
 constexpr int kLevels = 4;
 constexpr int kWidths[kLevels] = {32, 64, 128, 256};
 
 // ---- small CUDA-core kernels around the convolutions
-
-// The frames of one inpainting launch.  Their cell grids are concatenated: cell c of frame
-// f (c = ty * ntx + tx) is entry off[f] + c, so their hole cells form one list and one pass
-// of the network takes them all.
-constexpr int kMaxInpaintFrames = 32;
-
-struct FrameTable {
-    int n;
-    int off[kMaxInpaintFrames + 1];  // off[n]: cells of all frames
-    int w[kMaxInpaintFrames], h[kMaxInpaintFrames], ntx[kMaxInpaintFrames];
-    float near_[kMaxInpaintFrames];
-    uint32_t* rgba[kMaxInpaintFrames];
-    const uint8_t* mask[kMaxInpaintFrames];
-    const float* zt[kMaxInpaintFrames];
-    const float* zsrc[kMaxInpaintFrames];
-};
-
-// Frame of concatenated cell g.
-__device__ __forceinline__ int table_frame(const FrameTable& ft, int g)
-{
-    int lo = 0, hi = ft.n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (ft.off[mid] <= g) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
 
 // Per 64 x 64 cell of each frame (blockIdx.x: cell, blockIdx.y: frame): 1 if it holds a
 // hole pixel (mask == 1), at the cell's entry of the concatenated grids.
@@ -741,11 +732,6 @@ __device__ __forceinline__ uint16_t bf16_bits(float v)
     return *reinterpret_cast<const uint16_t*>(&b);
 }
 
-// Origin of the 64 x 64 window of grid cell (tx, ty): the cell itself, except that the
-// last column and row are shifted inward so the window ends at the frame's edge (a frame
-// narrower or lower than 64 keeps origin 0 and is padded).  A tile writes its cell only.
-__device__ __forceinline__ int window_origin(int t, int size) { return max(0, min(kTile * t, size - kTile)); }
-
 // The network input of listed tile ti, pixel (py, px) of its window: the six channels of
 // the definition (the plain path's right eye / 255: warped colors and the Patcher's fill
 // at holes; the hole mask; near / warped depth, 0 at holes; near / source depth), rounded
@@ -786,48 +772,15 @@ __global__ void tile_input_kernel(const __grid_constant__ FrameTable ft, const i
     for (int i = 0; i < 4; ++i) dst[i] = q[i];
 }
 
-// 2x2 max pooling of channels [0, C) of x (T x H x W, cstride channels) into y (T x H/2 x
-// W/2 x C), eight channels per thread.  bfloat16 values compare exactly as floats.
-__global__ void maxpool_kernel(const uint16_t* __restrict__ x, int T, int H, int W, int cstride, int C,
-                               uint16_t* __restrict__ y, const int* __restrict__ count)
+// The three colors of every pixel of the first T tiles to rgb (T x 64 x 64 x 3 floats), from
+// stored activations (the training forward, which keeps them for its backward pass).
+__global__ void output_kernel(const uint16_t* __restrict__ a, const float* __restrict__ wo, int T,
+                              float* __restrict__ rgb)
 {
-    const int Ho = H / 2, Wo = W / 2, cv = C / 8;
-    const long long total = (long long)T * Ho * Wo * cv;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int v = (int)(i % cv);
-        long long r = i / cv;
-        const int xo = (int)(r % Wo);
-        r /= Wo;
-        const int yo = (int)(r % Ho);
-        const int t = (int)(r / Ho);
-        if (count && t >= *count) continue;
-        float m[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) m[k] = -INFINITY;
-#pragma unroll
-        for (int ab = 0; ab < 4; ++ab) {
-            const size_t px = ((size_t)t * H + 2 * yo + (ab >> 1)) * W + 2 * xo + (ab & 1);
-            const uint4 q = *reinterpret_cast<const uint4*>(x + px * cstride + v * 8);
-            const uint32_t qw[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                m[k] = fmaxf(m[k], __uint_as_float((k & 1 ? qw[k >> 1] & 0xffff0000u : qw[k >> 1] << 16)));
-        }
-        uint4 o;
-        uint32_t* ow = reinterpret_cast<uint32_t*>(&o);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            ow[k] = (__float_as_uint(m[2 * k]) >> 16) | (__float_as_uint(m[2 * k + 1]) & 0xffff0000u);
-        *reinterpret_cast<uint4*>(y + (((size_t)t * Ho + yo) * Wo + xo) * C + v * 8) = o;
-    }
-}
-
-// The output layer at pixel p of tile ti: a 1x1 convolution of the 32 channels (FP32 sums
-// in channel order, then the bias) and the logistic sigmoid 1 / (1 + exp(-z)).
-__device__ __forceinline__ void net_colors(const uint16_t* __restrict__ a, const float* __restrict__ wo,
-                                           const float* __restrict__ bo, int ti, int p, float (&col)[3])
-{
+    const int ti = blockIdx.y;
+    if (ti >= T) return;
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= kTile * kTile) return;
     const uint4* src = reinterpret_cast<const uint4*>(a + ((size_t)ti * kTile * kTile + p) * 32);
     float v[32];
 #pragma unroll
@@ -840,57 +793,12 @@ __device__ __forceinline__ void net_colors(const uint16_t* __restrict__ a, const
             v[8 * i + 2 * k + 1] = __uint_as_float(qw[k] & 0xffff0000u);
         }
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int ci = 0; ci < 32; ++ci) acc = __fadd_rn(acc, __fmul_rn(wo[c * 32 + ci], v[ci]));
-        const float z = __fadd_rn(acc, bo[c]);
-        col[c] = __fdiv_rn(1.0f, __fadd_rn(1.0f, expf(-z)));
-    }
-}
-
-// The three colors of every pixel of the first T tiles to rgb (T x 64 x 64 x 3 floats).
-__global__ void output_kernel(const uint16_t* __restrict__ a, const float* __restrict__ wo,
-                              const float* __restrict__ bo, int T, float* __restrict__ rgb)
-{
-    const int ti = blockIdx.y;
-    if (ti >= T) return;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= kTile * kTile) return;
     float col[3];
-    net_colors(a, wo, bo, ti, p, col);
+    net_colors(v, wo, col);
     float* o = rgb + ((size_t)ti * kTile * kTile + p) * 3;
     o[0] = col[0];
     o[1] = col[1];
     o[2] = col[2];
-}
-
-// Compose into the frames: each hole pixel of a listed tile's cell takes rint(clamp(c, 0,
-// 1) * 255) per color and alpha 255 (the pixels of the window outside the cell belong to
-// the neighbouring tile).
-__global__ void compose_kernel(const uint16_t* __restrict__ a, const float* __restrict__ wo,
-                               const float* __restrict__ bo, const int* __restrict__ count,
-                               const int* __restrict__ list, const __grid_constant__ FrameTable ft)
-{
-    const int ti = blockIdx.y;
-    if (ti >= *count) return;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= kTile * kTile) return;
-    const int g = list[ti];
-    const int f = table_frame(ft, g);
-    const int tile = g - ft.off[f];
-    const int w = ft.w[f], h = ft.h[f], ntx = ft.ntx[f];
-    const int tx = tile % ntx, ty = tile / ntx;
-    const int gx = window_origin(tx, w) + (p & (kTile - 1)), gy = window_origin(ty, h) + (p >> 6);
-    if (gx < kTile * tx || gy < kTile * ty || gx >= w || gy >= h || !ft.mask[f][(size_t)gy * w + gx]) return;
-    float col[3];
-    net_colors(a, wo, bo, ti, p, col);
-    uint32_t out = 0xff000000u;
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-        out |= (uint32_t)rintf(__fmul_rn(fminf(fmaxf(col[c], 0.0f), 1.0f), 255.0f)) << (8 * c);
-    ft.rgba[f][(size_t)gy * w + gx] = out;
 }
 
 void host_bf16_impl(const float* src, size_t n, uint16_t* dst)
@@ -913,7 +821,7 @@ void host_bf16(const float* src, size_t n, uint16_t* dst) { host_bf16_impl(src, 
 
 cudaError_t unet_output_rgb(const UnetNet* n, int T, float* rgb, cudaStream_t s)
 {
-    output_kernel<<<dim3(16, (unsigned)T), 256, 0, s>>>(n->d0b, n->wout, n->wout + 96, T, rgb);
+    output_kernel<<<dim3(16, (unsigned)T), 256, 0, s>>>(n->d0b, n->wout, T, rgb);
     return cudaGetLastError();
 }
 
@@ -1030,41 +938,41 @@ UnetNet* unet_create(const float* params, size_t n_params, int max_tiles, int ma
     return n;
 }
 
-// The 14 convolutions and the pools over the first T tiles of in0 (tiles at or after
-// *count skipped when count is given); the last layer's activations end in d0b.
-cudaError_t unet_run(UnetNet* n, int T, const int* count, cudaStream_t s)
+// The 14 convolutions over the first T tiles of x (tiles at or after *count skipped when
+// count is given), the 2x2 pools in the epilogues of the layers they follow.  The output
+// layer rides on the last one: colors to out.rgb, or composed into out.frames; with
+// neither, the last layer's activations end in d0b.
+cudaError_t unet_run(UnetNet* n, const uint16_t* x, int T, const int* count, const NetOut& out, cudaStream_t s)
 {
-    const int Te = (T + 1) & ~1;
+    const int Te = (T + 1) & ~1;  // the 8 x 8 level takes two tiles per 128-pixel accumulator
     cudaError_t e = cudaSuccess;
-    auto conv = [&](int i, const uint16_t* x, int H, void* y, int cstride, int coff, int up) {
+    auto conv = [&](int i, const uint16_t* in, int H, void* y, int cstride, int coff, int up, void* pool) {
         if (e != cudaSuccess) return;
         const UnetLayer& L = n->conv[i];
-        e = unet_conv3x3(x, Te, H, H, L.cin_pad, L.wk, L.bias, y, L.cout, cstride, coff, up, 1, s, count);
+        ConvCall c{in, L.wk, y, L.bias, count, pool, i == 0 ? T : Te, H, H, L.cin_pad, L.cout, cstride, coff, up, 1};
+        if (i == 13) {
+            c.T = T;
+            c.wout = n->wout;
+            c.rgb = out.rgb;
+            c.frames = out.frames;
+            c.list = out.frames ? n->list : nullptr;
+        }
+        e = unet_conv3x3(c, s);
     };
-    auto pool = [&](const uint16_t* x, int H, int cstride, int C, uint16_t* y) {
-        if (e != cudaSuccess) return;
-        const long long total = (long long)Te * (H / 2) * (H / 2) * (C / 8);
-        const int blocks = (int)std::min<long long>((total + 255) / 256, 4096);
-        maxpool_kernel<<<blocks, 256, 0, s>>>(x, Te, H, H, cstride, C, y, count);
-        e = cudaGetLastError();
-    };
-    conv(0, n->in0, 64, n->e0a, 32, 0, 0);     // enc0a
-    conv(1, n->e0a, 64, n->cat0, 96, 0, 0);    // enc0b -> skip of level 0
-    pool(n->cat0, 64, 96, 32, n->p0);
-    conv(2, n->p0, 32, n->e1a, 64, 0, 0);      // enc1a
-    conv(3, n->e1a, 32, n->cat1, 192, 0, 0);   // enc1b -> skip of level 1
-    pool(n->cat1, 32, 192, 64, n->p1);
-    conv(4, n->p1, 16, n->e2a, 128, 0, 0);     // enc2a
-    conv(5, n->e2a, 16, n->cat2, 384, 0, 0);   // enc2b -> skip of level 2
-    pool(n->cat2, 16, 384, 128, n->p2);
-    conv(6, n->p2, 8, n->e3a, 256, 0, 0);      // enc3a
-    conv(7, n->e3a, 8, n->cat2, 384, 128, 1);  // enc3b, upsampled after the level-2 skip
-    conv(8, n->cat2, 16, n->d2a, 128, 0, 0);   // dec2a
-    conv(9, n->d2a, 16, n->cat1, 192, 64, 1);  // dec2b, upsampled after the level-1 skip
-    conv(10, n->cat1, 32, n->d1a, 64, 0, 0);   // dec1a
-    conv(11, n->d1a, 32, n->cat0, 96, 32, 1);  // dec1b, upsampled after the level-0 skip
-    conv(12, n->cat0, 64, n->d0a, 32, 0, 0);   // dec0a
-    conv(13, n->d0a, 64, n->d0b, 32, 0, 0);    // dec0b
+    conv(0, x, 64, n->e0a, 32, 0, 0, nullptr);          // enc0a
+    conv(1, n->e0a, 64, n->cat0, 96, 0, 0, n->p0);      // enc0b -> skip of level 0
+    conv(2, n->p0, 32, n->e1a, 64, 0, 0, nullptr);      // enc1a
+    conv(3, n->e1a, 32, n->cat1, 192, 0, 0, n->p1);     // enc1b -> skip of level 1
+    conv(4, n->p1, 16, n->e2a, 128, 0, 0, nullptr);     // enc2a
+    conv(5, n->e2a, 16, n->cat2, 384, 0, 0, n->p2);     // enc2b -> skip of level 2
+    conv(6, n->p2, 8, n->e3a, 256, 0, 0, nullptr);      // enc3a
+    conv(7, n->e3a, 8, n->cat2, 384, 128, 1, nullptr);  // enc3b, upsampled after the level-2 skip
+    conv(8, n->cat2, 16, n->d2a, 128, 0, 0, nullptr);   // dec2a
+    conv(9, n->d2a, 16, n->cat1, 192, 64, 1, nullptr);  // dec2b, upsampled after the level-1 skip
+    conv(10, n->cat1, 32, n->d1a, 64, 0, 0, nullptr);   // dec1a
+    conv(11, n->d1a, 32, n->cat0, 96, 32, 1, nullptr);  // dec1b, upsampled after the level-0 skip
+    conv(12, n->cat0, 64, n->d0a, 32, 0, 0, nullptr);   // dec0a
+    conv(13, n->d0a, 64, n->d0b, 32, 0, 0, nullptr);    // dec0b
     return e;
 }
 
@@ -1084,7 +992,8 @@ yoro_status yoro_unet_conv3x3(const void* x, int T, int H, int W, int Cin, const
 {
     if (!x || !wk || !bias || !y) return YORO_EINVAL;
     if (((uintptr_t)x | (uintptr_t)wk | (uintptr_t)y) & 15u) return YORO_EALIGN;
-    const cudaError_t e = yoro::unet_conv3x3(x, T, H, W, Cin, wk, bias, y, Cout, y_cstride, y_coff, upsample, relu,
+    const cudaError_t e = yoro::unet_conv3x3(yoro::ConvCall{x, wk, y, bias, nullptr, nullptr, T, H, W, Cin, Cout, y_cstride,
+                                                            y_coff, upsample, relu},
                                              (cudaStream_t)cuda_stream);
     if (e == cudaErrorInvalidValue) return YORO_EINVAL;
     return e == cudaSuccess ? YORO_OK : YORO_ECUDA;
@@ -1127,12 +1036,11 @@ yoro_status yoro_unet_forward(yoro_unet u, const void* x, int T, float* rgb, voi
     if (!u || !x || !rgb || T < 0 || T > u->net->max_tiles) return YORO_EINVAL;
     if (T == 0) return YORO_OK;
     if (((uintptr_t)x & 15u) || ((uintptr_t)rgb & 3u)) return YORO_EALIGN;
-    const cudaStream_t s = (cudaStream_t)cuda_stream;
-    if (cudaMemcpyAsync(u->net->in0, x, (size_t)T * 64 * 64 * 32 * 2, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return YORO_ECUDA;
-    if (yoro::unet_run(u->net, T, nullptr, s) != cudaSuccess) return YORO_ECUDA;
-    yoro::output_kernel<<<dim3(16, (unsigned)T), 256, 0, s>>>(u->net->d0b, u->net->wout, u->net->wout + 96, T, rgb);
-    return cudaGetLastError() == cudaSuccess ? YORO_OK : YORO_ECUDA;
+    const yoro::NetOut out{rgb, nullptr};
+    return yoro::unet_run(u->net, static_cast<const uint16_t*>(x), T, nullptr, out, (cudaStream_t)cuda_stream) ==
+                   cudaSuccess
+               ? YORO_OK
+               : YORO_ECUDA;
 }
 
 }  // extern "C"
@@ -1169,7 +1077,8 @@ void table_add(yoro::FrameTable& ft, const yoro_unet_frame& fr)
 
 // One pass of the network over the hole cells of the table's frames: the cells' flags, the
 // list of the flagged ones and its length on the device (launches cover every cell; those
-// past the list's length return at once), the inputs, the 14 layers, the composition.
+// past the list's length return at once), the inputs, and the 14 layers, the last of which
+// composes.
 yoro_status inpaint_table(yoro_unet_ctx* u, const yoro::FrameTable& ft, cudaStream_t s)
 {
     yoro::UnetNet* n = u->net;
@@ -1181,10 +1090,8 @@ yoro_status inpaint_table(yoro_unet_ctx* u, const yoro::FrameTable& ft, cudaStre
     yoro::tile_list_kernel<<<1, 1024, 0, s>>>(n->flags, total, n->list, n->count);
     yoro::tile_input_kernel<<<dim3(16, (unsigned)total), 256, 0, s>>>(ft, n->list, n->count, n->in0);
     if (cudaGetLastError() != cudaSuccess) return YORO_ECUDA;
-    if (yoro::unet_run(n, total, n->count, s) != cudaSuccess) return YORO_ECUDA;
-    yoro::compose_kernel<<<dim3(16, (unsigned)total), 256, 0, s>>>(n->d0b, n->wout, n->wout + 96, n->count, n->list,
-                                                                 ft);
-    return cudaGetLastError() == cudaSuccess ? YORO_OK : YORO_ECUDA;
+    const yoro::NetOut out{nullptr, &ft};
+    return yoro::unet_run(n, n->in0, total, n->count, out, s) == cudaSuccess ? YORO_OK : YORO_ECUDA;
 }
 
 }  // namespace

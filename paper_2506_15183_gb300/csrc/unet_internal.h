@@ -34,8 +34,14 @@ using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, 
                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiled tensor_map_encoder();
 
-// One 3x3 convolution (the arguments of unet_conv3x3) with an optional 2x2-pooled copy of
-// its output, T x H/2 x W/2 x Cout.
+struct FrameTable;
+
+// One 3x3 convolution: x (T tiles of H x W, NHWC bf16 with Cin channels), K-major weights wk,
+// bias, output y at channel y_coff of y_cstride channels (upsample: into the 2H x 2W grid).
+// count: optional device count of live tiles.  pool: optional T x H/2 x W/2 x Cout copy of
+// the output's 2x2 maximum.  rgb or frames: instead of y, the network's output layer (wout:
+// 3 x 32 weights and 3 biases) of every pixel, as colors (T x H x W x 3 floats) or composed
+// into the frames of the listed tiles.
 struct ConvCall {
     const void* x;
     const void* wk;
@@ -44,6 +50,16 @@ struct ConvCall {
     const int* count;
     void* pool;
     int T, H, W, Cin, Cout, y_cstride, y_coff, upsample, relu;
+    const float* wout = nullptr;
+    float* rgb = nullptr;
+    const FrameTable* frames = nullptr;
+    const int* list = nullptr;
+};
+
+// Where a pass of the network ends: colors, frames, or (neither) the activations in d0b.
+struct NetOut {
+    float* rgb;
+    const FrameTable* frames;
 };
 
 // conv_rows.cu: the row form of the convolution.  conv_rows_takes(): whether a shape that
@@ -56,10 +72,8 @@ size_t unet_param_count();
 void unet_layer_dims(int i, int* cin, int* cout);
 UnetNet* unet_create(const float* params, size_t n_params, int max_tiles, int max_grid_tiles);
 void unet_free(UnetNet* n);
-cudaError_t unet_run(UnetNet* n, int T, const int* count, cudaStream_t s);
-cudaError_t unet_conv3x3(const void* x, int T, int H, int W, int Cin, const void* wk, const float* bias, void* y,
-                         int Cout, int y_cstride, int y_coff, int upsample, int relu, cudaStream_t stream,
-                         const int* count = nullptr);
+cudaError_t unet_run(UnetNet* n, const uint16_t* x, int T, const int* count, const NetOut& out, cudaStream_t s);
+cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream);
 // The output layer (1x1 convolution, sigmoid) of T tiles' d0b activations into rgb (T x 64 x 64 x 3).
 cudaError_t unet_output_rgb(const UnetNet* n, int T, float* rgb, cudaStream_t s);
 // The host's round-to-nearest-even float -> bfloat16 rule (NaN kept NaN).

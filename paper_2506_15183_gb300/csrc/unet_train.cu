@@ -460,8 +460,8 @@ cudaError_t trainer_step(Trainer* t, const void* x, const uint8_t* gt, const uin
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(t->loss, 0, 4, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(t->nhole, 0, 4, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(n->in0, x, (size_t)npx * 32 * 2, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = unet_run(n, B, nullptr, s);
+    const uint16_t* xin = static_cast<const uint16_t*>(x);
+    if (e == cudaSuccess) e = unet_run(n, xin, B, nullptr, NetOut{nullptr, nullptr}, s);
     if (e == cudaSuccess) e = unet_output_rgb(n, B, t->rgb, s);
     if (e != cudaSuccess) return e;
     count_holes_kernel<<<blocks_for(npx), 256, 0, s>>>(hole, npx, t->nhole);
@@ -477,7 +477,7 @@ cudaError_t trainer_step(Trainer* t, const void* x, const uint8_t* gt, const uin
         const uint16_t* y;
         int ycs, ycoff, yup;
     };
-    const IO io[14] = {{n->in0, 32, n->e0a, 32, 0, 0},   {n->e0a, 32, n->cat0, 96, 0, 0},
+    const IO io[14] = {{xin, 32, n->e0a, 32, 0, 0},      {n->e0a, 32, n->cat0, 96, 0, 0},
                        {n->p0, 32, n->e1a, 64, 0, 0},    {n->e1a, 64, n->cat1, 192, 0, 0},
                        {n->p1, 64, n->e2a, 128, 0, 0},   {n->e2a, 128, n->cat2, 384, 0, 0},
                        {n->p2, 128, n->e3a, 256, 0, 0},  {n->e3a, 256, n->cat2, 384, 128, 1},
@@ -517,8 +517,9 @@ cudaError_t trainer_step(Trainer* t, const void* x, const uint8_t* gt, const uin
         for (int c0 = 0; c0 < L.cin && e == cudaSuccess;) {
             const int rem = L.cin - c0;
             const int w = rem >= 256 ? 256 : rem >= 128 ? 128 : rem >= 64 ? 64 : 32;
-            e = unet_conv3x3(t->dZ, B, side, side, L.cout, t->wt[i] + (size_t)c0 * 9 * L.cout, t->zero_bias, t->DX,
-                             w, L.cin, c0, 0, 0, s);
+            e = unet_conv3x3(ConvCall{t->dZ, t->wt[i] + (size_t)c0 * 9 * L.cout, t->DX, t->zero_bias, nullptr, nullptr, B,
+                                      side, side, L.cout, w, L.cin, c0, 0, 0},
+                             s);
             c0 += w;
         }
         if (e != cudaSuccess) return e;

@@ -65,3 +65,25 @@ def test_rows_match_64_bit_sums(un, T, H, W, cin, cout, up, relu):
     tol = 2 * 9 * cin * U * absum * (1 + 2.0 ** -7) + 2.0 ** -23 * big + half_step
     bad = (got - o).abs() > tol
     assert not bad.any(), f"{int(bad.sum())} of {bad.numel()} outside the bound"
+
+
+def test_colors_and_pools_do_not_depend_on_the_tile_count(un):
+    """The network's colors (output layer and pools in the row form's epilogue) of 39 tiles at
+    once, eight-row units, are bit for bit those of the same tiles alone and a few at a time
+    (two-row units, half-empty image groups)."""
+    from paper_2506_15183_gb300 import weights as W
+
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.zeros((39, 64, 64, 32), dtype=torch.bfloat16, device="cuda")
+    x[..., :6] = torch.rand((39, 64, 64, 6), generator=g, device="cuda")
+    net = un.Inpainter(W.load_flat(), max_tiles=39)
+    every = torch.empty((39, 64, 64, 3), device="cuda")
+    net.forward(x, every)
+    t0 = 0
+    for n in (1, 3, 10, 25):
+        some = torch.empty((n, 64, 64, 3), device="cuda")
+        net.forward(x[t0:t0 + n].contiguous(), some)
+        assert torch.equal(some, every[t0:t0 + n])
+        t0 += n
+    assert un.status() == 0
+    net.close()
