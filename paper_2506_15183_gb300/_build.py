@@ -29,7 +29,7 @@ LIBDIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(LIBDIR, "libyoro.so")
 DEBUG_LIB = os.path.join(LIBDIR, "libyoro_debug.so")
 SOURCES = ["api.cu", "fused.cu", "unfused.cu", "noalloc.cu", "server.cu", "imbuffer.cu", "pose.cu", "unet.cu", "conv_rows.cu",
-           "unet_train.cu"]
+           "conv_dw.cu", "unet_train.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-fmad=false", "-Xcompiler", "-fPIC",
               "-Xptxas", "-v", f"-I{INCLUDE}", f"-I{CSRC}"]

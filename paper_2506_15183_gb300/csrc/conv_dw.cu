@@ -1,0 +1,282 @@
+// Weight gradient of the inpainter's 3x3 layers on the tensor cores:
+//   dW[co][ci][dy][dx] = sum over pixels p of dZ[p][co] X[p + (dy - 1, dx - 1)][ci]
+// with bfloat16 dZ and X and FP32 accumulation: per layer a product of K = pixels (4,096 per
+// tile at the top level), M = co, N = 9 ci.
+//
+// Both operands lie in memory as NHWC rows, channels contiguous, so in shared memory the K
+// index (the pixel) strides by 64 bytes per 32 channels: MN-major operands of tcgen05.mma
+// with the 64-byte swizzle the copy engine writes, no transposition pass.  A box is 8 rows
+// of one image with one column of padding on each side (x = -1 and x = W arrive as zeros), so
+// the K index runs over 8 (W + 2) consecutive pixels, a multiple of 16 at every level, and
+// a tap is a constant distance dy (W + 2) + dx - 1 in it: the three dy are the three
+// 32-column blocks of N = 96 (block stride one row), the dx are three MMAs from starts one
+// pixel apart.  At the padding columns dZ is zero, so what X holds there adds nothing.
+//
+// A CTA accumulates one (32 or 64 or 128 co) x (32 ci) x 9 tile in 288 tensor-memory columns
+// over its share of the boxes; the shares' sums go to a workspace and dw_reduce_kernel adds
+// them in order (so the gradient is the same bits on every run).  M is always 128: with 32
+// or 64 output channels the other rows multiply whatever follows in shared memory and are
+// not read back.  One MMA takes 56 cycles at N = 96 whatever M holds.
+#include <algorithm>
+
+#include "tc.cuh"
+#include "unet_internal.h"
+
+namespace yoro {
+
+namespace {
+
+__device__ unsigned g_dw_status;  // waits that ran out in this file's kernel
+
+constexpr int kDwThreads = 128;
+constexpr int kDwRows = 8;                 // rows of a box
+constexpr int kDwN = 96;                   // N of an MMA: three dy times 32 ci
+constexpr int kDwTile = 9 * 32;            // columns of a tile: 9 taps times 32 ci
+
+// A level's shapes: W pixels wide, COB blocks of 32 output channels.
+template <int W, int COB, int STAGES>
+struct DwShape {
+    static constexpr int kPitch = W + 2;
+    static constexpr int kPix = kDwRows * kPitch;  // K of a box
+    static constexpr int kPlane = kPix * 64;       // one 32-channel block of dZ
+    static constexpr int kZ = COB * kPlane;
+    static constexpr int kXReal = (kDwRows + 2) * kPitch * 64;
+    static constexpr int kX = (kXReal + 64 + 1023) / 1024 * 1024;  // a pixel past the box is read (times zero)
+    static constexpr int kStage = (kZ + kX + 1023) / 1024 * 1024;
+    static constexpr int kStages = STAGES;
+    // block stride of A: the next plane; with one plane the next pixel (those rows are not read back)
+    static constexpr int kLboA = COB == 1 ? 64 : kPlane;
+    // rows 64..127 of two planes read two more planes' worth past the last stage
+    static constexpr int kSlack = COB == 2 ? std::max(0, 4 * kPlane - kStage) : 0;
+    static constexpr int kSmem = 1024 + 1024 + STAGES * kStage + kSlack;
+    static_assert(kPix % 16 == 0 && kPlane % 512 == 0, "whole K steps, whole swizzle atoms");
+    static_assert(kSmem <= 227 * 1024, "shared memory of one CTA");
+};
+
+__device__ __forceinline__ uint64_t desc_mn_sw64(uint32_t saddr, uint32_t block_stride)
+{
+    uint64_t d = (uint64_t)((saddr >> 4) & 0x3fffu);
+    d |= (uint64_t)(block_stride >> 4) << 16;  // next 32 channels
+    d |= (uint64_t)(512u >> 4) << 32;          // next 8 pixels
+    d |= (uint64_t)1u << 46;
+    d |= (uint64_t)4u << 61;
+    return d;
+}
+
+template <class S, int COB>
+__global__ void __launch_bounds__(kDwThreads, 1)
+    conv3x3_dw(const __grid_constant__ CUtensorMap tmZ, const __grid_constant__ CUtensorMap tmX, int H, int boxes,
+               int cbs, float* __restrict__ ws)
+{
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                                           ~static_cast<uintptr_t>(1023));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem);
+    uint64_t* empty = full + S::kStages;
+    uint64_t* done = empty + S::kStages;
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
+    unsigned char* stages = smem + 1024;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int cb = blockIdx.y % cbs, ct = blockIdx.y / cbs;
+    const int b0 = (int)((long long)boxes * blockIdx.x / gridDim.x);
+    const int b1 = (int)((long long)boxes * (blockIdx.x + 1) / gridDim.x);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S::kStages; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(done, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // the pixel after an X box, which a padding pixel's tap reads: finite
+    for (int i = threadIdx.x; i < S::kStages * 16; i += kDwThreads)
+        *reinterpret_cast<uint32_t*>(stages + (i >> 4) * S::kStage + S::kZ + S::kXReal + (i & 15) * 4) = 0u;
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tslot;
+    int issued = 0;
+
+    if (warp == 0) {
+        if (lane == 0) {  // copies
+            const int bands = H / kDwRows;
+            for (int b = b0; b < b1; ++b) {
+                const int i = b - b0, s = i % S::kStages;
+                if (!mbar_wait(&empty[s], ((i / S::kStages) & 1) ^ 1, globaltimer() + kWaitNs)) {
+                    atomicOr(&g_dw_status, kUnetTimeout);
+                    *abort_flag = 1;
+                    break;
+                }
+                const int n = b / bands, y0 = (b - n * bands) * kDwRows;
+                unsigned char* st = stages + s * S::kStage;
+                mbar_expect_tx(&full[s], (uint32_t)(S::kZ + S::kXReal));
+#pragma unroll
+                for (int j = 0; j < COB; ++j)
+                    tma_load_4d(st + j * S::kPlane, &tmZ, &full[s], (ct * COB + j) * 32, -1, y0, n);
+                tma_load_4d(st + S::kZ, &tmX, &full[s], cb * 32, -1, y0 - 1, n);
+                ++issued;
+            }
+        }
+    } else if (warp == 1) {  // MMAs: the whole warp runs the loop, one lane issues
+        constexpr uint32_t idesc = idesc_bf16(kDwN) | (1u << 15) | (1u << 16);  // both operands MN-major
+        const uint32_t el = elect_one();
+        const uint64_t da = desc_mn_sw64(smem_u32(stages), S::kLboA);
+        const uint64_t db = desc_mn_sw64(smem_u32(stages) + S::kZ, S::kPitch * 64);
+        bool ok = true;
+        for (int b = b0; b < b1; ++b) {
+            const int i = b - b0, s = i % S::kStages;
+            if (!(ok = mbar_wait_warp(&full[s], (i / S::kStages) & 1, globaltimer() + kWaitNs))) break;
+            tc_fence_after();
+            const uint64_t as = da + (uint64_t)((uint32_t)(s * S::kStage) >> 4);
+            const uint64_t bs = db + (uint64_t)((uint32_t)(s * S::kStage) >> 4);
+            for (int k = 0; k < S::kPix / 16; ++k) {
+                const uint32_t acc = (i > 0 || k > 0) ? 1u : 0u;
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx)
+                    mma_bf16_elected(el, tmem + dx * kDwN, as + 64 * k, bs + 64 * k + 4 * dx - 4, idesc, acc);
+            }
+            mma_commit_elected(el, &empty[s]);
+        }
+        mma_commit_elected(el, done);  // arrives once every MMA issued above has completed
+        if (!ok && el) {
+            atomicOr(&g_dw_status, kUnetTimeout);
+            *abort_flag = 1;
+        }
+    }
+    __syncwarp();
+    const bool ok = mbar_wait(done, 0, globaltimer() + 4 * kWaitNs);
+    if (!ok) {
+        atomicOr(&g_dw_status, kUnetTimeout);
+        *abort_flag = 1;
+    }
+    __syncthreads();
+    if (!*abort_flag && warp < COB) {  // row co of the tile, 9 x 32 sums, 128 bytes at a time
+        tc_fence_after();
+        const uint32_t tq = tmem + ((uint32_t)(warp * 32) << 16);
+        float* row = ws + ((((size_t)blockIdx.y * gridDim.x + blockIdx.x) * COB + warp) * 32 + lane) * kDwTile;
+#pragma unroll 1
+        for (int t = 0; t < 9; ++t) {  // column block dx 96 + dy 32 holds tap (dy, dx)
+            const int dy = t / 3, dx = t - 3 * dy;
+            uint32_t v[32];
+            tmem_ld32(tq + dx * kDwN + dy * 32, v);
+            const bool none = b0 == b1;  // no box: the accumulator was never written
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                reinterpret_cast<uint4*>(row + t * 32)[i] =
+                    none ? make_uint4(0u, 0u, 0u, 0u) : make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x == 0 && *abort_flag) {  // copies still in flight after a timeout: wait for them (bounded)
+        const uint64_t d = globaltimer() + kWaitNs;
+        for (int i = max(0, issued - S::kStages); i < issued; ++i) mbar_wait(&full[i % S::kStages], (i / S::kStages) & 1, d);
+    }
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    }
+}
+
+// dW[co][ci][tap] = the sum over the shares of ws[ct cbs + cb][share][co][tap][ci], in order.
+__global__ void dw_reduce_kernel(const float* __restrict__ ws, int shares, int co_tile, int cbs, int cin, int cout,
+                                 float* __restrict__ dW)
+{
+    const int n = cout * cbs * kDwTile;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+        const int c = e & 31, r = e >> 5;
+        const int tap = r % 9, r2 = r / 9;
+        const int col = r2 % co_tile, tile = r2 / co_tile;  // tile = ct cbs + cb
+        const int ci = (tile % cbs) * 32 + c, co = tile / cbs * co_tile + col;
+        if (ci >= cin) continue;  // the first layer's padding channels
+        const float* p = ws + ((size_t)tile * shares * co_tile + col) * kDwTile + tap * 32 + c;
+        const size_t step = (size_t)co_tile * kDwTile;
+        float s = 0.0f;
+        int i = 0;
+        for (; i + 4 <= shares; i += 4) {
+            const float v0 = p[0], v1 = p[step], v2 = p[2 * step], v3 = p[3 * step];
+            s += v0;
+            s += v1;
+            s += v2;
+            s += v3;
+            p += 4 * step;
+        }
+        for (; i < shares; ++i, p += step) s += *p;
+        dW[((size_t)co * cin + ci) * 9 + tap] = s;
+    }
+}
+
+template <int W, int COB, int STAGES>
+cudaError_t launch(const CUtensorMap& tz, const CUtensorMap& tx, int H, int boxes, int tiles, int cbs, int shares,
+                   float* ws, cudaStream_t s)
+{
+    using S = DwShape<W, COB, STAGES>;
+    const cudaError_t e =
+        cudaFuncSetAttribute(conv3x3_dw<S, COB>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem);
+    if (e != cudaSuccess) return e;
+    conv3x3_dw<S, COB><<<dim3((unsigned)shares, (unsigned)tiles), kDwThreads, S::kSmem, s>>>(tz, tx, H, boxes, cbs, ws);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t conv_dw_workspace(int sms) { return (size_t)sms * 128 * kDwTile * sizeof(float); }
+
+cudaError_t conv_dw_launch(const void* dZ, const void* X, int xcs, int T, int side, int cin, int cout, int sms, float* ws,
+                           float* dW, cudaStream_t s)
+{
+    EncodeTiled enc = tensor_map_encoder();
+    if (!enc) return cudaErrorNotSupported;
+    const int cob = cout == 32 ? 1 : cout == 64 ? 2 : 4;
+    if ((side != 64 || cob != 1) && (side != 32 || cob != 2) && ((side != 16 && side != 8) || cob != 4 || cout % 128))
+        return cudaErrorInvalidValue;
+    const int cbs = (cin + 31) / 32, tiles = cbs * (cout / (32 * cob));
+    const int boxes = T * (side / kDwRows);
+    const int shares = std::max(1, std::min(boxes, sms / tiles));
+    if ((size_t)shares * tiles > (size_t)sms) return cudaErrorInvalidValue;  // the workspace holds `sms` tiles
+    const cuuint32_t one[4] = {1, 1, 1, 1};
+    auto map = [&](CUtensorMap* m, const void* p, int cs, int rows) {
+        const cuuint64_t c = (cuuint64_t)cs, w = (cuuint64_t)side;
+        const cuuint64_t d[4] = {c, w, w, (cuuint64_t)T};
+        const cuuint64_t st[3] = {c * 2, w * c * 2, w * w * c * 2};
+        const cuuint32_t box[4] = {32, (cuuint32_t)side + 2, (cuuint32_t)rows, 1};
+        return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(p), d, st, box, one,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    CUtensorMap tz, tx;
+    if (!map(&tz, dZ, cout, kDwRows) || !map(&tx, X, xcs, kDwRows + 2)) return cudaErrorInvalidValue;
+    cudaError_t e;
+    if (side == 64) e = launch<64, 1, 2>(tz, tx, side, boxes, tiles, cbs, shares, ws, s);
+    else if (side == 32) e = launch<32, 2, 3>(tz, tx, side, boxes, tiles, cbs, shares, ws, s);
+    else if (side == 16) e = launch<16, 4, 4>(tz, tx, side, boxes, tiles, cbs, shares, ws, s);
+    else e = launch<8, 4, 4>(tz, tx, side, boxes, tiles, cbs, shares, ws, s);
+    if (e != cudaSuccess) return e;
+    const int n = cout * cbs * kDwTile;
+    dw_reduce_kernel<<<(n + 255) / 256, 256, 0, s>>>(ws, shares, 32 * cob, cbs, cin, cout, dW);
+    return cudaGetLastError();
+}
+
+unsigned conv_dw_status_take()
+{
+    unsigned v = 0, z = 0;
+    if (cudaMemcpyFromSymbol(&v, g_dw_status, sizeof v) != cudaSuccess ||
+        cudaMemcpyToSymbol(g_dw_status, &z, sizeof z) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return v;
+}
+
+}  // namespace yoro

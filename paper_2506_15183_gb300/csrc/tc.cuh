@@ -153,6 +153,19 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, u
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, deadline));
 }
 
+// An MMA issued by the lane whose `elected` is 1.
+__device__ __forceinline__ void mma_bf16_elected(uint32_t elected, uint32_t d_tmem, uint64_t a, uint64_t b,
+                                                 uint32_t idesc, uint32_t accum)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(accum), "r"(elected)
+        : "memory");
+}
+
 // An accumulating MMA issued by the lane whose `elected` is 1, with a lane mask: bit l of
 // (m0, m1, m2, m3) set leaves lane l (row l of D) as it is.
 __device__ __forceinline__ void mma_bf16_masked(uint32_t elected, uint32_t d_tmem, uint64_t a, uint64_t b,

@@ -500,7 +500,7 @@ unsigned unet_status_take()
         cudaGetLastError();
         return 0;
     }
-    return v | conv_rows_status_take();
+    return v | conv_rows_status_take() | conv_dw_status_take();
 }
 
 // One 3x3 convolution (zero padding 1) of x (T tiles of H x W, NHWC bf16 with Cin

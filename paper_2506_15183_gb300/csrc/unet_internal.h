@@ -68,6 +68,16 @@ bool conv_rows_takes(int H, int W, int Cout);
 cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStream_t stream);
 unsigned conv_rows_status_take();
 
+// conv_dw.cu: the weight gradient of one layer from its dZ (T x side x side x cout, dense) and
+// input X (channel stride xcs), into dW (cout, cin, 3, 3), overwritten.  ws: workspace of
+// conv_dw_workspace() bytes for the same sms.  The network's levels only (side 64, 32, 16, 8
+// with 32, 64, 128, 256 output channels).
+size_t conv_dw_workspace(int sms);
+cudaError_t conv_dw_launch(const void* dZ, const void* X, int xcs, int T, int side, int cin, int cout, int sms, float* ws,
+                           float* dW, cudaStream_t s);
+unsigned conv_dw_status_take();
+int sm_count();
+
 size_t unet_param_count();
 void unet_layer_dims(int i, int* cin, int* cout);
 UnetNet* unet_create(const float* params, size_t n_params, int max_tiles, int max_grid_tiles);

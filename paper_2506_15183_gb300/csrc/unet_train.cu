@@ -8,8 +8,8 @@
 //                 activations (the 1x1 layer's transpose);
 //   3x3 layer     dZ = dY where the layer's output is positive (ReLU'), rounded to
 //                 bfloat16; the bias gradient sums dZ; the weight gradient correlates the
-//                 layer's input with dZ over every pixel (FP32, CUDA cores: a K = pixels
-//                 reduction); the input gradient is a 3x3 convolution of dZ with the
+//                 layer's input with dZ over every pixel (a K = pixels product on the
+//                 tensor cores, conv_dw.cu); the input gradient is a 3x3 convolution of dZ with the
 //                 kernel flipped in both directions and its channels transposed, run by the
 //                 same tcgen05 kernel as the forward (no ReLU, zero bias; outputs wider than
 //                 256 channels in slices);
@@ -153,93 +153,6 @@ __global__ void relu_mask_kernel(const float* __restrict__ G, const uint16_t* __
     for (int i = threadIdx.x; i < C; i += blockDim.x) atomicAdd(&db[i], s[i]);
 }
 
-// The weight gradient with register tiles: dW[co][ci][tap] += sum over the block's pixels
-// of dZ[p][co] * X[p shifted by the tap][ci] (zero outside the tile).  A CTA takes a
-// CO_T x CI_T (co, ci) tile of one tap and a range of pixels, 32 pixels per step staged in
-// shared memory as floats (16-byte loads of 8 bfloat16 values; the tile side is a power
-// of two, so the shift is found with shifts and masks).  Thread (tc, ti) of group g keeps
-// the 4 x 4 products of co 4 tc .., ci 4 ti .. over the step's pixels g, g + G, ...
-// (G = 256 / (CO_T CI_T / 16) groups), each a fused multiply-add, and adds its sums to
-// dW at the end.  The channels a load covers lie inside X's channel stride (a layer whose
-// input channels are padded, the first, reads the zero padding); sums for ci >= cin are
-// dropped.
-template <int CO_T, int CI_T>
-__global__ void __launch_bounds__(256) dw_tiled_kernel(const uint16_t* __restrict__ dZ, const uint16_t* __restrict__ X,
-                                                      int xcs, int side_log2, int cin, int cout, long long npx,
-                                                      int pix_per_block, float* __restrict__ dW)
-{
-    constexpr int TC = CO_T / 4, TI = CI_T / 4, G = 256 / (TC * TI);
-    __shared__ __align__(16) float sZ[32][CO_T + 4];
-    __shared__ __align__(16) float sX[32][CI_T + 4];
-    const int ci0 = blockIdx.x * CI_T, co0 = blockIdx.y * CO_T;
-    const int tap = blockIdx.z % 9, split = blockIdx.z / 9;
-    const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-    const int side = 1 << side_log2;
-    const int t = threadIdx.x;
-    const int g = t / (TC * TI), r = t - g * (TC * TI);
-    const int tc = r / TI, ti = r - tc * TI;
-    const long long p_begin = (long long)split * pix_per_block;
-    const long long p_end = min(npx, p_begin + pix_per_block);
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
-    for (long long p0 = p_begin; p0 < p_end; p0 += 32) {
-        // dZ rows of the step: 32 pixels x CO_T channels, 8 per load
-        for (int l = t; l < 32 * (CO_T / 8); l += 256) {
-            const int k = l / (CO_T / 8), c = (l - k * (CO_T / 8)) * 8;
-            const long long p = p0 + k;
-            uint4 u = make_uint4(0u, 0u, 0u, 0u);
-            if (p < p_end) u = *reinterpret_cast<const uint4*>(dZ + p * cout + co0 + c);
-            float4* dst = reinterpret_cast<float4*>(&sZ[k][c]);
-            dst[0] = make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
-                                 __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
-            dst[1] = make_float4(__uint_as_float(u.z << 16), __uint_as_float(u.z & 0xffff0000u),
-                                 __uint_as_float(u.w << 16), __uint_as_float(u.w & 0xffff0000u));
-        }
-        // X at the tap's shift: 32 pixels x CI_T channels
-        for (int l = t; l < 32 * (CI_T / 8); l += 256) {
-            const int k = l / (CI_T / 8), c = (l - k * (CI_T / 8)) * 8;
-            const long long p = p0 + k;
-            uint4 u = make_uint4(0u, 0u, 0u, 0u);
-            if (p < p_end) {
-                const int x = (int)(p & (side - 1)), y = (int)((p >> side_log2) & (side - 1));
-                const long long tt = p >> (2 * side_log2);
-                const int ys = y + dy, xs = x + dx;
-                if (ys >= 0 && ys < side && xs >= 0 && xs < side)
-                    u = *reinterpret_cast<const uint4*>(X + (((tt << side_log2) + ys) * side + xs) * xcs + ci0 + c);
-            }
-            float4* dst = reinterpret_cast<float4*>(&sX[k][c]);
-            dst[0] = make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
-                                 __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
-            dst[1] = make_float4(__uint_as_float(u.z << 16), __uint_as_float(u.z & 0xffff0000u),
-                                 __uint_as_float(u.w << 16), __uint_as_float(u.w & 0xffff0000u));
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int k = g; k < 32; k += G) {
-            const float4 z = *reinterpret_cast<const float4*>(&sZ[k][4 * tc]);
-            const float4 x = *reinterpret_cast<const float4*>(&sX[k][4 * ti]);
-            const float zv[4] = {z.x, z.y, z.z, z.w}, xv[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = __fmaf_rn(zv[i], xv[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int co = co0 + 4 * tc + i;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int ci = ci0 + 4 * ti + j;
-            if (ci < cin) atomicAdd(&dW[((long long)co * cin + ci) * 9 + tap], acc[i][j]);
-        }
-    }
-}
-
 // G[p][c] += DX[p * dcs + dcoff + c]
 __global__ void add_kernel(float* __restrict__ G, const uint16_t* __restrict__ DX, int dcs, int dcoff, int C,
                            long long n)
@@ -349,6 +262,8 @@ struct Trainer {
     float* G[14];
     uint16_t *dZ, *DX;
     float *zero_bias, *rgb, *dzo, *loss;
+    float* ws;  // partial sums of the weight gradients
+    int sms;
     int* nhole;
     int step;
     float lr, b1, b2, eps;
@@ -366,7 +281,7 @@ void trainer_free(Trainer* t)
         cudaFree(t->wt[i]);
         cudaFree(t->G[i]);
     }
-    void* bufs[] = {t->params, t->grads, t->m, t->v, t->dZ, t->DX, t->zero_bias, t->rgb, t->dzo, t->loss, t->nhole};
+    void* bufs[] = {t->params, t->grads, t->m, t->v, t->dZ, t->DX, t->zero_bias, t->rgb, t->dzo, t->loss, t->nhole, t->ws};
     for (void* b : bufs) cudaFree(b);
     delete t;
 }
@@ -401,6 +316,7 @@ Trainer* trainer_create(const float* params, size_t np, int batch, float lr, flo
     t->b1 = b1;
     t->b2 = b2;
     t->eps = eps;
+    t->sms = sm_count();
     t->net = unet_create(params, np, batch, 1);
     bool ok = t->net != nullptr;
     size_t off = 0;
@@ -431,7 +347,8 @@ Trainer* trainer_create(const float* params, size_t np, int batch, float lr, flo
              cudaMalloc(&t->dZ, dz_max * 2) == cudaSuccess && cudaMalloc(&t->DX, dx_max * 2) == cudaSuccess &&
              cudaMalloc(&t->zero_bias, 384 * 4) == cudaSuccess && cudaMalloc(&t->rgb, B * 4096 * 3 * 4) == cudaSuccess &&
              cudaMalloc(&t->dzo, B * 4096 * 3 * 4) == cudaSuccess && cudaMalloc(&t->loss, 4) == cudaSuccess &&
-             cudaMalloc(&t->nhole, 4) == cudaSuccess;
+             cudaMalloc(&t->nhole, 4) == cudaSuccess &&
+             cudaMalloc(&t->ws, conv_dw_workspace(t->sms)) == cudaSuccess;
     if (ok)
         ok = cudaMemcpy(t->params, params, np * 4, cudaMemcpyHostToDevice) == cudaSuccess &&
              cudaMemset(t->m, 0, np * 4) == cudaSuccess && cudaMemset(t->v, 0, np * 4) == cudaSuccess &&
@@ -491,27 +408,9 @@ cudaError_t trainer_step(Trainer* t, const void* x, const uint8_t* gt, const uin
         const long long nz = P * L.cout;
         relu_mask_kernel<<<blocks_for(nz), 256, 0, s>>>(t->G[i], io[i].y, io[i].ycs, io[i].ycoff, io[i].yup, side,
                                                         L.cout, nz, t->dZ, t->grads + t->boff[i]);
-        {
-            // (co, ci) tiles of 64 where the channels allow, else 32; pixel ranges (multiples
-            // of 32) short enough for at least ~1,000 CTAs
-            const int cot = L.cout % 64 == 0 ? 64 : 32, cit = L.cin % 64 == 0 ? 64 : 32;
-            const int tiles = (L.cin + cit - 1) / cit * (L.cout / cot) * 9;
-            long long ppb = 4096;
-            while (ppb > 256 && tiles * ((P + ppb - 1) / ppb) < 1024) ppb /= 2;
-            const dim3 grid((L.cin + cit - 1) / cit, L.cout / cot, (unsigned)(9 * ((P + ppb - 1) / ppb)));
-            int ls = 0;
-            while ((1 << ls) < side) ++ls;
-            float* dw = t->grads + t->woff[i];
-            if (cot == 64 && cit == 64)
-                dw_tiled_kernel<64, 64><<<grid, 256, 0, s>>>(t->dZ, io[i].x, io[i].xcs, ls, L.cin, L.cout, P, (int)ppb, dw);
-            else if (cot == 64)
-                dw_tiled_kernel<64, 32><<<grid, 256, 0, s>>>(t->dZ, io[i].x, io[i].xcs, ls, L.cin, L.cout, P, (int)ppb, dw);
-            else if (cit == 64)
-                dw_tiled_kernel<32, 64><<<grid, 256, 0, s>>>(t->dZ, io[i].x, io[i].xcs, ls, L.cin, L.cout, P, (int)ppb, dw);
-            else
-                dw_tiled_kernel<32, 32><<<grid, 256, 0, s>>>(t->dZ, io[i].x, io[i].xcs, ls, L.cin, L.cout, P, (int)ppb, dw);
-        }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = conv_dw_launch(t->dZ, io[i].x, io[i].xcs, B, side, L.cin, L.cout, t->sms, t->ws, t->grads + t->woff[i], s);
+        if (e != cudaSuccess) return e;
         if (i == 0) break;
         // input gradient: slices of 256 / 128 / 64 / 32 output channels
         for (int c0 = 0; c0 < L.cin && e == cudaSuccess;) {
