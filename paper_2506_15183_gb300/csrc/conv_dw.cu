@@ -189,30 +189,27 @@ __global__ void __launch_bounds__(kDwThreads, 1)
     }
 }
 
-// dW[co][ci][tap] = the sum over the shares of ws[ct cbs + cb][share][co][tap][ci], in order.
-__global__ void dw_reduce_kernel(const float* __restrict__ ws, int shares, int co_tile, int cbs, int cin, int cout,
-                                 float* __restrict__ dW)
+// dW[co][ci][tap] = the sum over the shares of ws[ct cbs + cb][share][co][tap][ci]: a block
+// takes 32 consecutive ci, its eight warps every eighth share, and adds the warps' sums in
+// order (one thread per element over all shares was 13 us per layer, latency).
+__global__ void __launch_bounds__(256) dw_reduce_kernel(const float* __restrict__ ws, int shares, int co_tile, int cbs,
+                                                        int cin, float* __restrict__ dW)
 {
-    const int n = cout * cbs * kDwTile;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-        const int c = e & 31, r = e >> 5;
-        const int tap = r % 9, r2 = r / 9;
-        const int col = r2 % co_tile, tile = r2 / co_tile;  // tile = ct cbs + cb
-        const int ci = (tile % cbs) * 32 + c, co = tile / cbs * co_tile + col;
-        if (ci >= cin) continue;  // the first layer's padding channels
-        const float* p = ws + ((size_t)tile * shares * co_tile + col) * kDwTile + tap * 32 + c;
-        const size_t step = (size_t)co_tile * kDwTile;
-        float s = 0.0f;
-        int i = 0;
-        for (; i + 4 <= shares; i += 4) {
-            const float v0 = p[0], v1 = p[step], v2 = p[2 * step], v3 = p[3 * step];
-            s += v0;
-            s += v1;
-            s += v2;
-            s += v3;
-            p += 4 * step;
-        }
-        for (; i < shares; ++i, p += step) s += *p;
+    __shared__ float part[8][32];
+    const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int tap = blockIdx.x % 9, r = blockIdx.x / 9;
+    const int col = r % co_tile, tile = r / co_tile;  // tile = ct cbs + cb
+    const size_t step = (size_t)co_tile * kDwTile;
+    const float* p = ws + ((size_t)tile * shares * co_tile + col) * kDwTile + tap * 32 + c;
+    float s = 0.0f;
+#pragma unroll 4
+    for (int i = g; i < shares; i += 8) s += p[i * step];
+    part[g][c] = s;
+    __syncthreads();
+    const int ci = (tile % cbs) * 32 + c, co = tile / cbs * co_tile + col;
+    if (g == 0 && ci < cin) {  // the first layer's padding channels are dropped
+#pragma unroll
+        for (int i = 1; i < 8; ++i) s += part[i][c];
         dW[((size_t)co * cin + ci) * 9 + tap] = s;
     }
 }
@@ -263,8 +260,7 @@ cudaError_t conv_dw_launch(const void* dZ, const void* X, int xcs, int T, int si
     else if (side == 16) e = launch<16, 4, 4>(tz, tx, side, boxes, tiles, cbs, shares, ws, s);
     else e = launch<8, 4, 4>(tz, tx, side, boxes, tiles, cbs, shares, ws, s);
     if (e != cudaSuccess) return e;
-    const int n = cout * cbs * kDwTile;
-    dw_reduce_kernel<<<(n + 255) / 256, 256, 0, s>>>(ws, shares, 32 * cob, cbs, cin, cout, dW);
+    dw_reduce_kernel<<<(unsigned)(cout * cbs * 9), 256, 0, s>>>(ws, shares, 32 * cob, cbs, cin, dW);
     return cudaGetLastError();
 }
 

@@ -17,9 +17,9 @@
 //                 upsampling sums each 2x2 block, 2x2 max pooling sends each window's
 //                 gradient to its first maximum (row-major), and an encoder level's output
 //                 gathers its skip path and its pooling path.
-// Gradients of activations are FP32 (accumulated) and bfloat16 where a tensor-core
-// convolution reads them.  Adam keeps FP32 master weights; after each step the forward's
-// K-major bfloat16 weights and the backward's flipped, transposed ones are rebuilt.
+// Gradients of activations are bfloat16 where a tensor-core convolution writes or reads
+// them and FP32 sums in between.  Adam keeps FP32 master weights and rebuilds the forward's
+// K-major bfloat16 weights and the backward's flipped, transposed ones in the same pass.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -62,193 +62,273 @@ __global__ void count_holes_kernel(const uint8_t* __restrict__ hole, long long n
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(cnt, c);
 }
 
-// dz of the sigmoid input at every pixel (0 outside holes) and the loss.
-__global__ void loss_kernel(const float* __restrict__ rgb, const uint8_t* __restrict__ gt,
-                            const uint8_t* __restrict__ hole, long long npx, const int* __restrict__ cnt,
-                            float* __restrict__ dzo, float* __restrict__ loss)
+// Eight bfloat16 channels of a 16-byte load.
+__device__ __forceinline__ void unpack8(const uint16_t* p, float (&v)[8])
 {
-    const float inv_n = 1.0f / (3.0f * (float)max(*cnt, 1));
-    float l = 0.0f;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npx;
-         p += (long long)gridDim.x * blockDim.x) {
-        const bool h = hole[p] != 0;
+    const uint4 q = *reinterpret_cast<const uint4*>(p);
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float s = rgb[3 * p + c];
-            const float e = s - (float)gt[3 * p + c] / 255.0f;
-            dzo[3 * p + c] = h ? 2.0f * e * inv_n * s * (1.0f - s) : 0.0f;
-            if (h) l += e * e;
-        }
+    for (int k = 0; k < 4; ++k) {
+        v[2 * k] = __uint_as_float(w[k] << 16);
+        v[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
     }
-    l = warp_sum(l);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, l * inv_n);
 }
 
-// Output layer backward: the gradient of d0b (added to G) and of the 1x1 weights / biases.
-__global__ void out_bwd_kernel(const uint16_t* __restrict__ a, const float* __restrict__ wout,
-                               const float* __restrict__ dzo, long long npx, float* __restrict__ G,
-                               float* __restrict__ gw, float* __restrict__ gb)
+// dZ of eight channels of a pixel: v where the layer's output y is positive (ReLU'), rounded
+// to bfloat16 and stored; the bias gradient adds v.
+__device__ __forceinline__ void mask8(const float (&v)[8], const float (&y)[8], uint16_t* dz, float (&db)[8])
 {
-    __shared__ float s[99];
-    for (int i = threadIdx.x; i < 99; i += blockDim.x) s[i] = 0.0f;
-    __syncthreads();
-    for (long long base = blockIdx.x * (long long)blockDim.x; base < npx; base += (long long)gridDim.x * blockDim.x) {
-        const long long p = base + threadIdx.x;
-        float dz[3] = {0.0f, 0.0f, 0.0f};
-        float av[32];
-        if (p < npx) {
+    uint32_t w[4];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) dz[c] = dzo[3 * p + c];
-#pragma unroll
-            for (int ci = 0; ci < 32; ++ci) av[ci] = bf2f(a[p * 32 + ci]);
-#pragma unroll
-            for (int ci = 0; ci < 32; ++ci)
-                G[p * 32 + ci] += wout[ci] * dz[0] + wout[32 + ci] * dz[1] + wout[64 + ci] * dz[2];
-        } else {
-#pragma unroll
-            for (int ci = 0; ci < 32; ++ci) av[ci] = 0.0f;
-        }
-        const bool any = __any_sync(0xffffffffu, dz[0] != 0.0f || dz[1] != 0.0f || dz[2] != 0.0f);
-        if (!any) continue;  // warp-uniform: no hole pixel in this warp
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float b = warp_sum(dz[c]);
-            if ((threadIdx.x & 31) == 0) atomicAdd(&s[96 + c], b);
-            for (int ci = 0; ci < 32; ++ci) {
-                const float v = warp_sum(dz[c] * av[ci]);
-                if ((threadIdx.x & 31) == 0) atomicAdd(&s[c * 32 + ci], v);
-            }
-        }
+    for (int k = 0; k < 4; ++k) {
+        const float a = y[2 * k] > 0.0f ? v[2 * k] : 0.0f, b = y[2 * k + 1] > 0.0f ? v[2 * k + 1] : 0.0f;
+        db[2 * k] += a;
+        db[2 * k + 1] += b;
+        w[k] = (uint32_t)f2bf(a) | ((uint32_t)f2bf(b) << 16);
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 96; i += blockDim.x) atomicAdd(&gw[i], s[i]);
-    for (int i = threadIdx.x; i < 3; i += blockDim.x) atomicAdd(&gb[i], s[96 + i]);
+    *reinterpret_cast<uint4*>(dz) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// dZ = G where the layer's output Y is positive (bfloat16), and the bias gradient (sum of
-// dZ per channel).  Y: channel stride ycs, offset ycoff; up: Y is the 2x2-upsampled copy
-// (read at (2y, 2x)) of a layer whose pixels are side x side.
-__global__ void relu_mask_kernel(const float* __restrict__ G, const uint16_t* __restrict__ Y, int ycs, int ycoff,
-                                 int up, int side, int C, long long n, uint16_t* __restrict__ dZ,
-                                 float* __restrict__ db)
+// Adds every thread's sums of N channels (channel group threadIdx.x % groups, the groups a
+// power of two up to 32) into s[group * N ..] of shared memory, then adds s to dst.
+template <int N>
+__device__ __forceinline__ void block_sums(float (&v)[N], int groups, float* s, float* dst)
+{
+    for (int i = threadIdx.x; i < groups * N; i += blockDim.x) s[i] = 0.0f;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        for (int o = groups; o < 32; o <<= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+        if (lane < groups) atomicAdd(&s[(threadIdx.x & (groups - 1)) * N + k], v[k]);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < groups * N; i += blockDim.x) atomicAdd(&dst[i], s[i]);
+    __syncthreads();
+}
+
+// The gradient dZ of a layer's sums (before ReLU), with its bias gradient, from the input
+// gradients of the layers that read its output.  A thread takes eight channels of a pixel
+// (kDirect, kUp) or of a 2x2 window (kPooled); the blocks stride by whole pixels, so its
+// channels stay the same.  These passes are bound by memory (bfloat16 in, bfloat16 out),
+// so the routing, ReLU' and the bias sums are one pass with 16-byte accesses and nothing
+// is accumulated in global memory in between.
+//   kDirect   one consumer at the same pixels: D at channel doff of dcs
+//   kUp       the consumer read this layer's output upsampled: the sum of D's 2x2 block; the
+//             output itself is the upsampled copy (read at (2y, 2x))
+//   kPooled   an encoder level's last layer: its skip consumer's D plus, at the first maximum
+//             of each window of its output (row-major), the pooled consumer's P (dense)
+enum { kDirect, kUp, kPooled };
+
+template <int KIND>
+__global__ void __launch_bounds__(256) dz_kernel(const uint16_t* __restrict__ D, int dcs, int doff,
+                                                 const uint16_t* __restrict__ P, const uint16_t* __restrict__ Y, int ycs,
+                                                 int yoff, int side, int C, long long items, uint16_t* __restrict__ dZ,
+                                                 float* __restrict__ gb)
 {
     __shared__ float s[256];
-    for (int i = threadIdx.x; i < C; i += blockDim.x) s[i] = 0.0f;
-    __syncthreads();
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(e % C);
-        const long long p = e / C;
-        long long yo;
-        if (!up) {
-            yo = p * ycs;
+    const int cg = C >> 3;  // channel groups, a power of two
+    const int c = (threadIdx.x & (cg - 1)) << 3;
+    float db[8] = {};
+    // log2 of the groups and of the side (powers of two)
+    const int lc = __ffs(cg) - 1, ls = __ffs(KIND == kPooled ? side >> 1 : side) - 1;
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < items; i += gridDim.x * 256ll) {
+        const long long p = i >> lc;  // pixel, or window
+        float v[8], y[8];
+        if (KIND == kDirect) {
+            unpack8(D + p * dcs + doff + c, v);
+            unpack8(Y + p * ycs + yoff + c, y);
+            mask8(v, y, dZ + p * C + c, db);
+        } else if (KIND == kUp) {
+            const long long x = p & (side - 1), r = p >> ls, t = r >> ls, yy = r & (side - 1);
+            const long long q = (t * 2 * side + 2 * yy) * 2 * side + 2 * x;
+            float e[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = 0.0f;
+#pragma unroll
+            for (int ab = 0; ab < 4; ++ab) {
+                unpack8(D + (q + (ab >> 1) * 2 * side + (ab & 1)) * dcs + doff + c, e);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] += e[k];
+            }
+            unpack8(Y + q * ycs + yoff + c, y);
+            mask8(v, y, dZ + p * C + c, db);
         } else {
-            const long long x = p % side, r = p / side, y = r % side, t = r / side;
-            yo = ((t * 2 * side + 2 * y) * 2 * side + 2 * x) * ycs;
-        }
-        const float v = bf2f(Y[yo + ycoff + c]) > 0.0f ? G[e] : 0.0f;
-        dZ[e] = f2bf(v);
-        if (v != 0.0f) atomicAdd(&s[c], v);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < C; i += blockDim.x) atomicAdd(&db[i], s[i]);
-}
-
-// G[p][c] += DX[p * dcs + dcoff + c]
-__global__ void add_kernel(float* __restrict__ G, const uint16_t* __restrict__ DX, int dcs, int dcoff, int C,
-                           long long n)
-{
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
-        G[e] += bf2f(DX[(e / C) * dcs + dcoff + e % C]);
-}
-
-// Nearest upsampling's gradient: G (side x side) += the sum of DX's 2x2 block (2 side).
-__global__ void upbwd_kernel(float* __restrict__ G, const uint16_t* __restrict__ DX, int dcs, int dcoff, int side,
-                             int C, long long n)
-{
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(e % C);
-        const long long p = e / C, x = p % side, r = p / side, y = r % side, t = r / side;
-        float s = 0.0f;
+            const int h = side >> 1;
+            const long long x = p & (h - 1), r = p >> ls, t = r >> ls, yy = r & (h - 1);
+            const long long q0 = (t * side + 2 * yy) * side + 2 * x;
+            float g[8], w[4][8];
+            int best[8];
+            unpack8(P + p * C + c, g);
 #pragma unroll
-        for (int ab = 0; ab < 4; ++ab)
-            s += bf2f(DX[((t * 2 * side + 2 * y + (ab >> 1)) * 2 * side + 2 * x + (ab & 1)) * dcs + dcoff + c]);
-        G[e] += s;
-    }
-}
-
-// 2x2 max pooling's gradient: each pooled pixel's gradient (DX, side x side, C channels)
-// goes to the first maximum of its window of Y (2 side x 2 side, channel stride ycs), in
-// G (2 side x 2 side x C).
-__global__ void poolbwd_kernel(float* __restrict__ G, const uint16_t* __restrict__ DX, const uint16_t* __restrict__ Y,
-                               int ycs, int side, int C, long long n)
-{
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(e % C);
-        const long long p = e / C, x = p % side, r = p / side, y = r % side, t = r / side;
-        const int s2 = 2 * side;
-        long long best = -1;
-        float bv = 0.0f;
+            for (int ab = 0; ab < 4; ++ab) unpack8(Y + (q0 + (ab >> 1) * side + (ab & 1)) * ycs + yoff + c, w[ab]);
 #pragma unroll
-        for (int ab = 0; ab < 4; ++ab) {
-            const long long q = (t * s2 + 2 * y + (ab >> 1)) * s2 + 2 * x + (ab & 1);
-            const float v = bf2f(Y[q * ycs + c]);
-            if (best < 0 || v > bv) {
-                best = q;
-                bv = v;
+            for (int k = 0; k < 8; ++k) {
+                best[k] = 0;
+                float m = w[0][k];
+#pragma unroll
+                for (int ab = 1; ab < 4; ++ab)
+                    if (w[ab][k] > m) {
+                        m = w[ab][k];
+                        best[k] = ab;
+                    }
+            }
+#pragma unroll
+            for (int ab = 0; ab < 4; ++ab) {
+                const long long q = q0 + (ab >> 1) * side + (ab & 1);
+                unpack8(D + q * dcs + doff + c, v);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] += best[k] == ab ? g[k] : 0.0f;
+                mask8(v, w[ab], dZ + q * C + c, db);
             }
         }
-        G[best * C + c] += bf2f(DX[e]);
+    }
+    block_sums(db, cg, s, gb);
+}
+
+// The loss, and the backward pass through the output layer and the last layer's ReLU: dz of
+// the sigmoid input at every pixel (0 outside holes), the gradient of the 1x1 weights and
+// biases, and dZ of the last 3x3 layer with its bias gradient.  A thread takes eight
+// channels of a pixel (four threads a pixel; the first of them adds the loss).
+__global__ void __launch_bounds__(256) out_bwd_kernel(const float* __restrict__ rgb, const uint8_t* __restrict__ gt,
+                                                      const uint8_t* __restrict__ hole, long long npx,
+                                                      const int* __restrict__ cnt, const uint16_t* __restrict__ a,
+                                                      const float* __restrict__ wout, uint16_t* __restrict__ dZ,
+                                                      float* __restrict__ gw, float* __restrict__ gwb,
+                                                      float* __restrict__ gb, float* __restrict__ loss)
+{
+    __shared__ float s[128];
+    const float inv_n = 1.0f / (3.0f * (float)max(*cnt, 1));
+    const int c = (threadIdx.x & 3) << 3;
+    float w[3][8], dw[3][8] = {}, db[8] = {}, dwb[4] = {};  // dwb: three biases and the loss
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) w[j][k] = wout[32 * j + c + k];
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < 4 * npx; i += gridDim.x * 256ll) {
+        const long long p = i >> 2;
+        if (!hole[p]) {  // dz = 0
+            *reinterpret_cast<uint4*>(dZ + p * 32 + c) = make_uint4(0u, 0u, 0u, 0u);
+            continue;
+        }
+        float dz[3], v[8], y[8];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const float sg = rgb[3 * p + j];
+            const float e = sg - (float)gt[3 * p + j] / 255.0f;
+            dz[j] = 2.0f * e * inv_n * sg * (1.0f - sg);
+            if (c == 0) {
+                dwb[j] += dz[j];
+                dwb[3] += e * e;
+            }
+        }
+        unpack8(a + p * 32 + c, y);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            v[k] = w[0][k] * dz[0] + w[1][k] * dz[1] + w[2][k] * dz[2];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) dw[j][k] += dz[j] * y[k];
+        }
+        mask8(v, y, dZ + p * 32 + c, db);
+    }
+    block_sums(db, 4, s, gb);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) block_sums(dw[j], 4, s, gw + 32 * j);
+    dwb[3] *= inv_n;
+    // the sums sit in the threads of channel group 0; the others add zeros
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dwb[j] += __shfl_xor_sync(0xffffffffu, dwb[j], o);
+    if (threadIdx.x < 4) s[threadIdx.x] = 0.0f;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) atomicAdd(&s[j], dwb[j]);
+    __syncthreads();
+    if (threadIdx.x < 3) atomicAdd(&gwb[threadIdx.x], s[threadIdx.x]);
+    if (threadIdx.x == 3) atomicAdd(loss, s[3]);
+}
+
+// Adam and the layers' weights, one pass: a thread takes the nine taps of a (co, ci) pair of
+// one layer (its parameters, gradient and moments are 36 consecutive bytes each), or one
+// bias or parameter of the output layer, updates them (lr = 0: leaves them) and writes the
+// forms the kernels read:
+//   wk[co][tap][ci]       the forward's K-major weights (bfloat16; the first layer's padding
+//                         channels keep the zeros they were created with)
+//   wt[ci][8 - tap][co]   the kernel flipped in both directions: the input gradient is a 3x3
+//                         convolution of dZ with these
+//   bias, wout            FP32 biases; the output layer's bfloat16-rounded weights as floats
+struct WeightTable {
+    int pair0[15];  // first pair of each layer; [14]: pairs of all layers
+    int bias0[15];  // first bias of each layer; [14]: biases of all layers
+    int woff[14], boff[14], cin[14], cout[14], cin_pad[14];
+    uint16_t* wk[14];
+    uint16_t* wt[14];
+    float* bias[14];
+    int out_off;  // 96 weights, then 3 biases
+    float* wout;
+};
+
+struct AdamArgs {
+    float *p, *m, *v;
+    const float* g;
+    float lr, b1, b2, eps, c1, c2;
+    int update;
+};
+
+__device__ __forceinline__ float adam_step(const AdamArgs& a, int i)
+{
+    float p = a.p[i];
+    if (a.update) {
+        const float gi = a.g[i];
+        const float mi = a.b1 * a.m[i] + (1.0f - a.b1) * gi;
+        const float vi = a.b2 * a.v[i] + (1.0f - a.b2) * gi * gi;
+        a.m[i] = mi;
+        a.v[i] = vi;
+        p -= a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+        a.p[i] = p;
+    }
+    return p;
+}
+
+__global__ void __launch_bounds__(256) weights_kernel(const __grid_constant__ WeightTable w, const AdamArgs a)
+{
+    int i = blockIdx.x * 256 + threadIdx.x;
+    if (i < w.pair0[14]) {
+        int l = 0;
+        while (i >= w.pair0[l + 1]) ++l;
+        i -= w.pair0[l];
+        const int cin = w.cin[l], cout = w.cout[l], cp = w.cin_pad[l];
+        const int co = i / cin, ci = i - co * cin;
+        const int base = w.woff[l] + i * 9;
+        uint16_t* wk = w.wk[l] + (size_t)co * 9 * cp + ci;
+        uint16_t* wt = w.wt[l] + (size_t)ci * 9 * cout + co;
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            const uint16_t b = f2bf(adam_step(a, base + t));
+            wk[t * cp] = b;
+            wt[(8 - t) * cout] = b;
+        }
+        return;
+    }
+    i -= w.pair0[14];
+    if (i < w.bias0[14]) {
+        int l = 0;
+        while (i >= w.bias0[l + 1]) ++l;
+        i -= w.bias0[l];
+        w.bias[l][i] = adam_step(a, w.boff[l] + i);
+        return;
+    }
+    i -= w.bias0[14];
+    if (i < 99) {
+        const float p = adam_step(a, w.out_off + i);
+        w.wout[i] = i < 96 ? bf2f(f2bf(p)) : p;
     }
 }
 
-__global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, long long n, float lr, float b1, float b2, float eps, float c1,
-                            float c2)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.0f - b1) * gi;
-        const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    }
-}
-
-// Forward weights: (cout, cin, 3, 3) -> K-major (cout, 9, cin_pad) bfloat16, zero padding.
-__global__ void fwd_weights_kernel(const float* __restrict__ W, int cout, int cin, int cin_pad, uint16_t* __restrict__ wk)
-{
-    const long long n = (long long)cout * 9 * cin_pad;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int ci = (int)(i % cin_pad);
-        const long long r = i / cin_pad;
-        const int tap = (int)(r % 9), co = (int)(r / 9);
-        wk[i] = ci < cin ? f2bf(W[((long long)co * cin + ci) * 9 + tap]) : (uint16_t)0;
-    }
-}
-
-// Backward weights: wt[ci][tap'][co] = W[co][ci][8 - tap'] (the kernel flipped in both
-// directions), bfloat16: the input gradient is then a 3x3 convolution of dZ.
-__global__ void bwd_weights_kernel(const float* __restrict__ W, int cout, int cin, uint16_t* __restrict__ wt)
-{
-    const long long n = (long long)cin * 9 * cout;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int co = (int)(i % cout);
-        const long long r = i / cout;
-        const int tap = (int)(r % 9), ci = (int)(r / 9);
-        wt[i] = f2bf(W[((long long)co * cin + ci) * 9 + (8 - tap)]);
-    }
-}
-
-// Output layer: bfloat16-rounded weights as floats, then the FP32 biases.
-__global__ void out_weights_kernel(const float* __restrict__ W, const float* __restrict__ b, float* __restrict__ wout)
-{
-    const int i = threadIdx.x;
-    if (i < 96) wout[i] = bf2f(f2bf(W[i]));
-    if (i < 3) wout[96 + i] = b[i];
-}
-
-int blocks_for(long long n, int per = 256) { return (int)std::min<long long>((n + per - 1) / per, 8192); }
+// Blocks of a grid-stride pass: at most about four waves, so that the blocks' closing atomics
+// on the same few sums stay few.
+int blocks_for(long long n) { return (int)std::min<long long>((n + 255) / 256, 608); }
 
 }  // namespace
 
@@ -258,10 +338,12 @@ struct Trainer {
     size_t np;
     float *params, *grads, *m, *v;
     size_t woff[14], boff[14], wout_off, bout_off;
+    WeightTable table;
     uint16_t* wt[14];
-    float* G[14];
-    uint16_t *dZ, *DX;
-    float *zero_bias, *rgb, *dzo, *loss;
+    // bfloat16 gradients: dZ of the current layer; DX[0]: its input gradient; DX[1..3]: those
+    // of the decoder levels' first layers (8, 10, 12), which two layers read
+    uint16_t *dZ, *DX[4];
+    float *zero_bias, *rgb, *loss;  // loss and nhole follow the gradients in memory
     float* ws;  // partial sums of the weight gradients
     int sms;
     int* nhole;
@@ -273,32 +355,30 @@ namespace {
 
 int layer_side(int i) { return i < 8 ? (64 >> (i / 2)) : (64 >> (2 - (i - 8) / 2)); }
 
+// Where layer i's input gradient lives (Trainer::DX).
+int dx_buffer(int i) { return i == 8 ? 1 : i == 10 ? 2 : i == 12 ? 3 : 0; }
+
 void trainer_free(Trainer* t)
 {
     if (!t) return;
     unet_free(t->net);
-    for (int i = 0; i < 14; ++i) {
-        cudaFree(t->wt[i]);
-        cudaFree(t->G[i]);
-    }
-    void* bufs[] = {t->params, t->grads, t->m, t->v, t->dZ, t->DX, t->zero_bias, t->rgb, t->dzo, t->loss, t->nhole, t->ws};
+    for (uint16_t* w : t->wt) cudaFree(w);
+    for (uint16_t* d : t->DX) cudaFree(d);
+    void* bufs[] = {t->params, t->grads, t->m, t->v, t->dZ, t->zero_bias, t->rgb, t->ws};
     for (void* b : bufs) cudaFree(b);
     delete t;
 }
 
-cudaError_t rebuild_weights(Trainer* t, cudaStream_t s)
+// The layers' weights from the parameters, after an Adam step if update.
+cudaError_t update_weights(Trainer* t, bool update, cudaStream_t s)
 {
-    UnetNet* n = t->net;
-    for (int i = 0; i < 14; ++i) {
-        const UnetLayer& L = n->conv[i];
-        const float* W = t->params + t->woff[i];
-        fwd_weights_kernel<<<blocks_for((long long)L.cout * 9 * L.cin_pad), 256, 0, s>>>(W, L.cout, L.cin, L.cin_pad,
-                                                                                       L.wk);
-        bwd_weights_kernel<<<blocks_for((long long)L.cin * 9 * L.cout), 256, 0, s>>>(W, L.cout, L.cin, t->wt[i]);
-        const cudaError_t e = cudaMemcpyAsync(L.bias, t->params + t->boff[i], L.cout * 4, cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess) return e;
+    AdamArgs a{t->params, t->m, t->v, t->grads, t->lr, t->b1, t->b2, t->eps, 1.0f, 1.0f, update ? 1 : 0};
+    if (update) {
+        a.c1 = 1.0f - std::pow(t->b1, (float)t->step);
+        a.c2 = 1.0f - std::pow(t->b2, (float)t->step);
     }
-    out_weights_kernel<<<1, 128, 0, s>>>(t->params + t->wout_off, t->params + t->bout_off, n->wout);
+    const int n = t->table.pair0[14] + t->table.bias0[14] + 99;
+    weights_kernel<<<(n + 255) / 256, 256, 0, s>>>(t->table, a);
     return cudaGetLastError();
 }
 
@@ -331,29 +411,48 @@ Trainer* trainer_create(const float* params, size_t np, int batch, float lr, flo
     t->wout_off = off;
     t->bout_off = off + 96;
     const size_t B = batch;
-    size_t dz_max = 0, dx_max = 0;
+    size_t dz_max = 0, dx_max[4] = {};
+    WeightTable& w = t->table;
     for (int i = 0; i < 14 && ok; ++i) {
         int cin, cout;
         unet_layer_dims(i, &cin, &cout);
         const size_t P = B * layer_side(i) * layer_side(i);
         dz_max = std::max(dz_max, P * cout);
-        dx_max = std::max(dx_max, P * (size_t)((cin + 31) / 32 * 32));
-        ok = cudaMalloc(&t->wt[i], (size_t)cin * 9 * cout * 2) == cudaSuccess &&
-             cudaMalloc(&t->G[i], P * cout * 4) == cudaSuccess;
+        size_t& dx = dx_max[dx_buffer(i)];
+        dx = std::max(dx, P * (size_t)cin);
+        ok = cudaMalloc(&t->wt[i], (size_t)cin * 9 * cout * 2) == cudaSuccess;
+        const UnetLayer& L = t->net->conv[i];
+        w.pair0[i + 1] = w.pair0[i] + cout * cin;
+        w.bias0[i + 1] = w.bias0[i] + cout;
+        w.woff[i] = (int)t->woff[i];
+        w.boff[i] = (int)t->boff[i];
+        w.cin[i] = cin;
+        w.cout[i] = cout;
+        w.cin_pad[i] = L.cin_pad;
+        w.wk[i] = L.wk;
+        w.wt[i] = t->wt[i];
+        w.bias[i] = L.bias;
+    }
+    if (ok) {
+        w.out_off = (int)t->wout_off;
+        w.wout = t->net->wout;
+        for (int k = 0; k < 4 && ok; ++k) ok = cudaMalloc(&t->DX[k], dx_max[k] * 2) == cudaSuccess;
     }
     if (ok)
-        ok = cudaMalloc(&t->params, np * 4) == cudaSuccess && cudaMalloc(&t->grads, np * 4) == cudaSuccess &&
+        ok = cudaMalloc(&t->params, np * 4) == cudaSuccess && cudaMalloc(&t->grads, (np + 2) * 4) == cudaSuccess &&
              cudaMalloc(&t->m, np * 4) == cudaSuccess && cudaMalloc(&t->v, np * 4) == cudaSuccess &&
-             cudaMalloc(&t->dZ, dz_max * 2) == cudaSuccess && cudaMalloc(&t->DX, dx_max * 2) == cudaSuccess &&
-             cudaMalloc(&t->zero_bias, 384 * 4) == cudaSuccess && cudaMalloc(&t->rgb, B * 4096 * 3 * 4) == cudaSuccess &&
-             cudaMalloc(&t->dzo, B * 4096 * 3 * 4) == cudaSuccess && cudaMalloc(&t->loss, 4) == cudaSuccess &&
-             cudaMalloc(&t->nhole, 4) == cudaSuccess &&
+             cudaMalloc(&t->dZ, dz_max * 2) == cudaSuccess && cudaMalloc(&t->zero_bias, 384 * 4) == cudaSuccess &&
+             cudaMalloc(&t->rgb, B * 4096 * 3 * 4) == cudaSuccess &&
              cudaMalloc(&t->ws, conv_dw_workspace(t->sms)) == cudaSuccess;
-    if (ok)
+    if (ok) {
+        t->loss = t->grads + np;
+        t->nhole = reinterpret_cast<int*>(t->grads + np + 1);
         ok = cudaMemcpy(t->params, params, np * 4, cudaMemcpyHostToDevice) == cudaSuccess &&
              cudaMemset(t->m, 0, np * 4) == cudaSuccess && cudaMemset(t->v, 0, np * 4) == cudaSuccess &&
-             cudaMemset(t->zero_bias, 0, 384 * 4) == cudaSuccess && cudaMemset(t->grads, 0, np * 4) == cudaSuccess &&
-             rebuild_weights(t, nullptr) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
+             cudaMemset(t->zero_bias, 0, 384 * 4) == cudaSuccess &&
+             cudaMemset(t->grads, 0, (np + 2) * 4) == cudaSuccess && update_weights(t, false, nullptr) == cudaSuccess &&
+             cudaDeviceSynchronize() == cudaSuccess;
+    }
     if (!ok) {
         cudaGetLastError();
         trainer_free(t);
@@ -369,46 +468,62 @@ cudaError_t trainer_step(Trainer* t, const void* x, const uint8_t* gt, const uin
 {
     UnetNet* n = t->net;
     const long long npx = (long long)B * 4096;
-    cudaError_t e = cudaMemsetAsync(t->grads, 0, t->np * 4, s);
-    for (int i = 0; i < 14 && e == cudaSuccess; ++i) {
-        int cin, cout;
-        unet_layer_dims(i, &cin, &cout);
-        e = cudaMemsetAsync(t->G[i], 0, (size_t)B * layer_side(i) * layer_side(i) * cout * 4, s);
-    }
-    if (e == cudaSuccess) e = cudaMemsetAsync(t->loss, 0, 4, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(t->nhole, 0, 4, s);
     const uint16_t* xin = static_cast<const uint16_t*>(x);
+    // gradients, loss and hole count
+    cudaError_t e = cudaMemsetAsync(t->grads, 0, (t->np + 2) * 4, s);
     if (e == cudaSuccess) e = unet_run(n, xin, B, nullptr, NetOut{nullptr, nullptr}, s);
     if (e == cudaSuccess) e = unet_output_rgb(n, B, t->rgb, s);
     if (e != cudaSuccess) return e;
     count_holes_kernel<<<blocks_for(npx), 256, 0, s>>>(hole, npx, t->nhole);
-    loss_kernel<<<blocks_for(npx), 256, 0, s>>>(t->rgb, gt, hole, npx, t->nhole, t->dzo, t->loss);
-    out_bwd_kernel<<<blocks_for(npx), 256, 0, s>>>(n->d0b, n->wout, t->dzo, npx, t->G[13], t->grads + t->wout_off,
-                                                  t->grads + t->bout_off);
+    out_bwd_kernel<<<blocks_for(4 * npx), 256, 0, s>>>(t->rgb, gt, hole, npx, t->nhole, n->d0b, n->wout, t->dZ,
+                                                      t->grads + t->wout_off, t->grads + t->bout_off,
+                                                      t->grads + t->boff[13], t->loss);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
-    // per layer: forward input X (channel stride), output Y (stride, offset, upsampled copy)
+    // per layer: forward input X (channel stride), output Y (stride, offset)
     struct IO {
         const uint16_t* x;
         int xcs;
         const uint16_t* y;
-        int ycs, ycoff, yup;
+        int ycs, ycoff;
     };
-    const IO io[14] = {{xin, 32, n->e0a, 32, 0, 0},      {n->e0a, 32, n->cat0, 96, 0, 0},
-                       {n->p0, 32, n->e1a, 64, 0, 0},    {n->e1a, 64, n->cat1, 192, 0, 0},
-                       {n->p1, 64, n->e2a, 128, 0, 0},   {n->e2a, 128, n->cat2, 384, 0, 0},
-                       {n->p2, 128, n->e3a, 256, 0, 0},  {n->e3a, 256, n->cat2, 384, 128, 1},
-                       {n->cat2, 384, n->d2a, 128, 0, 0}, {n->d2a, 128, n->cat1, 192, 64, 1},
-                       {n->cat1, 192, n->d1a, 64, 0, 0}, {n->d1a, 64, n->cat0, 96, 32, 1},
-                       {n->cat0, 96, n->d0a, 32, 0, 0},  {n->d0a, 32, n->d0b, 32, 0, 0}};
+    const IO io[14] = {{xin, 32, n->e0a, 32, 0},       {n->e0a, 32, n->cat0, 96, 0},
+                       {n->p0, 32, n->e1a, 64, 0},     {n->e1a, 64, n->cat1, 192, 0},
+                       {n->p1, 64, n->e2a, 128, 0},    {n->e2a, 128, n->cat2, 384, 0},
+                       {n->p2, 128, n->e3a, 256, 0},   {n->e3a, 256, n->cat2, 384, 128},
+                       {n->cat2, 384, n->d2a, 128, 0}, {n->d2a, 128, n->cat1, 192, 64},
+                       {n->cat1, 192, n->d1a, 64, 0},  {n->d1a, 64, n->cat0, 96, 32},
+                       {n->cat0, 96, n->d0a, 32, 0},   {n->d0a, 32, n->d0b, 32, 0}};
+    // who reads layer i's output: the form of dZ, and the consumer's input gradient
+    struct Route {
+        int kind, from, off, pooled;  // consumer's layer, channel offset in its input, pooled consumer
+    };
+    const Route route[13] = {{kDirect, 1, 0, 0},  {kPooled, 12, 0, 2},  {kDirect, 3, 0, 0},  {kPooled, 10, 0, 4},
+                             {kDirect, 5, 0, 0},  {kPooled, 8, 0, 6},   {kDirect, 7, 0, 0},  {kUp, 8, 128, 0},
+                             {kDirect, 9, 0, 0},  {kUp, 10, 64, 0},     {kDirect, 11, 0, 0}, {kUp, 12, 32, 0},
+                             {kDirect, 13, 0, 0}};
     for (int i = 13; i >= 0; --i) {
         const UnetLayer& L = n->conv[i];
         const int side = layer_side(i);
         const long long P = (long long)B * side * side;
-        const long long nz = P * L.cout;
-        relu_mask_kernel<<<blocks_for(nz), 256, 0, s>>>(t->G[i], io[i].y, io[i].ycs, io[i].ycoff, io[i].yup, side,
-                                                        L.cout, nz, t->dZ, t->grads + t->boff[i]);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (i < 13) {
+            const Route& r = route[i];
+            const uint16_t* D = t->DX[dx_buffer(r.from)];
+            const int dcs = n->conv[r.from].cin;
+            const long long items = P * (L.cout / 8) / (r.kind == kPooled ? 4 : 1);
+            const int blocks = blocks_for(items);
+            float* gb = t->grads + t->boff[i];
+            if (r.kind == kDirect)
+                dz_kernel<kDirect><<<blocks, 256, 0, s>>>(D, dcs, r.off, nullptr, io[i].y, io[i].ycs, io[i].ycoff, side,
+                                                          L.cout, items, t->dZ, gb);
+            else if (r.kind == kUp)
+                dz_kernel<kUp><<<blocks, 256, 0, s>>>(D, dcs, r.off, nullptr, io[i].y, io[i].ycs, io[i].ycoff, side,
+                                                      L.cout, items, t->dZ, gb);
+            else
+                dz_kernel<kPooled><<<blocks, 256, 0, s>>>(D, dcs, r.off, t->DX[dx_buffer(r.pooled)], io[i].y, io[i].ycs,
+                                                          io[i].ycoff, side, L.cout, items, t->dZ, gb);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
         e = conv_dw_launch(t->dZ, io[i].x, io[i].xcs, B, side, L.cin, L.cout, t->sms, t->ws, t->grads + t->woff[i], s);
         if (e != cudaSuccess) return e;
         if (i == 0) break;
@@ -416,49 +531,16 @@ cudaError_t trainer_step(Trainer* t, const void* x, const uint8_t* gt, const uin
         for (int c0 = 0; c0 < L.cin && e == cudaSuccess;) {
             const int rem = L.cin - c0;
             const int w = rem >= 256 ? 256 : rem >= 128 ? 128 : rem >= 64 ? 64 : 32;
-            e = unet_conv3x3(ConvCall{t->dZ, t->wt[i] + (size_t)c0 * 9 * L.cout, t->DX, t->zero_bias, nullptr, nullptr, B,
-                                      side, side, L.cout, w, L.cin, c0, 0, 0},
+            e = unet_conv3x3(ConvCall{t->dZ, t->wt[i] + (size_t)c0 * 9 * L.cout, t->DX[dx_buffer(i)], t->zero_bias,
+                                      nullptr, nullptr, B, side, side, L.cout, w, L.cin, c0, 0, 0},
                              s);
             c0 += w;
         }
         if (e != cudaSuccess) return e;
-        // route the input gradient to the producers' output gradients
-        auto add = [&](int dst, int coff, int C) {
-            const long long nn = P * C;
-            add_kernel<<<blocks_for(nn), 256, 0, s>>>(t->G[dst], t->DX, L.cin, coff, C, nn);
-        };
-        auto upb = [&](int dst, int coff, int C) {
-            const long long nn = P / 4 * C;
-            upbwd_kernel<<<blocks_for(nn), 256, 0, s>>>(t->G[dst], t->DX, L.cin, coff, side / 2, C, nn);
-        };
-        auto pool = [&](int dst, const uint16_t* y, int ycs) {
-            const long long nn = P * L.cin;
-            poolbwd_kernel<<<blocks_for(nn), 256, 0, s>>>(t->G[dst], t->DX, y, ycs, side, L.cin, nn);
-        };
-        switch (i) {
-            case 13: add(12, 0, 32); break;
-            case 12: add(1, 0, 32); upb(11, 32, 64); break;
-            case 11: add(10, 0, 64); break;
-            case 10: add(3, 0, 64); upb(9, 64, 128); break;
-            case 9: add(8, 0, 128); break;
-            case 8: add(5, 0, 128); upb(7, 128, 256); break;
-            case 7: add(6, 0, 256); break;
-            case 6: pool(5, n->cat2, 384); break;
-            case 5: add(4, 0, 128); break;
-            case 4: pool(3, n->cat1, 192); break;
-            case 3: add(2, 0, 64); break;
-            case 2: pool(1, n->cat0, 96); break;
-            case 1: add(0, 0, 32); break;
-        }
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (t->lr != 0.0f) {
         ++t->step;
-        const float c1 = 1.0f - std::pow(t->b1, (float)t->step), c2 = 1.0f - std::pow(t->b2, (float)t->step);
-        adam_kernel<<<blocks_for((long long)t->np), 256, 0, s>>>(t->params, t->grads, t->m, t->v, (long long)t->np,
-                                                                t->lr, t->b1, t->b2, t->eps, c1, c2);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        e = rebuild_weights(t, s);
+        e = update_weights(t, true, s);
     }
     return e;
 }
