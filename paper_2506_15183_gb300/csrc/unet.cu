@@ -54,21 +54,23 @@ namespace {
 
 __device__ unsigned g_unet_status;  // kernel-side failures of this file's kernels
 
-constexpr int kStages = 4;
+constexpr int kStages = 4;     // one-tile form where several CTAs share an SM
+constexpr int kMaxStages = 12;  // either form
 constexpr int kABytes = kTileM * kKc * 2;  // 8 KB
 
 struct ConvArgs {
     int T, H, W;          // tiles and their size (the output has the input's size)
     int Cin, Cout;        // Cin: channels of the input tensor, a multiple of 32
+    int bn;               // output channels of a CTA: Cout, or a part of it (blockIdx.y) on small grids
     const float* bias;    // Cout
     __nv_bfloat16* y;     // NHWC output, channel stride y_cstride, channels from y_coff
     int y_cstride, y_coff;
     int upsample;         // 1: pixel (yy, xx) goes to (2yy + a, 2xx + b), a, b in {0, 1}
     int relu;
-    int ncols;            // tensor-memory columns allocated (a power of two >= mt Cout, >= 32)
+    int ncols;            // tensor-memory columns allocated (a power of two >= mt bn, >= 32)
     const int* count;     // optional: tiles at or after *count are skipped (the tile list's length)
     uint16_t* pool;       // optional (16-pixel rows only): T x H/2 x W/2 x Cout, the 2x2 maximum of the output
-    int mt, stages;       // halo form: 128-pixel accumulators per CTA and copy stages
+    int mt, stages;       // 128-pixel accumulators per CTA (halo form) and copy stages
 };
 
 // The epilogue of both forms: the CTA's mt accumulators of 128 pixels (pixel i of
@@ -76,7 +78,7 @@ struct ConvArgs {
 // back 32 channels at a time, the bias added, ReLU applied, rounded to BF16 and staged in
 // shared memory (`stg`, 1024-aligned: the copy stages, free once every MMA has
 // completed), one slice of 64 bytes per pixel for each 32 channels, in the 64-byte
-// swizzle (16-byte chunk k of pixel p at p 64 + (k ^ (p / 2 mod 4)) 16, so a warp's
+// swizzle (bias: the CTA's bn values; 16-byte chunk k of pixel p at p 64 + (k ^ (p / 2 mod 4)) 16, so a warp's
 // writes meet no bank twice).  One thread then writes every slice with TMA tensor
 // stores: a box {32 channels, W, rows, images} at channel y_coff + 32 s, or, for the
 // nearest upsampling, the same box four times through a 5-D view of the output that
@@ -85,14 +87,15 @@ struct ConvArgs {
 __device__ __forceinline__ void epilogue_store(const ConvArgs& a, const CUtensorMap* tmY, uint32_t tmem,
                                                unsigned char* stg, const float* bias, int mt, int n0, int y0)
 {
+    const int nb = blockIdx.y * a.bn;  // the CTA's first output channel
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m = warp * 32 + lane;  // this thread's pixel of each accumulator = its TMEM lane
     const int slice = mt * kTileM * 64;
-    for (int c0 = 0; c0 < a.Cout; c0 += 32) {
+    for (int c0 = 0; c0 < a.bn; c0 += 32) {
         unsigned char* sl = stg + (c0 >> 5) * slice;
         for (int j = 0; j < mt; ++j) {
             uint32_t r[32];
-            tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(j * a.Cout + c0), r);
+            tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(j * a.bn + c0), r);
             uint4 q[4];
             uint32_t* qw = reinterpret_cast<uint32_t*>(q);
 #pragma unroll
@@ -121,7 +124,7 @@ __device__ __forceinline__ void epilogue_store(const ConvArgs& a, const CUtensor
                 const size_t pp = ((size_t)n0 * (a.H >> 1) + (yy >> 1)) * 8 + ((lane & 15) >> 1);
                 // the four lanes of a pooled pixel write 16 bytes each
                 const int k = (lane & 1) + 2 * (lane >> 4);
-                reinterpret_cast<uint4*>(a.pool + pp * a.Cout + c0)[k] =
+                reinterpret_cast<uint4*>(a.pool + pp * a.Cout + nb + c0)[k] =
                     k == 0 ? q[0] : k == 1 ? q[1] : k == 2 ? q[2] : q[3];
             }
         }
@@ -129,13 +132,13 @@ __device__ __forceinline__ void epilogue_store(const ConvArgs& a, const CUtensor
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the writes, seen by the copy engine
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int c0 = 0; c0 < a.Cout; c0 += 32) {
+        for (int c0 = 0; c0 < a.bn; c0 += 32) {
             const unsigned char* sl = stg + (c0 >> 5) * slice;
             if (!a.upsample) {
-                tma_store_4d(tmY, sl, a.y_coff + c0, 0, y0, n0);
+                tma_store_4d(tmY, sl, a.y_coff + nb + c0, 0, y0, n0);
             } else {
 #pragma unroll
-                for (int ab = 0; ab < 4; ++ab) tma_store_5d(tmY, sl, a.y_coff + c0, ab & 1, 0, ab >> 1, n0 * a.H + y0);
+                for (int ab = 0; ab < 4; ++ab) tma_store_5d(tmY, sl, a.y_coff + nb + c0, ab & 1, 0, ab >> 1, n0 * a.H + y0);
             }
         }
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
@@ -151,17 +154,18 @@ __global__ void __launch_bounds__(128, 1)
     if (a.count && (int)((blockIdx.x * kTileM) / (a.H * a.W)) >= *a.count) return;  // no such tile (uniform)
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                            ~static_cast<uintptr_t>(1023));
-    const int b_bytes = a.Cout * kKc * 2;
+    const int S = a.stages, nb = blockIdx.y * a.bn;
+    const int b_bytes = a.bn * kKc * 2;
     const int stage_bytes = kABytes + ((b_bytes + 1023) & ~1023);
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * stage_bytes);
-    uint64_t* empty = full + kStages;
-    uint64_t* done = empty + kStages;
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * stage_bytes);
+    uint64_t* empty = full + S;
+    uint64_t* done = empty + S;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
     volatile int* counts = reinterpret_cast<volatile int*>(tslot + 1);  // [0] issued, [1] consumed
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -192,8 +196,8 @@ __global__ void __launch_bounds__(128, 1)
     if (warp == 0 && lane == 0) {  // copies
         int k = 0;
         for (; k < nk; ++k) {
-            const int s = k % kStages;
-            if (!mbar_wait(&empty[s], ((k / kStages) & 1) ^ 1, deadline)) {
+            const int s = k % S;
+            if (!mbar_wait(&empty[s], ((k / S) & 1) ^ 1, deadline)) {
                 atomicOr(&g_unet_status, kUnetTimeout);
                 break;
             }
@@ -202,25 +206,30 @@ __global__ void __launch_bounds__(128, 1)
             unsigned char* sa = smem + s * stage_bytes;
             mbar_expect_tx(&full[s], (uint32_t)(kABytes + b_bytes));
             tma_load_4d(sa, &tmA, &full[s], cb * kKc, dx - 1, y0 + dy - 1, n0);
-            tma_load_2d(sa + kABytes, &tmB, &full[s], tap * a.Cin + cb * kKc, 0);
+            tma_load_2d(sa + kABytes, &tmB, &full[s], tap * a.Cin + cb * kKc, nb);
             counts[0] = k + 1;
         }
-    } else if (warp == 1 && lane == 0) {  // MMAs
-        const uint32_t idesc = idesc_bf16(a.Cout);
+    } else if (warp == 1) {  // MMAs: the whole warp runs the loop, one lane issues
+        const uint32_t idesc = idesc_bf16(a.bn), el = elect_one();
+        const uint64_t dbase = desc_sw64(smem_u32(smem));
+        int s = 0, ph = 0;
         for (int k = 0; k < nk; ++k) {
-            const int s = k % kStages;
-            if (!mbar_wait(&full[s], (k / kStages) & 1, deadline)) {
-                atomicOr(&g_unet_status, kUnetTimeout);
+            if (!mbar_wait_warp(&full[s], ph, deadline)) {
+                if (el) atomicOr(&g_unet_status, kUnetTimeout);
                 break;
             }
             tc_fence_after();
-            const uint32_t sa = smem_u32(smem + s * stage_bytes), sb = sa + kABytes;
-            mma_bf16(tmem, desc_sw64(sa), desc_sw64(sb), idesc, k > 0 ? 1u : 0u);
-            mma_bf16(tmem, desc_sw64(sa + 32), desc_sw64(sb + 32), idesc, 1u);
-            mma_commit(&empty[s]);
-            counts[1] = k + 1;
+            const uint64_t da = dbase + (uint64_t)((uint32_t)(s * stage_bytes) >> 4), db = da + (kABytes >> 4);
+            mma_bf16_elected(el, tmem, da, db, idesc, k > 0 ? 1u : 0u);
+            mma_bf16_elected(el, tmem, da + 2, db + 2, idesc, 1u);
+            mma_commit_elected(el, &empty[s]);
+            if (el) counts[1] = k + 1;
+            if (++s == S) {
+                s = 0;
+                ph ^= 1;
+            }
         }
-        mma_commit(done);  // arrives once every MMA issued above has completed
+        mma_commit_elected(el, done);  // arrives once every MMA issued above has completed
     }
     __syncwarp();
 
@@ -228,14 +237,14 @@ __global__ void __launch_bounds__(128, 1)
     if (!ok) atomicOr(&g_unet_status, kUnetTimeout);
     if (ok) {
         tc_fence_after();
-        epilogue_store(a, &tmY, tmem, smem, a.bias, 1, n0, y0);
+        epilogue_store(a, &tmY, tmem, smem, a.bias + nb, 1, n0, y0);
     }
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0) {  // copies still in flight after a timeout: wait for them (bounded)
         const uint64_t d2 = globaltimer() + kWaitNs;
         for (int k = counts[1]; k < counts[0]; ++k)
-            if (!mbar_wait(&full[k % kStages], (k / kStages) & 1, d2)) break;
+            if (!mbar_wait(&full[k % S], (k / S) & 1, d2)) break;
     }
     __syncthreads();
     if (warp == 0) {
@@ -256,8 +265,6 @@ __global__ void __launch_bounds__(128, 1)
 // for W a multiple of 8, and the three dy taps share one copy.  Activation bytes copied
 // per output pixel: 3 (R + 2) / R boxes instead of 9; weight bytes: 1 / mt of the
 // one-tile form.
-constexpr int kMaxStages = 4;
-
 __global__ void __launch_bounds__(128, 1)
     conv3x3_halo(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmY, const ConvArgs a, int nbands)
@@ -274,7 +281,7 @@ __global__ void __launch_bounds__(128, 1)
                                                            ~static_cast<uintptr_t>(1023));
     const int a_bytes = (R + 2) * a.W * kKc * 2;
     const int a_span = (a_bytes + 1023) & ~1023;
-    const int b_tap = a.Cout * kKc * 2;
+    const int b_tap = a.bn * kKc * 2, nb = blockIdx.y * a.bn;
     const int stage_bytes = a_span + ((3 * b_tap + 1023) & ~1023);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * stage_bytes);
     uint64_t* empty = full + kMaxStages;
@@ -282,7 +289,7 @@ __global__ void __launch_bounds__(128, 1)
     uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
     volatile int* counts = reinterpret_cast<volatile int*>(tslot + 1);  // [0] issued, [1] consumed, [2] abort
     float* sbias = reinterpret_cast<float*>(smem + S * stage_bytes + 1024);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
     const int cb_n = a.Cin / kKc;
     const int nk = 3 * cb_n;  // K steps of a band: (channel block, dx)
@@ -296,7 +303,7 @@ __global__ void __launch_bounds__(128, 1)
         tma_load_4d(sa, &tmA, &full[s], cb * kKc, dx - 1, y0 - 1, n0);
 #pragma unroll
         for (int dy = 0; dy < 3; ++dy)
-            tma_load_2d(sa + a_span + dy * b_tap, &tmB, &full[s], (3 * dy + dx) * a.Cin + cb * kKc, 0);
+            tma_load_2d(sa + a_span + dy * b_tap, &tmB, &full[s], (3 * dy + dx) * a.Cin + cb * kKc, nb);
         counts[0] = kk + 1;
     };
     const int first = nk < S ? nk : S;  // copies issued before the CTA-wide barrier
@@ -323,7 +330,7 @@ __global__ void __launch_bounds__(128, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    for (int c = threadIdx.x; c < a.Cout; c += blockDim.x) sbias[c] = __ldg(a.bias + c);
+    for (int c = threadIdx.x; c < a.bn; c += blockDim.x) sbias[c] = __ldg(a.bias + nb + c);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -336,7 +343,7 @@ __global__ void __launch_bounds__(128, 1)
     // band's last K step, and the next band's first copy (into the other stage) is issued
     // by the MMA thread once that stage is free, so it lands during the last MMAs and the
     // epilogue.
-    const bool early = mt * kTileM * a.Cout * 2 <= stage_bytes && S >= 2;
+    const bool early = mt * kTileM * a.bn * 2 <= stage_bytes && S >= 2;
     int it = 0;
     for (int band = blockIdx.x; band < live; band += gridDim.x, ++it) {
         const int n0 = band / bands_per_tile, y0 = (band - n0 * bands_per_tile) * R;
@@ -351,18 +358,21 @@ __global__ void __launch_bounds__(128, 1)
                 }
                 issue(kk, n0, y0);
             }
-        } else if (warp == 1 && lane == 0) {  // MMAs
+        } else if (warp == 1) {  // MMAs: the whole warp runs the loop, one lane issues
             // Descriptors: a stage's bases plus constants in the 16-byte start-address
             // field (the smem window is below 256 KB, so the field never carries over).
-            const uint32_t idesc = idesc_bf16(a.Cout);
+            const uint32_t idesc = idesc_bf16(a.bn), el = elect_one();
             const uint64_t dbase = desc_sw64(smem_u32(smem));
             const uint32_t aW = (uint32_t)a.W * 4u, aT = (uint32_t)kTileM * 4u, bT = (uint32_t)b_tap >> 4;
-            const uint32_t d1 = tmem + (uint32_t)a.Cout;
+            const uint32_t d1 = tmem + (uint32_t)a.bn;
+            bool run = true;
             for (int k = 0; k < nk; ++k) {
                 const int kk = it * nk + k, s = kk % S;
-                if (!mbar_wait(&full[s], (kk / S) & 1, deadline)) {
-                    atomicOr(&g_unet_status, kUnetTimeout);
-                    counts[2] = 1;
+                if (!(run = mbar_wait_warp(&full[s], (kk / S) & 1, deadline))) {
+                    if (el) {
+                        atomicOr(&g_unet_status, kUnetTimeout);
+                        counts[2] = 1;
+                    }
                     break;
                 }
                 tc_fence_after();
@@ -373,19 +383,19 @@ __global__ void __launch_bounds__(128, 1)
                     const uint64_t bt = db + dy * bT;
                     const uint64_t a0 = da + dy * aW, a1 = a0 + aT;
                     const uint32_t acc = (k > 0 || dy > 0) ? 1u : 0u;
-                    mma_bf16(tmem, a0, bt, idesc, acc);
-                    mma_bf16(tmem, a0 + 2, bt + 2, idesc, 1u);
-                    mma_bf16(d1, a1, bt, idesc, acc);
-                    mma_bf16(d1, a1 + 2, bt + 2, idesc, 1u);
+                    mma_bf16_elected(el, tmem, a0, bt, idesc, acc);
+                    mma_bf16_elected(el, tmem, a0 + 2, bt + 2, idesc, 1u);
+                    mma_bf16_elected(el, d1, a1, bt, idesc, acc);
+                    mma_bf16_elected(el, d1, a1 + 2, bt + 2, idesc, 1u);
                 }
-                mma_commit(&empty[s]);
-                counts[1] = kk + 1;
+                mma_commit_elected(el, &empty[s]);
+                if (el) counts[1] = kk + 1;
             }
-            mma_commit(done);  // arrives once every MMA issued above has completed
+            mma_commit_elected(el, done);  // arrives once every MMA issued above has completed
             // early: the next band's first copy, into the stage the second-to-last K step
             // frees, while this band's last MMAs run
             const int next = band + (int)gridDim.x;
-            if (early && next < live && !counts[2]) {
+            if (early && next < live && run && el) {
                 const int kk = (it + 1) * nk, s = kk % S;
                 const int n1 = next / bands_per_tile, y1 = (next - n1 * bands_per_tile) * R;
                 if (mbar_wait(&empty[s], ((kk / S) & 1) ^ 1, deadline)) issue(kk, n1, y1);
@@ -447,11 +457,23 @@ EncodeTiled tensor_map_encoder()
 
 namespace {
 
-size_t conv_smem_bytes(int cout)
+// One-tile form: bytes of one copy stage, and of a CTA.
+int conv_stage_bytes(int bn) { return kABytes + ((bn * kKc * 2 + 1023) & ~1023); }
+
+size_t conv_smem_bytes(int bn, int stages)
 {
-    const int b_bytes = cout * kKc * 2;
-    const int stage = kABytes + ((b_bytes + 1023) & ~1023);
-    return 1024 + (size_t)kStages * stage + (2 * kStages + 1) * 8 + 16;
+    return 1024 + (size_t)stages * conv_stage_bytes(bn) + (2 * stages + 1) * 8 + 16;
+}
+
+// Output channels per CTA where `ctas` CTAs with all Cout would leave SMs idle: halved while
+// twice as many CTAs still get an SM of their own.  Each part runs the same K steps (its sums
+// are the same), but its copies are smaller, and a lone CTA's ring can be as deep as its SM's
+// shared memory: on few tiles these layers wait for their copies.
+int split_channels(int Cout, long long ctas, int sms)
+{
+    int bn = Cout;
+    while (bn > 32 && 2 * ctas * (Cout / bn) <= sms) bn /= 2;
+    return bn;
 }
 
 // Halo form: bytes of one copy stage (activation box of R + 2 rows, three weight boxes).
@@ -554,6 +576,17 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
     EncodeTiled enc = tensor_map_encoder();
     if (!enc) return cudaErrorNotSupported;
 
+    // the form, and the output channels of a CTA
+    const int sms = sm_count();
+    int mt = 0, stages = 0;
+    if (nb == 1) halo_shape(H, W, Cout, &mt, &stages);
+    if (mt && conv_rows_takes(H, W, Cout)) return conv_rows_launch(call, sms, kSmemPerBlock, stream);
+    // the output layer rides on the row form only; the other forms pool 16-pixel rows
+    if (call.rgb || call.frames || (call.pool && W != 16)) return cudaErrorInvalidValue;
+    const long long ctas = pixels / (std::max(mt, 1) * kTileM);
+    const int bn = split_channels(Cout, ctas, sms);
+    const bool alone = ctas * (Cout / bn) <= sms;  // every CTA has an SM of its own
+
     CUtensorMap ta, tb;
     const cuuint64_t adim[4] = {(cuuint64_t)Cin, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)T};
     const cuuint64_t astr[3] = {(cuuint64_t)Cin * 2, (cuuint64_t)W * Cin * 2, (cuuint64_t)H * W * Cin * 2};
@@ -565,7 +598,7 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
         return cudaErrorInvalidValue;
     const cuuint64_t bdim[2] = {(cuuint64_t)9 * Cin, (cuuint64_t)Cout};
     const cuuint64_t bstr[1] = {(cuuint64_t)9 * Cin * 2};
-    const cuuint32_t bbox[2] = {(cuuint32_t)kKc, (cuuint32_t)Cout};
+    const cuuint32_t bbox[2] = {(cuuint32_t)kKc, (cuuint32_t)bn};
     if (enc(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(wk), bdim, bstr, bbox, one4,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -605,17 +638,12 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
     a.y_coff = y_coff;
     a.upsample = upsample;
     a.relu = call.relu;
-    a.ncols = Cout < 32 ? 32 : Cout;
+    a.bn = bn;
+    a.ncols = bn;
     a.count = call.count;
     a.pool = static_cast<uint16_t*>(call.pool);
-    a.mt = 0;
-    a.stages = kStages;
-    int mt = 0, stages = 0;
-    if (nb == 1) halo_shape(H, W, Cout, &mt, &stages);
-    if (mt && conv_rows_takes(H, W, Cout))
-        return conv_rows_launch(call, sm_count(), kSmemPerBlock, stream);
-    // the output layer rides on the row form only; the other forms pool 16-pixel rows
-    if (call.rgb || call.frames || (call.pool && W != 16)) return cudaErrorInvalidValue;
+    a.mt = mt;
+    const unsigned parts = (unsigned)(Cout / bn);
     if (mt) {
         const int rows = mt * kTileM / W;
         CUtensorMap th;
@@ -626,37 +654,29 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
             return cudaErrorInvalidValue;
         CUtensorMap ty;
         if (!y_map(&ty, rows, 1)) return cudaErrorInvalidValue;
-        a.mt = mt;
+        const int stage = halo_stage_bytes(W, rows, bn);
+        a.ncols = mt * bn;
         a.stages = stages;
-        int nc = 32;
-        while (nc < mt * Cout) nc *= 2;
-        a.ncols = nc;
-        static bool halo_configured = false;
-        if (!halo_configured) {
-            const cudaError_t e =
-                cudaFuncSetAttribute(conv3x3_halo, cudaFuncAttributeMaxDynamicSharedMemorySize, kHaloSmemBudget);
-            if (e != cudaSuccess) return e;
-            halo_configured = true;
-        }
-        const size_t hsmem = halo_smem_bytes(halo_stage_bytes(W, rows, Cout), stages);
+        if (alone)
+            while (a.stages < kMaxStages && halo_smem_bytes(stage, a.stages + 1) <= (size_t)kSmemPerBlock) ++a.stages;
+        const cudaError_t e =
+            cudaFuncSetAttribute(conv3x3_halo, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerBlock);
+        if (e != cudaSuccess) return e;
+        const size_t hsmem = halo_smem_bytes(stage, a.stages);
         // as many CTAs as fit at once (shared memory; registers allow 5), each walking bands
-        const int nbands = (int)(pixels / (mt * kTileM));
         const int per_sm = std::min(5, (int)(kSmemPerSm / (hsmem + 1024)));
-        const int grid = std::min(nbands, std::max(per_sm, 1) * sm_count());
-        conv3x3_halo<<<(unsigned)grid, 128, hsmem, stream>>>(th, tb, ty, a, nbands);
+        const long long grid = std::min<long long>(ctas, (long long)std::max(per_sm, 1) * sms);
+        conv3x3_halo<<<dim3((unsigned)grid, parts), 128, hsmem, stream>>>(th, tb, ty, a, (int)ctas);
         return cudaGetLastError();
     }
-    const size_t smem = conv_smem_bytes(Cout);
-    static bool configured = false;
-    if (!configured) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(conv3x3_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_smem_bytes(256));
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    a.stages = kStages;
+    if (alone)
+        while (a.stages < kMaxStages && conv_smem_bytes(bn, a.stages + 1) <= (size_t)kSmemPerBlock) ++a.stages;
+    const cudaError_t e = cudaFuncSetAttribute(conv3x3_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerBlock);
+    if (e != cudaSuccess) return e;
     CUtensorMap ty;
     if (!y_map(&ty, hb, nb)) return cudaErrorInvalidValue;
-    conv3x3_tc<<<(unsigned)(pixels / kTileM), 128, smem, stream>>>(ta, tb, ty, a);
+    conv3x3_tc<<<dim3((unsigned)ctas, parts), 128, conv_smem_bytes(bn, a.stages), stream>>>(ta, tb, ty, a);
     return cudaGetLastError();
 }
 
