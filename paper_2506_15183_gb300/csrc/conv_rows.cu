@@ -8,8 +8,8 @@
 // their input, so here they share the MMA: M is one image row (128 / W images side by
 // side, so the lanes of an accumulator are the same pixels of every row), the accumulators
 // of R rows lie next to each other in tensor memory, and input row r is multiplied once
-// with the weights of taps dy = 2, 1, 0 (N = 3 Cout) into the accumulators of rows r - 1, r,
-// r + 1: 56 cycles where three MMAs took 164 (N = 96), 96 where they took 164 (N = 192).
+// with the weights of taps dy = 0, 1, 2 (N = 3 Cout) into the accumulators of rows r + 1, r,
+// r - 1 (later rows lie in lower columns): 56 cycles where three MMAs took 164 (N = 96), 96 where they took 164 (N = 192).
 //
 // The kernel columns share the copy of a row as well: tap dx reads the same shared-memory
 // row from a start one pixel (64 bytes) to the left or right (the swizzle is a function
@@ -21,8 +21,9 @@
 // Per output element the products are accumulated in the order (channel block, dx, dy,
 // K half) of conv3x3_halo, so both forms give the same bits.
 //
-// One CTA per SM walks units of (image group, R rows).  Warp 0 streams rows (8 KB each) and
-// weights, warp 1 issues the MMAs, warps 2-5 read back one of two accumulator sets (256
+// One CTA per SM walks units of (image group, R rows).  Warp 0 streams rows (two per
+// copy, 16 KB: a wait, an expect and a copy cost the issuing thread 300-450 cycles whatever
+// the size) and weights (nine taps per copy), warp 1 issues the MMAs, warps 2-5 read back one of two accumulator sets (256
 // columns each) while the other is being filled, zero it for its next use, and store: each
 // warp stages its 32 pixels of two rows and writes them with its own TMA store.  Where the
 // next level follows, the 2x2 maximum of the rows a warp holds goes to the pooled tensor
@@ -49,15 +50,16 @@ namespace {
 __device__ unsigned g_rows_status;  // waits that ran out in this file's kernel
 
 constexpr int kRowBytes = kTileM * kKc * 2;     // one row of 128 pixels x 32 channels
+constexpr int kPairBytes = 2 * kRowBytes;       // rows are copied two at a time
 constexpr int kAccCols = 256;                   // tensor-memory columns of an accumulator set
-constexpr int kMaxRows = 22;                    // row slots (bounds the barrier array)
+constexpr int kMaxPairs = 11;                   // row-pair slots (bounds the barrier array)
 constexpr int kStageBytes = 2 * 32 * kKc * 2;   // a warp's 32 pixels of two rows, 32 channels
 constexpr int kStores = 4 * 2 * kStageBytes;    // two staging buffers for each of four warps
 constexpr int kRowsThreads = 192;
 
 struct RowsArgs {
     int T, H, W, Cin;
-    int nrows;         // row slots
+    int pairs;         // row-pair slots
     int wslots;        // weight slots (9 taps of one channel block each); resident when wslots == Cin / 32
     int y_coff, upsample, relu;
     const float* bias;
@@ -94,7 +96,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
                  const __grid_constant__ CUtensorMap tmY, const RowsArgs a, const __grid_constant__ Frames ft)
 {
     extern __shared__ unsigned char smem_raw[];
-    const int W = a.W, H = a.H, NR = a.nrows, WS = a.wslots;
+    const int W = a.W, H = a.H, NP = a.pairs, WS = a.wslots;
     const int nimg = kTileM / W, bands = H / R;
     const int cb_n = a.Cin / kKc;
     const int tiles = a.count ? min(a.T, *a.count) : a.T;
@@ -105,8 +107,8 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
                                                            ~static_cast<uintptr_t>(1023));
     // 1 KB of barriers first: the row before slot 0 that a dx = 0 operand starts 64 bytes into
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);
-    uint64_t* empty = full + kMaxRows;
-    uint64_t* wfull = empty + kMaxRows;
+    uint64_t* empty = full + kMaxPairs;
+    uint64_t* wfull = empty + kMaxPairs;
     uint64_t* wempty = wfull + 4;
     uint64_t* afull = wempty + 4;
     uint64_t* aempty = afull + 2;
@@ -117,13 +119,13 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     float* swout = reinterpret_cast<float*>(smem + 608);  // kColors, kCompose: 99 floats after 32 biases
     unsigned char* rows = smem + 1024;
     constexpr int kWBytes = 9 * COUT * kKc * 2;
-    unsigned char* wts = rows + NR * kRowBytes;
+    unsigned char* wts = rows + NP * kPairBytes;
     unsigned char* stage = wts + WS * kWBytes;
     const bool resident = WS == cb_n;
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < NR; ++s) {
+        for (int s = 0; s < NP; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -170,27 +172,21 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
                 for (int cb = 0; cb < cb_n && ok; ++cb) {
                     if (!resident || u == (int)blockIdx.x) {
                         if (!(ok = mbar_wait(&wempty[ws], wph, deadline))) break;
-                        unsigned char* dst = wts + ws * kWBytes;
                         mbar_expect_tx(&wfull[ws], kWBytes);
-                        for (int dx = 0; dx < 3; ++dx)
-#pragma unroll
-                            for (int j = 0; j < 3; ++j)  // blocks of a kernel column: taps dy = 2, 1, 0
-                                tma_load_2d(dst + (dx * 3 + j) * COUT * kKc * 2, &tmB, &wfull[ws],
-                                            (3 * (2 - j) + dx) * a.Cin + cb * kKc, 0);
+                        tma_load_4d(wts + ws * kWBytes, &tmB, &wfull[ws], cb * kKc, 0, 0, 0);  // all nine taps
                         ++wissued;
                         if (++ws == WS) {
                             ws = 0;
                             wph ^= 1;
                         }
                     }
-                    for (int r = -1; r <= R; ++r) {
-                        const int y = y0 + r;
-                        if (y < 0 || y >= H) continue;  // zero padding: the row is left out
+                    // rows -1 and H arrive as zeros
+                    for (int r = -1; r <= R; r += 2) {
                         if (!(ok = mbar_wait(&empty[slot], ph, deadline))) break;
-                        mbar_expect_tx(&full[slot], kRowBytes);
-                        tma_load_4d(rows + slot * kRowBytes, &tmA, &full[slot], cb * kKc, 0, g * nimg, y);
+                        mbar_expect_tx(&full[slot], kPairBytes);
+                        tma_load_4d(rows + slot * kPairBytes, &tmA, &full[slot], cb * kKc, 0, g * nimg, y0 + r);
                         ++issued;
-                        if (++slot == NR) {
+                        if (++slot == NP) {
                             slot = 0;
                             ph ^= 1;
                         }
@@ -233,26 +229,28 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
                     ph = ph0;
 #pragma unroll
                     for (int r = -1; r <= R; ++r) {
-                        if ((r == -1 && top) || (r == R && bottom)) continue;
-                        if (dx == 0) {
+                        const bool second = (r & 1) == 0;  // of the pair in this slot
+                        if (dx == 0 && !second) {
                             ok = ok && mbar_wait_warp(&full[slot], ph, deadline);
                             tc_fence_after();
                         }
-                        if (ok) {
-                            // output rows r - 1 .. r + 1 inside the unit
+                        if (ok && !((r == -1 && top) || (r == R && bottom))) {
+                            // output rows r + 1 .. r - 1 inside the unit, in ascending columns
                             const int lo = r < 1 ? 0 : r - 1, hi = r + 1 > R - 1 ? R - 1 : r + 1, n = hi - lo + 1;
                             const uint32_t id = n == 3 ? id3 : n == 2 ? id2 : id1;
-                            const uint64_t da =
-                                drow + (uint64_t)((uint32_t)slot * (uint32_t)(kRowBytes >> 4) + (uint32_t)(4 * dx)) - 4;
-                            const uint64_t db = wb + (uint64_t)((lo - (r - 1)) * (COUT * kKc * 2 >> 4));
-                            const uint32_t d = acc + (uint32_t)(lo * COUT);
+                            const uint64_t da = drow + (uint64_t)((uint32_t)slot * (uint32_t)(kPairBytes >> 4) +
+                                                                  (uint32_t)((second ? kRowBytes >> 4 : 0) + 4 * dx)) - 4;
+                            const uint64_t db = wb + (uint64_t)((r + 1 - hi) * (COUT * kKc * 2 >> 4));
+                            const uint32_t d = acc + (uint32_t)((R - 1 - hi) * COUT);
                             mma_bf16_masked(el, d, da, db, id, m0, m1, m2, m3);
                             mma_bf16_masked(el, d, da + 2, db + 2, id, m0, m1, m2, m3);
-                            if (dx == 2) mma_commit_elected(el, &empty[slot]);
                         }
-                        if (++slot == NR) {
-                            slot = 0;
-                            ph ^= 1;
+                        if (second) {
+                            if (dx == 2 && ok) mma_commit_elected(el, &empty[slot]);
+                            if (++slot == NP) {
+                                slot = 0;
+                                ph ^= 1;
+                            }
                         }
                     }
                 }
@@ -323,7 +321,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
 #pragma unroll 1
                 for (int r = 0; r < R; ++r) {
                     uint32_t v[32], p[16];
-                    const uint32_t t = acc + (uint32_t)(r * COUT);
+                    const uint32_t t = acc + (uint32_t)((R - 1 - r) * COUT);
                     tmem_ld32_async(t, v);
                     bool put = live && r >= r0 && r < r1;
                     if constexpr (MODE == kCompose) {  // hole pixels only
@@ -356,7 +354,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
 #pragma unroll
                 for (int c0 = 0; c0 < COUT; c0 += 32) {
                     uint32_t v0[32], v1[32];
-                    const uint32_t t0 = acc + (uint32_t)(rr * COUT + c0), t1 = t0 + COUT;
+                    const uint32_t t0 = acc + (uint32_t)((R - 1 - rr) * COUT + c0), t1 = t0 - COUT;
                     tmem_ld32_async(t0, v0);
                     tmem_ld32_async(t1, v1);
                     tmem_wait_ld();
@@ -421,7 +419,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) {  // copies still in flight after a timeout: wait for them (bounded)
         const uint64_t d = globaltimer() + kWaitNs;
-        for (int i = max(0, issued - NR); i < issued; ++i) mbar_wait(&full[i % NR], (i / NR) & 1, d);
+        for (int i = max(0, issued - NP); i < issued; ++i) mbar_wait(&full[i % NP], (i / NP) & 1, d);
         for (int i = max(0, wissued - WS); i < wissued; ++i) mbar_wait(&wfull[i % WS], (i / WS) & 1, d);
     }
     __syncthreads();
@@ -431,9 +429,9 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     }
 }
 
-size_t rows_smem(int nrows, int wslots, int cout)
+size_t rows_smem(int pairs, int wslots, int cout)
 {
-    return 2048 + (size_t)nrows * kRowBytes + (size_t)wslots * 9 * cout * kKc * 2 + kStores;
+    return 2048 + (size_t)pairs * kPairBytes + (size_t)wslots * 9 * cout * kKc * 2 + kStores;
 }
 
 }  // namespace
@@ -463,8 +461,8 @@ cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStrea
     while (R > 2 && groups * (c.H / R) < sms) R /= 2;
     const int cb_n = c.Cin / kKc;
     a.wslots = cb_n <= 3 && 9 * c.Cin * c.Cout * 2 <= 80 * 1024 ? cb_n : 2;
-    a.nrows = std::min(kMaxRows, (int)((smem_max - (int)rows_smem(0, a.wslots, c.Cout)) / kRowBytes));
-    if (a.nrows < R + 2) return cudaErrorInvalidValue;
+    a.pairs = std::min(kMaxPairs, (int)((smem_max - (int)rows_smem(0, a.wslots, c.Cout)) / kPairBytes));
+    if (2 * a.pairs < R + 2) return cudaErrorInvalidValue;
     a.y_coff = c.y_coff;
     a.upsample = c.upsample;
     a.relu = c.relu;
@@ -478,19 +476,20 @@ cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStrea
 
     CUtensorMap ta, tb, ty;
     const cuuint32_t one[5] = {1, 1, 1, 1, 1};
-    // {channel, x, image, y}: a box of one row of nimg images is 128 consecutive pixels
+    // {channel, x, image, y}: a box of two rows of nimg images is 2 x 128 consecutive pixels
     const cuuint64_t ci = (cuuint64_t)c.Cin, W = (cuuint64_t)c.W, H = (cuuint64_t)c.H, T = (cuuint64_t)c.T;
     const cuuint64_t ad[4] = {ci, W, T, H};
     const cuuint64_t as[3] = {ci * 2, H * W * ci * 2, W * ci * 2};
-    const cuuint32_t abox[4] = {(cuuint32_t)kKc, (cuuint32_t)c.W, (cuuint32_t)nimg, 1};
+    const cuuint32_t abox[4] = {(cuuint32_t)kKc, (cuuint32_t)c.W, (cuuint32_t)nimg, 2};
     if (enc(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(c.x), ad, as, abox, one,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
-    const cuuint64_t bd[2] = {9 * ci, (cuuint64_t)c.Cout};
-    const cuuint64_t bs[1] = {9 * ci * 2};
-    const cuuint32_t bbox[2] = {(cuuint32_t)kKc, (cuuint32_t)c.Cout};
-    if (enc(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(c.wk), bd, bs, bbox, one,
+    // {channel, co, dy, dx}: a box of all taps lands as the three dy blocks of each dx
+    const cuuint64_t bd[4] = {ci, (cuuint64_t)c.Cout, 3, 3};
+    const cuuint64_t bs[3] = {9 * ci * 2, 3 * ci * 2, ci * 2};
+    const cuuint32_t bbox[4] = {(cuuint32_t)kKc, (cuuint32_t)c.Cout, 3, 3};
+    if (enc(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(c.wk), bd, bs, bbox, one,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
@@ -512,7 +511,7 @@ cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStrea
     }
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
 
-    const size_t smem = rows_smem(a.nrows, a.wslots, c.Cout);
+    const size_t smem = rows_smem(a.pairs, a.wslots, c.Cout);
     const int grid = std::min(groups * (c.H / R), sms);
     auto go = [&](auto kernel, const auto& frames) -> cudaError_t {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
