@@ -271,6 +271,8 @@ yoro_handle yoro_create_pose(int w, int h, float fx, float fy, float cx, float c
     c->pose_args.fy = fy;
     c->pose_args.cx = cx;
     c->pose_args.cy = cy;
+    c->pose_args.inv_fx = 1.0f / fx;
+    c->pose_args.inv_fy = 1.0f / fy;
     for (int i = 0; i < 9; ++i) c->pose_args.rot[i] = rotation[i];
     for (int i = 0; i < 3; ++i) c->pose_args.c[i] = position[i];
     c->pose_args.zbuf = nullptr;

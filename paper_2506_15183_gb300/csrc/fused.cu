@@ -32,6 +32,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "yoro_device.cuh"
 #include "yoro_internal.h"
@@ -124,10 +125,21 @@ __device__ __forceinline__ void find_edges(int x, int v, const Window& s, int w,
 }
 
 // Hole fill of pixel (v, x) with edges L, R (R < w).  Rows outside [0, h) are skipped.
-template <bool VAR>
+// SKIPS: `open` is set, and the result void, once kMaxSkips foreground candidates have been
+// passed over: such a kernel is crossed by the whole warp instead (fill_hole_warp, 32 columns a
+// step).  Almost every pixel settles after about ten candidates, but where the second eye
+// is rotated or shifted out of its row, holes up to 900 columns wide lie next to wide
+// occluders, their kernels hold more than a thousand foreground candidates, and one lane
+// walking them alone kept its band's CTA busy for 100 us (1832x1920, general pose: 148 -> 92
+// us and 113 -> 55 us on the frames with such holes).  The stereo pair's holes are
+// narrow (walks of 24 candidates at the 99th percentile), and there the counter cost 1 to 2 %.
+constexpr int kMaxSkips = 96;
+
+template <bool VAR, bool SKIPS>
 __device__ __forceinline__ uint32_t fill_from_edges(int x, int v, int L, int R, int h, int w, const Window& s,
-                                                    const KernelShape<VAR>& ks)
+                                                    const KernelShape<VAR>& ks, bool& open)
 {
+    int skips = kMaxSkips;
     const int wd = R - L;
     const float d_occ = (L >= 0) ? __uint_as_float(s.zrow(v)[L]) : 0.0f;
     FillAcc f;
@@ -152,7 +164,13 @@ __device__ __forceinline__ uint32_t fill_from_edges(int x, int v, int L, int R, 
                 const int bit = ks.nearest ? __ffs(m) - 1 : 31 - __clz(m);
                 m &= ~(1u << bit);
                 const int c = (wi << 5) + bit;
-                if (__uint_as_float(zr[c]) < d_occ) continue;  // foreground (O2)
+                if (__uint_as_float(zr[c]) < d_occ) {  // foreground (O2)
+                    if (SKIPS && --skips < 0) {
+                        open = true;
+                        return 0u;
+                    }
+                    continue;
+                }
                 if (!f.add(cr[c])) return f.result();          // weight reached exactly 0
                 uint32_t out;
                 if (f.wrem <= kSettleFrom && f.settled(out)) return out;
@@ -555,7 +573,7 @@ __device__ __forceinline__ void resolve_window(const FrameArgs& f, const float* 
 // One band [y0, y1) of one frame; shared memory holds the window rows ra..rb
 // (ra = y0-1 or 0, rb = y1 or h-1).  Ends with a barrier, so the next band may reuse
 // shared memory.
-template <int NT, bool VAR>
+template <int NT, bool VAR, bool SKIPS = false>
 __device__ __forceinline__ void fill_band(const FrameArgs& f, int y0, int y1, const Window& s, int* ctr,
                                           int* rowinfo);
 
@@ -602,7 +620,7 @@ __device__ __forceinline__ void run_band(const FrameArgs& f, int y0, int y1, Win
 // P3 of one band [y0, y1) whose window (s.ra set) holds the reached pixels' depths and
 // colors and every window row's reached bitmask.  Writes the band rows' holes to
 // f.out (reached pixels and masks are not touched).  Ends with a barrier.
-template <int NT, bool VAR>
+template <int NT, bool VAR, bool SKIPS>
 __device__ __forceinline__ void fill_band(const FrameArgs& f, int y0, int y1, const Window& s, int* ctr,
                                           int* rowinfo)
 {
@@ -742,10 +760,22 @@ __device__ __forceinline__ void fill_band(const FrameArgs& f, int y0, int y1, co
                 // one hole for the whole chunk: its kernel is scanned once by the warp
                 const int v0 = __shfl_sync(0xffffffffu, v, 0), L0 = __shfl_sync(0xffffffffu, L, 0),
                           R0 = __shfl_sync(0xffffffffu, R, 0);
+                bool open = false;
                 if (__all_sync(0xffffffffu, !act || (v == v0 && L == L0 && R == R0)))
                     o = fill_hole_warp<VAR>(x, act, v0, L0, R0, h, w, s, ks);
                 else if (act)
-                    o = fill_from_edges<VAR>(x, v, L, R, h, w, s, ks);
+                    o = fill_from_edges<VAR, SKIPS>(x, v, L, R, h, w, s, ks, open);
+                if (SKIPS) {  // kernels too full of foreground for one lane: each such hole by the warp
+                    for (uint32_t left = __ballot_sync(0xffffffffu, open); left;) {
+                        const int lead = __ffs(left) - 1;
+                        const int vl = __shfl_sync(0xffffffffu, v, lead), Ll = __shfl_sync(0xffffffffu, L, lead),
+                                  Rl = __shfl_sync(0xffffffffu, R, lead);
+                        const bool in = open && v == vl && L == Ll && R == Rl;
+                        const uint32_t r = fill_hole_warp<VAR>(x, in, vl, Ll, Rl, h, w, s, ks);
+                        if (in) o = r;
+                        left &= ~__ballot_sync(0xffffffffu, in);
+                    }
+                }
                 if (act && YORO_BOUND(v >= y0 && v < y1, kBadHoles)) f.out[(size_t)v * w + x] = o;
             } else {  // 64 cracks, two consecutive ones per lane
                 const int idx = ((chunk - ng) << 6) + 2 * lane;
@@ -908,12 +938,13 @@ __global__ void __launch_bounds__(NT, 1) fill_only(FrameArgs f, const float* __r
 // the key, the winner's color gathered from f.color), the band rows' colors of reached
 // pixels and their hole mask leave for global memory, and the holes are filled as in
 // fill_only.  It stands in for a gather pass that writes the image out and fill_only's
-// reading it back.
+// reading it back.  The loading takes about 19 us of the pass at 1832x1920; the rest is the
+// holes' fill, bound by the bands that hold the most of it.
 template <int NT, bool VAR>
 __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned long long* __restrict__ keys, int wpad)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    constexpr int NW = NT / 32;
+    constexpr int NW = NT / 32, RB = 5;  // bands of 13 rows: windows of three full batches
     int *ctr, *rowinfo;
     const KernelShape<VAR> ks(f);
     Window s = window_layout(smem_raw, f.band + 2 * ks.halo, wpad, f.w, ctr, rowinfo);
@@ -927,46 +958,56 @@ __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned l
         const int ra = max(y0 - ks.halo, 0), rb = min(y1 - 1 + ks.halo, h - 1);
         const int nr = rb - ra + 1;
         s.ra = ra;
-        const int items = nr * nwords;
-        for (int it0 = warp; it0 < items; it0 += 4 * NW) {
-            unsigned long long kv[4];
+        if (f.bulk && lane == 0)  // most winners come from rows near their target's
+            for (int j = warp; j < nr; j += NW) prefetch_l2(f.color + (size_t)(ra + j) * w, (uint32_t)w * 4u);
+        // as in the resolve, a warp owns the words g = warp, warp + NW, ... of every row and takes
+        // RB rows at a time, with offsets that advance by a row
+        for (int g = warp; g < nwords; g += NW) {
+            const int x = (g << 5) + lane;
+            const bool xin = x < w;
+            auto batch = [&](auto full, int j0, int nb) {
+                constexpr bool FULL = decltype(full)::value;
+                unsigned long long kv[RB];
+                uint32_t cv[RB];
+                const unsigned long long* kp = keys + ((ra + j0) * w + x);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int it = it0 + q * NW;
-                const int j = it / nwords, g = it - j * nwords;
-                const int x = (g << 5) + lane;
-                kv[q] = (it < items && x < w) ? keys[(size_t)(ra + j) * w + x] : kEmptyKey;
-            }
-            uint32_t cv[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t src = (uint32_t)kv[q];
-                cv[q] = (kv[q] != kEmptyKey && YORO_BOUND(src < n, kBadPose)) ? __ldg(f.color + src) : 0u;
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int it = it0 + q * NW;
-                if (it >= items) break;  // warp-uniform
-                const int j = it / nwords, g = it - j * nwords;
-                const int x = (g << 5) + lane;
-                const bool reached = kv[q] != kEmptyKey;
-                const uint32_t m = __ballot_sync(0xffffffffu, reached);
-                if (lane == 0 && YORO_BOUND(j < s.slots, kBadHoles)) s.bits[j * nwords + g] = m;
-                if (reached && YORO_BOUND(j * wpad + x < s.slots * wpad, kBadHoles)) {
-                    s.zt[j * wpad + x] = (uint32_t)(kv[q] >> 32);
-                    s.rgba[j * wpad + x] = cv[q];
+                for (int u = 0; u < RB; ++u) {
+                    kv[u] = ((FULL || u < nb) && xin) ? __ldg(kp) : kEmptyKey;
+                    kp += w;
                 }
-                const int v = ra + j;
-                if (v >= y0 && v < y1 && x < w) {  // a band row: the pixel and its mask byte leave
-                    const size_t o = (size_t)v * w + x;
-                    if (reached) f.out[o] = cv[q];
-                    f.mask[o] = reached ? 0 : 1;
+#pragma unroll
+                for (int u = 0; u < RB; ++u) {
+                    const uint32_t src = (uint32_t)kv[u];
+                    cv[u] = (kv[u] != kEmptyKey && YORO_BOUND(src < n, kBadPose)) ? __ldg(f.color + src) : 0u;
                 }
-            }
+                int so = j0 * wpad + x, vo = (ra + j0) * w + x;
+#pragma unroll
+                for (int u = 0; u < RB; ++u) {
+                    if (FULL || u < nb) {  // uniform
+                        const bool reached = kv[u] != kEmptyKey;
+                        const uint32_t m = __ballot_sync(0xffffffffu, reached);
+                        if (lane == 0 && YORO_BOUND(j0 + u < s.slots, kBadHoles)) s.bits[(j0 + u) * nwords + g] = m;
+                        if (reached && YORO_BOUND(so < s.slots * wpad, kBadHoles)) {
+                            s.zt[so] = (uint32_t)(kv[u] >> 32);
+                            s.rgba[so] = cv[u];
+                        }
+                        // a band row: the pixel and its mask byte leave
+                        if (ra + j0 + u >= y0 && ra + j0 + u < y1 && xin) {
+                            if (reached) f.out[vo] = cv[u];
+                            f.mask[vo] = reached ? 0 : 1;
+                        }
+                    }
+                    so += wpad;
+                    vo += w;
+                }
+            };
+            int j0 = 0;
+            for (; j0 + RB <= nr; j0 += RB) batch(std::true_type{}, j0, RB);
+            if (j0 < nr) batch(std::false_type{}, j0, nr - j0);
         }
         if (threadIdx.x == 0) *ctr = 0;
         __syncthreads();
-        fill_band<NT, VAR>(f, y0, y1, s, ctr, rowinfo);
+        fill_band<NT, VAR, true>(f, y0, y1, s, ctr, rowinfo);
     }
 }
 
@@ -975,14 +1016,17 @@ __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned l
 // every window pixel is sampled from its cell's winner into the window (depth, color,
 // reached bitmask; the band rows' reached pixels and masks leave for global memory),
 // and the band's holes are filled as the fused kernel fills them.  The steps and their
-// rounding are those of imbuffer.cu's separate kernels (the reading is stated there).
-template <int NT>
+// rounding are those of imbuffer.cu's separate kernels (the reading is stated there).  Bound
+// by its instructions: per 32-pixel word the sampling takes 105 and the cells 35 (four seeds
+// of 1832x1920, 4 px per cell: 70, 69, 71, 81 us before the balanced bands and the row
+// batches, 51, 48, 54, 59 us with them; without holes about 30).
+template <int NT, bool VAR>
 __global__ void __launch_bounds__(NT, 1) imb_band(FrameArgs f, int div, int interp, int wpad, int cells_off)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    constexpr int NW = NT / 32;
+    constexpr int NW = NT / 32, RB = 3;  // bands of 7 rows: windows of three full batches
     int *ctr, *rowinfo;
-    const KernelShape<true> ks(f);
+    const KernelShape<VAR> ks(f);
     const int slots = f.band + 2 * ks.halo;
     Window s = window_layout(smem_raw, slots, wpad, f.w, ctr, rowinfo);
     const int w = f.w, h = f.h, nwords = s.nwords, ws = (w + div - 1) / div;
@@ -1006,25 +1050,38 @@ __global__ void __launch_bounds__(NT, 1) imb_band(FrameArgs f, int div, int inte
         for (int i = threadIdx.x; i < nr * ws; i += NT) cells[i] = kEmptyKey;
         if (threadIdx.x == 0) *ctr = 0;
         __syncthreads();
-        // cells: Alg. 1 on each cell's pixel, Alg. 2 by a 64-bit minimum of the key;
-        // (row j, cell i) of flat index c advance without a division per cell
+        // cells: Alg. 1 on each cell's pixel, Alg. 2 by a 64-bit minimum of the key.  Only the
+        // target cell floor(t / s) is needed, so the exact t = (p + 0.5) - RN(k / zc) is
+        // computed only when the estimate cannot decide it (disparity_target's margin, which
+        // holds for t and so for t / s, s >= 1).  Four cells' loads are in flight at a time;
+        // (row j, cell i) of flat index c advance without a division per cell.
         const int dj = NT / ws, di = NT - dj * ws;
         int cj = (int)threadIdx.x / ws, ci = (int)threadIdx.x - cj * ws;
-        for (int c = threadIdx.x; c < nr * ws; c += NT) {
-            const int j = cj, i = ci;
-            cj += dj;
-            ci += di;
-            if (ci >= ws) {
-                ci -= ws;
-                ++cj;
+        for (int c = threadIdx.x; c < nr * ws; c += 4 * NT) {
+            float z[4];
+            int jq = cj, iq = ci;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                z[q] = c + q * NT < nr * ws
+                           ? __ldg(f.depth + (size_t)(ra + jq) * w + min((iq << lg) + (div >> 1), w - 1))
+                           : 0.0f;
+                advance(jq, iq, dj, di, ws);
             }
-            const int p = min(div * i + (div >> 1), w - 1);
-            const uint32_t zb = clamped_depth_bits(__ldg(f.depth + (size_t)(ra + j) * w + p), near_m1, far_m1);
-            const float disp = __fdiv_rn(f.k, __uint_as_float(zb));
-            const float t = __fsub_rn(__fadd_rn((float)p, 0.5f), disp);
-            const float tc = floorf(__fmul_rn(t, inv_s));
-            if (tc >= 0.0f && tc < (float)ws && YORO_BOUND(c < slots * ws, kBadScatter))
-                atomicMin(&cells[j * ws + (int)tc], zkey(zb, i));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (c + q * NT < nr * ws) {
+                    const float pc = __fadd_rn((float)min((ci << lg) + (div >> 1), w - 1), 0.5f);
+                    const uint32_t zb = clamped_depth_bits(z[q], near_m1, far_m1);
+                    const float zc = __uint_as_float(zb);
+                    const float te = __fmul_rn(__fmaf_rn(-f.k, rcp_approx(zc), pc), inv_s);
+                    float tc = floorf(te);
+                    if (!(fabsf(__fsub_rn(__fsub_rn(te, tc), 0.5f)) < f.half_m))
+                        tc = floorf(__fmul_rn(__fsub_rn(pc, __fdiv_rn(f.k, zc)), inv_s));
+                    if (tc >= 0.0f && tc < (float)ws && YORO_BOUND(cj < slots && ci < ws, kBadScatter))
+                        atomicMin(&cells[cj * ws + (int)tc], zkey(zb, ci));
+                }
+                advance(cj, ci, dj, di, ws);
+            }
         }
         __syncthreads();
         if (interp) {  // the winner's shift once per cell: its key's low word becomes disp
@@ -1037,62 +1094,104 @@ __global__ void __launch_bounds__(NT, 1) imb_band(FrameArgs f, int div, int inte
             }
             __syncthreads();
         }
-        // sampling: each window pixel from its cell's winner; warp per 32-pixel word
-        for (int it = warp; it < nr * nwords; it += NW) {
-            const int j = it / nwords, g = it - j * nwords;
+        // sampling: each window pixel from its cell's winner.  As in the resolve, a warp owns the
+        // words g = warp, warp + NW, ... of every row and takes RB rows at a time, their color
+        // loads issued before any is used, with offsets that advance by a row (an enumeration of
+        // (row, word) items took 153 instructions per word, this one 105).  div divides 32, so
+        // a lane's place in its cell is the same in every word: the neighbour's side and its
+        // weight |x + 0.5 - (div cj + div / 2)| / div are constants of the lane (all exact).
+        const float off = __fsub_rn(__fadd_rn((float)(lane & (div - 1)), 0.5f), 0.5f * (float)div);
+        const int nside = off == 0.0f ? 0 : off < 0.0f ? -1 : 1;
+        const float nwt = __fmul_rn(fabsf(off), inv_s);
+        const float wlast = (float)(w - 1);
+        for (int g = warp; g < nwords; g += NW) {
             const int x = (g << 5) + lane;
-            const int y = ra + j;
-            const unsigned long long* krow = cells + j * ws;
-            const uint32_t* crow = f.color + (size_t)y * w;
-            unsigned long long key = kEmptyKey;
-            if (x < w) key = krow[x >> lg];
-            const bool reached = key != kEmptyKey;
-            const uint32_t m = __ballot_sync(0xffffffffu, reached);
-            if (lane == 0 && YORO_BOUND(j < slots, kBadResolve)) s.bits[j * nwords + g] = m;
-            const bool band = y >= y0 && y < y1;
-            if (band && x < w) f.mask[(size_t)y * w + x] = reached ? 0 : 1;
-            if (!reached) continue;
-            const uint32_t zb = (uint32_t)(key >> 32);
-            const int cj = x >> lg;
-            uint32_t col;
-            if (!interp) {
-                col = __ldg(crow + min(div * (int)(uint32_t)key + (x - div * cj), w - 1));
-            } else {
-                const float dj = __uint_as_float((uint32_t)key);  // disp of the winner
-                const float off =
-                    __fsub_rn(__fadd_rn((float)x, 0.5f), __fadd_rn((float)(div * cj), 0.5f * (float)div));
-                const int nb = off < 0.0f ? cj - 1 : cj + 1;
-                float d = dj;
-                if (off != 0.0f && nb >= 0 && nb < ws && krow[nb] != kEmptyKey) {
-                    const float dn = __uint_as_float((uint32_t)krow[nb]);
-                    d = __fadd_rn(dj, __fmul_rn(__fsub_rn(dn, dj), __fmul_rn(fabsf(off), inv_s)));
-                }
-                const float u = __fadd_rn((float)x, d);
-                if (u <= 0.0f) {
-                    col = __ldg(crow);
-                } else if (u >= (float)(w - 1)) {
-                    col = __ldg(crow + w - 1);
-                } else {
-                    const float fl = floorf(u);
-                    const int i0 = (int)fl;
-                    const float fr = __fsub_rn(u, fl);
-                    const uint32_t c0 = __ldg(crow + i0), c1 = __ldg(crow + i0 + 1);
-                    col = 0u;
+            const bool xin = x < w;
+            const int cj = xin ? x >> lg : 0;
+            const bool side = nside != 0 && (unsigned)(cj + nside) < (unsigned)ws;
+            const float xf = (float)x;
+            auto batch = [&](auto full, int j0, int nb) {
+                constexpr bool FULL = decltype(full)::value;
+                uint32_t zb[RB], c0[RB], c1[RB];
+                float fr[RB];
+                uint32_t reach = 0u;  // bit u: this lane's pixel of row j0 + u is reached
+                const unsigned long long* kc = cells + j0 * ws + cj;
+                const uint32_t* crow = f.color + (ra + j0) * w;
 #pragma unroll
-                    for (int ch = 0; ch < 4; ++ch) {
-                        const float v0 = (float)((c0 >> (8 * ch)) & 255u), v1 = (float)((c1 >> (8 * ch)) & 255u);
-                        col |= (uint32_t)rintf(__fadd_rn(v0, __fmul_rn(__fsub_rn(v1, v0), fr))) << (8 * ch);
+                for (int u = 0; u < RB; ++u) {
+                    unsigned long long key = kEmptyKey;
+                    if ((FULL || u < nb) && xin) key = kc[0];
+                    zb[u] = (uint32_t)(key >> 32);
+                    fr[u] = 0.0f;
+                    c0[u] = c1[u] = 0u;
+                    if (key != kEmptyKey) {
+                        reach |= 1u << u;
+                        if (!interp) {
+                            c0[u] = __ldg(crow + min(((int)(uint32_t)key << lg) + (lane & (div - 1)), w - 1));
+                        } else {
+                            float d = __uint_as_float((uint32_t)key);  // disp of the winner
+                            if (side) {
+                                const unsigned long long kn = kc[nside];
+                                if (kn != kEmptyKey)
+                                    d = __fadd_rn(d, __fmul_rn(__fsub_rn(__uint_as_float((uint32_t)kn), d), nwt));
+                            }
+                            // the row's end texels: a coordinate clamped to [0, w - 1] (where the
+                            // fraction is 0, the second texel does not count)
+                            const float uc = fminf(fmaxf(__fadd_rn(xf, d), 0.0f), wlast);
+                            const float fl = floorf(uc);
+                            const int i0 = (int)fl;
+                            fr[u] = __fsub_rn(uc, fl);
+                            c0[u] = __ldg(crow + i0);
+                            c1[u] = __ldg(crow + min(i0 + 1, w - 1));
+                        }
                     }
+                    kc += ws;
+                    crow += w;
                 }
-            }
-            if (YORO_BOUND(j * wpad + x < slots * wpad, kBadResolve)) {
-                s.zt[j * wpad + x] = zb;
-                s.rgba[j * wpad + x] = col;
-            }
-            if (band) f.out[(size_t)y * w + x] = col;
+                int so = j0 * wpad + x, vo = (ra + j0) * w + x;
+#pragma unroll
+                for (int u = 0; u < RB; ++u) {
+                    if (FULL || u < nb) {  // uniform
+                        const bool reached = (reach >> u) & 1u;
+                        const uint32_t m = __ballot_sync(0xffffffffu, reached);
+                        if (lane == 0 && YORO_BOUND(j0 + u < slots, kBadResolve)) s.bits[(j0 + u) * nwords + g] = m;
+                        const bool band = ra + j0 + u >= y0 && ra + j0 + u < y1;
+                        if (band && xin) f.mask[vo] = reached ? 0 : 1;
+                        if (reached) {
+                            uint32_t col = c0[u];
+                            if (interp) {
+                                // per channel RN(v0 + RN((v1 - v0) fr)), rounded half to even: bytes under
+                                // the exponent of 2^23 give v1 - v0 exactly, and adding 2^23 to the result
+                                // (in [0, 255]) rounds it to an integer in the low byte
+                                uint32_t b[4];
+#pragma unroll
+                                for (int ch = 0; ch < 4; ++ch) {
+                                    const float e0 = __uint_as_float(__byte_perm(c0[u], 0x4B00u, 0x5440u + ch));
+                                    const float e1 = __uint_as_float(__byte_perm(c1[u], 0x4B00u, 0x5440u + ch));
+                                    const float r =
+                                        __fadd_rn(__fsub_rn(e0, 8388608.0f), __fmul_rn(__fsub_rn(e1, e0), fr[u]));
+                                    b[ch] = __float_as_uint(__fadd_rn(r, 8388608.0f));
+                                }
+                                col = __byte_perm(__byte_perm(b[0], b[1], 0x0040u), __byte_perm(b[2], b[3], 0x0040u),
+                                                  0x5410u);
+                            }
+                            if (YORO_BOUND(so < slots * wpad, kBadResolve)) {
+                                s.zt[so] = zb[u];
+                                s.rgba[so] = col;
+                            }
+                            if (band) f.out[vo] = col;
+                        }
+                    }
+                    so += wpad;
+                    vo += w;
+                }
+            };
+            int j0 = 0;
+            for (; j0 + RB <= nr; j0 += RB) batch(std::true_type{}, j0, RB);
+            if (j0 < nr) batch(std::false_type{}, j0, nr - j0);
         }
         __syncthreads();
-        fill_band<NT, true>(f, y0, y1, s, ctr, rowinfo);
+        fill_band<NT, VAR>(f, y0, y1, s, ctr, rowinfo);
     }
 }
 
@@ -1168,7 +1267,7 @@ cudaError_t fused_configure(int device, FusedLimits* lim)
                          (const void*)fused_batch<kBig, 1, false, true>,
                          (const void*)fill_only<kBig, false>,       (const void*)fill_only<kBig, true>,
                          (const void*)fill_keys<kBig, false>,       (const void*)fill_keys<kBig, true>,
-                         (const void*)imb_band<kBig>};
+                         (const void*)imb_band<kBig, false>,        (const void*)imb_band<kBig, true>};
     for (const void* fn : fns) {
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
         if (e != cudaSuccess) return e;
@@ -1185,6 +1284,28 @@ static int max_band(const FusedLimits& lim, int wpad, int halo)
     return b;
 }
 
+// Band height for h rows in bands of at most bmax rows on `sms` CTAs at a time: the height with
+// the least (waves of bands) x (rows a band works on, plus about three rows' worth of fixed
+// cost).  Bands of all bmax rows can leave the last wave nearly empty: 1920 rows in bands of
+// 10 are 192 bands, two waves for 152 SMs, and bands of 7 (275) are two waves of 9 rows
+// each instead of 12 (1832x1920 through the intermediate buffer, 4 px per cell: 69 -> 58 us with
+// the bands alone; fused 2064x2208 frames, 11 -> 8 rows: 48.7 -> 41.8 us).
+static int balanced_band(int h, int halo, int bmax, int sms)
+{
+    int best = 1;
+    long long cost = -1;
+    for (int b = 1; b <= bmax; ++b) {
+        const long long waves = ((h + b - 1) / b + sms - 1) / sms;
+        const long long c = waves * (b + 2 * halo + 3);
+        if (cost < 0 || c <= cost) {
+            cost = c;
+            best = b;
+        }
+        if (waves <= 1) break;  // taller bands only leave SMs idle
+    }
+    return best;
+}
+
 // Band height for a w x h frame: enough bands for every SM, each as tall as shared
 // memory allows up to that.  Two CTAs per SM when two such bands fit on an SM.
 FusedShape fused_shape(const FusedLimits& lim, int w, int h, int halo)
@@ -1193,7 +1314,11 @@ FusedShape fused_shape(const FusedLimits& lim, int w, int h, int halo)
     const int bmax = max_band(lim, wpad, halo);
     FusedShape s;
     int band = (h + lim.sms - 1) / lim.sms;
-    if (band > bmax) band = bmax;
+    if (band > bmax) {  // more than one wave: one CTA per SM fills it
+        s.band = balanced_band(h, halo, bmax, lim.sms);
+        s.two_per_sm = 0;
+        return s;
+    }
     if (band < 1) band = 1;
     // two CTAs of half the band height, if they fit beside each other
     const int half = (band + 1) / 2;
@@ -1274,26 +1399,24 @@ int imb_band_max(const FusedLimits& lim, int w, int halo, int div)
 
 cudaError_t imb_band_launch(FrameArgs f, int div, int interp, const FusedLimits& lim, cudaStream_t stream)
 {
-    const int per_sm = (f.h + lim.sms - 1) / lim.sms;
-    f.band = max(1, min(imb_band_max(lim, f.w, f.halo, div), per_sm));
+    f.band = balanced_band(f.h, f.halo, max(1, imb_band_max(lim, f.w, f.halo, div)), lim.sms);
     const size_t smem = imb_band_smem_bytes(f.w, f.band, f.halo, div);
     const int nbands = (f.h + f.band - 1) / f.band;
-    const int grid = nbands < lim.sms ? nbands : lim.sms;
-    if (grid < 1) return cudaSuccess;
-    imb_band<kBig><<<grid, kBig, smem, stream>>>(f, div, interp, fused_wpad(f.w),
-                                                 (int)imb_cells_offset(f.w, f.band, f.halo));
+    if (nbands < 1) return cudaSuccess;
+    const int wpad = fused_wpad(f.w), cells = (int)imb_cells_offset(f.w, f.band, f.halo);
+    if (f.halo == 1 && !f.nearest)
+        imb_band<kBig, false><<<nbands, kBig, smem, stream>>>(f, div, interp, wpad, cells);
+    else
+        imb_band<kBig, true><<<nbands, kBig, smem, stream>>>(f, div, interp, wpad, cells);
     return cudaGetLastError();
 }
 
 cudaError_t fill_only_launch(FrameArgs f, const float* zt, const FusedLimits& lim, cudaStream_t stream)
 {
     const int wpad = fused_wpad(f.w);
-    // bands as tall as shared memory allows, but at least one per SM
-    const int per_sm = (f.h + lim.sms - 1) / lim.sms;
-    f.band = max(1, min(max_band(lim, wpad, f.halo), per_sm));
+    f.band = balanced_band(f.h, f.halo, max(1, max_band(lim, wpad, f.halo)), lim.sms);
     const size_t smem = fused_smem_bytes(wpad, f.band, f.halo);
-    const int nbands = (f.h + f.band - 1) / f.band;
-    const int grid = nbands < lim.sms ? nbands : lim.sms;
+    const int grid = (f.h + f.band - 1) / f.band;
     if (grid < 1) return cudaSuccess;
     if (f.halo == 1 && !f.nearest) fill_only<kBig, false><<<grid, kBig, smem, stream>>>(f, zt, wpad);
     else fill_only<kBig, true><<<grid, kBig, smem, stream>>>(f, zt, wpad);
@@ -1303,12 +1426,9 @@ cudaError_t fill_only_launch(FrameArgs f, const float* zt, const FusedLimits& li
 cudaError_t fill_keys_launch(FrameArgs f, const unsigned long long* keys, const FusedLimits& lim, cudaStream_t stream)
 {
     const int wpad = fused_wpad(f.w);
-    // bands as tall as shared memory allows, but at least one per SM
-    const int per_sm = (f.h + lim.sms - 1) / lim.sms;
-    f.band = max(1, min(max_band(lim, wpad, f.halo), per_sm));
+    f.band = balanced_band(f.h, f.halo, max(1, max_band(lim, wpad, f.halo)), lim.sms);
     const size_t smem = fused_smem_bytes(wpad, f.band, f.halo);
-    const int nbands = (f.h + f.band - 1) / f.band;
-    const int grid = nbands < lim.sms ? nbands : lim.sms;
+    const int grid = (f.h + f.band - 1) / f.band;
     if (grid < 1) return cudaSuccess;
     if (f.halo == 1 && !f.nearest) fill_keys<kBig, false><<<grid, kBig, smem, stream>>>(f, keys, wpad);
     else fill_keys<kBig, true><<<grid, kBig, smem, stream>>>(f, keys, wpad);

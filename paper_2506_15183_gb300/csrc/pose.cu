@@ -38,27 +38,92 @@ __device__ __forceinline__ float dot3(const float* r, float q0, float q1, float 
     return __fadd_rn(__fadd_rn(__fmul_rn(r[0], q0), __fmul_rn(r[1], q1)), __fmul_rn(r[2], q2));
 }
 
-// Steps 1 and 2: one thread per source pixel.
-__global__ void pose_scatter_kernel(FrameArgs f, PoseArgs p)
+// a / b, correctly rounded, for a constant b whose correctly rounded reciprocal y is at hand:
+// the quotient estimate a y is corrected twice by its exact remainder (Markstein, "Computation
+// of elementary functions on the IBM RISC System/6000 processor", 1990: with y = RN(1/b) and a
+// faithful q, RN(q + RN(a - b q) y) is RN(a / b); the first correction makes q faithful).
+// Needs normal numbers throughout (pose_fast()).
+__device__ __forceinline__ float div_const(float a, float b, float y)
+{
+    float q = __fmul_rn(a, y);
+    q = __fmaf_rn(__fmaf_rn(-q, b, a), y, q);
+    return __fmaf_rn(__fmaf_rn(-q, b, a), y, q);
+}
+
+// floor(RN(RN(a / Z) + c)) as a float.  The estimate t = RN(a r + c), r = rcp.approx(Z) (within
+// 1 ulp), differs from RN(RN(a / Z) + c) by less than (2^-23 + 2^-24) |a / Z| + 2^-23 |t| (1 +
+// 2^-20), and |a / Z| <= (|t| + |c|) (1 + 2^-20): by less than 3.1e-7 (|t| + |c|).  Unless an
+// integer lies within m = 3.4e-7 (|t| + |c|) + 1e-6 of t, both have the same floor; else, and
+// where the estimate is not finite, the division decides.
+__device__ __forceinline__ float project(float a, float Z, float c)
+{
+    const float t = __fmaf_rn(a, rcp_approx(Z), c);
+    const float fl = floorf(t);
+    const float m = __fmaf_rn(__fadd_rn(fabsf(t), fabsf(c)), 3.4e-7f, 1.0e-6f);
+    const float fr = __fsub_rn(t, fl);
+    if (fr > m && fr < __fsub_rn(1.0f, m)) return fl;
+    return floorf(__fadd_rn(__fdiv_rn(a, Z), c));
+}
+
+// Steps 1 and 2.  A block takes 256 columns of kScatterRows rows, a thread one column of
+// them: its column's centre is set once and its loads are all in flight before the first is
+// used.  The pass is bound by its arithmetic: with four IEEE divisions and a 64-bit division
+// for the row per pixel it took 21.9 us at 1832x1920 (18.6 M warp instructions); now 16.6 us
+// (12.9 M).  FAST: the divisions by fx and fy
+// through their reciprocals, the two by p'.z only where an estimate leaves the target open.
+constexpr int kScatterRows = 4;
+
+template <bool FAST>
+__global__ void __launch_bounds__(256) pose_scatter_kernel(FrameArgs f, PoseArgs p, unsigned chunks)
 {
     const int w = f.w, h = f.h;
-    const size_t n = (size_t)w * (size_t)h;
+    const unsigned cols = (unsigned)(w + 255) >> 8;
     const uint32_t near_m1 = __float_as_uint(f.near_) - 1u, far_m1 = __float_as_uint(f.far_) - 1u;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int y = (int)(i / (size_t)w);
-        const int x = (int)(i - (size_t)y * w);
-        const float zc = __uint_as_float(clamped_depth_bits(f.depth[i], near_m1, far_m1));
-        const float px = __fdiv_rn(__fmul_rn(__fsub_rn(__fadd_rn((float)x, 0.5f), p.cx), zc), p.fx);
-        const float py = __fdiv_rn(__fmul_rn(__fsub_rn(__fadd_rn((float)y, 0.5f), p.cy), zc), p.fy);
-        const float q0 = __fsub_rn(px, p.c[0]), q1 = __fsub_rn(py, p.c[1]), q2 = __fsub_rn(zc, p.c[2]);
-        const float X = dot3(p.rot, q0, q1, q2), Y = dot3(p.rot + 3, q0, q1, q2), Z = dot3(p.rot + 6, q0, q1, q2);
-        if (!(Z > 0.0f)) continue;
-        const float u = floorf(__fadd_rn(__fdiv_rn(__fmul_rn(p.fx, X), Z), p.cx));
-        const float v = floorf(__fadd_rn(__fdiv_rn(__fmul_rn(p.fy, Y), Z), p.cy));
-        if (!(u >= 0.0f && u < (float)w && v >= 0.0f && v < (float)h)) continue;
-        const size_t o = (size_t)(int)v * w + (int)u;
-        if (YORO_BOUND(o < n, kBadPose)) atomicMin(&p.zbuf[o], zkey(__float_as_uint(Z), (int)i));
+    for (unsigned ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
+        const unsigned rg = ch / cols;
+        const int y0 = (int)rg * kScatterRows;
+        const int x = (int)((ch - rg * cols) << 8) + (int)threadIdx.x;
+        if (x >= w) continue;
+        const int nr = min(kScatterRows, h - y0);
+        const int i0 = y0 * w + x;  // w h < 2^31
+        float z[kScatterRows];
+#pragma unroll
+        for (int r = 0; r < kScatterRows; ++r) z[r] = r < nr ? __ldg(f.depth + i0 + r * w) : 0.0f;
+        const float xc = __fsub_rn(__fadd_rn((float)x, 0.5f), p.cx);
+#pragma unroll
+        for (int r = 0; r < kScatterRows; ++r) {
+            if (r >= nr) break;
+            const float zc = __uint_as_float(clamped_depth_bits(z[r], near_m1, far_m1));
+            const float ax = __fmul_rn(xc, zc);
+            const float ay = __fmul_rn(__fsub_rn(__fadd_rn((float)(y0 + r), 0.5f), p.cy), zc);
+            const float px = FAST ? div_const(ax, p.fx, p.inv_fx) : __fdiv_rn(ax, p.fx);
+            const float py = FAST ? div_const(ay, p.fy, p.inv_fy) : __fdiv_rn(ay, p.fy);
+            const float q0 = __fsub_rn(px, p.c[0]), q1 = __fsub_rn(py, p.c[1]), q2 = __fsub_rn(zc, p.c[2]);
+            const float X = dot3(p.rot, q0, q1, q2), Y = dot3(p.rot + 3, q0, q1, q2), Z = dot3(p.rot + 6, q0, q1, q2);
+            if (!(Z > 0.0f)) continue;
+            float u, v;
+            if (FAST) {
+                u = project(__fmul_rn(p.fx, X), Z, p.cx);
+                v = project(__fmul_rn(p.fy, Y), Z, p.cy);
+            } else {
+                u = floorf(__fadd_rn(__fdiv_rn(__fmul_rn(p.fx, X), Z), p.cx));
+                v = floorf(__fadd_rn(__fdiv_rn(__fmul_rn(p.fy, Y), Z), p.cy));
+            }
+            if (!(u >= 0.0f && u < (float)w && v >= 0.0f && v < (float)h)) continue;
+            const size_t o = (size_t)(int)v * w + (int)u;
+            if (YORO_BOUND(o < (size_t)w * (size_t)h, kBadPose))
+                atomicMin(&p.zbuf[o], zkey(__float_as_uint(Z), i0 + r * w));
+        }
     }
+}
+
+// Whether every division by fx and fy stays among normal numbers: the numerators are zero or
+// between 2^-25 near and (2^31 + |c|) far in magnitude.
+bool pose_fast(const FrameArgs& f, const PoseArgs& p)
+{
+    const float lo = 9.3e-10f, hi = 1.0e9f;  // 2^-30, 2^30
+    return p.fx >= lo && p.fx <= hi && p.fy >= lo && p.fy <= hi && f.near_ >= lo && f.far_ <= hi && p.cx >= -hi &&
+           p.cx <= hi && p.cy >= -hi && p.cy <= hi;
 }
 
 // Step 3: one thread per target pixel.
@@ -108,7 +173,10 @@ cudaError_t pose_launch(const FrameArgs& f, const PoseArgs& p, const FusedLimits
     cudaError_t e = cudaMemsetAsync(p.zbuf, 0xFF, n * sizeof(unsigned long long), stream);
     if (e != cudaSuccess) return e;
     const int threads = 256;
-    pose_scatter_kernel<<<blocks_for(n, threads), threads, 0, stream>>>(f, p);
+    const unsigned chunks = (unsigned)((f.w + 255) / 256) * (unsigned)((f.h + kScatterRows - 1) / kScatterRows);
+    const unsigned grid = chunks < (1u << 30) ? chunks : 1u << 30;
+    if (pose_fast(f, p)) pose_scatter_kernel<true><<<grid, threads, 0, stream>>>(f, p, chunks);
+    else pose_scatter_kernel<false><<<grid, threads, 0, stream>>>(f, p, chunks);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // a band fits shared memory: the band fill reads the keys itself (gather included)
     if (band_fill) return fill_keys_launch(f, p.zbuf, lim, stream);

@@ -125,6 +125,7 @@ cudaError_t fill_pixels_launch(const FrameArgs& f, const float* zt, cudaStream_t
 // General second-eye pose (pose.cu): p' = rot (p - c) with the shared intrinsics.
 struct PoseArgs {
     float fx, fy, cx, cy;
+    float inv_fx, inv_fy;       // 1 / fx, 1 / fy, correctly rounded
     float rot[9];               // row-major
     float c[3];                 // second eye position in left-eye camera coordinates
     unsigned long long* zbuf;   // h * w keys (p'.z bits << 32 | source index)
