@@ -189,28 +189,37 @@ __global__ void __launch_bounds__(kDwThreads, 1)
     }
 }
 
-// dW[co][ci][tap] = the sum over the shares of ws[ct cbs + cb][share][co][tap][ci]: a block
-// takes 32 consecutive ci, its eight warps every eighth share, and adds the warps' sums in
-// order (one thread per element over all shares was 13 us per layer, latency).
+// dW[co][ci][tap] = the sum over the shares of ws[ct cbs + cb][share][co][tap][ci].  A block
+// takes 128 consecutive floats of a tile (32 loads of 16 bytes), its eight warps every eighth
+// share, and adds the warps' sums in order.  Bound by reading the workspace from L2 (up to 22
+// MB a layer); one thread per element over all shares was 13 us a layer, latency.
 __global__ void __launch_bounds__(256) dw_reduce_kernel(const float* __restrict__ ws, int shares, int co_tile, int cbs,
                                                         int cin, float* __restrict__ dW)
 {
-    __shared__ float part[8][32];
-    const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const int tap = blockIdx.x % 9, r = blockIdx.x / 9;
-    const int col = r % co_tile, tile = r / co_tile;  // tile = ct cbs + cb
-    const size_t step = (size_t)co_tile * kDwTile;
-    const float* p = ws + ((size_t)tile * shares * co_tile + col) * kDwTile + tap * 32 + c;
-    float s = 0.0f;
+    __shared__ float4 part[8][32];
+    const int l = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int quads = co_tile * (kDwTile / 4);  // of a tile
+    const int tile = blockIdx.x / (quads / 32), q = (blockIdx.x - tile * (quads / 32)) * 32 + l;
+    const float4* p = reinterpret_cast<const float4*>(ws) + (size_t)tile * shares * quads + q;
+    float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll 4
-    for (int i = g; i < shares; i += 8) s += p[i * step];
-    part[g][c] = s;
+    for (int i = g; i < shares; i += 8) {
+        const float4 v = p[(size_t)i * quads];
+        s.x += v.x;
+        s.y += v.y;
+        s.z += v.z;
+        s.w += v.w;
+    }
+    part[g][l] = s;
     __syncthreads();
-    const int ci = (tile % cbs) * 32 + c, co = tile / cbs * co_tile + col;
-    if (g == 0 && ci < cin) {  // the first layer's padding channels are dropped
+    if (threadIdx.x < 128) {  // thread k: float k of the 128
+        const int k = threadIdx.x, e = (q - l) * 4 + k;  // place in the tile: [co][tap][ci]
+        float t = 0.0f;
 #pragma unroll
-        for (int i = 1; i < 8; ++i) s += part[i][c];
-        dW[((size_t)co * cin + ci) * 9 + tap] = s;
+        for (int i = 0; i < 8; ++i) t += reinterpret_cast<const float*>(&part[i][0])[k];
+        const int c = e & 31, r = e >> 5, tap = r % 9, col = r / 9;
+        const int ci = (tile % cbs) * 32 + c, co = tile / cbs * co_tile + col;  // tile = ct cbs + cb
+        if (ci < cin) dW[((size_t)co * cin + ci) * 9 + tap] = t;  // the first layer's padding channels are dropped
     }
 }
 
@@ -240,7 +249,10 @@ cudaError_t conv_dw_launch(const void* dZ, const void* X, int xcs, int T, int si
         return cudaErrorInvalidValue;
     const int cbs = (cin + 31) / 32, tiles = cbs * (cout / (32 * cob));
     const int boxes = T * (side / kDwRows);
-    const int shares = std::max(1, std::min(boxes, sms / tiles));
+    // shares of the pixels: a CTA for every SM, but at the two lowest levels at least four boxes
+    // each, whose sums (147 KB a share) would cost more to write and add than their MMAs
+    const int least = side <= 16 ? 4 : 1;
+    const int shares = std::max(1, std::min(boxes / least, sms / tiles));
     if ((size_t)shares * tiles > (size_t)sms) return cudaErrorInvalidValue;  // the workspace holds `sms` tiles
     const cuuint32_t one[4] = {1, 1, 1, 1};
     auto map = [&](CUtensorMap* m, const void* p, int cs, int rows) {
@@ -260,7 +272,7 @@ cudaError_t conv_dw_launch(const void* dZ, const void* X, int xcs, int T, int si
     else if (side == 16) e = launch<16, 4, 4>(tz, tx, side, boxes, tiles, cbs, shares, ws, s);
     else e = launch<8, 4, 4>(tz, tx, side, boxes, tiles, cbs, shares, ws, s);
     if (e != cudaSuccess) return e;
-    dw_reduce_kernel<<<(unsigned)(cout * cbs * 9), 256, 0, s>>>(ws, shares, 32 * cob, cbs, cin, dW);
+    dw_reduce_kernel<<<(unsigned)(tiles * (32 * cob * kDwTile / 128)), 256, 0, s>>>(ws, shares, 32 * cob, cbs, cin, dW);
     return cudaGetLastError();
 }
 

@@ -249,18 +249,19 @@ __global__ void __launch_bounds__(256) out_bwd_kernel(const float* __restrict__ 
     if (threadIdx.x == 3) atomicAdd(loss, s[3]);
 }
 
-// Adam and the layers' weights, one pass: a thread takes the nine taps of a (co, ci) pair of
-// one layer (its parameters, gradient and moments are 36 consecutive bytes each), or one
-// bias or parameter of the output layer, updates them (lr = 0: leaves them) and writes the
-// forms the kernels read:
+// Adam and the layers' weights, one pass.  A block takes 32 x 32 (co, ci) of one layer (a run
+// of 288 consecutive parameters per co; the first layer has 6 ci), updates them (lr = 0: leaves
+// them) with coalesced accesses to the parameters, gradient and moments, and writes from
+// shared memory, 64 bytes at a time, the forms the kernels read:
 //   wk[co][tap][ci]       the forward's K-major weights (bfloat16; the first layer's padding
 //                         channels keep the zeros they were created with)
 //   wt[ci][8 - tap][co]   the kernel flipped in both directions: the input gradient is a 3x3
 //                         convolution of dZ with these
-//   bias, wout            FP32 biases; the output layer's bfloat16-rounded weights as floats
+// The last block takes the biases and the output layer (FP32 biases; bfloat16-rounded weights
+// as floats).  31 us for 1.9 M parameters; one thread per (co, ci), which wrote wt two bytes at
+// a time, took 49, and eight elements' loads in flight per thread 40.
 struct WeightTable {
-    int pair0[15];  // first pair of each layer; [14]: pairs of all layers
-    int bias0[15];  // first bias of each layer; [14]: biases of all layers
+    int block0[15];  // first block of each layer; [14]: the last block
     int woff[14], boff[14], cin[14], cout[14], cin_pad[14];
     uint16_t* wk[14];
     uint16_t* wt[14];
@@ -291,38 +292,39 @@ __device__ __forceinline__ float adam_step(const AdamArgs& a, int i)
     return p;
 }
 
-__global__ void __launch_bounds__(256) weights_kernel(const __grid_constant__ WeightTable w, const AdamArgs a)
+constexpr int kWeightThreads = 576;  // two of a tile's rows of 288
+
+__global__ void __launch_bounds__(kWeightThreads) weights_kernel(const __grid_constant__ WeightTable w, const AdamArgs a)
 {
-    int i = blockIdx.x * 256 + threadIdx.x;
-    if (i < w.pair0[14]) {
-        int l = 0;
-        while (i >= w.pair0[l + 1]) ++l;
-        i -= w.pair0[l];
-        const int cin = w.cin[l], cout = w.cout[l], cp = w.cin_pad[l];
-        const int co = i / cin, ci = i - co * cin;
-        const int base = w.woff[l] + i * 9;
-        uint16_t* wk = w.wk[l] + (size_t)co * 9 * cp + ci;
-        uint16_t* wt = w.wt[l] + (size_t)ci * 9 * cout + co;
-#pragma unroll
-        for (int t = 0; t < 9; ++t) {
-            const uint16_t b = f2bf(adam_step(a, base + t));
-            wk[t * cp] = b;
-            wt[(8 - t) * cout] = b;
+    __shared__ uint16_t s[32][290];  // [co][ci 9 + tap]; 145 words per row: no bank conflict along co
+    if ((int)blockIdx.x == w.block0[14]) {
+        for (int l = 0; l < 14; ++l)
+            for (int i = threadIdx.x; i < w.cout[l]; i += kWeightThreads) w.bias[l][i] = adam_step(a, w.boff[l] + i);
+        if (threadIdx.x < 99) {
+            const int i = threadIdx.x;
+            const float p = adam_step(a, w.out_off + i);
+            w.wout[i] = i < 96 ? bf2f(f2bf(p)) : p;
         }
         return;
     }
-    i -= w.pair0[14];
-    if (i < w.bias0[14]) {
-        int l = 0;
-        while (i >= w.bias0[l + 1]) ++l;
-        i -= w.bias0[l];
-        w.bias[l][i] = adam_step(a, w.boff[l] + i);
-        return;
+    int l = 0;
+    while ((int)blockIdx.x >= w.block0[l + 1]) ++l;
+    const int cin = w.cin[l], cout = w.cout[l], cp = w.cin_pad[l];
+    const int cbs = (cin + 31) >> 5, b = blockIdx.x - w.block0[l];
+    const int co0 = b / cbs * 32, ci0 = b % cbs * 32;
+    const int nci = min(32, cin - ci0), run = nci * 9;
+    const int base = w.woff[l] + (co0 * cin + ci0) * 9;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < 32 * run; i += kWeightThreads) {
+        const int co = i / run, k = i - co * run;
+        s[co][k] = f2bf(adam_step(a, base + co * cin * 9 + k));
     }
-    i -= w.bias0[14];
-    if (i < 99) {
-        const float p = adam_step(a, w.out_off + i);
-        w.wout[i] = i < 96 ? bf2f(f2bf(p)) : p;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int r = warp; r < 32 * 9; r += kWeightThreads / 32) {
+        const int row = r / 9, tap = r - row * 9;
+        if (lane < nci) w.wk[l][((size_t)(co0 + row) * 9 + tap) * cp + ci0 + lane] = s[row][lane * 9 + tap];
+        if (row < nci) w.wt[l][((size_t)(ci0 + row) * 9 + 8 - tap) * cout + co0 + lane] = s[lane][row * 9 + tap];
     }
 }
 
@@ -377,8 +379,7 @@ cudaError_t update_weights(Trainer* t, bool update, cudaStream_t s)
         a.c1 = 1.0f - std::pow(t->b1, (float)t->step);
         a.c2 = 1.0f - std::pow(t->b2, (float)t->step);
     }
-    const int n = t->table.pair0[14] + t->table.bias0[14] + 99;
-    weights_kernel<<<(n + 255) / 256, 256, 0, s>>>(t->table, a);
+    weights_kernel<<<t->table.block0[14] + 1, kWeightThreads, 0, s>>>(t->table, a);
     return cudaGetLastError();
 }
 
@@ -422,8 +423,7 @@ Trainer* trainer_create(const float* params, size_t np, int batch, float lr, flo
         dx = std::max(dx, P * (size_t)cin);
         ok = cudaMalloc(&t->wt[i], (size_t)cin * 9 * cout * 2) == cudaSuccess;
         const UnetLayer& L = t->net->conv[i];
-        w.pair0[i + 1] = w.pair0[i] + cout * cin;
-        w.bias0[i + 1] = w.bias0[i] + cout;
+        w.block0[i + 1] = w.block0[i] + cout / 32 * ((cin + 31) / 32);
         w.woff[i] = (int)t->woff[i];
         w.boff[i] = (int)t->boff[i];
         w.cin[i] = cin;
