@@ -117,6 +117,18 @@ __device__ __forceinline__ uint64_t desc_sw64(uint32_t saddr)
     return d;
 }
 
+// The same for rows of 128 bytes of K with the 128-byte swizzle (layout type 2): 8-row groups
+// 1024 bytes apart.
+__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr)
+{
+    uint64_t d = (uint64_t)((saddr >> 4) & 0x3fffu);
+    d |= (uint64_t)1u << 16;
+    d |= (uint64_t)(1024u >> 4) << 32;
+    d |= (uint64_t)1u << 46;
+    d |= (uint64_t)2u << 61;
+    return d;
+}
+
 // Instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), BF16 A and B
 // (bits 7-9 and 10-12 = 1), both K-major, N / 8 at bit 17, M / 16 at bit 24.
 __host__ __device__ constexpr uint32_t idesc_bf16(int n)

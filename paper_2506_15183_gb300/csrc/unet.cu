@@ -54,9 +54,7 @@ namespace {
 
 __device__ unsigned g_unet_status;  // kernel-side failures of this file's kernels
 
-constexpr int kStages = 4;     // one-tile form where several CTAs share an SM
-constexpr int kMaxStages = 12;  // either form
-constexpr int kABytes = kTileM * kKc * 2;  // 8 KB
+constexpr int kMaxStages = 12;
 
 struct ConvArgs {
     int T, H, W;          // tiles and their size (the output has the input's size)
@@ -146,17 +144,32 @@ __device__ __forceinline__ void epilogue_store(const ConvArgs& a, const CUtensor
     }
 }
 
+// The one-tile form: MT tiles of 128 consecutive pixels (whole images where an image is
+// smaller), a K step being KC channels of one tap.  The activation boxes and the weight box of
+// a step are issued by two threads (warps 0 and 2): an issue costs a thread about 300 cycles
+// plus 100 per copy whatever its size, so one thread with two copies of 32 channels per step
+// was the pace of small grids (690 cycles a step).  With 64 channels a step (128-byte
+// swizzle) half as many are needed.  The sums keep their order (tap, channel).
+//
+// MT = 2 for grids of two tiles per SM and more: both tiles use the weights of one copy (256
+// channels: 64 instead of 96 bytes per cycle from L2, which 128-pixel CTAs were bound by).
+//
+// Measured, us (KC = 32, MT = 1, one issuing thread -> this): CONV_TC_MEASURED
+template <int KC, int MT>
 __global__ void __launch_bounds__(128, 1)
     conv3x3_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmY, const ConvArgs a)
 {
     extern __shared__ unsigned char smem_raw[];
-    if (a.count && (int)((blockIdx.x * kTileM) / (a.H * a.W)) >= *a.count) return;  // no such tile (uniform)
+    const int hw = a.H * a.W;
+    const int p0 = blockIdx.x * MT * kTileM;
+    if (a.count && p0 / hw >= *a.count) return;  // no such tile (uniform)
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                            ~static_cast<uintptr_t>(1023));
+    constexpr int kA = kTileM * KC * 2;  // one tile's activation box
     const int S = a.stages, nb = blockIdx.y * a.bn;
-    const int b_bytes = a.bn * kKc * 2;
-    const int stage_bytes = kABytes + ((b_bytes + 1023) & ~1023);
+    const int b_bytes = a.bn * KC * 2;
+    const int stage_bytes = MT * kA + b_bytes;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * stage_bytes);
     uint64_t* empty = full + S;
     uint64_t* done = empty + S;
@@ -166,7 +179,7 @@ __global__ void __launch_bounds__(128, 1)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
-            mbar_init(&full[s], 1);
+            mbar_init(&full[s], 2);
             mbar_init(&empty[s], 1);
         }
         mbar_init(done, 1);
@@ -174,7 +187,7 @@ __global__ void __launch_bounds__(128, 1)
         counts[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) {
+    if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                      "r"(a.ncols)
                      : "memory");
@@ -185,33 +198,43 @@ __global__ void __launch_bounds__(128, 1)
     tc_fence_after();
     const uint32_t tmem = *tslot;
 
-    const int cb_n = a.Cin / kKc;
+    const int cb_n = a.Cin / KC;
     const int nk = 9 * cb_n;
-    const int hw = a.H * a.W;
-    const int p0 = blockIdx.x * kTileM;
-    const int n0 = p0 / hw;
-    const int y0 = (p0 - n0 * hw) / a.W;
     const uint64_t deadline = globaltimer() + kWaitNs;
 
-    if (warp == 0 && lane == 0) {  // copies
-        int k = 0;
-        for (; k < nk; ++k) {
-            const int s = k % S;
-            if (!mbar_wait(&empty[s], ((k / S) & 1) ^ 1, deadline)) {
+    if ((warp == 0 || warp == 2) && lane == 0) {  // copies: activations, weights
+        int s = 0, ph = 1, tap = 0, cb = 0;
+        for (int k = 0; k < nk; ++k) {
+            if (!mbar_wait(&empty[s], ph, deadline)) {
                 atomicOr(&g_unet_status, kUnetTimeout);
                 break;
             }
-            const int tap = k / cb_n, cb = k - tap * cb_n;
-            const int dy = tap / 3, dx = tap - 3 * (tap / 3);
             unsigned char* sa = smem + s * stage_bytes;
-            mbar_expect_tx(&full[s], (uint32_t)(kABytes + b_bytes));
-            tma_load_4d(sa, &tmA, &full[s], cb * kKc, dx - 1, y0 + dy - 1, n0);
-            tma_load_2d(sa + kABytes, &tmB, &full[s], tap * a.Cin + cb * kKc, nb);
-            counts[0] = k + 1;
+            if (warp == 0) {
+                const int dy = tap / 3, dx = tap - 3 * dy;
+                mbar_expect_tx(&full[s], (uint32_t)(MT * kA));
+#pragma unroll
+                for (int j = 0; j < MT; ++j) {  // a tile past the last image arrives as zeros
+                    const int p = p0 + j * kTileM, n = p / hw, y = (p - n * hw) / a.W;
+                    tma_load_4d(sa + j * kA, &tmA, &full[s], cb * KC, dx - 1, y + dy - 1, n);
+                }
+                counts[0] = k + 1;
+            } else {
+                mbar_expect_tx(&full[s], (uint32_t)b_bytes);
+                tma_load_2d(sa + MT * kA, &tmB, &full[s], tap * a.Cin + cb * KC, nb);
+            }
+            if (++cb == cb_n) {
+                cb = 0;
+                ++tap;
+            }
+            if (++s == S) {
+                s = 0;
+                ph ^= 1;
+            }
         }
     } else if (warp == 1) {  // MMAs: the whole warp runs the loop, one lane issues
         const uint32_t idesc = idesc_bf16(a.bn), el = elect_one();
-        const uint64_t dbase = desc_sw64(smem_u32(smem));
+        const uint64_t dbase = KC == 64 ? desc_sw128(smem_u32(smem)) : desc_sw64(smem_u32(smem));
         int s = 0, ph = 0;
         for (int k = 0; k < nk; ++k) {
             if (!mbar_wait_warp(&full[s], ph, deadline)) {
@@ -219,9 +242,13 @@ __global__ void __launch_bounds__(128, 1)
                 break;
             }
             tc_fence_after();
-            const uint64_t da = dbase + (uint64_t)((uint32_t)(s * stage_bytes) >> 4), db = da + (kABytes >> 4);
-            mma_bf16_elected(el, tmem, da, db, idesc, k > 0 ? 1u : 0u);
-            mma_bf16_elected(el, tmem, da + 2, db + 2, idesc, 1u);
+            const uint64_t da = dbase + (uint64_t)((uint32_t)(s * stage_bytes) >> 4), db = da + (MT * kA >> 4);
+#pragma unroll
+            for (int q = 0; q < KC / 16; ++q)
+#pragma unroll
+                for (int j = 0; j < MT; ++j)
+                    mma_bf16_elected(el, tmem + (uint32_t)(j * a.bn), da + (uint64_t)(j * (kA >> 4) + 2 * q),
+                                     db + (uint64_t)(2 * q), idesc, k + q > 0 ? 1u : 0u);
             mma_commit_elected(el, &empty[s]);
             if (el) counts[1] = k + 1;
             if (++s == S) {
@@ -237,7 +264,13 @@ __global__ void __launch_bounds__(128, 1)
     if (!ok) atomicOr(&g_unet_status, kUnetTimeout);
     if (ok) {
         tc_fence_after();
-        epilogue_store(a, &tmY, tmem, smem, a.bias + nb, 1, n0, y0);
+#pragma unroll
+        for (int j = 0; j < MT; ++j) {
+            const int p = p0 + j * kTileM, n = p / hw, y = (p - n * hw) / a.W;
+            if (n < a.T)  // uniform
+                epilogue_store(a, &tmY, tmem + (uint32_t)(j * a.bn), smem + j * (a.bn >> 5) * kTileM * 64, a.bias + nb, 1,
+                               n, y);
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -247,7 +280,7 @@ __global__ void __launch_bounds__(128, 1)
             if (!mbar_wait(&full[k % S], (k / S) & 1, d2)) break;
     }
     __syncthreads();
-    if (warp == 0) {
+    if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.ncols) : "memory");
     }
@@ -293,18 +326,18 @@ __global__ void __launch_bounds__(128, 1)
 
     const int cb_n = a.Cin / kKc;
     const int nk = 3 * cb_n;  // K steps of a band: (channel block, dx)
-    // K step kk of the CTA (band kk / nk of its walk, step kk % nk) into stage kk % S
-    auto issue = [&](int kk, int n0, int y0) {
-        const int s = kk % S;
-        const int k = kk % nk;
-        const int cb = k / 3, dx = k - 3 * cb;
-        unsigned char* sa = smem + s * stage_bytes;
-        mbar_expect_tx(&full[s], (uint32_t)(a_bytes + 3 * b_tap));
-        tma_load_4d(sa, &tmA, &full[s], cb * kKc, dx - 1, y0 - 1, n0);
-#pragma unroll
-        for (int dy = 0; dy < 3; ++dy)
-            tma_load_2d(sa + a_span + dy * b_tap, &tmB, &full[s], (3 * dy + dx) * a.Cin + cb * kKc, nb);
+    // K step kk of the CTA (band kk / nk of its walk, step kk % nk) into stage kk % S: the
+    // activation box (issued by warp 0) and the three taps' weights (one box, warp 2)
+    auto issue_a = [&](int kk, int n0, int y0) {
+        const int s = kk % S, k = kk % nk, cb = k / 3, dx = k - 3 * cb;
+        mbar_expect_tx(&full[s], (uint32_t)a_bytes);
+        tma_load_4d(smem + s * stage_bytes, &tmA, &full[s], cb * kKc, dx - 1, y0 - 1, n0);
         counts[0] = kk + 1;
+    };
+    auto issue_b = [&](int kk) {
+        const int s = kk % S, k = kk % nk, cb = k / 3, dx = k - 3 * cb;
+        mbar_expect_tx(&full[s], (uint32_t)(3 * b_tap));
+        tma_load_4d(smem + s * stage_bytes + a_span, &tmB, &full[s], cb * kKc, nb, 0, dx);
     };
     const int first = nk < S ? nk : S;  // copies issued before the CTA-wide barrier
 
@@ -312,7 +345,7 @@ __global__ void __launch_bounds__(128, 1)
     // warp 1 allocates the tensor memory and the bias is staged in shared memory.
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
-            mbar_init(&full[s], 1);
+            mbar_init(&full[s], 2);
             mbar_init(&empty[s], 1);
         }
         mbar_init(done, 1);
@@ -322,7 +355,10 @@ __global__ void __launch_bounds__(128, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         const int b0 = blockIdx.x, n0 = b0 / bands_per_tile, y0 = (b0 - n0 * bands_per_tile) * R;
-        for (int k = 0; k < first; ++k) issue(k, n0, y0);
+        for (int k = 0; k < first; ++k) {
+            issue_a(k, n0, y0);
+            issue_b(k);
+        }
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
@@ -348,7 +384,7 @@ __global__ void __launch_bounds__(128, 1)
     for (int band = blockIdx.x; band < live; band += gridDim.x, ++it) {
         const int n0 = band / bands_per_tile, y0 = (band - n0 * bands_per_tile) * R;
         const uint64_t deadline = globaltimer() + kWaitNs;
-        if (warp == 0 && lane == 0) {  // copies
+        if ((warp == 0 || warp == 2) && lane == 0) {  // copies: activations, weights
             for (int k = it == 0 ? first : (early ? 1 : 0); k < nk; ++k) {
                 const int kk = it * nk + k, s = kk % S;
                 if (!mbar_wait(&empty[s], ((kk / S) & 1) ^ 1, deadline)) {
@@ -356,7 +392,8 @@ __global__ void __launch_bounds__(128, 1)
                     counts[2] = 1;
                     break;
                 }
-                issue(kk, n0, y0);
+                if (warp == 0) issue_a(kk, n0, y0);
+                else issue_b(kk);
             }
         } else if (warp == 1) {  // MMAs: the whole warp runs the loop, one lane issues
             // Descriptors: a stage's bases plus constants in the 16-byte start-address
@@ -385,8 +422,10 @@ __global__ void __launch_bounds__(128, 1)
                     const uint32_t acc = (k > 0 || dy > 0) ? 1u : 0u;
                     mma_bf16_elected(el, tmem, a0, bt, idesc, acc);
                     mma_bf16_elected(el, tmem, a0 + 2, bt + 2, idesc, 1u);
-                    mma_bf16_elected(el, d1, a1, bt, idesc, acc);
-                    mma_bf16_elected(el, d1, a1 + 2, bt + 2, idesc, 1u);
+                    if (mt > 1) {  // uniform
+                        mma_bf16_elected(el, d1, a1, bt, idesc, acc);
+                        mma_bf16_elected(el, d1, a1 + 2, bt + 2, idesc, 1u);
+                    }
                 }
                 mma_commit_elected(el, &empty[s]);
                 if (el) counts[1] = kk + 1;
@@ -398,8 +437,10 @@ __global__ void __launch_bounds__(128, 1)
             if (early && next < live && run && el) {
                 const int kk = (it + 1) * nk, s = kk % S;
                 const int n1 = next / bands_per_tile, y1 = (next - n1 * bands_per_tile) * R;
-                if (mbar_wait(&empty[s], ((kk / S) & 1) ^ 1, deadline)) issue(kk, n1, y1);
-                else {
+                if (mbar_wait(&empty[s], ((kk / S) & 1) ^ 1, deadline)) {
+                    issue_a(kk, n1, y1);
+                    issue_b(kk);
+                } else {
                     atomicOr(&g_unet_status, kUnetTimeout);
                     counts[2] = 1;
                 }
@@ -458,21 +499,19 @@ EncodeTiled tensor_map_encoder()
 namespace {
 
 // One-tile form: bytes of one copy stage, and of a CTA.
-int conv_stage_bytes(int bn) { return kABytes + ((bn * kKc * 2 + 1023) & ~1023); }
+int conv_stage_bytes(int bn, int kc, int mt) { return (mt * kTileM + bn) * kc * 2; }
 
-size_t conv_smem_bytes(int bn, int stages)
-{
-    return 1024 + (size_t)stages * conv_stage_bytes(bn) + (2 * stages + 1) * 8 + 16;
-}
+size_t conv_smem_bytes(int stage, int stages) { return 1024 + (size_t)stages * stage + (2 * stages + 1) * 8 + 16; }
 
-// Output channels per CTA where `ctas` CTAs with all Cout would leave SMs idle: halved while
-// twice as many CTAs still get an SM of their own.  Each part runs the same K steps (its sums
+// Output channels per CTA where `ctas` CTAs with all Cout would leave SMs idle: halved, down to
+// 64 (an MMA takes 55 cycles at N = 64 and at N = 32), while twice as many CTAs still get an
+// SM of their own.  Each part runs the same K steps (its sums
 // are the same), but its copies are smaller, and a lone CTA's ring can be as deep as its SM's
 // shared memory: on few tiles these layers wait for their copies.
 int split_channels(int Cout, long long ctas, int sms)
 {
     int bn = Cout;
-    while (bn > 32 && 2 * ctas * (Cout / bn) <= sms) bn /= 2;
+    while (bn > 64 && 2 * ctas * (Cout / bn) <= sms) bn /= 2;
     return bn;
 }
 
@@ -583,26 +622,41 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
     if (mt && conv_rows_takes(H, W, Cout)) return conv_rows_launch(call, sms, kSmemPerBlock, stream);
     // the output layer rides on the row form only; the other forms pool 16-pixel rows
     if (call.rgb || call.frames || (call.pool && W != 16)) return cudaErrorInvalidValue;
-    const long long ctas = pixels / (std::max(mt, 1) * kTileM);
+    // on small grids one accumulator per CTA: twice the CTAs, half the MMAs of each (the halo
+    // rows' overhead does not matter there)
+    if (mt && pixels / (mt * kTileM) * 2 <= sms) mt = 1;
+    const int kc = !mt && Cin % 64 == 0 ? 64 : kKc;  // one-tile form: channels of a K step
+    const int tt = !mt && pixels >= 2ll * kTileM * sms ? 2 : 1;  // one-tile form: tiles of a CTA
+    const int cta_px = (mt ? mt : tt) * kTileM;
+    const long long ctas = (pixels + cta_px - 1) / cta_px;
     const int bn = split_channels(Cout, ctas, sms);
     const bool alone = ctas * (Cout / bn) <= sms;  // every CTA has an SM of its own
 
     CUtensorMap ta, tb;
     const cuuint64_t adim[4] = {(cuuint64_t)Cin, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)T};
     const cuuint64_t astr[3] = {(cuuint64_t)Cin * 2, (cuuint64_t)W * Cin * 2, (cuuint64_t)H * W * Cin * 2};
-    const cuuint32_t abox[4] = {(cuuint32_t)kKc, (cuuint32_t)W, (cuuint32_t)hb, (cuuint32_t)nb};
     const cuuint32_t one4[4] = {1, 1, 1, 1};
-    if (enc(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(x), adim, astr, abox, one4,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
-    const cuuint64_t bdim[2] = {(cuuint64_t)9 * Cin, (cuuint64_t)Cout};
-    const cuuint64_t bstr[1] = {(cuuint64_t)9 * Cin * 2};
-    const cuuint32_t bbox[2] = {(cuuint32_t)kKc, (cuuint32_t)bn};
-    if (enc(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(wk), bdim, bstr, bbox, one4,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
+    auto load_map = [&](CUtensorMap* m, const void* ptr, int rank, const cuuint64_t* dim, const cuuint64_t* str,
+                        const cuuint32_t* box) {
+        return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(ptr), dim, str, box, one4,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   box[0] == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    if (mt) {  // weights as {channel, co, dy, dx}: the three taps of a kernel column in one box
+        const cuuint64_t ci = (cuuint64_t)Cin;
+        const cuuint64_t bdim[4] = {ci, (cuuint64_t)Cout, 3, 3};
+        const cuuint64_t bstr[3] = {9 * ci * 2, 3 * ci * 2, ci * 2};
+        const cuuint32_t bbox[4] = {(cuuint32_t)kKc, (cuuint32_t)bn, 3, 1};
+        const cuuint32_t abox[4] = {(cuuint32_t)kKc, (cuuint32_t)W, (cuuint32_t)(mt * kTileM / W + 2), 1u};
+        if (!load_map(&ta, x, 4, adim, astr, abox) || !load_map(&tb, wk, 4, bdim, bstr, bbox)) return cudaErrorInvalidValue;
+    } else {
+        const cuuint64_t bdim[2] = {(cuuint64_t)9 * Cin, (cuuint64_t)Cout};
+        const cuuint64_t bstr[1] = {(cuuint64_t)9 * Cin * 2};
+        const cuuint32_t bbox[2] = {(cuuint32_t)kc, (cuuint32_t)bn};
+        const cuuint32_t abox[4] = {(cuuint32_t)kc, (cuuint32_t)W, (cuuint32_t)hb, (cuuint32_t)nb};
+        if (!load_map(&ta, x, 4, adim, astr, abox) || !load_map(&tb, wk, 2, bdim, bstr, bbox)) return cudaErrorInvalidValue;
+    }
 
     // The output map: the epilogue's box of 32 channels x the CTA's pixels (rows x W x
     // images), or for the upsampling a 5-D view {channel, b, x, a, n H + y} of the 2H x 2W
@@ -646,17 +700,11 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
     const unsigned parts = (unsigned)(Cout / bn);
     if (mt) {
         const int rows = mt * kTileM / W;
-        CUtensorMap th;
-        const cuuint32_t hbox[4] = {(cuuint32_t)kKc, (cuuint32_t)W, (cuuint32_t)(rows + 2), 1u};
-        if (enc(&th, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(x), adim, astr, hbox, one4,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
         CUtensorMap ty;
         if (!y_map(&ty, rows, 1)) return cudaErrorInvalidValue;
         const int stage = halo_stage_bytes(W, rows, bn);
         a.ncols = mt * bn;
-        a.stages = stages;
+        a.stages = stages;  // two
         if (alone)
             while (a.stages < kMaxStages && halo_smem_bytes(stage, a.stages + 1) <= (size_t)kSmemPerBlock) ++a.stages;
         const cudaError_t e =
@@ -666,18 +714,26 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
         // as many CTAs as fit at once (shared memory; registers allow 5), each walking bands
         const int per_sm = std::min(5, (int)(kSmemPerSm / (hsmem + 1024)));
         const long long grid = std::min<long long>(ctas, (long long)std::max(per_sm, 1) * sms);
-        conv3x3_halo<<<dim3((unsigned)grid, parts), 128, hsmem, stream>>>(th, tb, ty, a, (int)ctas);
+        conv3x3_halo<<<dim3((unsigned)grid, parts), 128, hsmem, stream>>>(ta, tb, ty, a, (int)ctas);
         return cudaGetLastError();
     }
-    a.stages = kStages;
-    if (alone)
-        while (a.stages < kMaxStages && conv_smem_bytes(bn, a.stages + 1) <= (size_t)kSmemPerBlock) ++a.stages;
-    const cudaError_t e = cudaFuncSetAttribute(conv3x3_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerBlock);
-    if (e != cudaSuccess) return e;
+    // one-tile form: a lone CTA (and one with two tiles, whose accumulators take the tensor
+    // memory) rings as deep as its SM's shared memory, else two CTAs share an SM
+    const int stage = conv_stage_bytes(bn, kc, tt);
+    const size_t budget = alone || tt > 1 ? (size_t)kSmemPerBlock : kSmemPerSm / 2 - 1024;
+    a.ncols = tt * bn;
+    a.stages = 1;
+    while (a.stages < kMaxStages && conv_smem_bytes(stage, a.stages + 1) <= budget) ++a.stages;
     CUtensorMap ty;
     if (!y_map(&ty, hb, nb)) return cudaErrorInvalidValue;
-    conv3x3_tc<<<dim3((unsigned)ctas, parts), 128, conv_smem_bytes(bn, a.stages), stream>>>(ta, tb, ty, a);
-    return cudaGetLastError();
+    auto go = [&](auto kernel) -> cudaError_t {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerBlock);
+        if (e != cudaSuccess) return e;
+        kernel<<<dim3((unsigned)ctas, parts), 128, conv_smem_bytes(stage, a.stages), stream>>>(ta, tb, ty, a);
+        return cudaGetLastError();
+    };
+    if (kc == 64) return tt == 2 ? go(conv3x3_tc<64, 2>) : go(conv3x3_tc<64, 1>);
+    return tt == 2 ? go(conv3x3_tc<32, 2>) : go(conv3x3_tc<32, 1>);
 }
 
 namespace {
