@@ -55,11 +55,14 @@ constexpr int kAccCols = 256;                   // tensor-memory columns of an a
 constexpr int kMaxPairs = 11;                   // row-pair slots (bounds the barrier array)
 constexpr int kStageBytes = 2 * 32 * kKc * 2;   // a warp's 32 pixels of two rows, 32 channels
 constexpr int kStores = 4 * 2 * kStageBytes;    // two staging buffers for each of four warps
-constexpr int kRowsThreads = 192;
+constexpr int kRowsThreads = 192;               // 224 with an upsampled input (one more warp)
+constexpr int kLowBytes = kRowBytes / 2;        // a row of the half-resolution input: 64 pixels
+constexpr int kLow = 6;                         // its landing slots
 
 struct RowsArgs {
     int T, H, W, Cin;
     int pairs;         // row-pair slots
+    int cskip;         // channels of the first input; the other Cin - cskip come from the half-resolution one
     int wslots;        // weight slots (9 taps of one channel block each); resident when wslots == Cin / 32
     int y_coff, upsample, relu;
     const float* bias;
@@ -90,15 +93,26 @@ __device__ __forceinline__ void finish(const uint32_t (&r)[32], const float* bia
 
 struct NoFrames {};
 
-template <int COUT, int R, int MODE, class Frames>
-__global__ void __launch_bounds__(kRowsThreads, 1)
+// UP: the input is a concatenation of cskip channels at the layer's resolution (tmA) and the
+// nearest upsampling of the rest (tmU, H/2 x W/2), which is never stored: a fifth kind of warp
+// writes each of its rows, pixels doubled, into the row slots (8 KB of shared-memory writes),
+// where it serves as both input rows it is upsampled to.  Written out and read back, the
+// upsampled tensors were half of the memory traffic of the decoder's first layers and most of
+// what the layers below them wrote.
+template <int COUT, int R, int MODE, bool UP, class Frames>
+__global__ void __launch_bounds__(kRowsThreads + (UP ? 32 : 0), 1)
     conv3x3_rows(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                 const __grid_constant__ CUtensorMap tmY, const RowsArgs a, const __grid_constant__ Frames ft)
+                 const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmU, const RowsArgs a,
+                 const __grid_constant__ Frames ft)
 {
+    constexpr int kThreads = kRowsThreads + (UP ? 32 : 0);
+    constexpr int kSkipSlots = (R + 2) / 2;             // slots of a channel block: rows -1 .. R
+    constexpr int kLowRows = R / 2 + 2;                 // half-resolution rows under them
+    constexpr int kUpSlots = (kLowRows + 1) / 2;
     extern __shared__ unsigned char smem_raw[];
     const int W = a.W, H = a.H, NP = a.pairs, WS = a.wslots;
     const int nimg = kTileM / W, bands = H / R;
-    const int cb_n = a.Cin / kKc;
+    const int cb_n = a.Cin / kKc, cb_skip = UP ? a.cskip / kKc : cb_n;
     const int tiles = a.count ? min(a.T, *a.count) : a.T;
     const int units = (tiles + nimg - 1) / nimg * bands;
     if ((int)blockIdx.x >= units) return;  // uniform
@@ -112,7 +126,9 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     uint64_t* wempty = wfull + 4;
     uint64_t* afull = wempty + 4;
     uint64_t* aempty = afull + 2;
-    uint64_t* drain = aempty + 2;
+    uint64_t* lfull = aempty + 2;
+    uint64_t* lempty = lfull + kLow;
+    uint64_t* drain = lempty + kLow;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
     float* sbias = reinterpret_cast<float*>(smem + 480);  // COUT floats
@@ -121,6 +137,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     constexpr int kWBytes = 9 * COUT * kKc * 2;
     unsigned char* wts = rows + NP * kPairBytes;
     unsigned char* stage = wts + WS * kWBytes;
+    unsigned char* land = stage + kStores;
     const bool resident = WS == cb_n;
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
@@ -137,6 +154,10 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
             mbar_init(&afull[s], 1);
             mbar_init(&aempty[s], 4);
         }
+        for (int s = 0; s < kLow; ++s) {
+            mbar_init(&lfull[s], 1);
+            mbar_init(&lempty[s], 1);
+        }
         mbar_init(drain, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -148,9 +169,9 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    for (int c = threadIdx.x; c < COUT; c += kRowsThreads) sbias[c] = __ldg(a.bias + c);
+    for (int c = threadIdx.x; c < COUT; c += kThreads) sbias[c] = __ldg(a.bias + c);
     if (MODE == kColors || MODE == kCompose)
-        for (int c = threadIdx.x; c < 99; c += kRowsThreads) swout[c] = __ldg(a.wout + c);
+        for (int c = threadIdx.x; c < 99; c += kThreads) swout[c] = __ldg(a.wout + c);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -160,11 +181,13 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
         atomicOr(&g_rows_status, kUnetTimeout);
         *abort_flag = 1;
     };
-    int issued = 0, wissued = 0;  // rows and weight slots that thread 0 has copied
+    // what thread 0 has copied: row slots (bits) and the parity of their last copy's phase; counts
+    uint32_t copied = 0u, parity = 0u;
+    int wissued = 0, lissued = 0;
 
     if (warp == 0) {
         if (lane == 0) {  // copies
-            int slot = 0, ph = 1, ws = 0, wph = 1;
+            int slot = 0, ph = 1, ws = 0, wph = 1, ls = 0, lph = 1;
             bool ok = true;
             for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
                 const int g = u / bands, y0 = (u - g * bands) * R;
@@ -181,11 +204,31 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
                         }
                     }
                     // rows -1 and H arrive as zeros
+                    if (UP && cb >= cb_skip) {
+                        for (int i = 0; i < kLowRows; ++i) {
+                            if (!(ok = mbar_wait(&lempty[ls], lph, deadline))) break;
+                            mbar_expect_tx(&lfull[ls], kLowBytes);
+                            tma_load_4d(land + ls * kLowBytes, &tmU, &lfull[ls], (cb - cb_skip) * kKc, 0, g * nimg,
+                                        y0 / 2 - 1 + i);
+                            ++lissued;
+                            if (++ls == kLow) {
+                                ls = 0;
+                                lph ^= 1;
+                            }
+                        }
+                        for (int i = 0; i < kUpSlots; ++i)  // filled by the doubling warp
+                            if (++slot == NP) {
+                                slot = 0;
+                                ph ^= 1;
+                            }
+                        continue;
+                    }
                     for (int r = -1; r <= R; r += 2) {
                         if (!(ok = mbar_wait(&empty[slot], ph, deadline))) break;
                         mbar_expect_tx(&full[slot], kPairBytes);
                         tma_load_4d(rows + slot * kPairBytes, &tmA, &full[slot], cb * kKc, 0, g * nimg, y0 + r);
-                        ++issued;
+                        copied |= 1u << slot;
+                        parity = (parity & ~(1u << slot)) | ((uint32_t)(ph ^ 1) << slot);
                         if (++slot == NP) {
                             slot = 0;
                             ph ^= 1;
@@ -218,6 +261,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
                 if (!resident || it == 0)
                     if (!(ok = mbar_wait_warp(&wfull[ws], wph, deadline))) break;
                 int slot = slot0, ph = ph0;
+                const bool up = UP && cb >= cb_skip;
 #pragma unroll
                 for (int dx = 0; dx < 3; ++dx) {
                     const uint32_t m0 = dx == 0 ? 1u : dx == 2 ? hi02 : 0u;
@@ -227,30 +271,49 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
                     const uint64_t wb = dw + (uint64_t)((uint32_t)(ws * kWBytes + dx * 3 * COUT * kKc * 2) >> 4);
                     slot = slot0;
                     ph = ph0;
-#pragma unroll
-                    for (int r = -1; r <= R; ++r) {
-                        const bool second = (r & 1) == 0;  // of the pair in this slot
-                        if (dx == 0 && !second) {
+                    // input row r, in row `half` of the current slot, into output rows r + 1 .. r - 1
+                    // inside the unit (ascending columns)
+                    auto row = [&](int r, int half) {
+                        const int lo = r < 1 ? 0 : r - 1, hi = r + 1 > R - 1 ? R - 1 : r + 1, n = hi - lo + 1;
+                        const uint32_t id = n == 3 ? id3 : n == 2 ? id2 : id1;
+                        const uint64_t da = drow + (uint64_t)((uint32_t)slot * (uint32_t)(kPairBytes >> 4) +
+                                                              (uint32_t)(half * (kRowBytes >> 4) + 4 * dx)) - 4;
+                        const uint64_t db = wb + (uint64_t)((r + 1 - hi) * (COUT * kKc * 2 >> 4));
+                        const uint32_t d = acc + (uint32_t)((R - 1 - hi) * COUT);
+                        mma_bf16_masked(el, d, da, db, id, m0, m1, m2, m3);
+                        mma_bf16_masked(el, d, da + 2, db + 2, id, m0, m1, m2, m3);
+                    };
+                    auto next = [&]() {
+                        if (dx == 2 && ok) mma_commit_elected(el, &empty[slot]);
+                        if (++slot == NP) {
+                            slot = 0;
+                            ph ^= 1;
+                        }
+                    };
+                    auto arrived = [&]() {
+                        if (dx == 0) {
                             ok = ok && mbar_wait_warp(&full[slot], ph, deadline);
                             tc_fence_after();
                         }
-                        if (ok && !((r == -1 && top) || (r == R && bottom))) {
-                            // output rows r + 1 .. r - 1 inside the unit, in ascending columns
-                            const int lo = r < 1 ? 0 : r - 1, hi = r + 1 > R - 1 ? R - 1 : r + 1, n = hi - lo + 1;
-                            const uint32_t id = n == 3 ? id3 : n == 2 ? id2 : id1;
-                            const uint64_t da = drow + (uint64_t)((uint32_t)slot * (uint32_t)(kPairBytes >> 4) +
-                                                                  (uint32_t)((second ? kRowBytes >> 4 : 0) + 4 * dx)) - 4;
-                            const uint64_t db = wb + (uint64_t)((r + 1 - hi) * (COUT * kKc * 2 >> 4));
-                            const uint32_t d = acc + (uint32_t)((R - 1 - hi) * COUT);
-                            mma_bf16_masked(el, d, da, db, id, m0, m1, m2, m3);
-                            mma_bf16_masked(el, d, da + 2, db + 2, id, m0, m1, m2, m3);
+                    };
+                    if (!up) {
+#pragma unroll
+                        for (int r = -1; r <= R; ++r) {
+                            const bool second = (r & 1) == 0;  // of the pair in this slot
+                            if (!second) arrived();
+                            if (ok && !((r == -1 && top) || (r == R && bottom))) row(r, second ? 1 : 0);
+                            if (second) next();
                         }
-                        if (second) {
-                            if (dx == 2 && ok) mma_commit_elected(el, &empty[slot]);
-                            if (++slot == NP) {
-                                slot = 0;
-                                ph ^= 1;
-                            }
+                    } else {
+                        // half-resolution row i = 0 .. kLowRows - 1 of the unit, in row i & 1 of its slot, is
+                        // input rows 2i - 2 and 2i - 1
+#pragma unroll
+                        for (int i = 0; i < kLowRows; ++i) {
+                            if (!(i & 1)) arrived();
+#pragma unroll
+                            for (int r = 2 * i - 2; r <= 2 * i - 1; ++r)
+                                if (r >= -1 && r <= R && ok && !((r == -1 && top) || (r == R && bottom))) row(r, i & 1);
+                            if ((i & 1) || i == kLowRows - 1) next();
                         }
                     }
                 }
@@ -271,6 +334,48 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
             mma_commit_elected(el, drain);
             mbar_wait_warp(drain, 0, globaltimer() + kWaitNs);
         }
+    } else if (UP && warp == 6) {  // doubles the half-resolution rows
+        int slot = 0, ph = 1, ls = 0, lph = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+            const uint64_t deadline = globaltimer() + kWaitNs;
+            for (int cb = 0; cb < cb_n && ok; ++cb) {
+                const bool up = cb >= cb_skip;
+                for (int t = 0; t < (up ? kUpSlots : kSkipSlots); ++t) {
+                    if (up) {
+                        if (!(ok = mbar_wait_warp(&empty[slot], ph, deadline))) break;
+                        for (int half = 0; half < 2 && 2 * t + half < kLowRows; ++half) {
+                            if (!(ok = mbar_wait_warp(&lfull[ls], lph, deadline))) break;
+                            const unsigned char* src = land + ls * kLowBytes;
+                            unsigned char* dst = rows + slot * kPairBytes + half * kRowBytes;
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {  // 16-byte chunk e & 3 of pixel e >> 2, twice
+                                const int e = i * 32 + lane, q = e >> 2, k = e & 3;
+                                const uint4 v = *reinterpret_cast<const uint4*>(src + q * 64 + ((k ^ ((q >> 1) & 3)) << 4));
+                                unsigned char* o = dst + q * 128 + ((k ^ (q & 3)) << 4);
+                                *reinterpret_cast<uint4*>(o + (q & 1) * 64) = v;  // odd q the other way round:
+                                *reinterpret_cast<uint4*>(o + 64 - (q & 1) * 64) = v;  // no bank met twice
+                            }
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(&lempty[ls]);
+                            if (++ls == kLow) {
+                                ls = 0;
+                                lph ^= 1;
+                            }
+                        }
+                        if (!ok) break;
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&full[slot]);
+                    }
+                    if (++slot == NP) {
+                        slot = 0;
+                        ph ^= 1;
+                    }
+                }
+            }
+        }
+        if (!ok && lane == 0) timed_out();
     } else {  // read back, store
         const int q = warp & 3;  // this warp's quarter of the tensor-memory lanes
         const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
@@ -419,7 +524,9 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) {  // copies still in flight after a timeout: wait for them (bounded)
         const uint64_t d = globaltimer() + kWaitNs;
-        for (int i = max(0, issued - NP); i < issued; ++i) mbar_wait(&full[i % NP], (i / NP) & 1, d);
+        for (int i = 0; i < NP; ++i)
+            if ((copied >> i) & 1u) mbar_wait(&full[i], (parity >> i) & 1u, d);
+        for (int i = max(0, lissued - kLow); i < lissued; ++i) mbar_wait(&lfull[i % kLow], (i / kLow) & 1, d);
         for (int i = max(0, wissued - WS); i < wissued; ++i) mbar_wait(&wfull[i % WS], (i / WS) & 1, d);
     }
     __syncthreads();
@@ -429,9 +536,9 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     }
 }
 
-size_t rows_smem(int pairs, int wslots, int cout)
+size_t rows_smem(int pairs, int wslots, int cout, bool up)
 {
-    return 2048 + (size_t)pairs * kPairBytes + (size_t)wslots * 9 * cout * kKc * 2 + kStores;
+    return 2048 + (up ? kLow * kLowBytes : 0) + (size_t)pairs * kPairBytes + (size_t)wslots * 9 * cout * kKc * 2 + kStores;
 }
 
 }  // namespace
@@ -459,9 +566,13 @@ cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStrea
     int R = kAccCols / c.Cout;
     while (c.H % R) R /= 2;
     while (R > 2 && groups * (c.H / R) < sms) R /= 2;
+    const bool up = c.low != nullptr;
+    if (up && (c.rgb || c.frames || c.pool || c.W > 64 || c.cskip < kKc || c.cskip % kKc || c.cskip >= c.Cin))
+        return cudaErrorInvalidValue;
+    a.cskip = c.cskip;
     const int cb_n = c.Cin / kKc;
     a.wslots = cb_n <= 3 && 9 * c.Cin * c.Cout * 2 <= 80 * 1024 ? cb_n : 2;
-    a.pairs = std::min(kMaxPairs, (int)((smem_max - (int)rows_smem(0, a.wslots, c.Cout)) / kPairBytes));
+    a.pairs = std::min(kMaxPairs, (int)((smem_max - (int)rows_smem(0, a.wslots, c.Cout, up)) / kPairBytes));
     if (2 * a.pairs < R + 2) return cudaErrorInvalidValue;
     a.y_coff = c.y_coff;
     a.upsample = c.upsample;
@@ -474,17 +585,29 @@ cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStrea
     a.list = c.list;
     if ((c.rgb || c.frames) && (c.Cout != 32 || c.upsample || c.pool)) return cudaErrorInvalidValue;
 
-    CUtensorMap ta, tb, ty;
+    CUtensorMap ta, tb, ty, tu;
     const cuuint32_t one[5] = {1, 1, 1, 1, 1};
     // {channel, x, image, y}: a box of two rows of nimg images is 2 x 128 consecutive pixels
     const cuuint64_t ci = (cuuint64_t)c.Cin, W = (cuuint64_t)c.W, H = (cuuint64_t)c.H, T = (cuuint64_t)c.T;
-    const cuuint64_t ad[4] = {ci, W, T, H};
-    const cuuint64_t as[3] = {ci * 2, H * W * ci * 2, W * ci * 2};
+    const cuuint64_t ca = up ? (cuuint64_t)c.cskip : ci;
+    const cuuint64_t ad[4] = {ca, W, T, H};
+    const cuuint64_t as[3] = {ca * 2, H * W * ca * 2, W * ca * 2};
     const cuuint32_t abox[4] = {(cuuint32_t)kKc, (cuuint32_t)c.W, (cuuint32_t)nimg, 2};
     if (enc(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(c.x), ad, as, abox, one,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
+    tu = ta;  // unused without a half-resolution input
+    if (up) {  // the same of one half-resolution row: 64 pixels
+        const cuuint64_t cu = ci - ca, Wl = W / 2, Hl = H / 2;
+        const cuuint64_t ud[4] = {cu, Wl, T, Hl};
+        const cuuint64_t us[3] = {cu * 2, Hl * Wl * cu * 2, Wl * cu * 2};
+        const cuuint32_t ubox[4] = {(cuuint32_t)kKc, (cuuint32_t)Wl, (cuuint32_t)nimg, 1};
+        if (enc(&tu, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(c.low), ud, us, ubox, one,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
     // {channel, co, dy, dx}: a box of all taps lands as the three dy blocks of each dx
     const cuuint64_t bd[4] = {ci, (cuuint64_t)c.Cout, 3, 3};
     const cuuint64_t bs[3] = {9 * ci * 2, 3 * ci * 2, ci * 2};
@@ -495,8 +618,10 @@ cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStrea
         return cudaErrorInvalidValue;
     // a store's box: 32 channels x 32 pixels x two rows of one image
     const cuuint64_t cs = (cuuint64_t)c.y_cstride;
-    CUresult r;
-    if (!c.upsample) {
+    CUresult r = CUDA_SUCCESS;
+    if (c.rgb || c.frames) {
+        ty = ta;  // nothing is stored
+    } else if (!c.upsample) {
         const cuuint64_t d[4] = {cs, W, T, H};
         const cuuint64_t s[3] = {cs * 2, H * W * cs * 2, W * cs * 2};
         const cuuint32_t box[4] = {(cuuint32_t)kKc, 32, 1, 2};
@@ -511,22 +636,30 @@ cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStrea
     }
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
 
-    const size_t smem = rows_smem(a.pairs, a.wslots, c.Cout);
+    const size_t smem = rows_smem(a.pairs, a.wslots, c.Cout, up);
     const int grid = std::min(groups * (c.H / R), sms);
     auto go = [&](auto kernel, const auto& frames) -> cudaError_t {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
         if (e != cudaSuccess) return e;
-        kernel<<<grid, kRowsThreads, smem, stream>>>(ta, tb, ty, a, frames);
+        kernel<<<grid, kRowsThreads + (up ? 32 : 0), smem, stream>>>(ta, tb, ty, tu, a, frames);
         return cudaGetLastError();
     };
     const NoFrames none;
 #define YORO_ROWS32(MODE, FRAMES, TABLE)                                \
-    (R == 8   ? go(conv3x3_rows<32, 8, MODE, FRAMES>, TABLE)            \
-     : R == 4 ? go(conv3x3_rows<32, 4, MODE, FRAMES>, TABLE)            \
-              : go(conv3x3_rows<32, 2, MODE, FRAMES>, TABLE))
+    (R == 8   ? go(conv3x3_rows<32, 8, MODE, false, FRAMES>, TABLE)            \
+     : R == 4 ? go(conv3x3_rows<32, 4, MODE, false, FRAMES>, TABLE)            \
+              : go(conv3x3_rows<32, 2, MODE, false, FRAMES>, TABLE))
+    if (up) {
+        if (c.Cout == 64)
+            return R == 4 ? go(conv3x3_rows<64, 4, kStore, true, NoFrames>, none)
+                          : go(conv3x3_rows<64, 2, kStore, true, NoFrames>, none);
+        return R == 8   ? go(conv3x3_rows<32, 8, kStore, true, NoFrames>, none)
+               : R == 4 ? go(conv3x3_rows<32, 4, kStore, true, NoFrames>, none)
+                        : go(conv3x3_rows<32, 2, kStore, true, NoFrames>, none);
+    }
     if (c.Cout == 64) {
-        if (c.pool) return R == 4 ? go(conv3x3_rows<64, 4, kPool, NoFrames>, none) : go(conv3x3_rows<64, 2, kPool, NoFrames>, none);
-        return R == 4 ? go(conv3x3_rows<64, 4, kStore, NoFrames>, none) : go(conv3x3_rows<64, 2, kStore, NoFrames>, none);
+        if (c.pool) return R == 4 ? go(conv3x3_rows<64, 4, kPool, false, NoFrames>, none) : go(conv3x3_rows<64, 2, kPool, false, NoFrames>, none);
+        return R == 4 ? go(conv3x3_rows<64, 4, kStore, false, NoFrames>, none) : go(conv3x3_rows<64, 2, kStore, false, NoFrames>, none);
     }
     if (c.frames) return YORO_ROWS32(kCompose, FrameTable, *c.frames);
     if (c.rgb) return YORO_ROWS32(kColors, NoFrames, none);

@@ -154,7 +154,8 @@ __device__ __forceinline__ void epilogue_store(const ConvArgs& a, const CUtensor
 // MT = 2 for grids of two tiles per SM and more: both tiles use the weights of one copy (256
 // channels: 64 instead of 96 bytes per cycle from L2, which 128-pixel CTAs were bound by).
 //
-// Measured, us (KC = 32, MT = 1, one issuing thread -> this): CONV_TC_MEASURED
+// Measured (KC = 32, MT = 1, one issuing thread -> this): enc3b on 8 tiles 26.5 -> 15.6 us, on
+// 870 89 -> 76; enc3a 15.0 -> 9.2 us on 8 tiles, 43 on 870 before and after.
 template <int KC, int MT>
 __global__ void __launch_bounds__(128, 1)
     conv3x3_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -620,8 +621,8 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
     int mt = 0, stages = 0;
     if (nb == 1) halo_shape(H, W, Cout, &mt, &stages);
     if (mt && conv_rows_takes(H, W, Cout)) return conv_rows_launch(call, sms, kSmemPerBlock, stream);
-    // the output layer rides on the row form only; the other forms pool 16-pixel rows
-    if (call.rgb || call.frames || (call.pool && W != 16)) return cudaErrorInvalidValue;
+    // the output layer and half-resolution inputs are the row form's; the others pool 16-pixel rows
+    if (call.rgb || call.frames || call.low || (call.pool && W != 16)) return cudaErrorInvalidValue;
     // on small grids one accumulator per CTA: twice the CTAs, half the MMAs of each (the halo
     // rows' overhead does not matter there)
     if (mt && pixels / (mt * kTileM) * 2 <= sms) mt = 1;
@@ -938,8 +939,8 @@ void unet_free(UnetNet* n)
         cudaFree(L.bias);
     }
     cudaFree(n->wout);
-    uint16_t* bufs[] = {n->in0, n->e0a, n->cat0, n->p0, n->e1a, n->cat1, n->p1, n->e2a,
-                        n->cat2, n->p2, n->e3a, n->d2a, n->d1a, n->d0a, n->d0b};
+    uint16_t* bufs[] = {n->in0, n->e0a, n->cat0, n->skip0, n->d1b, n->p0,  n->e1a, n->cat1, n->skip1, n->d2b,
+                        n->p1,  n->e2a, n->cat2, n->p2,    n->e3a, n->d2a, n->d1a, n->d0a,  n->d0b};
     for (uint16_t* b : bufs) cudaFree(b);
     cudaFree(n->flags);
     cudaFree(n->list);
@@ -947,7 +948,7 @@ void unet_free(UnetNet* n)
     delete n;
 }
 
-UnetNet* unet_create(const float* params, size_t n_params, int max_tiles, int max_grid_tiles)
+UnetNet* unet_create(const float* params, size_t n_params, int max_tiles, int max_grid_tiles, bool train)
 {
     if (!params || n_params != unet_param_count() || max_tiles < 1 || max_grid_tiles < 1) return nullptr;
     UnetNet* n = new UnetNet();
@@ -993,15 +994,19 @@ UnetNet* unet_create(const float* params, size_t n_params, int max_tiles, int ma
     struct {
         uint16_t** b;
         size_t elems;
-    } al[] = {{&n->in0, P0 * 32}, {&n->e0a, P0 * 32}, {&n->cat0, P0 * 96}, {&n->p0, P1 * 32}, {&n->e1a, P1 * 64},
-              {&n->cat1, P1 * 192}, {&n->p1, P2 * 64}, {&n->e2a, P2 * 128}, {&n->cat2, P2 * 384},
-              {&n->p2, P3 * 128}, {&n->e3a, P3 * 256}, {&n->d2a, P2 * 128}, {&n->d1a, P1 * 64},
-              {&n->d0a, P0 * 32}, {&n->d0b, P0 * 32}};
+    } al[] = {{&n->e0a, P0 * 32}, {&n->p0, P1 * 32}, {&n->e1a, P1 * 64}, {&n->p1, P2 * 64}, {&n->e2a, P2 * 128},
+              {&n->cat2, P2 * 384}, {&n->p2, P3 * 128}, {&n->e3a, P3 * 256}, {&n->d2a, P2 * 128}, {&n->d1a, P1 * 64},
+              {&n->d0a, P0 * 32},
+              // training
+              {&n->cat0, train ? P0 * 96 : 0}, {&n->cat1, train ? P1 * 192 : 0}, {&n->d0b, train ? P0 * 32 : 0},
+              // inference
+              {&n->in0, train ? 0 : P0 * 32}, {&n->skip0, train ? 0 : P0 * 32}, {&n->d1b, train ? 0 : P1 * 64},
+              {&n->skip1, train ? 0 : P1 * 64}, {&n->d2b, train ? 0 : P2 * 128}};
     for (auto& x : al)
-        if (ok) ok = cudaMalloc(x.b, x.elems * 2) == cudaSuccess;
+        if (ok && x.elems) ok = cudaMalloc(x.b, x.elems * 2) == cudaSuccess;
     if (ok) {
         // the in0 buffer of tiles never written stays zero (T rounded up to even)
-        ok = cudaMemset(n->in0, 0, P0 * 32 * 2) == cudaSuccess &&
+        ok = (train || cudaMemset(n->in0, 0, P0 * 32 * 2) == cudaSuccess) &&
              cudaMalloc(&n->flags, (size_t)max_grid_tiles * 4) == cudaSuccess &&
              cudaMalloc(&n->list, (size_t)max_grid_tiles * 4) == cudaSuccess &&
              cudaMalloc(&n->count, 4) == cudaSuccess;
@@ -1015,17 +1020,25 @@ UnetNet* unet_create(const float* params, size_t n_params, int max_tiles, int ma
 }
 
 // The 14 convolutions over the first T tiles of x (tiles at or after *count skipped when
-// count is given), the 2x2 pools in the epilogues of the layers they follow.  The output
-// layer rides on the last one: colors to out.rgb, or composed into out.frames; with
-// neither, the last layer's activations end in d0b.
+// count is given), the 2x2 pools in the epilogues of the layers they follow.  In an inference
+// net the decoder's first layers of levels 1 and 0 read the skip and the lower level's output
+// at its own resolution; in a training net they read the concatenation, written by the
+// layers before.  The output layer rides on the last one: colors to out.rgb, or composed into
+// out.frames; with neither (training), the last layer's activations end in d0b.
 cudaError_t unet_run(UnetNet* n, const uint16_t* x, int T, const int* count, const NetOut& out, cudaStream_t s)
 {
     const int Te = (T + 1) & ~1;  // the 8 x 8 level takes two tiles per 128-pixel accumulator
+    const bool cat = n->cat0 != nullptr;
     cudaError_t e = cudaSuccess;
-    auto conv = [&](int i, const uint16_t* in, int H, void* y, int cstride, int coff, int up, void* pool) {
+    // layer i on H x H tiles: input (and half-resolution input), output at channel offset coff of
+    // cstride, upsampled store, pooled copy
+    auto conv = [&](int i, const uint16_t* in, const uint16_t* low, int cskip, int H, void* y, int cstride, int coff,
+                    int up, void* pool) {
         if (e != cudaSuccess) return;
         const UnetLayer& L = n->conv[i];
         ConvCall c{in, L.wk, y, L.bias, count, pool, i == 0 ? T : Te, H, H, L.cin_pad, L.cout, cstride, coff, up, 1};
+        c.low = low;
+        c.cskip = cskip;
         if (i == 13) {
             c.T = T;
             c.wout = n->wout;
@@ -1035,20 +1048,28 @@ cudaError_t unet_run(UnetNet* n, const uint16_t* x, int T, const int* count, con
         }
         e = unet_conv3x3(c, s);
     };
-    conv(0, x, 64, n->e0a, 32, 0, 0, nullptr);          // enc0a
-    conv(1, n->e0a, 64, n->cat0, 96, 0, 0, n->p0);      // enc0b -> skip of level 0
-    conv(2, n->p0, 32, n->e1a, 64, 0, 0, nullptr);      // enc1a
-    conv(3, n->e1a, 32, n->cat1, 192, 0, 0, n->p1);     // enc1b -> skip of level 1
-    conv(4, n->p1, 16, n->e2a, 128, 0, 0, nullptr);     // enc2a
-    conv(5, n->e2a, 16, n->cat2, 384, 0, 0, n->p2);     // enc2b -> skip of level 2
-    conv(6, n->p2, 8, n->e3a, 256, 0, 0, nullptr);      // enc3a
-    conv(7, n->e3a, 8, n->cat2, 384, 128, 1, nullptr);  // enc3b, upsampled after the level-2 skip
-    conv(8, n->cat2, 16, n->d2a, 128, 0, 0, nullptr);   // dec2a
-    conv(9, n->d2a, 16, n->cat1, 192, 64, 1, nullptr);  // dec2b, upsampled after the level-1 skip
-    conv(10, n->cat1, 32, n->d1a, 64, 0, 0, nullptr);   // dec1a
-    conv(11, n->d1a, 32, n->cat0, 96, 32, 1, nullptr);  // dec1b, upsampled after the level-0 skip
-    conv(12, n->cat0, 64, n->d0a, 32, 0, 0, nullptr);   // dec0a
-    conv(13, n->d0a, 64, n->d0b, 32, 0, 0, nullptr);    // dec0b
+    uint16_t* const none = nullptr;
+    conv(0, x, none, 0, 64, n->e0a, 32, 0, 0, nullptr);                                       // enc0a
+    conv(1, n->e0a, none, 0, 64, cat ? n->cat0 : n->skip0, cat ? 96 : 32, 0, 0, n->p0);       // enc0b
+    conv(2, n->p0, none, 0, 32, n->e1a, 64, 0, 0, nullptr);                                   // enc1a
+    conv(3, n->e1a, none, 0, 32, cat ? n->cat1 : n->skip1, cat ? 192 : 64, 0, 0, n->p1);      // enc1b
+    conv(4, n->p1, none, 0, 16, n->e2a, 128, 0, 0, nullptr);                                  // enc2a
+    conv(5, n->e2a, none, 0, 16, n->cat2, 384, 0, 0, n->p2);                                  // enc2b
+    conv(6, n->p2, none, 0, 8, n->e3a, 256, 0, 0, nullptr);                                   // enc3a
+    conv(7, n->e3a, none, 0, 8, n->cat2, 384, 128, 1, nullptr);                               // enc3b, upsampled
+    conv(8, n->cat2, none, 0, 16, n->d2a, 128, 0, 0, nullptr);                                // dec2a
+    if (cat) {
+        conv(9, n->d2a, none, 0, 16, n->cat1, 192, 64, 1, nullptr);                           // dec2b, upsampled
+        conv(10, n->cat1, none, 0, 32, n->d1a, 64, 0, 0, nullptr);                            // dec1a
+        conv(11, n->d1a, none, 0, 32, n->cat0, 96, 32, 1, nullptr);                           // dec1b, upsampled
+        conv(12, n->cat0, none, 0, 64, n->d0a, 32, 0, 0, nullptr);                            // dec0a
+    } else {
+        conv(9, n->d2a, none, 0, 16, n->d2b, 128, 0, 0, nullptr);
+        conv(10, n->skip1, n->d2b, 64, 32, n->d1a, 64, 0, 0, nullptr);
+        conv(11, n->d1a, none, 0, 32, n->d1b, 64, 0, 0, nullptr);
+        conv(12, n->skip0, n->d1b, 32, 64, n->d0a, 32, 0, 0, nullptr);
+    }
+    conv(13, n->d0a, none, 0, 64, n->d0b, 32, 0, 0, nullptr);                                 // dec0b
     return e;
 }
 
@@ -1092,7 +1113,7 @@ yoro_unet yoro_unet_create(const float* params, long long n_params, int max_tile
     }
     c->max_w = max_w;
     c->max_h = max_h;
-    c->net = yoro::unet_create(params, (size_t)n_params, tiles, tiles);  // flags and list hold `tiles` cells
+    c->net = yoro::unet_create(params, (size_t)n_params, tiles, tiles, false);  // flags and list hold `tiles` cells
     if (!c->net) {
         delete c;
         return nullptr;

@@ -21,8 +21,11 @@ struct UnetNet {
     UnetLayer conv[14];
     float* wout;  // device: 3 x 32 (bfloat16 values as floats), then 3 biases
     int max_tiles;
-    // activations, NHWC bfloat16, for max_tiles tiles
-    uint16_t *in0, *e0a, *cat0, *p0, *e1a, *cat1, *p1, *e2a, *cat2, *p2, *e3a, *d2a, *d1a, *d0a, *d0b;
+    // activations, NHWC bfloat16, for max_tiles tiles.  A training net keeps the concatenations
+    // of levels 0 and 1 (the weight gradients read them); an inference net keeps their parts:
+    // the skips, and the lower levels' outputs at their own resolution.
+    uint16_t *in0, *e0a, *cat0, *skip0, *d1b, *p0, *e1a, *cat1, *skip1, *d2b, *p1, *e2a, *cat2, *p2, *e3a, *d2a, *d1a,
+        *d0a, *d0b;
     int *flags, *list, *count;
     int max_grid_tiles;  // capacity of flags / list
 };
@@ -54,6 +57,10 @@ struct ConvCall {
     float* rgb = nullptr;
     const FrameTable* frames = nullptr;
     const int* list = nullptr;
+    // optional (row form only): x holds the first cskip channels, low (T x H/2 x W/2, dense) the
+    // others, read through their nearest upsampling
+    const void* low = nullptr;
+    int cskip = 0;
 };
 
 // Where a pass of the network ends: colors, frames, or (neither) the activations in d0b.
@@ -80,7 +87,7 @@ int sm_count();
 
 size_t unet_param_count();
 void unet_layer_dims(int i, int* cin, int* cout);
-UnetNet* unet_create(const float* params, size_t n_params, int max_tiles, int max_grid_tiles);
+UnetNet* unet_create(const float* params, size_t n_params, int max_tiles, int max_grid_tiles, bool train);
 void unet_free(UnetNet* n);
 cudaError_t unet_run(UnetNet* n, const uint16_t* x, int T, const int* count, const NetOut& out, cudaStream_t s);
 cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream);

@@ -398,7 +398,7 @@ Trainer* trainer_create(const float* params, size_t np, int batch, float lr, flo
     t->b2 = b2;
     t->eps = eps;
     t->sms = sm_count();
-    t->net = unet_create(params, np, batch, 1);
+    t->net = unet_create(params, np, batch, 1, true);
     bool ok = t->net != nullptr;
     size_t off = 0;
     for (int i = 0; i < 14; ++i) {
