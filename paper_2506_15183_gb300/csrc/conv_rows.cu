@@ -55,7 +55,11 @@ constexpr int kAccCols = 256;                   // tensor-memory columns of an a
 constexpr int kMaxPairs = 11;                   // row-pair slots (bounds the barrier array)
 constexpr int kStageBytes = 2 * 32 * kKc * 2;   // a warp's 32 pixels of two rows, 32 channels
 constexpr int kStores = 4 * 2 * kStageBytes;    // two staging buffers for each of four warps
-constexpr int kRowsThreads = 192;               // 224 with an upsampled input (one more warp)
+// Warps: one copies, one issues MMAs, four read back and store; the output layer's epilogues
+// take eight (its 96 products and sums per pixel kept four busy longer than the MMAs: dec0b on
+// 870 tiles 127 us), an upsampled input one more that doubles its rows.
+__host__ __device__ constexpr int epilogue_warps(int mode) { return mode >= 2 ? 8 : 4; }
+__host__ __device__ constexpr int rows_threads(int mode, bool up) { return 64 + 32 * epilogue_warps(mode) + (up ? 32 : 0); }
 constexpr int kLowBytes = kRowBytes / 2;        // a row of the half-resolution input: 64 pixels
 constexpr int kLow = 6;                         // its landing slots
 
@@ -75,6 +79,7 @@ struct RowsArgs {
 
 // What the epilogue does with a pixel's channels.
 enum { kStore, kPool, kColors, kCompose };
+static_assert(kColors == 2, "epilogue_warps()");
 
 // One 32-channel slice of one pixel: bias, ReLU, rounding to bfloat16.
 __device__ __forceinline__ void finish(const uint32_t (&r)[32], const float* bias, int relu, uint32_t (&q)[16])
@@ -100,12 +105,12 @@ struct NoFrames {};
 // upsampled tensors were half of the memory traffic of the decoder's first layers and most of
 // what the layers below them wrote.
 template <int COUT, int R, int MODE, bool UP, class Frames>
-__global__ void __launch_bounds__(kRowsThreads + (UP ? 32 : 0), 1)
+__global__ void __launch_bounds__(rows_threads(MODE, UP), 1)
     conv3x3_rows(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmU, const RowsArgs a,
                  const __grid_constant__ Frames ft)
 {
-    constexpr int kThreads = kRowsThreads + (UP ? 32 : 0);
+    constexpr int kThreads = rows_threads(MODE, UP), kEpi = epilogue_warps(MODE);
     constexpr int kSkipSlots = (R + 2) / 2;             // slots of a channel block: rows -1 .. R
     constexpr int kLowRows = R / 2 + 2;                 // half-resolution rows under them
     constexpr int kUpSlots = (kLowRows + 1) / 2;
@@ -152,7 +157,7 @@ __global__ void __launch_bounds__(kRowsThreads + (UP ? 32 : 0), 1)
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(&afull[s], 1);
-            mbar_init(&aempty[s], 4);
+            mbar_init(&aempty[s], kEpi);
         }
         for (int s = 0; s < kLow; ++s) {
             mbar_init(&lfull[s], 1);
@@ -246,89 +251,94 @@ __global__ void __launch_bounds__(kRowsThreads + (UP ? 32 : 0), 1)
         // lanes x = 0 and x = W - 1 of each image
         const uint32_t lo2 = W == 128 ? 0u : 1u, lo13 = W == 32 ? 1u : 0u;
         const uint32_t hi3 = 0x80000000u, hi1 = W == 128 ? 0u : hi3, hi02 = W == 32 ? hi3 : 0u;
-        int slot0 = 0, ph0 = 0, ws = 0, wph = 0;
-        bool ok = true;
-        int it = 0;
-        for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++it) {
-            const int g = u / bands, y0 = (u - g * bands) * R;
-            const bool top = y0 == 0, bottom = y0 + R == H;  // row -1 or R lies outside the image
-            const uint32_t acc = tmem + (uint32_t)((it & 1) * kAccCols);
-            const uint64_t deadline = globaltimer() + kWaitNs;
-            if (!(ok = mbar_wait_warp(&aempty[it & 1], (it >> 1) & 1, deadline))) break;
-            tc_fence_after();
-            for (int cb = 0; cb < cb_n && ok; ++cb) {
-                if (resident) ws = cb;
-                if (!resident || it == 0)
-                    if (!(ok = mbar_wait_warp(&wfull[ws], wph, deadline))) break;
-                int slot = slot0, ph = ph0;
-                const bool up = UP && cb >= cb_skip;
+        // false once a wait ran out.  Every value below is the same in all lanes and no issue
+        // hangs on a condition that only a vote makes uniform, so the loop stays in the uniform
+        // datapath.
+        auto issue_all = [&]() -> bool {
+            int slot0 = 0, ph0 = 0, ws = 0, wph = 0, it = 0;
+            for (int u = blockIdx.x; u < units; u += gridDim.x, ++it) {
+                const int g = u / bands, y0 = (u - g * bands) * R;
+                const bool top = y0 == 0, bottom = y0 + R == H;  // row -1 or R lies outside the image
+                const uint32_t acc = tmem + (uint32_t)((it & 1) * kAccCols);
+                const uint64_t deadline = globaltimer() + kWaitNs;
+                if (!mbar_wait_warp(&aempty[it & 1], (it >> 1) & 1, deadline)) return false;
+                tc_fence_after();
+                for (int cb = 0; cb < cb_n; ++cb) {
+                    if (resident) ws = cb;
+                    if (!resident || it == 0)
+                        if (!mbar_wait_warp(&wfull[ws], wph, deadline)) return false;
+                    const bool up = UP && cb >= cb_skip;
+                    int slot = slot0, ph = ph0;
 #pragma unroll
-                for (int dx = 0; dx < 3; ++dx) {
-                    const uint32_t m0 = dx == 0 ? 1u : dx == 2 ? hi02 : 0u;
-                    const uint32_t m1 = dx == 0 ? lo13 : dx == 2 ? hi1 : 0u;
-                    const uint32_t m2 = dx == 0 ? lo2 : dx == 2 ? hi02 : 0u;
-                    const uint32_t m3 = dx == 0 ? lo13 : dx == 2 ? hi3 : 0u;
-                    const uint64_t wb = dw + (uint64_t)((uint32_t)(ws * kWBytes + dx * 3 * COUT * kKc * 2) >> 4);
-                    slot = slot0;
-                    ph = ph0;
-                    // input row r, in row `half` of the current slot, into output rows r + 1 .. r - 1
-                    // inside the unit (ascending columns)
-                    auto row = [&](int r, int half) {
-                        const int lo = r < 1 ? 0 : r - 1, hi = r + 1 > R - 1 ? R - 1 : r + 1, n = hi - lo + 1;
-                        const uint32_t id = n == 3 ? id3 : n == 2 ? id2 : id1;
-                        const uint64_t da = drow + (uint64_t)((uint32_t)slot * (uint32_t)(kPairBytes >> 4) +
-                                                              (uint32_t)(half * (kRowBytes >> 4) + 4 * dx)) - 4;
-                        const uint64_t db = wb + (uint64_t)((r + 1 - hi) * (COUT * kKc * 2 >> 4));
-                        const uint32_t d = acc + (uint32_t)((R - 1 - hi) * COUT);
-                        mma_bf16_masked(el, d, da, db, id, m0, m1, m2, m3);
-                        mma_bf16_masked(el, d, da + 2, db + 2, id, m0, m1, m2, m3);
-                    };
-                    auto next = [&]() {
-                        if (dx == 2 && ok) mma_commit_elected(el, &empty[slot]);
-                        if (++slot == NP) {
-                            slot = 0;
-                            ph ^= 1;
+                    for (int dx = 0; dx < 3; ++dx) {
+                        const uint32_t m0 = dx == 0 ? 1u : dx == 2 ? hi02 : 0u;
+                        const uint32_t m1 = dx == 0 ? lo13 : dx == 2 ? hi1 : 0u;
+                        const uint32_t m2 = dx == 0 ? lo2 : dx == 2 ? hi02 : 0u;
+                        const uint32_t m3 = dx == 0 ? lo13 : dx == 2 ? hi3 : 0u;
+                        const uint64_t wb = dw + (uint64_t)((uint32_t)(ws * kWBytes + dx * 3 * COUT * kKc * 2) >> 4);
+                        slot = slot0;
+                        ph = ph0;
+                        // input row r, in row `half` of the current slot, into output rows r + 1 .. r - 1
+                        // inside the unit (ascending columns)
+                        auto row = [&](int r, int half) {
+                            const int lo = r < 1 ? 0 : r - 1, hi = r + 1 > R - 1 ? R - 1 : r + 1, n = hi - lo + 1;
+                            const uint32_t id = n == 3 ? id3 : n == 2 ? id2 : id1;
+                            const uint64_t da = drow + (uint64_t)((uint32_t)slot * (uint32_t)(kPairBytes >> 4) +
+                                                                  (uint32_t)(half * (kRowBytes >> 4) + 4 * dx)) - 4;
+                            const uint64_t db = wb + (uint64_t)((r + 1 - hi) * (COUT * kKc * 2 >> 4));
+                            const uint32_t d = acc + (uint32_t)((R - 1 - hi) * COUT);
+                            mma_bf16_masked(el, d, da, db, id, m0, m1, m2, m3);
+                            mma_bf16_masked(el, d, da + 2, db + 2, id, m0, m1, m2, m3);
+                        };
+                        auto next = [&]() {
+                            if (dx == 2) mma_commit_elected(el, &empty[slot]);
+                            if (++slot == NP) {
+                                slot = 0;
+                                ph ^= 1;
+                            }
+                        };
+                        if (!up) {
+#pragma unroll
+                            for (int r = -1; r <= R; ++r) {
+                                const bool second = (r & 1) == 0;  // of the pair in this slot
+                                if (dx == 0 && !second) {
+                                    if (!mbar_wait_warp(&full[slot], ph, deadline)) return false;
+                                    tc_fence_after();
+                                }
+                                if (!(r == -1 && top) && !(r == R && bottom)) row(r, second ? 1 : 0);
+                                if (second) next();
+                            }
+                        } else {
+                            // half-resolution row i = 0 .. kLowRows - 1 of the unit, in row i & 1 of its slot,
+                            // is input rows 2i - 2 and 2i - 1
+#pragma unroll
+                            for (int i = 0; i < kLowRows; ++i) {
+                                if (dx == 0 && !(i & 1)) {
+                                    if (!mbar_wait_warp(&full[slot], ph, deadline)) return false;
+                                    tc_fence_after();
+                                }
+#pragma unroll
+                                for (int r = 2 * i - 2; r <= 2 * i - 1; ++r)
+                                    if (r >= -1 && r <= R && !(r == -1 && top) && !(r == R && bottom)) row(r, i & 1);
+                                if ((i & 1) || i == kLowRows - 1) next();
+                            }
                         }
-                    };
-                    auto arrived = [&]() {
-                        if (dx == 0) {
-                            ok = ok && mbar_wait_warp(&full[slot], ph, deadline);
-                            tc_fence_after();
-                        }
-                    };
-                    if (!up) {
-#pragma unroll
-                        for (int r = -1; r <= R; ++r) {
-                            const bool second = (r & 1) == 0;  // of the pair in this slot
-                            if (!second) arrived();
-                            if (ok && !((r == -1 && top) || (r == R && bottom))) row(r, second ? 1 : 0);
-                            if (second) next();
-                        }
-                    } else {
-                        // half-resolution row i = 0 .. kLowRows - 1 of the unit, in row i & 1 of its slot, is
-                        // input rows 2i - 2 and 2i - 1
-#pragma unroll
-                        for (int i = 0; i < kLowRows; ++i) {
-                            if (!(i & 1)) arrived();
-#pragma unroll
-                            for (int r = 2 * i - 2; r <= 2 * i - 1; ++r)
-                                if (r >= -1 && r <= R && ok && !((r == -1 && top) || (r == R && bottom))) row(r, i & 1);
-                            if ((i & 1) || i == kLowRows - 1) next();
+                    }
+                    slot0 = slot;
+                    ph0 = ph;
+                    if (!resident) {
+                        mma_commit_elected(el, &wempty[ws]);
+                        if (++ws == WS) {
+                            ws = 0;
+                            wph ^= 1;
                         }
                     }
                 }
-                slot0 = slot;
-                ph0 = ph;
-                if (!resident) {
-                    if (ok) mma_commit_elected(el, &wempty[ws]);
-                    if (++ws == WS) {
-                        ws = 0;
-                        wph ^= 1;
-                    }
-                }
+                mma_commit_elected(el, &afull[it & 1]);
             }
-            if (ok) mma_commit_elected(el, &afull[it & 1]);
-        }
+            return true;
+        };
+        const bool ok = issue_all();
         if (!ok) {  // the MMAs issued so far: wait for them (bounded)
             if (el) timed_out();
             mma_commit_elected(el, drain);
@@ -423,8 +433,9 @@ __global__ void __launch_bounds__(kRowsThreads + (UP ? 32 : 0), 1)
                     mask = ft.mask[f] + (ptrdiff_t)gy * pitch + gx;
                     rgba = ft.rgba[f] + (ptrdiff_t)gy * pitch + gx;
                 }
+                // the two groups of four warps take every other row
 #pragma unroll 1
-                for (int r = 0; r < R; ++r) {
+                for (int r = (warp - 2) >> 2; r < R; r += kEpi / 4) {
                     uint32_t v[32], p[16];
                     const uint32_t t = acc + (uint32_t)((R - 1 - r) * COUT);
                     tmem_ld32_async(t, v);
@@ -641,7 +652,7 @@ cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStrea
     auto go = [&](auto kernel, const auto& frames) -> cudaError_t {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
         if (e != cudaSuccess) return e;
-        kernel<<<grid, kRowsThreads + (up ? 32 : 0), smem, stream>>>(ta, tb, ty, tu, a, frames);
+        kernel<<<grid, rows_threads(c.frames || c.rgb ? kColors : kStore, up), smem, stream>>>(ta, tb, ty, tu, a, frames);
         return cudaGetLastError();
     };
     const NoFrames none;
