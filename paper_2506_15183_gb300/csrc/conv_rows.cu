@@ -177,6 +177,8 @@ __global__ void __launch_bounds__(rows_threads(MODE, UP), 1)
     for (int c = threadIdx.x; c < COUT; c += kThreads) sbias[c] = __ldg(a.bias + c);
     if (MODE == kColors || MODE == kCompose)
         for (int c = threadIdx.x; c < 99; c += kThreads) swout[c] = __ldg(a.wout + c);
+    pdl_wait();
+    pdl_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -652,8 +654,8 @@ cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStrea
     auto go = [&](auto kernel, const auto& frames) -> cudaError_t {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
         if (e != cudaSuccess) return e;
-        kernel<<<grid, rows_threads(c.frames || c.rgb ? kColors : kStore, up), smem, stream>>>(ta, tb, ty, tu, a, frames);
-        return cudaGetLastError();
+        return launch_conv(kernel, dim3((unsigned)grid), rows_threads(c.frames || c.rgb ? kColors : kStore, up), smem,
+                           stream, c.pdl, ta, tb, ty, tu, a, frames);
     };
     const NoFrames none;
 #define YORO_ROWS32(MODE, FRAMES, TABLE)                                \

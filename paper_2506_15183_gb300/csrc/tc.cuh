@@ -99,6 +99,12 @@ __device__ __forceinline__ void tma_store_5d(const CUtensorMap* map, const void*
                  : "memory");
 }
 
+// Programmatic dependent launch: wait until the kernel before in the stream has completed and
+// its writes are visible (at once where this kernel was launched without the attribute), and
+// let the kernel after start its prologue.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -255,6 +261,26 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b)
     const __nv_bfloat162 m =
         __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
     return *reinterpret_cast<const uint32_t*>(&m);
+}
+
+// Launch of a kernel whose predecessor in the stream it may overlap with its prologue (pdl): the
+// kernel calls pdl_wait() before it touches what the predecessor writes.
+template <class... P, class... A>
+cudaError_t launch_conv(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, bool pdl,
+                        const A&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 }  // namespace yoro

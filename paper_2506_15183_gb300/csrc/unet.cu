@@ -194,6 +194,8 @@ __global__ void __launch_bounds__(128, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_wait();
+    pdl_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -355,6 +357,7 @@ __global__ void __launch_bounds__(128, 1)
         counts[2] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        pdl_wait();
         const int b0 = blockIdx.x, n0 = b0 / bands_per_tile, y0 = (b0 - n0 * bands_per_tile) * R;
         for (int k = 0; k < first; ++k) {
             issue_a(k, n0, y0);
@@ -368,6 +371,8 @@ __global__ void __launch_bounds__(128, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     for (int c = threadIdx.x; c < a.bn; c += blockDim.x) sbias[c] = __ldg(a.bias + nb + c);
+    pdl_wait();
+    pdl_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -715,8 +720,8 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
         // as many CTAs as fit at once (shared memory; registers allow 5), each walking bands
         const int per_sm = std::min(5, (int)(kSmemPerSm / (hsmem + 1024)));
         const long long grid = std::min<long long>(ctas, (long long)std::max(per_sm, 1) * sms);
-        conv3x3_halo<<<dim3((unsigned)grid, parts), 128, hsmem, stream>>>(ta, tb, ty, a, (int)ctas);
-        return cudaGetLastError();
+        return launch_conv(conv3x3_halo, dim3((unsigned)grid, parts), 128, hsmem, stream, call.pdl, ta, tb, ty, a,
+                           (int)ctas);
     }
     // one-tile form: a lone CTA (and one with two tiles, whose accumulators take the tensor
     // memory) rings as deep as its SM's shared memory, else two CTAs share an SM
@@ -730,8 +735,8 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
     auto go = [&](auto kernel) -> cudaError_t {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerBlock);
         if (e != cudaSuccess) return e;
-        kernel<<<dim3((unsigned)ctas, parts), 128, conv_smem_bytes(stage, a.stages), stream>>>(ta, tb, ty, a);
-        return cudaGetLastError();
+        return launch_conv(kernel, dim3((unsigned)ctas, parts), 128, conv_smem_bytes(stage, a.stages), stream, call.pdl,
+                           ta, tb, ty, a);
     };
     if (kc == 64) return tt == 2 ? go(conv3x3_tc<64, 2>) : go(conv3x3_tc<64, 1>);
     return tt == 2 ? go(conv3x3_tc<32, 2>) : go(conv3x3_tc<32, 1>);
@@ -1039,6 +1044,7 @@ cudaError_t unet_run(UnetNet* n, const uint16_t* x, int T, const int* count, con
         ConvCall c{in, L.wk, y, L.bias, count, pool, i == 0 ? T : Te, H, H, L.cin_pad, L.cout, cstride, coff, up, 1};
         c.low = low;
         c.cskip = cskip;
+        c.pdl = i > 0;  // the kernel before is the layer before
         if (i == 13) {
             c.T = T;
             c.wout = n->wout;

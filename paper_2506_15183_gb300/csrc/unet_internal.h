@@ -61,6 +61,9 @@ struct ConvCall {
     // others, read through their nearest upsampling
     const void* low = nullptr;
     int cskip = 0;
+    // the kernel before in the stream is a convolution whose prologue-time state (weights, biases,
+    // count) this one does not depend on: start the prologue while it ends
+    bool pdl = false;
 };
 
 // Where a pass of the network ends: colors, frames, or (neither) the activations in d0b.
