@@ -101,6 +101,8 @@ __global__ void __launch_bounds__(kDwThreads, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_wait();
+    pdl_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -196,6 +198,8 @@ __global__ void __launch_bounds__(kDwThreads, 1)
 __global__ void __launch_bounds__(256) dw_reduce_kernel(const float* __restrict__ ws, int shares, int co_tile, int cbs,
                                                         int cin, float* __restrict__ dW)
 {
+    pdl_wait();
+    pdl_launch();
     __shared__ float4 part[8][32];
     const int l = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int quads = co_tile * (kDwTile / 4);  // of a tile
@@ -231,8 +235,8 @@ cudaError_t launch(const CUtensorMap& tz, const CUtensorMap& tx, int H, int boxe
     const cudaError_t e =
         cudaFuncSetAttribute(conv3x3_dw<S, COB>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem);
     if (e != cudaSuccess) return e;
-    conv3x3_dw<S, COB><<<dim3((unsigned)shares, (unsigned)tiles), kDwThreads, S::kSmem, s>>>(tz, tx, H, boxes, cbs, ws);
-    return cudaGetLastError();
+    return launch_kernel(conv3x3_dw<S, COB>, dim3((unsigned)shares, (unsigned)tiles), kDwThreads, S::kSmem, s, true, tz, tx,
+                         H, boxes, cbs, ws);
 }
 
 }  // namespace
@@ -272,8 +276,8 @@ cudaError_t conv_dw_launch(const void* dZ, const void* X, int xcs, int T, int si
     else if (side == 16) e = launch<16, 4, 4>(tz, tx, side, boxes, tiles, cbs, shares, ws, s);
     else e = launch<8, 4, 4>(tz, tx, side, boxes, tiles, cbs, shares, ws, s);
     if (e != cudaSuccess) return e;
-    dw_reduce_kernel<<<(unsigned)(tiles * (32 * cob * kDwTile / 128)), 256, 0, s>>>(ws, shares, 32 * cob, cbs, cin, dW);
-    return cudaGetLastError();
+    return launch_kernel(dw_reduce_kernel, dim3((unsigned)(tiles * (32 * cob * kDwTile / 128))), 256, 0, s, true, (const float*)ws, shares, 32 * cob, cbs, cin,
+                         dW);
 }
 
 unsigned conv_dw_status_take()

@@ -654,7 +654,7 @@ cudaError_t conv_rows_launch(const ConvCall& c, int sms, int smem_max, cudaStrea
     auto go = [&](auto kernel, const auto& frames) -> cudaError_t {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
         if (e != cudaSuccess) return e;
-        return launch_conv(kernel, dim3((unsigned)grid), rows_threads(c.frames || c.rgb ? kColors : kStore, up), smem,
+        return launch_kernel(kernel, dim3((unsigned)grid), rows_threads(c.frames || c.rgb ? kColors : kStore, up), smem,
                            stream, c.pdl, ta, tb, ty, tu, a, frames);
     };
     const NoFrames none;

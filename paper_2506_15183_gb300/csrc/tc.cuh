@@ -266,7 +266,7 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b)
 // Launch of a kernel whose predecessor in the stream it may overlap with its prologue (pdl): the
 // kernel calls pdl_wait() before it touches what the predecessor writes.
 template <class... P, class... A>
-cudaError_t launch_conv(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, bool pdl,
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, bool pdl,
                         const A&... args)
 {
     cudaLaunchConfig_t cfg = {};

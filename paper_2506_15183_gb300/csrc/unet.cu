@@ -720,7 +720,7 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
         // as many CTAs as fit at once (shared memory; registers allow 5), each walking bands
         const int per_sm = std::min(5, (int)(kSmemPerSm / (hsmem + 1024)));
         const long long grid = std::min<long long>(ctas, (long long)std::max(per_sm, 1) * sms);
-        return launch_conv(conv3x3_halo, dim3((unsigned)grid, parts), 128, hsmem, stream, call.pdl, ta, tb, ty, a,
+        return launch_kernel(conv3x3_halo, dim3((unsigned)grid, parts), 128, hsmem, stream, call.pdl, ta, tb, ty, a,
                            (int)ctas);
     }
     // one-tile form: a lone CTA (and one with two tiles, whose accumulators take the tensor
@@ -735,7 +735,7 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
     auto go = [&](auto kernel) -> cudaError_t {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerBlock);
         if (e != cudaSuccess) return e;
-        return launch_conv(kernel, dim3((unsigned)ctas, parts), 128, conv_smem_bytes(stage, a.stages), stream, call.pdl,
+        return launch_kernel(kernel, dim3((unsigned)ctas, parts), 128, conv_smem_bytes(stage, a.stages), stream, call.pdl,
                            ta, tb, ty, a);
     };
     if (kc == 64) return tt == 2 ? go(conv3x3_tc<64, 2>) : go(conv3x3_tc<64, 1>);
@@ -772,6 +772,8 @@ __global__ void tile_flags_kernel(const __grid_constant__ FrameTable ft, int* __
 __global__ void tile_list_kernel(const int* __restrict__ flags, int ntiles, int* __restrict__ list,
                                  int* __restrict__ count)
 {
+    pdl_wait();
+    pdl_launch();
     __shared__ int warp_sums[32];
     __shared__ int base;
     if (threadIdx.x == 0) base = 0;
@@ -822,6 +824,8 @@ __device__ __forceinline__ uint16_t bf16_bits(float v)
 __global__ void tile_input_kernel(const __grid_constant__ FrameTable ft, const int* __restrict__ list,
                                   const int* __restrict__ count, uint16_t* __restrict__ x)
 {
+    pdl_wait();
+    pdl_launch();
     const int ti = blockIdx.y;
     if (ti >= *count) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;  // pixel of the tile
@@ -859,6 +863,8 @@ __global__ void tile_input_kernel(const __grid_constant__ FrameTable ft, const i
 __global__ void output_kernel(const uint16_t* __restrict__ a, const float* __restrict__ wo, int T,
                               float* __restrict__ rgb)
 {
+    pdl_wait();
+    pdl_launch();
     const int ti = blockIdx.y;
     if (ti >= T) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -903,8 +909,7 @@ void host_bf16(const float* src, size_t n, uint16_t* dst) { host_bf16_impl(src, 
 
 cudaError_t unet_output_rgb(const UnetNet* n, int T, float* rgb, cudaStream_t s)
 {
-    output_kernel<<<dim3(16, (unsigned)T), 256, 0, s>>>(n->d0b, n->wout, T, rgb);
-    return cudaGetLastError();
+    return launch_kernel(output_kernel, dim3(16, (unsigned)T), 256, 0, s, true, n->d0b, n->wout, T, rgb);
 }
 
 size_t unet_param_count()
@@ -1190,9 +1195,11 @@ yoro_status inpaint_table(yoro_unet_ctx* u, const yoro::FrameTable& ft, cudaStre
     for (int f = 0; f < ft.n; ++f) maxcells = std::max(maxcells, ft.off[f + 1] - ft.off[f]);
     if (total == 0) return YORO_OK;
     yoro::tile_flags_kernel<<<dim3((unsigned)maxcells, (unsigned)ft.n), 256, 0, s>>>(ft, n->flags);
-    yoro::tile_list_kernel<<<1, 1024, 0, s>>>(n->flags, total, n->list, n->count);
-    yoro::tile_input_kernel<<<dim3(16, (unsigned)total), 256, 0, s>>>(ft, n->list, n->count, n->in0);
-    if (cudaGetLastError() != cudaSuccess) return YORO_ECUDA;
+    if (yoro::launch_kernel(yoro::tile_list_kernel, dim3(1), 1024, 0, s, true, n->flags, total, n->list, n->count) !=
+            cudaSuccess ||
+        yoro::launch_kernel(yoro::tile_input_kernel, dim3(16, (unsigned)total), 256, 0, s, true, ft, n->list, n->count,
+                            n->in0) != cudaSuccess)
+        return YORO_ECUDA;
     const yoro::NetOut out{nullptr, &ft};
     return yoro::unet_run(n, n->in0, total, n->count, out, s) == cudaSuccess ? YORO_OK : YORO_ECUDA;
 }

@@ -30,6 +30,7 @@
 #include <new>
 #include <vector>
 
+#include "tc.cuh"
 #include "unet_internal.h"
 #include "yoro.h"
 #include "yoro_unet.h"
@@ -55,6 +56,8 @@ __device__ __forceinline__ float warp_sum(float v)
 
 __global__ void count_holes_kernel(const uint8_t* __restrict__ hole, long long n, int* __restrict__ cnt)
 {
+    pdl_wait();
+    pdl_launch();
     int c = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         c += hole[i] != 0;
@@ -126,6 +129,8 @@ __global__ void __launch_bounds__(256) dz_kernel(const uint16_t* __restrict__ D,
                                                  int yoff, int side, int C, long long items, uint16_t* __restrict__ dZ,
                                                  float* __restrict__ gb)
 {
+    pdl_wait();
+    pdl_launch();
     __shared__ float s[256];
     const int cg = C >> 3;  // channel groups, a power of two
     const int c = (threadIdx.x & (cg - 1)) << 3;
@@ -197,6 +202,8 @@ __global__ void __launch_bounds__(256) out_bwd_kernel(const float* __restrict__ 
                                                       float* __restrict__ gw, float* __restrict__ gwb,
                                                       float* __restrict__ gb, float* __restrict__ loss)
 {
+    pdl_wait();
+    pdl_launch();
     __shared__ float s[128];
     const float inv_n = 1.0f / (3.0f * (float)max(*cnt, 1));
     const int c = (threadIdx.x & 3) << 3;
@@ -296,6 +303,8 @@ constexpr int kWeightThreads = 576;  // two of a tile's rows of 288
 
 __global__ void __launch_bounds__(kWeightThreads) weights_kernel(const __grid_constant__ WeightTable w, const AdamArgs a)
 {
+    pdl_wait();
+    pdl_launch();
     __shared__ uint16_t s[32][290];  // [co][ci 9 + tap]; 145 words per row: no bank conflict along co
     if ((int)blockIdx.x == w.block0[14]) {
         for (int l = 0; l < 14; ++l)
@@ -330,7 +339,7 @@ __global__ void __launch_bounds__(kWeightThreads) weights_kernel(const __grid_co
 
 // Blocks of a grid-stride pass: at most about four waves, so that the blocks' closing atomics
 // on the same few sums stay few.
-int blocks_for(long long n) { return (int)std::min<long long>((n + 255) / 256, 608); }
+unsigned blocks_for(long long n) { return (unsigned)std::min<long long>((n + 255) / 256, 608); }
 
 }  // namespace
 
@@ -379,8 +388,7 @@ cudaError_t update_weights(Trainer* t, bool update, cudaStream_t s)
         a.c1 = 1.0f - std::pow(t->b1, (float)t->step);
         a.c2 = 1.0f - std::pow(t->b2, (float)t->step);
     }
-    weights_kernel<<<t->table.block0[14] + 1, kWeightThreads, 0, s>>>(t->table, a);
-    return cudaGetLastError();
+    return launch_kernel(weights_kernel, dim3((unsigned)t->table.block0[14] + 1), kWeightThreads, 0, s, true, t->table, a);
 }
 
 }  // namespace
@@ -474,11 +482,12 @@ cudaError_t trainer_step(Trainer* t, const void* x, const uint8_t* gt, const uin
     if (e == cudaSuccess) e = unet_run(n, xin, B, nullptr, NetOut{nullptr, nullptr}, s);
     if (e == cudaSuccess) e = unet_output_rgb(n, B, t->rgb, s);
     if (e != cudaSuccess) return e;
-    count_holes_kernel<<<blocks_for(npx), 256, 0, s>>>(hole, npx, t->nhole);
-    out_bwd_kernel<<<blocks_for(4 * npx), 256, 0, s>>>(t->rgb, gt, hole, npx, t->nhole, n->d0b, n->wout, t->dZ,
-                                                      t->grads + t->wout_off, t->grads + t->bout_off,
-                                                      t->grads + t->boff[13], t->loss);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_kernel(count_holes_kernel, dim3(blocks_for(npx)), 256, 0, s, true, hole, npx, t->nhole);
+    if (e == cudaSuccess)
+        e = launch_kernel(out_bwd_kernel, dim3(blocks_for(4 * npx)), 256, 0, s, true, (const float*)t->rgb, gt, hole, npx,
+                          (const int*)t->nhole, (const uint16_t*)n->d0b, (const float*)n->wout, t->dZ,
+                          t->grads + t->wout_off, t->grads + t->bout_off, t->grads + t->boff[13], t->loss);
+    if (e != cudaSuccess) return e;
 
     // per layer: forward input X (channel stride), output Y (stride, offset)
     struct IO {
@@ -511,18 +520,13 @@ cudaError_t trainer_step(Trainer* t, const void* x, const uint8_t* gt, const uin
             const uint16_t* D = t->DX[dx_buffer(r.from)];
             const int dcs = n->conv[r.from].cin;
             const long long items = P * (L.cout / 8) / (r.kind == kPooled ? 4 : 1);
-            const int blocks = blocks_for(items);
+            const unsigned blocks = blocks_for(items);
             float* gb = t->grads + t->boff[i];
-            if (r.kind == kDirect)
-                dz_kernel<kDirect><<<blocks, 256, 0, s>>>(D, dcs, r.off, nullptr, io[i].y, io[i].ycs, io[i].ycoff, side,
-                                                          L.cout, items, t->dZ, gb);
-            else if (r.kind == kUp)
-                dz_kernel<kUp><<<blocks, 256, 0, s>>>(D, dcs, r.off, nullptr, io[i].y, io[i].ycs, io[i].ycoff, side,
-                                                      L.cout, items, t->dZ, gb);
-            else
-                dz_kernel<kPooled><<<blocks, 256, 0, s>>>(D, dcs, r.off, t->DX[dx_buffer(r.pooled)], io[i].y, io[i].ycs,
-                                                          io[i].ycoff, side, L.cout, items, t->dZ, gb);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            const uint16_t* pooled = r.kind == kPooled ? t->DX[dx_buffer(r.pooled)] : nullptr;
+            const auto kernel = r.kind == kDirect ? dz_kernel<kDirect> : r.kind == kUp ? dz_kernel<kUp> : dz_kernel<kPooled>;
+            e = launch_kernel(kernel, dim3(blocks), 256, 0, s, true, D, dcs, r.off, pooled, io[i].y, io[i].ycs, io[i].ycoff,
+                              side, L.cout, items, t->dZ, gb);
+            if (e != cudaSuccess) return e;
         }
         e = conv_dw_launch(t->dZ, io[i].x, io[i].xcs, B, side, L.cin, L.cout, t->sms, t->ws, t->grads + t->woff[i], s);
         if (e != cudaSuccess) return e;
@@ -531,9 +535,10 @@ cudaError_t trainer_step(Trainer* t, const void* x, const uint8_t* gt, const uin
         for (int c0 = 0; c0 < L.cin && e == cudaSuccess;) {
             const int rem = L.cin - c0;
             const int w = rem >= 256 ? 256 : rem >= 128 ? 128 : rem >= 64 ? 64 : 32;
-            e = unet_conv3x3(ConvCall{t->dZ, t->wt[i] + (size_t)c0 * 9 * L.cout, t->DX[dx_buffer(i)], t->zero_bias,
-                                      nullptr, nullptr, B, side, side, L.cout, w, L.cin, c0, 0, 0},
-                             s);
+            ConvCall c{t->dZ, t->wt[i] + (size_t)c0 * 9 * L.cout, t->DX[dx_buffer(i)], t->zero_bias, nullptr, nullptr, B,
+                       side, side, L.cout, w, L.cin, c0, 0, 0};
+            c.pdl = true;
+            e = unet_conv3x3(c, s);
             c0 += w;
         }
         if (e != cudaSuccess) return e;
