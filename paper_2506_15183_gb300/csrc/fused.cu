@@ -845,6 +845,7 @@ __device__ __forceinline__ Window window_layout(unsigned char* smem, int slots, 
 template <int NT, int MINB, bool VAR, bool ZT = false, bool WIDE = false, bool RANGE = false>
 __global__ void __launch_bounds__(NT, MINB) fused_single(FrameArgs f, int wpad, int row0, int row1)
 {
+    after_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     int *ctr, *rowinfo;
     const Window s = window_layout(smem_raw, f.band + 2 * KernelShape<VAR>(f).halo, wpad, f.w, ctr, rowinfo);
@@ -859,6 +860,7 @@ __global__ void __launch_bounds__(NT, MINB) fused_single(FrameArgs f, int wpad, 
 template <int NT, int MINB, bool ZT = false, bool WIDE = false>
 __global__ void __launch_bounds__(NT, MINB) fused_batch(const __grid_constant__ BatchArgs a, int wpad)
 {
+    after_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     for (int item = blockIdx.x; item < a.total_items; item += gridDim.x) {
         int lo = 0, hi = a.n - 1;  // frame whose item range holds `item`
@@ -887,6 +889,7 @@ __global__ void __launch_bounds__(NT, MINB) fused_batch(const __grid_constant__ 
 template <int NT, bool VAR>
 __global__ void __launch_bounds__(NT, 1) fill_only(FrameArgs f, const float* __restrict__ zt, int wpad)
 {
+    after_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int NW = NT / 32;
     int *ctr, *rowinfo;
@@ -946,6 +949,7 @@ __global__ void __launch_bounds__(NT, 1) fill_only(FrameArgs f, const float* __r
 template <int NT, bool VAR>
 __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned long long* __restrict__ keys, int wpad)
 {
+    after_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int NW = NT / 32, RB = 5;  // bands of 13 rows: windows of three full batches
     int *ctr, *rowinfo;
@@ -1026,6 +1030,7 @@ __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned l
 template <int NT, bool VAR>
 __global__ void __launch_bounds__(NT, 1) imb_band(FrameArgs f, int div, int interp, int wpad, int cells_off)
 {
+    after_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int NW = NT / 32, RB = 3;  // bands of 7 rows: windows of three full batches
     int *ctr, *rowinfo;
@@ -1351,7 +1356,10 @@ cudaError_t fused_launch(const FrameArgs& f, const FusedLimits& lim, int two_per
     const int grid = nbands < slots ? nbands : slots;
     if (f.zt_out && var) return cudaErrorInvalidValue;  // the depth output exists for the default kernel
     const bool wide = (f.w + 31) / 32 > 2 * (kBig / 32);  // wider than 2 words per warp
-    auto go = [&](auto kernel, int threads) { kernel<<<grid, threads, smem, stream>>>(f, wpad, row0, row1); };
+    cudaError_t launched = cudaSuccess;
+    auto go = [&](auto kernel, int threads) {
+        launched = launch_after(kernel, (unsigned)grid, threads, smem, stream, f, wpad, row0, row1);
+    };
     if (row0 != 0 || row1 != f.h) {
         if (f.zt_out) return cudaErrorInvalidValue;
         if (two_per_sm) {
@@ -1372,7 +1380,7 @@ cudaError_t fused_launch(const FrameArgs& f, const FusedLimits& lim, int two_per
         else if (wide) go(fused_single<kBig, 1, false, false, true>, kBig);
         else go(fused_single<kBig, 1, false>, kBig);
     }
-    return cudaGetLastError();
+    return launched;
 }
 
 cudaError_t fused_launch_batch(const BatchArgs& a, int wmax, const FusedLimits& lim, cudaStream_t stream, bool zt)
@@ -1385,16 +1393,13 @@ cudaError_t fused_launch_batch(const BatchArgs& a, int wmax, const FusedLimits& 
     // rest of the batch.
     const int grid = a.total_items;
     if (grid < 1) return cudaSuccess;
-    if (two) {
-        if (zt) fused_batch<kSmall, 2, true><<<grid, kSmall, smem, stream>>>(a, wpad);
-        else fused_batch<kSmall, 2><<<grid, kSmall, smem, stream>>>(a, wpad);
-    } else {
-        if (zt) fused_batch<kBig, 1, true><<<grid, kBig, smem, stream>>>(a, wpad);
-        else if ((wmax + 31) / 32 > 2 * (kBig / 32))  // a frame wider than 2 words per warp
-            fused_batch<kBig, 1, false, true><<<grid, kBig, smem, stream>>>(a, wpad);
-        else fused_batch<kBig, 1><<<grid, kBig, smem, stream>>>(a, wpad);
-    }
-    return cudaGetLastError();
+    const bool wide = (wmax + 31) / 32 > 2 * (kBig / 32);  // a frame wider than 2 words per warp
+    auto go = [&](auto kernel, int threads) {
+        return launch_after(kernel, (unsigned)grid, threads, smem, stream, a, wpad);
+    };
+    if (two) return zt ? go(fused_batch<kSmall, 2, true>, kSmall) : go(fused_batch<kSmall, 2>, kSmall);
+    if (zt) return go(fused_batch<kBig, 1, true>, kBig);
+    return wide ? go(fused_batch<kBig, 1, false, true>, kBig) : go(fused_batch<kBig, 1>, kBig);
 }
 
 int fused_max_band(const FusedLimits& lim, int w, int halo) { return max_band(lim, fused_wpad(w), halo); }
@@ -1424,11 +1429,8 @@ cudaError_t imb_band_launch(FrameArgs f, int div, int interp, const FusedLimits&
     const int nbands = (f.h + f.band - 1) / f.band;
     if (nbands < 1) return cudaSuccess;
     const int wpad = fused_wpad(f.w), cells = (int)imb_cells_offset(f.w, f.band, f.halo);
-    if (f.halo == 1 && !f.nearest)
-        imb_band<kBig, false><<<nbands, kBig, smem, stream>>>(f, div, interp, wpad, cells);
-    else
-        imb_band<kBig, true><<<nbands, kBig, smem, stream>>>(f, div, interp, wpad, cells);
-    return cudaGetLastError();
+    const auto kernel = f.halo == 1 && !f.nearest ? imb_band<kBig, false> : imb_band<kBig, true>;
+    return launch_after(kernel, (unsigned)nbands, kBig, smem, stream, f, div, interp, wpad, cells);
 }
 
 cudaError_t fill_only_launch(FrameArgs f, const float* zt, const FusedLimits& lim, cudaStream_t stream)
@@ -1438,9 +1440,8 @@ cudaError_t fill_only_launch(FrameArgs f, const float* zt, const FusedLimits& li
     const size_t smem = fused_smem_bytes(wpad, f.band, f.halo);
     const int grid = (f.h + f.band - 1) / f.band;
     if (grid < 1) return cudaSuccess;
-    if (f.halo == 1 && !f.nearest) fill_only<kBig, false><<<grid, kBig, smem, stream>>>(f, zt, wpad);
-    else fill_only<kBig, true><<<grid, kBig, smem, stream>>>(f, zt, wpad);
-    return cudaGetLastError();
+    const auto kernel = f.halo == 1 && !f.nearest ? fill_only<kBig, false> : fill_only<kBig, true>;
+    return launch_after(kernel, (unsigned)grid, kBig, smem, stream, f, zt, wpad);
 }
 
 cudaError_t fill_keys_launch(FrameArgs f, const unsigned long long* keys, const FusedLimits& lim, cudaStream_t stream)
@@ -1450,9 +1451,8 @@ cudaError_t fill_keys_launch(FrameArgs f, const unsigned long long* keys, const 
     const size_t smem = fused_smem_bytes(wpad, f.band, f.halo);
     const int grid = (f.h + f.band - 1) / f.band;
     if (grid < 1) return cudaSuccess;
-    if (f.halo == 1 && !f.nearest) fill_keys<kBig, false><<<grid, kBig, smem, stream>>>(f, keys, wpad);
-    else fill_keys<kBig, true><<<grid, kBig, smem, stream>>>(f, keys, wpad);
-    return cudaGetLastError();
+    const auto kernel = f.halo == 1 && !f.nearest ? fill_keys<kBig, false> : fill_keys<kBig, true>;
+    return launch_after(kernel, (unsigned)grid, kBig, smem, stream, f, keys, wpad);
 }
 
 }  // namespace yoro

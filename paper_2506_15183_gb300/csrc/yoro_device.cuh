@@ -10,6 +10,30 @@
 
 namespace yoro {
 
+// Programmatic dependent launch: a kernel launched with launch_after() may be set up while the
+// kernel before it in the stream ends; it starts with after_wait(), which returns once that
+// kernel has completed and its writes are visible.  The frame kernels do not release their
+// successors early: a waiting CTA would hold an SM that other streams' frames could use.
+__device__ __forceinline__ void after_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), unsigned grid, int threads, size_t smem, cudaStream_t stream,
+                         const A&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
 constexpr unsigned long long kEmptyKey = ~0ull;
 
 // rcp.approx.ftz: one MUFU op, within 1 ulp of 1/x for normal x (a denormal
