@@ -70,6 +70,7 @@ struct Window {
     uint32_t* rgba;
     uint32_t* bits;
     uint32_t* pre;  // band row vj's hole prefix sums per word at pre + vj*nwords
+    uint32_t* zmax; // fills with ZMAX: per word of window row j, its largest reached depth (bits; 0: none)
     int wpad, nwords, ra, slots;
     __device__ __forceinline__ const uint32_t* zrow(int v) const { return zt + (v - ra) * wpad; }
     __device__ __forceinline__ const uint32_t* crow(int v) const { return rgba + (v - ra) * wpad; }
@@ -125,21 +126,15 @@ __device__ __forceinline__ void find_edges(int x, int v, const Window& s, int w,
 }
 
 // Hole fill of pixel (v, x) with edges L, R (R < w).  Rows outside [0, h) are skipped.
-// SKIPS: `open` is set, and the result void, once kMaxSkips foreground candidates have been
-// passed over: such a kernel is crossed by the whole warp instead (fill_hole_warp, 32 columns a
-// step).  Almost every pixel settles after about ten candidates, but where the second eye
-// is rotated or shifted out of its row, holes up to 900 columns wide lie next to wide
-// occluders, their kernels hold more than a thousand foreground candidates, and one lane
-// walking them alone kept its band's CTA busy for 100 us (1832x1920, general pose: 148 -> 92
-// us and 113 -> 55 us on the frames with such holes).  The stereo pair's holes are
-// narrow (walks of 24 candidates at the 99th percentile), and there the counter cost 1 to 2 %.
-constexpr int kMaxSkips = 96;
-
-template <bool VAR, bool SKIPS>
+// ZMAX: words whose reached pixels are all foreground are passed over by their largest depth.
+// The stereo pair's holes are narrow (24 candidates walked at the 99th percentile), but where
+// the second eye is rotated or shifted out of its row, holes up to 900 columns wide lie
+// beside wide occluders and their kernels hold more than a thousand foreground candidates;
+// walked one by one they kept single bands' CTAs busy for 100 us (figures at fill_keys).
+template <bool VAR, bool ZMAX>
 __device__ __forceinline__ uint32_t fill_from_edges(int x, int v, int L, int R, int h, int w, const Window& s,
-                                                    const KernelShape<VAR>& ks, bool& open)
+                                                    const KernelShape<VAR>& ks)
 {
-    int skips = kMaxSkips;
     const int wd = R - L;
     const float d_occ = (L >= 0) ? __uint_as_float(s.zrow(v)[L]) : 0.0f;
     FillAcc f;
@@ -157,6 +152,7 @@ __device__ __forceinline__ uint32_t fill_from_edges(int x, int v, int L, int R, 
 #pragma unroll 1
         for (int step = 0; step <= whi - wlo; ++step) {
             const int wi = ks.nearest ? wlo + step : whi - step;
+            if (ZMAX && __uint_as_float(s.zmax[(vv - s.ra) * s.nwords + wi]) < d_occ) continue;
             uint32_t m = b[wi];
             if (wi == whi) m &= mhi;
             if (wi == wlo) m &= mlo;
@@ -164,13 +160,7 @@ __device__ __forceinline__ uint32_t fill_from_edges(int x, int v, int L, int R, 
                 const int bit = ks.nearest ? __ffs(m) - 1 : 31 - __clz(m);
                 m &= ~(1u << bit);
                 const int c = (wi << 5) + bit;
-                if (__uint_as_float(zr[c]) < d_occ) {  // foreground (O2)
-                    if (SKIPS && --skips < 0) {
-                        open = true;
-                        return 0u;
-                    }
-                    continue;
-                }
+                if (__uint_as_float(zr[c]) < d_occ) continue;  // foreground (O2)
                 if (!f.add(cr[c])) return f.result();          // weight reached exactly 0
                 uint32_t out;
                 if (f.wrem <= kSettleFrom && f.settled(out)) return out;
@@ -187,7 +177,7 @@ __device__ __forceinline__ uint32_t fill_from_edges(int x, int v, int L, int R, 
 // lanes; each lane accumulates it with its own t and stops at its own exact exit.  A
 // kernel full of foreground candidates is thus crossed 32 columns per step instead of
 // one candidate per step.
-template <bool VAR>
+template <bool VAR, bool ZMAX>
 __device__ __forceinline__ uint32_t fill_hole_warp(int x, bool act, int v, int L, int R, int h, int w,
                                                    const Window& s, const KernelShape<VAR>& ks)
 {
@@ -200,37 +190,64 @@ __device__ __forceinline__ uint32_t fill_hole_warp(int x, bool act, int v, int L
     uint32_t res = 0u;
     const int jhi = min(R + wd, w - 1);
     const int jlast = min(v + ks.halo, h - 1) - s.ra;
-    for (int j = max(v - ks.halo, 0) - s.ra; j <= jlast; ++j) {
-        for (int g0 = 0; g0 <= jhi - R; g0 += 32) {
-            // lane 0 takes the group's first column in kernel order
-            const int c = ks.nearest ? R + g0 + lane : jhi - g0 - lane;
-            bool contrib = false;
-            uint32_t col = 0u;
-            if ((ks.nearest ? c <= jhi : c >= R) &&
-                YORO_BOUND(j >= 0 && j < s.slots && c >= 0 && c < s.wpad, kBadHoles)) {
-                const int i = j * s.wpad + c;
-                const bool reached = (s.bits[j * s.nwords + (c >> 5)] >> (c & 31)) & 1u;
-                contrib = reached && !(__uint_as_float(s.zt[i]) < d_occ);  // not foreground (O2)
-                if (contrib) col = s.rgba[i];
-            }
-            uint32_t cm = __ballot_sync(0xffffffffu, contrib);
-            while (cm) {  // contributors in kernel order
-                const int k = __ffs(cm) - 1;
-                cm &= cm - 1u;
-                const uint32_t cc = __shfl_sync(0xffffffffu, col, k);
-                if (!done) {
-                    if (!f.add(cc)) {  // weight reached exactly 0
-                        res = f.result();
+    // contributor of this lane's column c of window row j, if it is one
+    auto gate = [&](int j, int c, bool in, uint32_t& col) {
+        bool contrib = false;
+        col = 0u;
+        if (in && YORO_BOUND(j >= 0 && j < s.slots && c >= 0 && c < s.wpad, kBadHoles)) {
+            const int i = j * s.wpad + c;
+            const bool reached = (s.bits[j * s.nwords + (c >> 5)] >> (c & 31)) & 1u;
+            contrib = reached && !(__uint_as_float(s.zt[i]) < d_occ);  // not foreground (O2)
+            if (contrib) col = s.rgba[i];
+        }
+        return __ballot_sync(0xffffffffu, contrib);
+    };
+    // accumulates a group's contributors in kernel order; true once every lane is done
+    auto take = [&](uint32_t cm, uint32_t col) {
+        while (cm) {
+            const int k = __ffs(cm) - 1;
+            cm &= cm - 1u;
+            const uint32_t cc = __shfl_sync(0xffffffffu, col, k);
+            if (!done) {
+                if (!f.add(cc)) {  // weight reached exactly 0
+                    res = f.result();
+                    done = true;
+                } else {
+                    uint32_t out;
+                    if (f.wrem <= kSettleFrom && f.settled(out)) {
+                        res = out;
                         done = true;
-                    } else {
-                        uint32_t out;
-                        if (f.wrem <= kSettleFrom && f.settled(out)) {
-                            res = out;
-                            done = true;
-                        }
                     }
                 }
-                if (__all_sync(0xffffffffu, done)) return res;
+            }
+            if (__all_sync(0xffffffffu, done)) return true;
+        }
+        return false;
+    };
+    for (int j = max(v - ks.halo, 0) - s.ra; j <= jlast; ++j) {
+        if (!ZMAX) {
+            for (int g0 = 0; g0 <= jhi - R; g0 += 32) {
+                // lane 0 takes the group's first column in kernel order
+                const int c = ks.nearest ? R + g0 + lane : jhi - g0 - lane;
+                uint32_t col;
+                const uint32_t cm = gate(j, c, ks.nearest ? c <= jhi : c >= R, col);
+                if (take(cm, col)) return res;
+            }
+        } else {
+            // 32 words per step by their largest depth, then the columns of those that are not
+            // all foreground
+            const int wlo = R >> 5, whi = jhi >> 5;
+            for (int g0 = 0; g0 <= whi - wlo; g0 += 32) {
+                const int wi = ks.nearest ? wlo + g0 + lane : whi - g0 - lane;
+                const bool some = wi >= wlo && wi <= whi && YORO_BOUND(j >= 0 && j < s.slots, kBadHoles) &&
+                                  !(__uint_as_float(s.zmax[j * s.nwords + wi]) < d_occ);
+                for (uint32_t wm = __ballot_sync(0xffffffffu, some); wm; wm &= wm - 1u) {
+                    const int k = __ffs(wm) - 1, word = ks.nearest ? wlo + g0 + k : whi - g0 - k;
+                    const int c = (word << 5) + (ks.nearest ? lane : 31 - lane);
+                    uint32_t col;
+                    const uint32_t cm = gate(j, c, c >= R && c <= jhi, col);
+                    if (take(cm, col)) return res;
+                }
             }
         }
     }
@@ -573,7 +590,7 @@ __device__ __forceinline__ void resolve_window(const FrameArgs& f, const float* 
 // One band [y0, y1) of one frame; shared memory holds the window rows ra..rb
 // (ra = y0-1 or 0, rb = y1 or h-1).  Ends with a barrier, so the next band may reuse
 // shared memory.
-template <int NT, bool VAR, bool SKIPS = false>
+template <int NT, bool VAR, bool ZMAX = false>
 __device__ __forceinline__ void fill_band(const FrameArgs& f, int y0, int y1, const Window& s, int* ctr,
                                           int* rowinfo);
 
@@ -620,7 +637,7 @@ __device__ __forceinline__ void run_band(const FrameArgs& f, int y0, int y1, Win
 // P3 of one band [y0, y1) whose window (s.ra set) holds the reached pixels' depths and
 // colors and every window row's reached bitmask.  Writes the band rows' holes to
 // f.out (reached pixels and masks are not touched).  Ends with a barrier.
-template <int NT, bool VAR, bool SKIPS>
+template <int NT, bool VAR, bool ZMAX>
 __device__ __forceinline__ void fill_band(const FrameArgs& f, int y0, int y1, const Window& s, int* ctr,
                                           int* rowinfo)
 {
@@ -760,22 +777,10 @@ __device__ __forceinline__ void fill_band(const FrameArgs& f, int y0, int y1, co
                 // one hole for the whole chunk: its kernel is scanned once by the warp
                 const int v0 = __shfl_sync(0xffffffffu, v, 0), L0 = __shfl_sync(0xffffffffu, L, 0),
                           R0 = __shfl_sync(0xffffffffu, R, 0);
-                bool open = false;
                 if (__all_sync(0xffffffffu, !act || (v == v0 && L == L0 && R == R0)))
-                    o = fill_hole_warp<VAR>(x, act, v0, L0, R0, h, w, s, ks);
+                    o = fill_hole_warp<VAR, ZMAX>(x, act, v0, L0, R0, h, w, s, ks);
                 else if (act)
-                    o = fill_from_edges<VAR, SKIPS>(x, v, L, R, h, w, s, ks, open);
-                if (SKIPS) {  // kernels too full of foreground for one lane: each such hole by the warp
-                    for (uint32_t left = __ballot_sync(0xffffffffu, open); left;) {
-                        const int lead = __ffs(left) - 1;
-                        const int vl = __shfl_sync(0xffffffffu, v, lead), Ll = __shfl_sync(0xffffffffu, L, lead),
-                                  Rl = __shfl_sync(0xffffffffu, R, lead);
-                        const bool in = open && v == vl && L == Ll && R == Rl;
-                        const uint32_t r = fill_hole_warp<VAR>(x, in, vl, Ll, Rl, h, w, s, ks);
-                        if (in) o = r;
-                        left &= ~__ballot_sync(0xffffffffu, in);
-                    }
-                }
+                    o = fill_from_edges<VAR, ZMAX>(x, v, L, R, h, w, s, ks);
                 if (act && YORO_BOUND(v >= y0 && v < y1, kBadHoles)) f.out[(size_t)v * w + x] = o;
             } else {  // 64 cracks, two consecutive ones per lane
                 const int idx = ((chunk - ng) << 6) + 2 * lane;
@@ -835,6 +840,7 @@ __device__ __forceinline__ Window window_layout(unsigned char* smem, int slots, 
     s.ra = 0;
     s.slots = slots;
     s.pre = s.bits + slots * ((wpad + 31) / 32);
+    s.zmax = nullptr;
     ctr = reinterpret_cast<int*>(s.pre + slots * ((wpad + 31) / 32));
     rowinfo = ctr + 4;
     return s;
@@ -945,7 +951,10 @@ __global__ void __launch_bounds__(NT, 1) fill_only(FrameArgs f, const float* __r
 // pixels and their hole mask leave for global memory, and the holes are filled as in
 // fill_only.  It stands in for a gather pass that writes the image out and fill_only's
 // reading it back.  The loading takes about 19 us of the pass at 1832x1920; the rest is the
-// holes' fill, bound by the bands that hold the most of it.
+// holes' fill, bound by the bands that hold the most of it.  With each word's largest reached
+// depth at hand (one warp reduction and 4 bytes per word) the fill passes over words that
+// // are all foreground: eight seeds of 1832x1920 took 103, 52, 66, 56, 72, 95, 52 and 60 us with one
+// lane or one warp crossing them column by column, 64, 53, 61, 54, 68, 61, 50 and 48 so.
 template <int NT, bool VAR>
 __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned long long* __restrict__ keys, int wpad)
 {
@@ -955,6 +964,7 @@ __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned l
     int *ctr, *rowinfo;
     const KernelShape<VAR> ks(f);
     Window s = window_layout(smem_raw, f.band + 2 * ks.halo, wpad, f.w, ctr, rowinfo);
+    s.zmax = reinterpret_cast<uint32_t*>(rowinfo + 2 * s.slots);  // after the window (keys_smem_bytes)
     const int w = f.w, h = f.h, nwords = s.nwords;
     const size_t n = (size_t)w * (size_t)h;  // source indices are below n (checked in the debug-bounds build)
     (void)n;
@@ -993,7 +1003,11 @@ __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned l
                     if (FULL || u < nb) {  // uniform
                         const bool reached = kv[u] != kEmptyKey;
                         const uint32_t m = __ballot_sync(0xffffffffu, reached);
-                        if (lane == 0 && YORO_BOUND(j0 + u < s.slots, kBadHoles)) s.bits[(j0 + u) * nwords + g] = m;
+                        const uint32_t zm = __reduce_max_sync(0xffffffffu, reached ? (uint32_t)(kv[u] >> 32) : 0u);
+                        if (lane == 0 && YORO_BOUND(j0 + u < s.slots, kBadHoles)) {
+                            s.bits[(j0 + u) * nwords + g] = m;
+                            s.zmax[(j0 + u) * nwords + g] = zm;
+                        }
                         if (reached && YORO_BOUND(so < s.slots * wpad, kBadHoles)) {
                             s.zt[so] = (uint32_t)(kv[u] >> 32);
                             s.rgba[so] = cv[u];
@@ -1444,11 +1458,24 @@ cudaError_t fill_only_launch(FrameArgs f, const float* zt, const FusedLimits& li
     return launch_after(kernel, (unsigned)grid, kBig, smem, stream, f, zt, wpad);
 }
 
+// fill_keys: the window and its words' largest depths.
+static size_t keys_smem_bytes(int wpad, int band, int halo)
+{
+    return fused_smem_bytes(wpad, band, halo) + (size_t)(band + 2 * halo) * (size_t)((wpad + 31) / 32) * 4;
+}
+
+bool fill_keys_fits(const FusedLimits& lim, int w, int halo)
+{
+    return keys_smem_bytes(fused_wpad(w), 1, halo) <= (size_t)lim.smem_per_block;
+}
+
 cudaError_t fill_keys_launch(FrameArgs f, const unsigned long long* keys, const FusedLimits& lim, cudaStream_t stream)
 {
     const int wpad = fused_wpad(f.w);
-    f.band = balanced_band(f.h, f.halo, max(1, max_band(lim, wpad, f.halo)), lim.sms);
-    const size_t smem = fused_smem_bytes(wpad, f.band, f.halo);
+    int bmax = 1;
+    while (bmax < 4096 && keys_smem_bytes(wpad, bmax + 1, f.halo) <= (size_t)lim.smem_per_block) ++bmax;
+    f.band = balanced_band(f.h, f.halo, bmax, lim.sms);
+    const size_t smem = keys_smem_bytes(wpad, f.band, f.halo);
     const int grid = (f.h + f.band - 1) / f.band;
     if (grid < 1) return cudaSuccess;
     const auto kernel = f.halo == 1 && !f.nearest ? fill_keys<kBig, false> : fill_keys<kBig, true>;

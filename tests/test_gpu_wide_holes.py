@@ -1,6 +1,6 @@
 """General poses and the intermediate buffer where their band kernels change course, byte for
 byte against the oracle (needs a GPU): holes hundreds of columns wide beside wide occluders
-(kernels that one lane hands over to its warp), the scatter's two ways to divide, and frames
+(kernels whose words are passed over by their largest depth), the scatter's two ways to divide, and frames
 whose bands take several waves (band heights below the tallest)."""
 import math
 
