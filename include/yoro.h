@@ -195,10 +195,8 @@ yoro_status yoro_synthesize_unfused(yoro_handle h, const void* color_rgba8, cons
 /*
  * yoro_synthesize() for HOST buffers: copies color and depth to device staging
  * owned by the handle (allocated on first use), runs the fused kernel, and copies
- * the right eye and mask back, in the order of cuda_stream.  Page-locked (pinned) host
- * buffers give asynchronous copies (of large frames in parts, on two streams of the
- * handle that are forked from and joined to cuda_stream, so that copies in, kernels and
- * copies out overlap); the call returns before the copies finish,
+ * the right eye and mask back, all on cuda_stream.  Page-locked (pinned) host
+ * buffers give asynchronous copies; the call returns before the copies finish,
  * so the caller synchronises the stream before reading the outputs.  Calls that
  * share a handle must not overlap on the GPU (they share the staging).
  */

@@ -18,14 +18,6 @@
 using yoro::FrameArgs;
 using yoro::FusedLimits;
 
-// Copy streams and events of a handle's host-buffer calls (run_host_pipelined).
-constexpr int kHostParts = 8;
-
-struct HostPipe {
-    cudaStream_t in, out;
-    cudaEvent_t start, done, have[kHostParts], made[kHostParts];
-};
-
 struct yoro_ctx {
     int w, h;
     float fx, fy, cx, cy, ipd, near_, far_;
@@ -40,7 +32,6 @@ struct yoro_ctx {
     yoro::FusedShape shape;
     unsigned long long* d_zbuf;    // unfused path, h*w keys, allocated on first use
     unsigned char* d_stage;        // host-buffer path, 13*h*w bytes (+ padding), on first use
-    HostPipe* pipe;                // host-buffer path, copy streams and events, on first use
     void* d_imb;                   // intermediate-buffer path: cell keys and depths, on first use
     void* d_pose;                  // general-pose path: keys and depths, on first use
 };
@@ -173,97 +164,6 @@ yoro_status run_frame(yoro_ctx* c, FrameArgs f, cudaStream_t s)
     return yoro::fused_launch(f, c->lim, c->shape.two_per_sm, s) == cudaSuccess ? YORO_OK : YORO_ECUDA;
 }
 
-void free_pipe(HostPipe* p)
-{
-    if (!p) return;
-    if (p->in) cudaStreamDestroy(p->in);
-    if (p->out) cudaStreamDestroy(p->out);
-    if (p->start) cudaEventDestroy(p->start);
-    if (p->done) cudaEventDestroy(p->done);
-    for (int i = 0; i < kHostParts; ++i) {
-        if (p->have[i]) cudaEventDestroy(p->have[i]);
-        if (p->made[i]) cudaEventDestroy(p->made[i]);
-    }
-    delete p;
-}
-
-// The handle's copy streams and events, made on first use; null if they cannot be made.
-HostPipe* host_pipe(yoro_ctx* c)
-{
-    if (c->pipe) return c->pipe;
-    HostPipe* p = new (std::nothrow) HostPipe();
-    if (!p) return nullptr;
-    auto event = [](cudaEvent_t* e) { return cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess; };
-    bool ok = cudaStreamCreateWithFlags(&p->in, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&p->out, cudaStreamNonBlocking) == cudaSuccess && event(&p->start) &&
-              event(&p->done);
-    for (int i = 0; ok && i < kHostParts; ++i) ok = event(&p->have[i]) && event(&p->made[i]);
-    if (!ok) {
-        cudaGetLastError();
-        free_pipe(p);
-        return nullptr;
-    }
-    c->pipe = p;
-    return p;
-}
-
-bool page_locked(const void* p)
-{
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeHost;
-}
-
-// Rows per part of a host frame: two or more parts of about 9 MB of input, the last one half as
-// tall as the others (its kernel and its copy out overlap nothing); 0 where one part is all.
-// Every part costs about 8 us of copy and event set-up: parts of 3, 4 and 6 MB were slower.
-int host_part_rows(int w, int h)
-{
-    const int parts = std::min((int)(8.0 * w * h / 9.0e6), kHostParts);
-    return parts < 2 ? 0 : (2 * h + 2 * parts - 2) / (2 * parts - 1);
-}
-
-// A frame in page-locked host memory, in parts of `rows` output rows: while a part's rows are
-// synthesized, the next part's are copied in and the last part's are copied out, each
-// direction on a stream of the handle's, forked from and joined to the caller's stream (so
-// the call as a whole keeps that stream's order, also under capture).  A part's input ends
-// `halo` rows below its output, the rows its kernel windows reach.  One after the other the
-// copies in, the kernel and the copies out of a 1832x1920 frame took 278 us; the two copy
-// directions alone, overlapped, take 144.
-yoro_status run_host_pipelined(yoro_ctx* c, HostPipe* p, FrameArgs f, int rows, const unsigned char* hcolor,
-                               const float* hdepth, unsigned char* hout, unsigned char* hmask, cudaStream_t s)
-{
-    const int w = c->w, h = c->h;
-    auto copy = [&](void* dst, const void* src, int r0, int r1, int bytes, cudaMemcpyKind kind, cudaStream_t st) {
-        const size_t o = (size_t)r0 * w * bytes;
-        return cudaMemcpyAsync((char*)dst + o, (const char*)src + o, (size_t)(r1 - r0) * w * bytes, kind, st) ==
-               cudaSuccess;
-    };
-    auto after = [](cudaEvent_t e, cudaStream_t from, cudaStream_t to) {
-        return cudaEventRecord(e, from) == cudaSuccess && cudaStreamWaitEvent(to, e, 0) == cudaSuccess;
-    };
-    bool ok = after(p->start, s, p->in) && cudaStreamWaitEvent(p->out, p->start, 0) == cudaSuccess;
-    int have = 0;
-    for (int k = 0, y0 = 0; ok && y0 < h; ++k, y0 += rows) {
-        const int y1 = std::min(y0 + rows, h), need = std::min(y1 + f.halo, h);
-        ok = copy((void*)f.color, hcolor, have, need, 4, cudaMemcpyHostToDevice, p->in) &&
-             copy((void*)f.depth, hdepth, have, need, 4, cudaMemcpyHostToDevice, p->in) && after(p->have[k], p->in, s);
-        have = need;
-        if (!ok) break;
-        const yoro::FusedShape shape = yoro::fused_shape(c->lim, w, y1 - y0, c->halo);
-        f.band = shape.band;
-        ok = yoro::fused_launch(f, c->lim, shape.two_per_sm, s, y0, y1) == cudaSuccess && after(p->made[k], s, p->out) &&
-             copy(hout, f.out, y0, y1, 4, cudaMemcpyDeviceToHost, p->out) &&
-             copy(hmask, f.mask, y0, y1, 1, cudaMemcpyDeviceToHost, p->out);
-    }
-    // the caller's stream waits for what was enqueued, also after a failure
-    const bool joined = after(p->done, p->in, s) && after(p->done, p->out, s);
-    return ok && joined ? YORO_OK : YORO_ECUDA;
-}
-
 }  // namespace
 
 namespace yoro {
@@ -387,7 +287,6 @@ void yoro_destroy(yoro_handle c)
     if (!c) return;
     if (c->d_zbuf) cudaFree(c->d_zbuf);
     if (c->d_stage) cudaFree(c->d_stage);
-    free_pipe(c->pipe);
     if (c->d_imb) cudaFree(c->d_imb);
     if (c->d_pose) cudaFree(c->d_pose);
     delete c;
@@ -499,22 +398,12 @@ yoro_status yoro_synthesize_host(yoro_handle c, const void* hcolor, const float*
     unsigned char* dout = c->d_stage + 2 * seg;
     unsigned char* dmask = c->d_stage + 3 * seg;
     cudaStream_t s = (cudaStream_t)stream;
-    FrameArgs f;
-    st = make_frame(c->w, c->h, c->k, c->near_, c->far_, dc, dd, dout, dmask, &f);
-    if (st != YORO_OK) return st;
-    // Parts of page-locked frames overlap their copies and kernels where the handle's kernel
-    // works on bands of rows; pageable memory is copied by the calling thread, one copy at
-    // a time, and the general pose and over-wide frames need the whole input.
-    const int rows = c->fused_ok && !c->pose && !uses_imb(c) ? host_part_rows(c->w, c->h) : 0;
-    if (rows > 0 && page_locked(hcolor) && page_locked(hdepth) && page_locked(hout) && page_locked(hmask)) {
-        if (HostPipe* pipe = host_pipe(c)) {
-            apply_options(c, &f);
-            return run_host_pipelined(c, pipe, f, rows, (const unsigned char*)hcolor, hdepth, (unsigned char*)hout, hmask, s);
-        }
-    }
     if (cudaMemcpyAsync(dc, hcolor, 4 * n, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemcpyAsync(dd, hdepth, 4 * n, cudaMemcpyHostToDevice, s) != cudaSuccess)
         return YORO_ECUDA;
+    FrameArgs f;
+    st = make_frame(c->w, c->h, c->k, c->near_, c->far_, dc, dd, dout, dmask, &f);
+    if (st != YORO_OK) return st;
     apply_options(c, &f);
     st = run_frame(c, f, s);
     if (st != YORO_OK) return st;

@@ -846,20 +846,17 @@ __device__ __forceinline__ Window window_layout(unsigned char* smem, int slots, 
     return s;
 }
 
-// RANGE: output rows [row0, row1) only (a part of a host frame); an instance of its own, since
-// the two arguments cost whole frames 0.4 %.
-template <int NT, int MINB, bool VAR, bool ZT = false, bool WIDE = false, bool RANGE = false>
-__global__ void __launch_bounds__(NT, MINB) fused_single(FrameArgs f, int wpad, int row0, int row1)
+template <int NT, int MINB, bool VAR, bool ZT = false, bool WIDE = false>
+__global__ void __launch_bounds__(NT, MINB) fused_single(FrameArgs f, int wpad)
 {
     after_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     int *ctr, *rowinfo;
     const Window s = window_layout(smem_raw, f.band + 2 * KernelShape<VAR>(f).halo, wpad, f.w, ctr, rowinfo);
-    const int first = RANGE ? row0 : 0, end = RANGE ? row1 : f.h;
-    const int nbands = (end - first + f.band - 1) / f.band;
+    const int nbands = (f.h + f.band - 1) / f.band;
     for (int b = blockIdx.x; b < nbands; b += gridDim.x) {
-        const int y0 = first + b * f.band;
-        run_band<NT, VAR, ZT, WIDE>(f, y0, min(y0 + f.band, end), s, ctr, rowinfo);
+        const int y0 = b * f.band;
+        run_band<NT, VAR, ZT, WIDE>(f, y0, min(y0 + f.band, f.h), s, ctr, rowinfo);
     }
 }
 
@@ -1287,11 +1284,6 @@ cudaError_t fused_configure(int device, FusedLimits* lim)
                          (const void*)fused_batch<kBig, 1, true>,   (const void*)fused_batch<kSmall, 2, true>,
                          (const void*)fused_single<kBig, 1, false, false, true>,
                          (const void*)fused_batch<kBig, 1, false, true>,
-                         (const void*)fused_single<kSmall, 2, true, false, false, true>,
-                         (const void*)fused_single<kSmall, 2, false, false, false, true>,
-                         (const void*)fused_single<kBig, 1, true, false, false, true>,
-                         (const void*)fused_single<kBig, 1, false, false, true, true>,
-                         (const void*)fused_single<kBig, 1, false, false, false, true>,
                          (const void*)fill_only<kBig, false>,       (const void*)fill_only<kBig, true>,
                          (const void*)fill_keys<kBig, false>,       (const void*)fill_keys<kBig, true>,
                          (const void*)imb_band<kBig, false>,        (const void*)imb_band<kBig, true>};
@@ -1359,42 +1351,26 @@ FusedShape fused_shape(const FusedLimits& lim, int w, int h, int halo)
     return s;
 }
 
-cudaError_t fused_launch(const FrameArgs& f, const FusedLimits& lim, int two_per_sm, cudaStream_t stream, int row0, int row1)
+cudaError_t fused_launch(const FrameArgs& f, const FusedLimits& lim, int two_per_sm, cudaStream_t stream)
 {
     const int wpad = fused_wpad(f.w);
     const size_t smem = fused_smem_bytes(wpad, f.band, f.halo);
     const bool var = f.halo != 1 || f.nearest != 0;  // a Patcher variant: its own instantiation
-    if (row1 < 0) row1 = f.h;
-    const int nbands = (row1 - row0 + f.band - 1) / f.band;
+    const int nbands = (f.h + f.band - 1) / f.band;
     const int slots = lim.sms * (two_per_sm ? 2 : 1);
     const int grid = nbands < slots ? nbands : slots;
     if (f.zt_out && var) return cudaErrorInvalidValue;  // the depth output exists for the default kernel
     const bool wide = (f.w + 31) / 32 > 2 * (kBig / 32);  // wider than 2 words per warp
-    cudaError_t launched = cudaSuccess;
     auto go = [&](auto kernel, int threads) {
-        launched = launch_after(kernel, (unsigned)grid, threads, smem, stream, f, wpad, row0, row1);
+        return launch_after(kernel, (unsigned)grid, threads, smem, stream, f, wpad);
     };
-    if (row0 != 0 || row1 != f.h) {
-        if (f.zt_out) return cudaErrorInvalidValue;
-        if (two_per_sm) {
-            if (var) go(fused_single<kSmall, 2, true, false, false, true>, kSmall);
-            else go(fused_single<kSmall, 2, false, false, false, true>, kSmall);
-        } else {
-            if (var) go(fused_single<kBig, 1, true, false, false, true>, kBig);
-            else if (wide) go(fused_single<kBig, 1, false, false, true, true>, kBig);
-            else go(fused_single<kBig, 1, false, false, false, true>, kBig);
-        }
-    } else if (two_per_sm) {
-        if (f.zt_out) go(fused_single<kSmall, 2, false, true>, kSmall);
-        else if (var) go(fused_single<kSmall, 2, true>, kSmall);
-        else go(fused_single<kSmall, 2, false>, kSmall);
-    } else {
-        if (f.zt_out) go(fused_single<kBig, 1, false, true>, kBig);
-        else if (var) go(fused_single<kBig, 1, true>, kBig);
-        else if (wide) go(fused_single<kBig, 1, false, false, true>, kBig);
-        else go(fused_single<kBig, 1, false>, kBig);
+    if (two_per_sm) {
+        if (f.zt_out) return go(fused_single<kSmall, 2, false, true>, kSmall);
+        return var ? go(fused_single<kSmall, 2, true>, kSmall) : go(fused_single<kSmall, 2, false>, kSmall);
     }
-    return launched;
+    if (f.zt_out) return go(fused_single<kBig, 1, false, true>, kBig);
+    if (var) return go(fused_single<kBig, 1, true>, kBig);
+    return wide ? go(fused_single<kBig, 1, false, false, true>, kBig) : go(fused_single<kBig, 1, false>, kBig);
 }
 
 cudaError_t fused_launch_batch(const BatchArgs& a, int wmax, const FusedLimits& lim, cudaStream_t stream, bool zt)

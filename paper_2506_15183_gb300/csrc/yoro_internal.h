@@ -74,9 +74,7 @@ size_t fused_smem_bytes(int wpad, int band, int halo = 1);
 cudaError_t fused_configure(int device, FusedLimits* lim);
 FusedShape fused_shape(const FusedLimits& lim, int w, int h, int halo = 1);
 int fused_max_band(const FusedLimits& lim, int w, int halo = 1);
-// Output rows [row0, row1) of the frame (row1 < 0: to its last row).
-cudaError_t fused_launch(const FrameArgs& f, const FusedLimits& lim, int two_per_sm, cudaStream_t stream, int row0 = 0,
-                         int row1 = -1);
+cudaError_t fused_launch(const FrameArgs& f, const FusedLimits& lim, int two_per_sm, cudaStream_t stream);
 // zt: the instantiation that writes each frame's warped depth where its zt_out is set.
 cudaError_t fused_launch_batch(const BatchArgs& a, int wmax, const FusedLimits& lim, cudaStream_t stream,
                                bool zt = false);
