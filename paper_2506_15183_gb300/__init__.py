@@ -122,6 +122,9 @@ def _check(code: int, where: str) -> None:
 
 def _stream(stream) -> int:
     if stream is None:
+        # the current stream's handle without a Stream object around it (0.1 instead of 3 us a call)
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
@@ -133,7 +136,7 @@ def _dev_ptr(t: torch.Tensor, dtype, shape, name: str) -> int:
         raise TypeError(f"{name} must be a torch tensor")
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype or tuple(t.shape) != tuple(shape) or not t.is_contiguous():
+    if t.dtype != dtype or t.shape != shape or not t.is_contiguous():
         raise ValueError(f"{name} must be a contiguous {dtype} tensor of shape {tuple(shape)}, "
                          f"got {t.dtype} {tuple(t.shape)}")
     return t.data_ptr()
@@ -348,8 +351,11 @@ class Synthesizer:
             self.handle = yoro_create_ex(w, h, fx, fy, cx, cy, ipd, near, far, kernel_rows, nearest_first)
 
     def __call__(self, color: torch.Tensor, depth: torch.Tensor, stream=None, unfused: bool = False):
-        out = torch.empty((self.h, self.w, 4), dtype=torch.uint8, device=color.device)
-        mask = torch.empty((self.h, self.w), dtype=torch.uint8, device=color.device)
+        if color.dtype == torch.uint8:
+            out, mask = color.new_empty((self.h, self.w, 4)), color.new_empty((self.h, self.w))
+        else:  # refused below
+            out = torch.empty((self.h, self.w, 4), dtype=torch.uint8, device=color.device)
+            mask = torch.empty((self.h, self.w), dtype=torch.uint8, device=color.device)
         fn = yoro_synthesize_unfused if unfused else yoro_synthesize
         fn(self.handle, color, depth, out, mask, stream)
         return out, mask
