@@ -102,10 +102,10 @@ __global__ void __launch_bounds__(kDwThreads, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     pdl_wait();
-    pdl_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch();  // this CTA's tensor memory is allocated
     const uint32_t tmem = *tslot;
     int issued = 0;
 

@@ -178,10 +178,10 @@ __global__ void __launch_bounds__(rows_threads(MODE, UP), 1)
     if (MODE == kColors || MODE == kCompose)
         for (int c = threadIdx.x; c < 99; c += kThreads) swout[c] = __ldg(a.wout + c);
     pdl_wait();
-    pdl_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch();  // this CTA's tensor memory is allocated
     const uint32_t tmem = *tslot;
 
     auto timed_out = [&]() {

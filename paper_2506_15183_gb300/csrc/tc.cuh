@@ -101,7 +101,9 @@ __device__ __forceinline__ void tma_store_5d(const CUtensorMap* map, const void*
 
 // Programmatic dependent launch: wait until the kernel before in the stream has completed and
 // its writes are visible (at once where this kernel was launched without the attribute), and
-// let the kernel after start its prologue.
+// let the kernel after start its prologue.  A kernel with tensor memory lets its successor
+// start only once the CTA has allocated it: a successor's CTA on the same SM allocates before it
+// waits, and must never hold columns that a CTA it waits for still needs.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

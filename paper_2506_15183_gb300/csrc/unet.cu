@@ -195,10 +195,10 @@ __global__ void __launch_bounds__(128, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     pdl_wait();
-    pdl_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch();  // this CTA's tensor memory is allocated
     const uint32_t tmem = *tslot;
 
     const int cb_n = a.Cin / KC;
@@ -372,10 +372,10 @@ __global__ void __launch_bounds__(128, 1)
     }
     for (int c = threadIdx.x; c < a.bn; c += blockDim.x) sbias[c] = __ldg(a.bias + nb + c);
     pdl_wait();
-    pdl_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch();  // this CTA's tensor memory is allocated
     const uint32_t tmem = *tslot;
 
     // The CTA walks bands blockIdx.x, + gridDim.x, ...: per band its K steps, then the
