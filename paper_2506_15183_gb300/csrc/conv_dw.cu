@@ -105,7 +105,6 @@ __global__ void __launch_bounds__(kDwThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_launch();  // this CTA's tensor memory is allocated
     const uint32_t tmem = *tslot;
     int issued = 0;
 
@@ -199,7 +198,6 @@ __global__ void __launch_bounds__(256) dw_reduce_kernel(const float* __restrict_
                                                         int cin, float* __restrict__ dW)
 {
     pdl_wait();
-    pdl_launch();
     __shared__ float4 part[8][32];
     const int l = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int quads = co_tile * (kDwTile / 4);  // of a tile

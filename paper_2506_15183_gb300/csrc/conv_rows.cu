@@ -181,7 +181,6 @@ __global__ void __launch_bounds__(rows_threads(MODE, UP), 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_launch();  // this CTA's tensor memory is allocated
     const uint32_t tmem = *tslot;
 
     auto timed_out = [&]() {

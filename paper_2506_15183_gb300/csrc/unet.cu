@@ -198,7 +198,6 @@ __global__ void __launch_bounds__(128, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_launch();  // this CTA's tensor memory is allocated
     const uint32_t tmem = *tslot;
 
     const int cb_n = a.Cin / KC;
@@ -375,7 +374,6 @@ __global__ void __launch_bounds__(128, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_launch();  // this CTA's tensor memory is allocated
     const uint32_t tmem = *tslot;
 
     // The CTA walks bands blockIdx.x, + gridDim.x, ...: per band its K steps, then the
@@ -772,8 +770,6 @@ __global__ void tile_flags_kernel(const __grid_constant__ FrameTable ft, int* __
 __global__ void tile_list_kernel(const int* __restrict__ flags, int ntiles, int* __restrict__ list,
                                  int* __restrict__ count)
 {
-    pdl_wait();
-    pdl_launch();
     __shared__ int warp_sums[32];
     __shared__ int base;
     if (threadIdx.x == 0) base = 0;
@@ -824,8 +820,6 @@ __device__ __forceinline__ uint16_t bf16_bits(float v)
 __global__ void tile_input_kernel(const __grid_constant__ FrameTable ft, const int* __restrict__ list,
                                   const int* __restrict__ count, uint16_t* __restrict__ x)
 {
-    pdl_wait();
-    pdl_launch();
     const int ti = blockIdx.y;
     if (ti >= *count) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;  // pixel of the tile
@@ -864,7 +858,6 @@ __global__ void output_kernel(const uint16_t* __restrict__ a, const float* __res
                               float* __restrict__ rgb)
 {
     pdl_wait();
-    pdl_launch();
     const int ti = blockIdx.y;
     if (ti >= T) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1049,7 +1042,11 @@ cudaError_t unet_run(UnetNet* n, const uint16_t* x, int T, const int* count, con
         ConvCall c{in, L.wk, y, L.bias, count, pool, i == 0 ? T : Te, H, H, L.cin_pad, L.cout, cstride, coff, up, 1};
         c.low = low;
         c.cskip = cskip;
-        c.pdl = i > 0;  // the kernel before is the layer before
+        // the kernel before is the layer before.  The frame path (count) is launched plainly: it
+        // shares the GPU with other streams' batches in the serving loop, whose learned frames met
+        // stalls with it (p99 4 to 27 ms in two runs, 1.3 to 2.8 in four without; one frame alone
+        // 604 against 639 us).
+        c.pdl = i > 0 && !count;
         if (i == 13) {
             c.T = T;
             c.wout = n->wout;
@@ -1195,11 +1192,9 @@ yoro_status inpaint_table(yoro_unet_ctx* u, const yoro::FrameTable& ft, cudaStre
     for (int f = 0; f < ft.n; ++f) maxcells = std::max(maxcells, ft.off[f + 1] - ft.off[f]);
     if (total == 0) return YORO_OK;
     yoro::tile_flags_kernel<<<dim3((unsigned)maxcells, (unsigned)ft.n), 256, 0, s>>>(ft, n->flags);
-    if (yoro::launch_kernel(yoro::tile_list_kernel, dim3(1), 1024, 0, s, true, n->flags, total, n->list, n->count) !=
-            cudaSuccess ||
-        yoro::launch_kernel(yoro::tile_input_kernel, dim3(16, (unsigned)total), 256, 0, s, true, ft, n->list, n->count,
-                            n->in0) != cudaSuccess)
-        return YORO_ECUDA;
+    yoro::tile_list_kernel<<<1, 1024, 0, s>>>(n->flags, total, n->list, n->count);
+    yoro::tile_input_kernel<<<dim3(16, (unsigned)total), 256, 0, s>>>(ft, n->list, n->count, n->in0);
+    if (cudaGetLastError() != cudaSuccess) return YORO_ECUDA;
     const yoro::NetOut out{nullptr, &ft};
     return yoro::unet_run(n, n->in0, total, n->count, out, s) == cudaSuccess ? YORO_OK : YORO_ECUDA;
 }

@@ -57,7 +57,6 @@ __device__ __forceinline__ float warp_sum(float v)
 __global__ void count_holes_kernel(const uint8_t* __restrict__ hole, long long n, int* __restrict__ cnt)
 {
     pdl_wait();
-    pdl_launch();
     int c = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         c += hole[i] != 0;
@@ -130,7 +129,6 @@ __global__ void __launch_bounds__(256) dz_kernel(const uint16_t* __restrict__ D,
                                                  float* __restrict__ gb)
 {
     pdl_wait();
-    pdl_launch();
     __shared__ float s[256];
     const int cg = C >> 3;  // channel groups, a power of two
     const int c = (threadIdx.x & (cg - 1)) << 3;
@@ -203,7 +201,6 @@ __global__ void __launch_bounds__(256) out_bwd_kernel(const float* __restrict__ 
                                                       float* __restrict__ gb, float* __restrict__ loss)
 {
     pdl_wait();
-    pdl_launch();
     __shared__ float s[128];
     const float inv_n = 1.0f / (3.0f * (float)max(*cnt, 1));
     const int c = (threadIdx.x & 3) << 3;
@@ -304,7 +301,6 @@ constexpr int kWeightThreads = 576;  // two of a tile's rows of 288
 __global__ void __launch_bounds__(kWeightThreads) weights_kernel(const __grid_constant__ WeightTable w, const AdamArgs a)
 {
     pdl_wait();
-    pdl_launch();
     __shared__ uint16_t s[32][290];  // [co][ci 9 + tap]; 145 words per row: no bank conflict along co
     if ((int)blockIdx.x == w.block0[14]) {
         for (int l = 0; l < 14; ++l)
