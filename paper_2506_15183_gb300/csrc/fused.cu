@@ -950,8 +950,8 @@ __global__ void __launch_bounds__(NT, 1) fill_only(FrameArgs f, const float* __r
 // reading it back.  The loading takes about 19 us of the pass at 1832x1920; the rest is the
 // holes' fill, bound by the bands that hold the most of it.  With each word's largest reached
 // depth at hand (one warp reduction and 4 bytes per word) the fill passes over words that
-// // are all foreground: eight seeds of 1832x1920 took 103, 52, 66, 56, 72, 95, 52 and 60 us with one
-// lane or one warp crossing them column by column, 64, 53, 61, 54, 68, 61, 50 and 48 so.
+// are all foreground: eight seeds of 1832x1920 took 103, 52, 66, 56, 72, 95, 52 and 60 us with
+// one lane or one warp crossing them column by column, 64, 53, 61, 54, 68, 61, 50 and 48 so.
 template <int NT, bool VAR>
 __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned long long* __restrict__ keys, int wpad)
 {

@@ -117,11 +117,17 @@ __global__ void __launch_bounds__(256) pose_scatter_kernel(FrameArgs f, PoseArgs
     }
 }
 
-// Whether every division by fx and fy stays among normal numbers: the numerators are zero or
-// between 2^-25 near and (2^31 + |c|) far in magnitude.
+// Whether every division by fx and fy stays among normal numbers (the numerators are zero or
+// between 2^-25 near and (2^31 + |c|) far in magnitude), and p'.z below 2^126, where
+// rcp.approx.ftz would flush its reciprocal to zero: |p| < 2^93, so |p'.z| < 3 2^30 (2^93 +
+// 2^30) < 2^125.  Rotations and positions are only checked to be finite when a handle is made.
 bool pose_fast(const FrameArgs& f, const PoseArgs& p)
 {
     const float lo = 9.3e-10f, hi = 1.0e9f;  // 2^-30, 2^30
+    for (float r : p.rot)
+        if (!(r >= -hi && r <= hi)) return false;
+    for (float c : p.c)
+        if (!(c >= -hi && c <= hi)) return false;
     return p.fx >= lo && p.fx <= hi && p.fy >= lo && p.fy <= hi && f.near_ >= lo && f.far_ <= hi && p.cx >= -hi &&
            p.cx <= hi && p.cy >= -hi && p.cy <= hi;
 }

@@ -62,6 +62,28 @@ def test_pose_bytes(yoro, w, h, fx, near, rows, yaw, pitch, c):
     syn.close()
 
 
+@pytest.mark.parametrize("rot,c", [
+    (np.eye(3), (-3e38, 0.0, -1e38)),                     # p'.z = 1e38: its reciprocal is a subnormal number
+    (np.diag([1e38, 1.0, 1e38]), (-2.5, 0.0, -1.0)),      # the same by the rotation
+    (np.eye(3) * 9e8, (0.063, 0.0, 0.0))])                # just inside the range of the estimates
+def test_pose_bytes_far_out_of_scale(yoro, rot, c):
+    """Rotations and positions are free as long as they are finite: where 1 / p'.z underflows the
+    targets come from the divisions themselves."""
+    import oracle
+
+    w, h, one = 48, 20, np.float32(1.0)
+    color, depth = _occluders(w, h, 5)
+    depth = (depth * 0.001).astype(np.float32)
+    rot, c = np.array(rot, np.float32), np.array(c, np.float32)
+    syn = yoro.Synthesizer(w, h, 1.0, 1.0, 16.5, 8.5, 0.0, near=1e-4, far=1000.0, pose=(rot, c))
+    out, mask = syn(torch.from_numpy(color).cuda(), torch.from_numpy(depth).cuda())
+    ref, rmask = oracle.synthesize_pose(color, depth, one, one, np.float32(16.5), np.float32(8.5), rot, c,
+                                        np.float32(1e-4), np.float32(1000.0))
+    assert np.array_equal(mask.cpu().numpy(), rmask)
+    assert np.array_equal(out.cpu().numpy(), ref)
+    syn.close()
+
+
 @pytest.mark.parametrize("w,h,div,interp", [(3000, 640, 4, True), (3001, 640, 2, True), (2999, 500, 16, False),
                                             (1832, 330, 4, True)])
 def test_imbuffer_bytes_over_several_waves(yoro, w, h, div, interp):
