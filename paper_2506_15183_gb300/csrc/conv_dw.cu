@@ -6,11 +6,15 @@
 // Both operands lie in memory as NHWC rows, channels contiguous, so in shared memory the K
 // index (the pixel) strides by 64 bytes per 32 channels: MN-major operands of tcgen05.mma
 // with the 64-byte swizzle the copy engine writes, no transposition pass.  A box is 8 rows
-// of one image with one column of padding on each side (x = -1 and x = W arrive as zeros), so
-// the K index runs over 8 (W + 2) consecutive pixels, a multiple of 16 at every level, and
-// a tap is a constant distance dy (W + 2) + dx - 1 in it: the three dy are the three
-// 32-column blocks of N = 96 (block stride one row), the dx are three MMAs from starts one
-// pixel apart.  At the padding columns dZ is zero, so what X holds there adds nothing.
+// of one image: of dZ its W columns alone, of X the ten rows around them with a column of
+// padding on each side (what lies outside the image arrives as zeros).  A K step is 16 pixels
+// of dZ (of one row; of two where W = 8, whose X rows are 16 pixels apart for that) and the
+// 16 pixels of X at a constant distance: the three dy are the three 32-column blocks of N =
+// 96 (block stride one row), the dx are three MMAs from starts one pixel apart.  So every
+// product is one of the sum's, a gradient pixel with an input pixel or with the padding's
+// zero: an infinite input reaches the taps it lies under and no others.  (With padding columns
+// in dZ too, one box walked as one run of pixels, their zeros met the columns 0 and W - 1 of
+// X, and 0 x infinity put NaN into taps that never meet such a pixel.)
 //
 // A CTA accumulates one (32 or 64 or 128 co) x (32 ci) x 9 tile in 288 tensor-memory columns
 // over its share of the boxes; the shares' sums go to a workspace and dw_reduce_kernel adds
@@ -36,28 +40,29 @@ constexpr int kDwTile = 9 * 32;            // columns of a tile: 9 taps times 32
 // A level's shapes: W pixels wide, COB blocks of 32 output channels.
 template <int W, int COB, int STAGES>
 struct DwShape {
-    static constexpr int kPitch = W + 2;
-    static constexpr int kPix = kDwRows * kPitch;  // K of a box
-    static constexpr int kPlane = kPix * 64;       // one 32-channel block of dZ
+    static constexpr int kPitch = W == 8 ? 16 : W + 2;  // pixels of an X row
+    static constexpr int kSteps = kDwRows * W / 16;     // K steps of a box
+    static constexpr int kPlane = kDwRows * W * 64;     // one 32-channel block of dZ
     static constexpr int kZ = COB * kPlane;
-    static constexpr int kXReal = (kDwRows + 2) * kPitch * 64;
-    static constexpr int kX = (kXReal + 64 + 1023) / 1024 * 1024;  // a pixel past the box is read (times zero)
+    static constexpr int kX = (kDwRows + 2) * kPitch * 64;
     static constexpr int kStage = (kZ + kX + 1023) / 1024 * 1024;
+    // 16-byte units from the box's first X pixel to that of K step k
+    __device__ static constexpr uint32_t x_start(int k) { return 4u * (uint32_t)(W == 8 ? 2 * k * kPitch : 16 * k / W * kPitch + 16 * k % W); }
     static constexpr int kStages = STAGES;
     // block stride of A: the next plane; with one plane the next pixel (those rows are not read back)
     static constexpr int kLboA = COB == 1 ? 64 : kPlane;
     // rows 64..127 of two planes read two more planes' worth past the last stage
     static constexpr int kSlack = COB == 2 ? std::max(0, 4 * kPlane - kStage) : 0;
     static constexpr int kSmem = 1024 + 1024 + STAGES * kStage + kSlack;
-    static_assert(kPix % 16 == 0 && kPlane % 512 == 0, "whole K steps, whole swizzle atoms");
+    static_assert((W % 16 == 0 || W == 8) && kPlane % 1024 == 0, "K steps of 16 pixels, whole swizzle atoms");
     static_assert(kSmem <= 227 * 1024, "shared memory of one CTA");
 };
 
-__device__ __forceinline__ uint64_t desc_mn_sw64(uint32_t saddr, uint32_t block_stride)
+__device__ __forceinline__ uint64_t desc_mn_sw64(uint32_t saddr, uint32_t block_stride, uint32_t group_stride)
 {
     uint64_t d = (uint64_t)((saddr >> 4) & 0x3fffu);
     d |= (uint64_t)(block_stride >> 4) << 16;  // next 32 channels
-    d |= (uint64_t)(512u >> 4) << 32;          // next 8 pixels
+    d |= (uint64_t)(group_stride >> 4) << 32;  // next 8 pixels
     d |= (uint64_t)1u << 46;
     d |= (uint64_t)4u << 61;
     return d;
@@ -91,10 +96,6 @@ __global__ void __launch_bounds__(kDwThreads, 1)
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // the pixel after an X box, which a padding pixel's tap reads: finite
-    for (int i = threadIdx.x; i < S::kStages * 16; i += kDwThreads)
-        *reinterpret_cast<uint32_t*>(stages + (i >> 4) * S::kStage + S::kZ + S::kXReal + (i & 15) * 4) = 0u;
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                      "r"(512)
@@ -120,10 +121,10 @@ __global__ void __launch_bounds__(kDwThreads, 1)
                 }
                 const int n = b / bands, y0 = (b - n * bands) * kDwRows;
                 unsigned char* st = stages + s * S::kStage;
-                mbar_expect_tx(&full[s], (uint32_t)(S::kZ + S::kXReal));
+                mbar_expect_tx(&full[s], (uint32_t)(S::kZ + S::kX));
 #pragma unroll
                 for (int j = 0; j < COB; ++j)
-                    tma_load_4d(st + j * S::kPlane, &tmZ, &full[s], (ct * COB + j) * 32, -1, y0, n);
+                    tma_load_4d(st + j * S::kPlane, &tmZ, &full[s], (ct * COB + j) * 32, 0, y0, n);
                 tma_load_4d(st + S::kZ, &tmX, &full[s], cb * 32, -1, y0 - 1, n);
                 ++issued;
             }
@@ -131,8 +132,8 @@ __global__ void __launch_bounds__(kDwThreads, 1)
     } else if (warp == 1) {  // MMAs: the whole warp runs the loop, one lane issues
         constexpr uint32_t idesc = idesc_bf16(kDwN) | (1u << 15) | (1u << 16);  // both operands MN-major
         const uint32_t el = elect_one();
-        const uint64_t da = desc_mn_sw64(smem_u32(stages), S::kLboA);
-        const uint64_t db = desc_mn_sw64(smem_u32(stages) + S::kZ, S::kPitch * 64);
+        const uint64_t da = desc_mn_sw64(smem_u32(stages), S::kLboA, 512);
+        const uint64_t db = desc_mn_sw64(smem_u32(stages) + S::kZ, S::kPitch * 64, S::kPitch == 16 ? 1024 : 512);
         bool ok = true;
         for (int b = b0; b < b1; ++b) {
             const int i = b - b0, s = i % S::kStages;
@@ -140,11 +141,11 @@ __global__ void __launch_bounds__(kDwThreads, 1)
             tc_fence_after();
             const uint64_t as = da + (uint64_t)((uint32_t)(s * S::kStage) >> 4);
             const uint64_t bs = db + (uint64_t)((uint32_t)(s * S::kStage) >> 4);
-            for (int k = 0; k < S::kPix / 16; ++k) {
+            for (int k = 0; k < S::kSteps; ++k) {
                 const uint32_t acc = (i > 0 || k > 0) ? 1u : 0u;
 #pragma unroll
                 for (int dx = 0; dx < 3; ++dx)
-                    mma_bf16_elected(el, tmem + dx * kDwN, as + 64 * k, bs + 64 * k + 4 * dx - 4, idesc, acc);
+                    mma_bf16_elected(el, tmem + dx * kDwN, as + 64 * k, bs + S::x_start(k) + 4 * dx, idesc, acc);
             }
             mma_commit_elected(el, &empty[s]);
         }
@@ -257,17 +258,17 @@ cudaError_t conv_dw_launch(const void* dZ, const void* X, int xcs, int T, int si
     const int shares = std::max(1, std::min(boxes / least, sms / tiles));
     if ((size_t)shares * tiles > (size_t)sms) return cudaErrorInvalidValue;  // the workspace holds `sms` tiles
     const cuuint32_t one[4] = {1, 1, 1, 1};
-    auto map = [&](CUtensorMap* m, const void* p, int cs, int rows) {
+    auto map = [&](CUtensorMap* m, const void* p, int cs, int cols, int rows) {
         const cuuint64_t c = (cuuint64_t)cs, w = (cuuint64_t)side;
         const cuuint64_t d[4] = {c, w, w, (cuuint64_t)T};
         const cuuint64_t st[3] = {c * 2, w * c * 2, w * w * c * 2};
-        const cuuint32_t box[4] = {32, (cuuint32_t)side + 2, (cuuint32_t)rows, 1};
+        const cuuint32_t box[4] = {32, (cuuint32_t)cols, (cuuint32_t)rows, 1};
         return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(p), d, st, box, one,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
     CUtensorMap tz, tx;
-    if (!map(&tz, dZ, cout, kDwRows) || !map(&tx, X, xcs, kDwRows + 2)) return cudaErrorInvalidValue;
+    if (!map(&tz, dZ, cout, side, kDwRows) || !map(&tx, X, xcs, side == 8 ? 16 : side + 2, kDwRows + 2)) return cudaErrorInvalidValue;
     cudaError_t e;
     if (side == 64) e = launch<64, 1, 2>(tz, tx, side, boxes, tiles, cbs, shares, ws, s);
     else if (side == 32) e = launch<32, 2, 3>(tz, tx, side, boxes, tiles, cbs, shares, ws, s);
