@@ -351,9 +351,9 @@ class Synthesizer:
             self.handle = yoro_create_ex(w, h, fx, fy, cx, cy, ipd, near, far, kernel_rows, nearest_first)
 
     def __call__(self, color: torch.Tensor, depth: torch.Tensor, stream=None, unfused: bool = False):
-        if color.dtype == torch.uint8:
+        if type(color) is torch.Tensor and color.dtype == torch.uint8:
             out, mask = color.new_empty((self.h, self.w, 4)), color.new_empty((self.h, self.w))
-        else:  # refused below
+        else:  # a subclass (its new_empty makes more of its kind), or refused below
             out = torch.empty((self.h, self.w, 4), dtype=torch.uint8, device=color.device)
             mask = torch.empty((self.h, self.w), dtype=torch.uint8, device=color.device)
         fn = yoro_synthesize_unfused if unfused else yoro_synthesize
