@@ -21,6 +21,7 @@
 
 #include <cstdint>
 
+#include "pose_grid.h"
 #include "yoro_device.cuh"
 #include "yoro_internal.h"
 
@@ -71,49 +72,43 @@ __device__ __forceinline__ float project(float a, float Z, float c)
 // for the row per pixel it took 21.9 us at 1832x1920 (18.6 M warp instructions); now 16.6 us
 // (12.9 M).  FAST: the divisions by fx and fy
 // through their reciprocals, the two by p'.z only where an estimate leaves the target open.
-constexpr int kScatterRows = 4;
-
 template <bool FAST>
-__global__ void __launch_bounds__(256) pose_scatter_kernel(FrameArgs f, PoseArgs p, unsigned chunks)
+__global__ void __launch_bounds__(kScatterCols) pose_scatter_kernel(FrameArgs f, PoseArgs p, unsigned cols)
 {
     const int w = f.w, h = f.h;
-    const unsigned cols = (unsigned)(w + 255) >> 8;
     const uint32_t near_m1 = __float_as_uint(f.near_) - 1u, far_m1 = __float_as_uint(f.far_) - 1u;
-    for (unsigned ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
-        const unsigned rg = ch / cols;
-        const int y0 = (int)rg * kScatterRows;
-        const int x = (int)((ch - rg * cols) << 8) + (int)threadIdx.x;
-        if (x >= w) continue;
-        const int nr = min(kScatterRows, h - y0);
-        const int i0 = y0 * w + x;  // w h < 2^31
-        float z[kScatterRows];
+    const unsigned rg = blockIdx.x / cols, xu = (blockIdx.x - rg * cols) * kScatterCols + threadIdx.x;
+    if (xu >= (unsigned)w) return;
+    const int x = (int)xu, y0 = (int)rg * kScatterRows;
+    const int nr = min(kScatterRows, h - y0);
+    const int i0 = y0 * w + x;  // w h < 2^31
+    float z[kScatterRows];
 #pragma unroll
-        for (int r = 0; r < kScatterRows; ++r) z[r] = r < nr ? __ldg(f.depth + i0 + r * w) : 0.0f;
-        const float xc = __fsub_rn(__fadd_rn((float)x, 0.5f), p.cx);
+    for (int r = 0; r < kScatterRows; ++r) z[r] = r < nr ? __ldg(f.depth + i0 + r * w) : 0.0f;
+    const float xc = __fsub_rn(__fadd_rn((float)x, 0.5f), p.cx);
 #pragma unroll
-        for (int r = 0; r < kScatterRows; ++r) {
-            if (r >= nr) break;
-            const float zc = __uint_as_float(clamped_depth_bits(z[r], near_m1, far_m1));
-            const float ax = __fmul_rn(xc, zc);
-            const float ay = __fmul_rn(__fsub_rn(__fadd_rn((float)(y0 + r), 0.5f), p.cy), zc);
-            const float px = FAST ? div_const(ax, p.fx, p.inv_fx) : __fdiv_rn(ax, p.fx);
-            const float py = FAST ? div_const(ay, p.fy, p.inv_fy) : __fdiv_rn(ay, p.fy);
-            const float q0 = __fsub_rn(px, p.c[0]), q1 = __fsub_rn(py, p.c[1]), q2 = __fsub_rn(zc, p.c[2]);
-            const float X = dot3(p.rot, q0, q1, q2), Y = dot3(p.rot + 3, q0, q1, q2), Z = dot3(p.rot + 6, q0, q1, q2);
-            if (!(Z > 0.0f)) continue;
-            float u, v;
-            if (FAST) {
-                u = project(__fmul_rn(p.fx, X), Z, p.cx);
-                v = project(__fmul_rn(p.fy, Y), Z, p.cy);
-            } else {
-                u = floorf(__fadd_rn(__fdiv_rn(__fmul_rn(p.fx, X), Z), p.cx));
-                v = floorf(__fadd_rn(__fdiv_rn(__fmul_rn(p.fy, Y), Z), p.cy));
-            }
-            if (!(u >= 0.0f && u < (float)w && v >= 0.0f && v < (float)h)) continue;
-            const size_t o = (size_t)(int)v * w + (int)u;
-            if (YORO_BOUND(o < (size_t)w * (size_t)h, kBadPose))
-                atomicMin(&p.zbuf[o], zkey(__float_as_uint(Z), i0 + r * w));
+    for (int r = 0; r < kScatterRows; ++r) {
+        if (r >= nr) break;
+        const float zc = __uint_as_float(clamped_depth_bits(z[r], near_m1, far_m1));
+        const float ax = __fmul_rn(xc, zc);
+        const float ay = __fmul_rn(__fsub_rn(__fadd_rn((float)(y0 + r), 0.5f), p.cy), zc);
+        const float px = FAST ? div_const(ax, p.fx, p.inv_fx) : __fdiv_rn(ax, p.fx);
+        const float py = FAST ? div_const(ay, p.fy, p.inv_fy) : __fdiv_rn(ay, p.fy);
+        const float q0 = __fsub_rn(px, p.c[0]), q1 = __fsub_rn(py, p.c[1]), q2 = __fsub_rn(zc, p.c[2]);
+        const float X = dot3(p.rot, q0, q1, q2), Y = dot3(p.rot + 3, q0, q1, q2), Z = dot3(p.rot + 6, q0, q1, q2);
+        if (!(Z > 0.0f)) continue;
+        float u, v;
+        if (FAST) {
+            u = project(__fmul_rn(p.fx, X), Z, p.cx);
+            v = project(__fmul_rn(p.fy, Y), Z, p.cy);
+        } else {
+            u = floorf(__fadd_rn(__fdiv_rn(__fmul_rn(p.fx, X), Z), p.cx));
+            v = floorf(__fadd_rn(__fdiv_rn(__fmul_rn(p.fy, Y), Z), p.cy));
         }
+        if (!(u >= 0.0f && u < (float)w && v >= 0.0f && v < (float)h)) continue;
+        const size_t o = (size_t)(int)v * w + (int)u;
+        if (YORO_BOUND(o < (size_t)w * (size_t)h, kBadPose))
+            atomicMin(&p.zbuf[o], zkey(__float_as_uint(Z), i0 + r * w));
     }
 }
 
@@ -179,10 +174,9 @@ cudaError_t pose_launch(const FrameArgs& f, const PoseArgs& p, const FusedLimits
     cudaError_t e = cudaMemsetAsync(p.zbuf, 0xFF, n * sizeof(unsigned long long), stream);
     if (e != cudaSuccess) return e;
     const int threads = 256;
-    const unsigned chunks = (unsigned)((f.w + 255) / 256) * (unsigned)((f.h + kScatterRows - 1) / kScatterRows);
-    const unsigned grid = chunks < (1u << 30) ? chunks : 1u << 30;
-    if (pose_fast(f, p)) pose_scatter_kernel<true><<<grid, threads, 0, stream>>>(f, p, chunks);
-    else pose_scatter_kernel<false><<<grid, threads, 0, stream>>>(f, p, chunks);
+    const ScatterGrid g = scatter_grid(f.w, f.h);
+    if (pose_fast(f, p)) pose_scatter_kernel<true><<<g.blocks, kScatterCols, 0, stream>>>(f, p, g.cols);
+    else pose_scatter_kernel<false><<<g.blocks, kScatterCols, 0, stream>>>(f, p, g.cols);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // a band fits shared memory: the band fill reads the keys itself (gather included)
     if (band_fill && fill_keys_fits(lim, f.w, f.halo)) return fill_keys_launch(f, p.zbuf, lim, stream);
