@@ -41,6 +41,7 @@
 #include <new>
 #include <vector>
 
+#include "ring.h"
 #include "tc.cuh"
 #include "unet_device.cuh"
 #include "unet_internal.h"
@@ -175,7 +176,8 @@ __global__ void __launch_bounds__(128, 1)
     uint64_t* empty = full + S;
     uint64_t* done = empty + S;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
-    volatile int* counts = reinterpret_cast<volatile int*>(tslot + 1);  // [0] issued, [1] consumed
+    // steps issued by warp 0 (activations), consumed, issued by warp 2 (weights)
+    volatile int* counts = reinterpret_cast<volatile int*>(tslot + 1);
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -186,6 +188,7 @@ __global__ void __launch_bounds__(128, 1)
         mbar_init(done, 1);
         counts[0] = 0;
         counts[1] = 0;
+        counts[2] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -224,6 +227,7 @@ __global__ void __launch_bounds__(128, 1)
             } else {
                 mbar_expect_tx(&full[s], (uint32_t)b_bytes);
                 tma_load_2d(sa + MT * kA, &tmB, &full[s], tap * a.Cin + cb * KC, nb);
+                counts[2] = k + 1;
             }
             if (++cb == cb_n) {
                 cb = 0;
@@ -276,10 +280,10 @@ __global__ void __launch_bounds__(128, 1)
     }
     tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0) {  // copies still in flight after a timeout: wait for them (bounded)
+    if (threadIdx.x == 0 && counts[1] < nk) {  // copies still in flight after a timeout: wait for them (bounded)
         const uint64_t d2 = globaltimer() + kWaitNs;
-        for (int k = counts[1]; k < counts[0]; ++k)
-            if (!mbar_wait(&full[k % S], (k / S) & 1, d2)) break;
+        ring_drain(counts[1], counts[0], counts[2], [&](int k) { mbar_arrive(&full[k % S]); },
+                   [&](int k) { mbar_wait(&full[k % S], (k / S) & 1, d2); });
     }
     __syncthreads();
     if (warp == 1) {
@@ -322,7 +326,8 @@ __global__ void __launch_bounds__(128, 1)
     uint64_t* empty = full + kMaxStages;
     uint64_t* done = empty + kMaxStages;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
-    volatile int* counts = reinterpret_cast<volatile int*>(tslot + 1);  // [0] issued, [1] consumed, [2] abort
+    // activation boxes issued, steps consumed, abort, weight boxes issued
+    volatile int* counts = reinterpret_cast<volatile int*>(tslot + 1);
     float* sbias = reinterpret_cast<float*>(smem + S * stage_bytes + 1024);
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
@@ -340,6 +345,7 @@ __global__ void __launch_bounds__(128, 1)
         const int s = kk % S, k = kk % nk, cb = k / 3, dx = k - 3 * cb;
         mbar_expect_tx(&full[s], (uint32_t)(3 * b_tap));
         tma_load_4d(smem + s * stage_bytes + a_span, &tmB, &full[s], cb * kKc, nb, 0, dx);
+        counts[3] = kk + 1;
     };
     const int first = nk < S ? nk : S;  // copies issued before the CTA-wide barrier
 
@@ -354,6 +360,7 @@ __global__ void __launch_bounds__(128, 1)
         counts[0] = 0;
         counts[1] = 0;
         counts[2] = 0;
+        counts[3] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         pdl_wait();
@@ -473,8 +480,8 @@ __global__ void __launch_bounds__(128, 1)
     __syncthreads();
     if (threadIdx.x == 0 && counts[2]) {  // copies still in flight after a timeout: wait for them (bounded)
         const uint64_t d2 = globaltimer() + kWaitNs;
-        for (int k = counts[1]; k < counts[0]; ++k)
-            if (!mbar_wait(&full[k % S], (k / S) & 1, d2)) break;
+        ring_drain(counts[1], counts[0], counts[3], [&](int k) { mbar_arrive(&full[k % S]); },
+                   [&](int k) { mbar_wait(&full[k % S], (k / S) & 1, d2); });
     }
     __syncthreads();
     if (warp == 1) {  // the allocating warp frees
