@@ -102,7 +102,7 @@ __device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity)
 template <class S, int COB>
 __global__ void __launch_bounds__(kDwThreads, 1)
     conv3x3_dw(const __grid_constant__ CUtensorMap tmZ, const __grid_constant__ CUtensorMap tmX, int H, int boxes,
-               int cbs, float* __restrict__ ws)
+               int cbs, float* ws)
 {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -280,8 +280,8 @@ __device__ __forceinline__ float value(const Sum2& a) { return isfinite(a.s) ? _
 // A block takes 128 consecutive floats of a tile (32 loads of 16 bytes), its eight warps every
 // eighth share, and adds the warps' sums in order.  Bound by reading the workspace from L2 (up to 22
 // MB a layer); one thread per element over all shares was 13 us a layer, latency.
-__global__ void __launch_bounds__(256) dw_reduce_kernel(const float* __restrict__ ws, int shares, int co_tile, int cbs,
-                                                        int cin, float* __restrict__ dW)
+__global__ void __launch_bounds__(256) dw_reduce_kernel(const float* ws, int shares, int co_tile, int cbs, int cin,
+                                                        float* dW)
 {
     pdl_wait();
     __shared__ float4 part[8][32], rest[8][32];

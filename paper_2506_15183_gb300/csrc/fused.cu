@@ -362,7 +362,7 @@ __device__ __forceinline__ void scatter_rows(const FrameArgs& f, const float* dc
 #pragma unroll
         for (int u = 0; u < U; ++u)
             z[c][u] = ((c == 0 || two) && YORO_BOUND(j + u < nr, kBadScatter))
-                          ? __ldg(dcol + c * NT + (size_t)u * w)
+                          ? dcol[c * NT + (size_t)u * w]
                           : 0.0f;
 #pragma unroll
     for (int c = 0; c < 2; ++c)
@@ -407,7 +407,7 @@ __device__ __forceinline__ void scatter_flat(const FrameArgs& f, const float* de
         ru[u] = r;
         xu[u] = x0 + q;
         z[u] = ((FULL || i + u * NT < n) && YORO_BOUND(i + u * NT < n, kBadScatter))
-                   ? __ldg(depth + (size_t)r * w + x0 + q)
+                   ? depth[(size_t)r * w + x0 + q]
                    : 0.0f;
         advance(r, q, dr, dq, rw);
     }
@@ -509,8 +509,8 @@ __device__ __forceinline__ void resolve_batch(const FrameArgs& f, const float* d
             zs[q][u] = 0.0f;
             cs[q][u] = 0u;
             if ((FULL || u < nb) && YORO_BOUND(o < nr * w, kBadResolve)) {
-                zs[q][u] = __ldg(depth + o);
-                cs[q][u] = __ldg(color + o);
+                zs[q][u] = depth[o];
+                cs[q][u] = color[o];
             }
         }
         go += w;
@@ -890,7 +890,7 @@ __global__ void __launch_bounds__(NT, MINB) fused_batch(const __grid_constant__ 
 // before any is used), then filled exactly as the fused kernel fills its bands.  VAR as
 // in the fused kernel: false compiles the paper's kernel shape as constants.
 template <int NT, bool VAR>
-__global__ void __launch_bounds__(NT, 1) fill_only(FrameArgs f, const float* __restrict__ zt, int wpad)
+__global__ void __launch_bounds__(NT, 1) fill_only(FrameArgs f, const float* zt, int wpad)
 {
     after_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -953,7 +953,7 @@ __global__ void __launch_bounds__(NT, 1) fill_only(FrameArgs f, const float* __r
 // are all foreground: eight seeds of 1832x1920 took 103, 52, 66, 56, 72, 95, 52 and 60 us with
 // one lane or one warp crossing them column by column, 64, 53, 61, 54, 68, 61, 50 and 48 so.
 template <int NT, bool VAR>
-__global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned long long* __restrict__ keys, int wpad)
+__global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned long long* keys, int wpad)
 {
     after_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -986,13 +986,13 @@ __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned l
                 const unsigned long long* kp = keys + ((ra + j0) * w + x);
 #pragma unroll
                 for (int u = 0; u < RB; ++u) {
-                    kv[u] = ((FULL || u < nb) && xin) ? __ldg(kp) : kEmptyKey;
+                    kv[u] = ((FULL || u < nb) && xin) ? *kp : kEmptyKey;
                     kp += w;
                 }
 #pragma unroll
                 for (int u = 0; u < RB; ++u) {
                     const uint32_t src = (uint32_t)kv[u];
-                    cv[u] = (kv[u] != kEmptyKey && YORO_BOUND(src < n, kBadPose)) ? __ldg(f.color + src) : 0u;
+                    cv[u] = (kv[u] != kEmptyKey && YORO_BOUND(src < n, kBadPose)) ? f.color[src] : 0u;
                 }
                 int so = j0 * wpad + x, vo = (ra + j0) * w + x;
 #pragma unroll
@@ -1082,7 +1082,7 @@ __global__ void __launch_bounds__(NT, 1) imb_band(FrameArgs f, int div, int inte
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 z[q] = c + q * NT < nr * ws
-                           ? __ldg(f.depth + (size_t)(ra + jq) * w + min((iq << lg) + (div >> 1), w - 1))
+                           ? f.depth[(size_t)(ra + jq) * w + min((iq << lg) + (div >> 1), w - 1)]
                            : 0.0f;
                 advance(jq, iq, dj, di, ws);
             }
@@ -1146,7 +1146,7 @@ __global__ void __launch_bounds__(NT, 1) imb_band(FrameArgs f, int div, int inte
                     if (key != kEmptyKey) {
                         reach |= 1u << u;
                         if (!interp) {
-                            c0[u] = __ldg(crow + min(((int)(uint32_t)key << lg) + (lane & (div - 1)), w - 1));
+                            c0[u] = crow[min(((int)(uint32_t)key << lg) + (lane & (div - 1)), w - 1)];
                         } else {
                             float d = __uint_as_float((uint32_t)key);  // disp of the winner
                             if (side) {
@@ -1160,8 +1160,8 @@ __global__ void __launch_bounds__(NT, 1) imb_band(FrameArgs f, int div, int inte
                             const float fl = floorf(uc);
                             const int i0 = (int)fl;
                             fr[u] = __fsub_rn(uc, fl);
-                            c0[u] = __ldg(crow + i0);
-                            c1[u] = __ldg(crow + min(i0 + 1, w - 1));
+                            c0[u] = crow[i0];
+                            c1[u] = crow[min(i0 + 1, w - 1)];
                         }
                     }
                     kc += ws;

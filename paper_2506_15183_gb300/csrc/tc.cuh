@@ -101,7 +101,9 @@ __device__ __forceinline__ void tma_store_5d(const CUtensorMap* map, const void*
 
 // Programmatic dependent launch: a kernel launched by launch_kernel(pdl) is set up while the
 // kernel before it in the stream ends, and waits here until that kernel has completed and its
-// writes are visible (at once where it was launched without the attribute).  No kernel
+// writes are visible (at once where it was launched without the attribute).  What the kernel
+// before may have written is read by ordinary loads only: the read-only path (__ldg, const
+// __restrict__) may be taken for constant while this kernel is resident, before the wait too.  No kernel
 // releases its successor early (griddepcontrol.launch_dependents): the successor's waiting
 // CTAs would hold whole SMs (217 KB of shared memory each) that other streams' frames need, and
 // tensor memory that a CTA they wait for may still need, for 6 us of 114 on 8 tiles alone.

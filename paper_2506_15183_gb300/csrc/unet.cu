@@ -861,8 +861,7 @@ __global__ void tile_input_kernel(const __grid_constant__ FrameTable ft, const i
 
 // The three colors of every pixel of the first T tiles to rgb (T x 64 x 64 x 3 floats), from
 // stored activations (the training forward, which keeps them for its backward pass).
-__global__ void output_kernel(const uint16_t* __restrict__ a, const float* __restrict__ wo, int T,
-                              float* __restrict__ rgb)
+__global__ void output_kernel(const uint16_t* a, const float* wo, int T, float* rgb)
 {
     pdl_wait();
     const int ti = blockIdx.y;

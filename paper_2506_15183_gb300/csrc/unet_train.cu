@@ -54,7 +54,7 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
-__global__ void count_holes_kernel(const uint8_t* __restrict__ hole, long long n, int* __restrict__ cnt)
+__global__ void count_holes_kernel(const uint8_t* hole, long long n, int* cnt)
 {
     pdl_wait();
     int c = 0;
@@ -123,10 +123,9 @@ __device__ __forceinline__ void block_sums(float (&v)[N], int groups, float* s, 
 enum { kDirect, kUp, kPooled };
 
 template <int KIND>
-__global__ void __launch_bounds__(256) dz_kernel(const uint16_t* __restrict__ D, int dcs, int doff,
-                                                 const uint16_t* __restrict__ P, const uint16_t* __restrict__ Y, int ycs,
-                                                 int yoff, int side, int C, long long items, uint16_t* __restrict__ dZ,
-                                                 float* __restrict__ gb)
+__global__ void __launch_bounds__(256) dz_kernel(const uint16_t* D, int dcs, int doff, const uint16_t* P,
+                                                 const uint16_t* Y, int ycs, int yoff, int side, int C, long long items,
+                                                 uint16_t* dZ, float* gb)
 {
     pdl_wait();
     __shared__ float s[256];
@@ -193,12 +192,9 @@ __global__ void __launch_bounds__(256) dz_kernel(const uint16_t* __restrict__ D,
 // the sigmoid input at every pixel (0 outside holes), the gradient of the 1x1 weights and
 // biases, and dZ of the last 3x3 layer with its bias gradient.  A thread takes eight
 // channels of a pixel (four threads a pixel; the first of them adds the loss).
-__global__ void __launch_bounds__(256) out_bwd_kernel(const float* __restrict__ rgb, const uint8_t* __restrict__ gt,
-                                                      const uint8_t* __restrict__ hole, long long npx,
-                                                      const int* __restrict__ cnt, const uint16_t* __restrict__ a,
-                                                      const float* __restrict__ wout, uint16_t* __restrict__ dZ,
-                                                      float* __restrict__ gw, float* __restrict__ gwb,
-                                                      float* __restrict__ gb, float* __restrict__ loss)
+__global__ void __launch_bounds__(256) out_bwd_kernel(const float* rgb, const uint8_t* gt, const uint8_t* hole, long long npx,
+                                                      const int* cnt, const uint16_t* a, const float* wout, uint16_t* dZ,
+                                                      float* gw, float* gwb, float* gb, float* loss)
 {
     pdl_wait();
     __shared__ float s[128];

@@ -12,7 +12,9 @@ namespace yoro {
 
 // Programmatic dependent launch: a kernel launched with launch_after() may be set up while the
 // kernel before it in the stream ends; it starts with after_wait(), which returns once that
-// kernel has completed and its writes are visible.  The frame kernels do not release their
+// kernel has completed and its writes are visible.  Their inputs are read by ordinary loads: the
+// read-only path (__ldg, const __restrict__) may be taken for constant from before the wait on.
+// The frame kernels do not release their
 // successors early: a waiting CTA would hold an SM that other streams' frames could use.
 __device__ __forceinline__ void after_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
