@@ -952,7 +952,8 @@ __global__ void __launch_bounds__(NT, 1) fill_only(FrameArgs f, const float* zt,
 // depth at hand (one warp reduction and 4 bytes per word) the fill passes over words that
 // are all foreground: eight seeds of 1832x1920 took 103, 52, 66, 56, 72, 95, 52 and 60 us with
 // one lane or one warp crossing them column by column, 64, 53, 61, 54, 68, 61, 50 and 48 so.
-template <int NT, bool VAR>
+// ZMAX = false, without them, is for the widths whose window just fits shared memory.
+template <int NT, bool VAR, bool ZMAX>
 __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned long long* keys, int wpad)
 {
     after_wait();
@@ -961,7 +962,7 @@ __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned l
     int *ctr, *rowinfo;
     const KernelShape<VAR> ks(f);
     Window s = window_layout(smem_raw, f.band + 2 * ks.halo, wpad, f.w, ctr, rowinfo);
-    s.zmax = reinterpret_cast<uint32_t*>(rowinfo + 2 * s.slots);  // after the window (keys_smem_bytes)
+    if (ZMAX) s.zmax = reinterpret_cast<uint32_t*>(rowinfo + 2 * s.slots);  // after the window (keys_smem_bytes)
     const int w = f.w, h = f.h, nwords = s.nwords;
     const size_t n = (size_t)w * (size_t)h;  // source indices are below n (checked in the debug-bounds build)
     (void)n;
@@ -1000,10 +1001,11 @@ __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned l
                     if (FULL || u < nb) {  // uniform
                         const bool reached = kv[u] != kEmptyKey;
                         const uint32_t m = __ballot_sync(0xffffffffu, reached);
-                        const uint32_t zm = __reduce_max_sync(0xffffffffu, reached ? (uint32_t)(kv[u] >> 32) : 0u);
+                        uint32_t zm = 0u;
+                        if (ZMAX) zm = __reduce_max_sync(0xffffffffu, reached ? (uint32_t)(kv[u] >> 32) : 0u);
                         if (lane == 0 && YORO_BOUND(j0 + u < s.slots, kBadHoles)) {
                             s.bits[(j0 + u) * nwords + g] = m;
-                            s.zmax[(j0 + u) * nwords + g] = zm;
+                            if (ZMAX) s.zmax[(j0 + u) * nwords + g] = zm;
                         }
                         if (reached && YORO_BOUND(so < s.slots * wpad, kBadHoles)) {
                             s.zt[so] = (uint32_t)(kv[u] >> 32);
@@ -1025,7 +1027,7 @@ __global__ void __launch_bounds__(NT, 1) fill_keys(FrameArgs f, const unsigned l
         }
         if (threadIdx.x == 0) *ctr = 0;
         __syncthreads();
-        fill_band<NT, VAR, true>(f, y0, y1, s, ctr, rowinfo);
+        fill_band<NT, VAR, ZMAX>(f, y0, y1, s, ctr, rowinfo);
     }
 }
 
@@ -1285,7 +1287,8 @@ cudaError_t fused_configure(int device, FusedLimits* lim)
                          (const void*)fused_single<kBig, 1, false, false, true>,
                          (const void*)fused_batch<kBig, 1, false, true>,
                          (const void*)fill_only<kBig, false>,       (const void*)fill_only<kBig, true>,
-                         (const void*)fill_keys<kBig, false>,       (const void*)fill_keys<kBig, true>,
+                         (const void*)fill_keys<kBig, false, true>, (const void*)fill_keys<kBig, true, true>,
+                         (const void*)fill_keys<kBig, false, false>, (const void*)fill_keys<kBig, true, false>,
                          (const void*)imb_band<kBig, false>,        (const void*)imb_band<kBig, true>};
     for (const void* fn : fns) {
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
@@ -1434,27 +1437,39 @@ cudaError_t fill_only_launch(FrameArgs f, const float* zt, const FusedLimits& li
     return launch_after(kernel, (unsigned)grid, kBig, smem, stream, f, zt, wpad);
 }
 
-// fill_keys: the window and its words' largest depths.
-static size_t keys_smem_bytes(int wpad, int band, int halo)
+// fill_keys: the window and, if any, its words' largest depths.
+static size_t keys_smem_bytes(int wpad, int band, int halo, bool zmax)
 {
-    return fused_smem_bytes(wpad, band, halo) + (size_t)(band + 2 * halo) * (size_t)((wpad + 31) / 32) * 4;
+    return fused_smem_bytes(wpad, band, halo) + (zmax ? (size_t)(band + 2 * halo) * (size_t)((wpad + 31) / 32) * 4 : 0);
 }
 
-bool fill_keys_fits(const FusedLimits& lim, int w, int halo)
+static bool keys_zmax(const FusedLimits& lim, int w, int halo)
 {
-    return keys_smem_bytes(fused_wpad(w), 1, halo) <= (size_t)lim.smem_per_block;
+    return keys_smem_bytes(fused_wpad(w), 1, halo, true) <= (size_t)lim.smem_per_block;
 }
+
+// The largest depths take 1.5 % more shared memory, so some frames' one-row window fits without
+// them only (9,249 to 9,384 columns for 3 kernel rows, 1,849 to 1,872 for 15).  Those with up to 7
+// rows go without, still filled by bands; with more rows, where a band is mostly halo, a gather
+// and one thread per hole pixel is faster.  h = 1024, wide occluders / 40-pixel runs of depths,
+// bands against gather, us: 3 rows at 9317 columns 344 / 420 against 786 / 862, 5 rows at 5589
+// 248 / 348 against 390 / 516, 7 rows at 3989 447 / 331 against 410 / 374, 9 rows at 3105
+// 307 / 340 against 276 / 281, 15 rows at 1861 205 / 356 against 212 / 281.
+bool fill_keys_takes(const FusedLimits& lim, int w, int halo) { return keys_zmax(lim, w, halo) || halo <= 3; }
 
 cudaError_t fill_keys_launch(FrameArgs f, const unsigned long long* keys, const FusedLimits& lim, cudaStream_t stream)
 {
     const int wpad = fused_wpad(f.w);
+    const bool zmax = keys_zmax(lim, f.w, f.halo);
     int bmax = 1;
-    while (bmax < 4096 && keys_smem_bytes(wpad, bmax + 1, f.halo) <= (size_t)lim.smem_per_block) ++bmax;
+    while (bmax < 4096 && keys_smem_bytes(wpad, bmax + 1, f.halo, zmax) <= (size_t)lim.smem_per_block) ++bmax;
     f.band = balanced_band(f.h, f.halo, bmax, lim.sms);
-    const size_t smem = keys_smem_bytes(wpad, f.band, f.halo);
+    const size_t smem = keys_smem_bytes(wpad, f.band, f.halo, zmax);
     const int grid = (f.h + f.band - 1) / f.band;
     if (grid < 1) return cudaSuccess;
-    const auto kernel = f.halo == 1 && !f.nearest ? fill_keys<kBig, false> : fill_keys<kBig, true>;
+    const bool var = f.halo != 1 || f.nearest;
+    const auto kernel = zmax ? (var ? fill_keys<kBig, true, true> : fill_keys<kBig, false, true>)
+                             : (var ? fill_keys<kBig, true, false> : fill_keys<kBig, false, false>);
     return launch_after(kernel, (unsigned)grid, kBig, smem, stream, f, keys, wpad);
 }
 

@@ -179,7 +179,7 @@ cudaError_t pose_launch(const FrameArgs& f, const PoseArgs& p, const FusedLimits
     else pose_scatter_kernel<false><<<g.blocks, kScatterCols, 0, stream>>>(f, p, g.cols);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // a band fits shared memory: the band fill reads the keys itself (gather included)
-    if (band_fill && fill_keys_fits(lim, f.w, f.halo)) return fill_keys_launch(f, p.zbuf, lim, stream);
+    if (band_fill && fill_keys_takes(lim, f.w, f.halo)) return fill_keys_launch(f, p.zbuf, lim, stream);
     pose_gather_kernel<<<blocks_for(n, threads), threads, 0, stream>>>(f, p);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return fill_pixels_launch(f, p.zt, stream);

@@ -117,7 +117,8 @@ cudaError_t fill_only_launch(FrameArgs f, const float* zt, const FusedLimits& li
 // The same fill read straight from a frame-wide z-buffer of 64-bit keys (depth bits above
 // the source index, ~0 at holes): also writes the reached pixels' colors (gathered from
 // f.color) and the hole mask.
-bool fill_keys_fits(const FusedLimits& lim, int w, int halo);
+// fill_keys_takes(): whether a frame whose window fits shared memory goes that way.
+bool fill_keys_takes(const FusedLimits& lim, int w, int halo);
 cudaError_t fill_keys_launch(FrameArgs f, const unsigned long long* keys, const FusedLimits& lim, cudaStream_t stream);
 // The holes of a frame resolved in global memory (colors in f.out, depths in zt, mask
 // in f.mask), one thread per pixel: for frames too wide for a band window.
