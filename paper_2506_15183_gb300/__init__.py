@@ -122,9 +122,13 @@ def _check(code: int, where: str) -> None:
 
 def _stream(stream) -> int:
     if stream is None:
-        # the current stream's handle without a Stream object around it (0.1 instead of 3 us a call)
+        # the current stream's handle without a Stream object around it (0.1 instead of 3 us a call),
+        # by private getters where this torch has them
         if torch.cuda.is_initialized():
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            try:
+                return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            except AttributeError:
+                pass
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream

@@ -1,8 +1,25 @@
-"""The Python binding's own decisions: the type of the tensors a Synthesizer returns."""
+"""The Python binding's own decisions: the current stream's handle with and without torch's
+raw-handle getters, and the type of the tensors a Synthesizer returns."""
+import types
+
 import pytest
 import torch
 
 import paper_2506_15183_gb300 as yoro
+
+
+@pytest.mark.parametrize("missing", [(), ("_cuda_getCurrentRawStream",), ("_cuda_getDevice",)])
+def test_current_stream_needs_no_private_getter(monkeypatch, missing):
+    """A torch without the raw getters (private names) takes the public way to the same handle."""
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: types.SimpleNamespace(cuda_stream=77))
+    for name, value in (("_cuda_getCurrentRawStream", lambda d: 70 + d), ("_cuda_getDevice", lambda: 7)):
+        if name in missing:
+            monkeypatch.delattr(torch._C, name, raising=False)
+        else:
+            monkeypatch.setattr(torch._C, name, value, raising=False)
+    assert yoro._stream(None) == 77
+    assert yoro._stream(5) == 5
 
 
 class Frame(torch.Tensor):
