@@ -152,7 +152,9 @@ __device__ __forceinline__ uint32_t fill_from_edges(int x, int v, int L, int R, 
 #pragma unroll 1
         for (int step = 0; step <= whi - wlo; ++step) {
             const int wi = ks.nearest ? wlo + step : whi - step;
-            if (ZMAX && __uint_as_float(s.zmax[(vv - s.ra) * s.nwords + wi]) < d_occ) continue;
+            if (ZMAX && YORO_BOUND(wi >= 0 && wi < s.nwords, kBadHoles) &&
+                __uint_as_float(s.zmax[(vv - s.ra) * s.nwords + wi]) < d_occ)
+                continue;
             uint32_t m = b[wi];
             if (wi == whi) m &= mhi;
             if (wi == wlo) m &= mlo;
