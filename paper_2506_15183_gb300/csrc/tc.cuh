@@ -146,16 +146,6 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int n)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(accum)
-        : "memory");
-}
-
 // For a warp that issues MMAs in uniform control flow (all lanes run the loop, so the
 // descriptors stay in uniform registers): 1 in one lane of the warp, 0 in the others.
 __device__ __forceinline__ uint32_t elect_one()
@@ -175,7 +165,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, u
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, deadline));
 }
 
-// An MMA issued by the lane whose `elected` is 1.
+// An MMA issued by the lane whose `elected` is 1; it accumulates if `accum` is not 0.
 __device__ __forceinline__ void mma_bf16_elected(uint32_t elected, uint32_t d_tmem, uint64_t a, uint64_t b,
                                                  uint32_t idesc, uint32_t accum)
 {
@@ -210,12 +200,6 @@ __device__ __forceinline__ void mma_commit_elected(uint32_t elected, uint64_t* b
         "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(smem_u32(bar)),
         "r"(elected)
         : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t* bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
 }
 
 // 32 consecutive accumulator columns of this warp's 32 TMEM lanes (one lane per thread);

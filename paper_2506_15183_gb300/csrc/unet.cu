@@ -62,8 +62,7 @@ struct ConvArgs {
     int Cin, Cout;        // Cin: channels of the input tensor, a multiple of 32
     int bn;               // output channels of a CTA: Cout, or a part of it (blockIdx.y) on small grids
     const float* bias;    // Cout
-    __nv_bfloat16* y;     // NHWC output, channel stride y_cstride, channels from y_coff
-    int y_cstride, y_coff;
+    int y_coff;           // first output channel in y (the output's tensor map)
     int upsample;         // 1: pixel (yy, xx) goes to (2yy + a, 2xx + b), a, b in {0, 1}
     int relu;
     int ncols;            // tensor-memory columns allocated (a power of two >= mt bn, >= 32)
@@ -698,8 +697,6 @@ cudaError_t unet_conv3x3(const ConvCall& call, cudaStream_t stream)
     a.Cin = Cin;
     a.Cout = Cout;
     a.bias = call.bias;
-    a.y = static_cast<__nv_bfloat16*>(y);
-    a.y_cstride = y_cstride;
     a.y_coff = y_coff;
     a.upsample = upsample;
     a.relu = call.relu;
