@@ -66,7 +66,7 @@ long long yoro_unet_param_count(void);
  * An inpainter on the current device.  params: host floats as above (weights are rounded
  * to bfloat16 here, biases stay FP32); the handle keeps its own copy.  It owns device
  * buffers for max(max_tiles, the tiles of a max_w x max_h frame) 64 x 64 tiles (about
- * 2.9 MB per tile).  NULL if an argument is wrong or an allocation fails.
+ * 2.1 MB per tile).  NULL if an argument is wrong or an allocation fails.
  */
 yoro_unet yoro_unet_create(const float* params, long long n_params, int max_tiles, int max_w, int max_h);
 void yoro_unet_destroy(yoro_unet u);

@@ -2,30 +2,31 @@
 // 64 x 64 tiles, BF16 weights and activations, FP32 accumulation.
 //
 // Each 3x3 convolution is an implicit GEMM: M = output pixels (128 per accumulator), N =
-// output channels (32..256, one MMA tile), K = taps x input channels, taken 32 channels
-// (64 bytes: the swizzle span) at a time.  Operands are TMA tiled loads into shared
-// memory with 64-byte swizzle (the zero padding of the convolution is the part of a box
-// outside the tensor, which TMA fills with zeros); one thread issues the copies, another
-// the tcgen05.mma (kind::f16, BF16 operands, FP32 accumulator in tensor memory, two
-// K = 16 steps per 32-channel slice), with mbarriers between them.  The epilogue reads
-// the accumulators with tcgen05.ld, adds the bias, applies ReLU, rounds to BF16 and
-// stores NHWC at a channel offset of a wider buffer (so a decoder's concatenation is
-// written in place), or, for the layer below a decoder level, to the 2 x 2 pixels of the
-// nearest upsampling.  Three forms:
+// output channels (32..256, or a part of them on small grids), K = taps x input channels,
+// taken 32 or 64 channels (64 or 128 bytes: the swizzle span) at a time.  Operands are TMA
+// tiled loads into shared memory, swizzled by the copy engine (the zero padding of the
+// convolution is the part of a box outside the tensor, which TMA fills with zeros); one thread
+// each issues the activation and the weight copies, one warp the tcgen05.mma (kind::f16, BF16
+// operands, FP32 accumulator in tensor memory, K = 16), with mbarriers between them.  The
+// epilogue reads the accumulators with tcgen05.ld, adds the bias, applies ReLU, rounds to BF16
+// and stores NHWC at a channel offset of a wider buffer (so a concatenation is written in
+// place), or, for the layer below a decoder level, to the 2 x 2 pixels of the nearest
+// upsampling.  Three forms:
 //   - conv3x3_rows (conv_rows.cu), for 32 or 64 output channels on tiles 32 to 128 pixels
 //     wide: one image row per accumulator, the three taps of a kernel column in one MMA.
-//   - conv3x3_halo, for the other tiles of whole rows of one image: a band of 256 / W rows goes
-//     into two accumulators (each CTA walks bands blockIdx.x, + gridDim.x, ..., as many
-//     CTAs as fit on the SMs at once); a K step is one (channel block, dx) pair, a single box of
-//     the rows plus one above and below, shared by the three dy taps through the start
-//     address of the MMA operand (whole 512-byte swizzle atoms apart), and the three
-//     taps' weight boxes.  Each input pixel is copied 3 (R + 2) / R times instead of 9.
-//   - conv3x3_tc, one CTA per 128-pixel tile (the 8 x 8 level, where 128 pixels are two
-//     tiles, and 256 output channels): a K step is one (channel block, tap), the
-//     activation box {32 channels, W, rows, tiles} at the tap's offset and the weight box
-//     {32, Cout} of the K-major weights (k = tap * Cin + ci), in a 4-stage ring.
-// The last two use CTAs of 128 threads, several per SM, so the copies of one overlap the set-up,
-// MMAs and epilogue of the others.
+//   - conv3x3_halo, for the other tiles of whole rows of one image: a band of 128 or 256 pixels
+//     goes into one or two accumulators (each CTA walks bands blockIdx.x, + gridDim.x, ..., as
+//     many CTAs as fit on the SMs at once); a K step is one (32-channel block, dx) pair, a single
+//     box of the band's R rows plus one above and below, shared by the three dy taps through the
+//     start address of the MMA operand (whole 512-byte swizzle atoms apart), and one box of the
+//     three taps' weights.  Each input pixel is copied 3 (R + 2) / R times instead of 9.
+//   - conv3x3_tc, one CTA per one or two 128-pixel tiles (the 8 x 8 level, where 128 pixels are
+//     two images, and 256 output channels): a K step is one (block of 32 or 64 channels, tap),
+//     the activation boxes {channels, W, rows, images} at the tap's offset and the weight box
+//     {channels, the CTA's output channels} of the K-major weights (k = tap * Cin + ci).
+// The last two use CTAs of 128 threads and rings of up to 12 stages: two, and several CTAs per SM,
+// where there are enough of them that the copies of one overlap the set-up, MMAs and
+// epilogue of the others; deeper where a CTA has its SM to itself.
 //
 // Every wait on an mbarrier has a deadline (1 s of %globaltimer): a wait that runs out
 // records kUnetTimeout in a status word, the kernel waits (again bounded) for the copies
@@ -537,17 +538,18 @@ size_t halo_smem_bytes(int stage_bytes, int stages)
     return 1024 + (size_t)stages * stage_bytes + 1024 + 256 * 4;
 }
 
-// Shared memory a halo-form CTA may take: at least two CTAs share an SM (228 KB, 1 KB
-// reserved per CTA); with two stages, three fit for Cout <= 64.
+// Shared memory a halo-form CTA of two stages may take: two CTAs share an SM (228 KB, 1 KB
+// reserved per CTA).
 constexpr int kHaloSmemBudget = 112 * 1024;
 
 // The halo form's shape for a layer, or mt = 0 where the one-tile form runs: whole-row
 // tiles of one image (W in 16..128), two accumulators of 128 pixels (R = 256 / W rows,
 // a divisor of H), Cout <= 128 (2 Cout tensor-memory columns), two copy stages within
-// the budget.  Two accumulators with two stages (three CTAs per SM for Cout <= 64, two
-// for Cout = 128) measured fastest on every layer of the network, against one or four
-// accumulators and two to four stages at one to four CTAs per SM: more CTAs per SM
-// overlap one CTA's set-up, last MMAs and epilogue with the others' copies.
+// the budget.  It also says which layers the row form may take.  At 128 output channels, which
+// the halo form still runs, two accumulators with two stages (two CTAs per SM) measured
+// fastest against one or four accumulators and two to four stages at one to four CTAs per SM:
+// more CTAs per SM overlap one CTA's set-up, last MMAs and epilogue with the others' copies.
+// unet_conv3x3 takes one accumulator and a deeper ring on grids that leave SMs idle.
 void halo_shape(int H, int W, int Cout, int* mt, int* stages)
 {
     *mt = 0;

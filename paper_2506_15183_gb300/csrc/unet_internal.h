@@ -61,8 +61,8 @@ struct ConvCall {
     // others, read through their nearest upsampling
     const void* low = nullptr;
     int cskip = 0;
-    // the kernel before in the stream is a convolution whose prologue-time state (weights, biases,
-    // count) this one does not depend on: start the prologue while it ends
+    // the kernel before in the stream writes nothing that this one reads in its prologue (biases,
+    // output weights, count): start the prologue while it ends
     bool pdl = false;
 };
 
