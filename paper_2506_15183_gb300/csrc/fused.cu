@@ -1332,7 +1332,11 @@ static int max_band(const FusedLimits& lim, int wpad, int halo)
 // cost).  Bands of all bmax rows can leave the last wave nearly empty: 1920 rows in bands of
 // 10 are 192 bands, two waves for 152 SMs, and bands of 7 (275) are two waves of 9 rows
 // each instead of 12 (1832x1920 through the intermediate buffer, 4 px per cell: 69 -> 58 us with
-// the bands alone; fused 2064x2208 frames, 11 -> 8 rows: 48.7 -> 41.8 us).
+// the bands alone).  A frame whose slowest band falls into the last wave can lose what the others
+// gain: of 24 seeds each, against bands of bmax rows dealt by stride, plain frames of 2064x2208
+// take 0.68 to 0.95 of the time (mean 0.82), 1832x1920 with 5 kernel rows 0.67 to 1.23 (0.84; three
+// seeds above 1), through the buffer 1832x1920 0.58 to 0.98 (2 and 4 px per cell: 0.81 and
+// 0.72), 2064x2208 0.63 to 1.10 (0.81 and 0.88; one seed each above 1).
 static int balanced_band(int h, int halo, int bmax, int sms)
 {
     int best = 1;
@@ -1381,8 +1385,10 @@ cudaError_t fused_launch(const FrameArgs& f, const FusedLimits& lim, int two_per
     const size_t smem = fused_smem_bytes(wpad, f.band, f.halo);
     const bool var = f.halo != 1 || f.nearest != 0;  // a Patcher variant: its own instantiation
     const int nbands = (f.h + f.band - 1) / f.band;
-    const int slots = lim.sms * (two_per_sm ? 2 : 1);
-    const int grid = nbands < slots ? nbands : slots;
+    // One CTA per band, as in the other band kernels: the hardware deals the later waves' bands to
+    // whichever SM is free.  Striding over the bands left a slow band's CTA with its next one
+    // (2064x2208, 24 seeds: mean 45.3 -> 42.6 us, one seed 48.1 -> 38.3).
+    const int grid = nbands;
     if (f.zt_out && var) return cudaErrorInvalidValue;  // the depth output exists for the default kernel
     const bool wide = (f.w + 31) / 32 > 2 * (kBig / 32);  // wider than 2 words per warp
     auto go = [&](auto kernel, int threads) {
