@@ -647,7 +647,7 @@ def run_inpaint(args):
                      "frac": round(tflops / peak, 4), "peak_source": "MEASURED_PEAKS.json bf16_tflops (burst)",
                      "traffic": None,
                      "traffic_note": "the network is 14 convolution launches and small kernels; DRAM bytes per "
-                                     "convolution launch are in profiles/conv3x3_rows_inpaint_304tiles.md"},
+                                     "convolution launch are in profiles/conv3x3_network.md"},
         "frame_path_ms": {"p50": round(lat[len(lat) // 2], 3), "p99": round(lat[int(0.99 * (len(lat) - 1))], 3),
                           "what": "yoro_synthesize_zt + yoro_unet_inpaint on one 1832x1920 frame (hole tiles only)"},
     }), flush=True)

@@ -9,7 +9,8 @@
 // side, so the lanes of an accumulator are the same pixels of every row), the accumulators
 // of R rows lie next to each other in tensor memory, and input row r is multiplied once
 // with the weights of taps dy = 0, 1, 2 (N = 3 Cout) into the accumulators of rows r + 1, r,
-// r - 1 (later rows lie in lower columns): 56 cycles where three MMAs took 164 (N = 96), 96 where they took 164 (N = 192).
+// r - 1 (later rows lie in lower columns): 56 cycles where three MMAs took 164 (N = 96), 96
+// where they took 164 (N = 192).
 //
 // The kernel columns share the copy of a row as well: tap dx reads the same shared-memory
 // row from a start one pixel (64 bytes) to the left or right (the swizzle is a function
@@ -31,11 +32,14 @@
 //
 // The issuing warp runs its loop as a whole (one lane elected per instruction): in uniform
 // control flow the descriptors are built in uniform registers, where a single-lane branch
-// cost about 100 more cycles per MMA (dec0a below 337 us).
+// cost about 100 more cycles per MMA (155 against 56 at N = 96).
 //
-// Measured, 870 tiles, halo form -> row form, us: enc0a 143 -> 83, enc0b 144 -> 106, enc1a 51
-// -> 34, enc1b 78 -> 50, dec1a 166 -> 129, dec1b 141 -> 118, dec0a 305 -> 174, dec0b 152 -> 83
-// (dec0b moves 456 MB: 67 us at the measured copy bandwidth).
+// Measured, 870 tiles, halo form -> row form as the network runs it, us: enc0a 143 -> 71, enc0b
+// 144 -> 83 (with the pooling), enc1a 51 -> 33, enc1b 78 -> 49 (with the pooling), dec1a 166 ->
+// 137 and dec0a 305 -> 186 (half-resolution input), dec1b 141 -> 46 (stored at its own
+// resolution), dec0b 152 -> 95 (with the output layer).  enc0a moves its 405 MB at 5.7 TB/s;
+// dec0a keeps the tensor pipe 43 % and shared memory 57 % busy, dec1a 59 and 59 % (304 tiles):
+// neither unit is full, the one CTA's roles wait on one another.
 #include <algorithm>
 #include <cmath>
 
